@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "lgf_fixed.cuh"
 #include "lgf_internal.h"
 
 namespace lgf {
@@ -181,6 +182,151 @@ __device__ __forceinline__ R delta_norm2(R a0, R a1, R a2, C2<R> d01, C2<R> d02,
   return fma((R)2, off, dia);
 }
 
+// Divergence of one site: the sums over its eight links that Delta is made of
+// (W = sum_mu [U_mu(x - mu^) - U_mu(x)]: Im W_ii and W_ij - conj(W_ji)) and
+// the Re Tr sum of its forward links, in FP64.
+struct SiteDiv {
+  double f, im0, im1, im2;
+  double2 w01, w02, w12;
+};
+
+// In the link precision (FP64 sum over mu of each link's trace).
+template <typename R, int ROWS>
+__device__ __forceinline__ void site_divergence(const Geom& g, const MatField<R, ROWS>& U, int64_t s, const int c[4],
+                                                double& fsum, R& im0, R& im1, R& im2, C2<R>& w01, C2<R>& w02,
+                                                C2<R>& w12) {
+  fsum = 0;
+  im0 = im1 = im2 = 0;
+  w01 = w02 = w12 = mkc<R>(0, 0);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    M3<R> u;
+    U.load_ro(mu, s, u);
+    fsum += (double)(u.e[0][0].x + u.e[1][1].x + u.e[2][2].x);
+    im0 -= u.e[0][0].y; im1 -= u.e[1][1].y; im2 -= u.e[2][2].y;
+    w01 = csub<R>(w01, csub<R>(u.e[0][1], cconj<R>(u.e[1][0])));
+    w02 = csub<R>(w02, csub<R>(u.e[0][2], cconj<R>(u.e[2][0])));
+    w12 = csub<R>(w12, csub<R>(u.e[1][2], cconj<R>(u.e[2][1])));
+    M3<R> b;
+    U.load_ro(mu, site_back(g, s, c, mu), b);
+    im0 += b.e[0][0].y; im1 += b.e[1][1].y; im2 += b.e[2][2].y;
+    w01 = cadd<R>(w01, csub<R>(b.e[0][1], cconj<R>(b.e[1][0])));
+    w02 = cadd<R>(w02, csub<R>(b.e[0][2], cconj<R>(b.e[2][0])));
+    w12 = cadd<R>(w12, csub<R>(b.e[1][2], cconj<R>(b.e[2][1])));
+  }
+}
+
+// The FP64 path of links outside the fixed-point range.
+template <int ROWS>
+__device__ __noinline__ void site_divergence_fp64(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                                  SiteDiv& o) {
+  int c[4];
+  site_coords(g, s, c);
+  site_divergence<double, ROWS>(g, U, s, c, o.f, o.im0, o.im1, o.im2, o.w01, o.w02, o.w12);
+}
+
+// FP64 links, summed in 64-bit fixed point (unit 2^-58) on the integer pipe:
+// 132 entries of eight links enter the sums, exactly but for what lies below
+// 2^-58 in an entry, against one FP64 rounding per addition (2^-54 for sums
+// of order one).  12-real links rebuild row 3 in fixed point as well.
+// Where the anti-symmetric real parts of all eight links are below 2^-12 (a
+// field near the identity), FP64 sums are relative to numbers that small and
+// round finer than 2^-58: that site takes the FP64 path, as do entries
+// outside the fixed-point range.
+// Bound by the ALU pipe (65 % busy in ncu) beside HBM (41 %).  32^4: 18-real
+// 195 us (FP64 sums on the FP64 pipe: 355 us), 12-real 314 us (665 us).
+template <int ROWS>
+__device__ __forceinline__ void site_divergence_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                                   const int c[4], SiteDiv& o) {
+  int64_t f = 0, i0 = 0, i1 = 0, i2 = 0, x01 = 0, y01 = 0, x02 = 0, y02 = 0, x12 = 0, y12 = 0;
+  uint32_t m = 0, t = 0, w = 0;
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    const int mu = k >> 1;
+    int64_t sf, sb;
+    site_nbrs_sel(g, s, c, mu, sf, sb);
+    const bool fwd = (k & 1) == 0;  // the site's own link, else the one that ends in it
+    const int64_t sl = fwd ? s : sb;
+    double2 e[3][3];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        e[r][j] = __ldg(&U.p[U.off(mu, r, j, sl)]);
+        m = fx_max(m, e[r][j]);
+      }
+    int64_t f00, f11, f22, d0, d1, d2, ax, ay, bx, by, cx, cy;
+    d0 = fx58_from(e[0][0].y);
+    d1 = fx58_from(e[1][1].y);
+    if (ROWS == 3) {
+      f00 = f11 = f22 = 0;
+      if (fwd) {
+        f00 = fx58_from(e[0][0].x);
+        f11 = fx58_from(e[1][1].x);
+        f22 = fx58_from(e[2][2].x);
+      }
+      d2 = fx58_from(e[2][2].y);
+      ax = fx58_from(e[0][1].x) - fx58_from(e[1][0].x);
+      ay = fx58_from(e[0][1].y) + fx58_from(e[1][0].y);
+      bx = fx58_from(e[0][2].x) - fx58_from(e[2][0].x);
+      by = fx58_from(e[0][2].y) + fx58_from(e[2][0].y);
+      cx = fx58_from(e[1][2].x) - fx58_from(e[2][1].x);
+      cy = fx58_from(e[1][2].y) + fx58_from(e[2][1].y);
+    } else {
+      int64_t q[2][3][2];
+      FxC w[2][3];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          q[r][j][0] = fx58_from(e[r][j].x);
+          q[r][j][1] = fx58_from(e[r][j].y);
+          w[r][j] = FxC{fx_operand58(q[r][j][0]), fx_operand58(q[r][j][1])};
+        }
+      int64_t z[3][2];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        FxAcc re = fx_zero(), im = fx_zero();
+        fx_cross_conj(re, im, w[0][(j + 1) % 3], w[0][(j + 2) % 3], w[1][(j + 1) % 3], w[1][(j + 2) % 3]);
+        z[j][0] = fx_sum60(re, t) >> 2;
+        z[j][1] = fx_sum60(im, t) >> 2;
+      }
+      f00 = fwd ? q[0][0][0] : 0;
+      f11 = fwd ? q[1][1][0] : 0;
+      f22 = fwd ? z[2][0] : 0;
+      d2 = z[2][1];
+      ax = q[0][1][0] - q[1][0][0];
+      ay = q[0][1][1] + q[1][0][1];
+      bx = q[0][2][0] - z[0][0];
+      by = q[0][2][1] + z[0][1];
+      cx = q[1][2][0] - z[1][0];
+      cy = q[1][2][1] + z[1][1];
+    }
+    w |= (uint32_t)(ax >> 32) ^ (uint32_t)(ax >> 63);
+    w |= (uint32_t)(bx >> 32) ^ (uint32_t)(bx >> 63);
+    w |= (uint32_t)(cx >> 32) ^ (uint32_t)(cx >> 63);
+    if (fwd) {
+      f += f00 + f11 + f22;
+      i0 -= d0; i1 -= d1; i2 -= d2;
+      x01 -= ax; y01 -= ay; x02 -= bx; y02 -= by; x12 -= cx; y12 -= cy;
+    } else {
+      i0 += d0; i1 += d1; i2 += d2;
+      x01 += ax; y01 += ay; x02 += bx; y02 += by; x12 += cx; y12 += cy;
+    }
+  }
+  if (fx_bad(m, t) || w < (1u << (58 - 12 - 32))) {
+    site_divergence_fp64<ROWS>(g, U, s, o);
+    return;
+  }
+  o.f = fx_to_double_fp<58>(f);
+  o.im0 = fx_to_double_fp<58>(i0);
+  o.im1 = fx_to_double_fp<58>(i1);
+  o.im2 = fx_to_double_fp<58>(i2);
+  o.w01 = make_double2(fx_to_double_fp<58>(x01), fx_to_double_fp<58>(y01));
+  o.w02 = make_double2(fx_to_double_fp<58>(x02), fx_to_double_fp<58>(y02));
+  o.w12 = make_double2(fx_to_double_fp<58>(x12), fx_to_double_fp<58>(y12));
+}
+
 template <typename R, int ROWS>
 __global__ void __launch_bounds__(MEASURE_THREADS)
 measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt, C2<R>* __restrict__ delta,
@@ -206,23 +352,16 @@ measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt,
     site_coords(g, s, c);
     // W = sum_mu [U_mu(x - mu^) - U_mu(x)]; only the entries that enter its
     // traceless anti-Hermitian part are accumulated.
-    R im0 = 0, im1 = 0, im2 = 0;           // Im W_ii
-    C2<R> w01 = mkc<R>(0, 0), w02 = mkc<R>(0, 0), w12 = mkc<R>(0, 0);  // W_ij - conj(W_ji)
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      M3<R> u;
-      U.load_ro(mu, s, u);
-      fsum += (double)(u.e[0][0].x + u.e[1][1].x + u.e[2][2].x);
-      im0 -= u.e[0][0].y; im1 -= u.e[1][1].y; im2 -= u.e[2][2].y;
-      w01 = csub<R>(w01, csub<R>(u.e[0][1], cconj<R>(u.e[1][0])));
-      w02 = csub<R>(w02, csub<R>(u.e[0][2], cconj<R>(u.e[2][0])));
-      w12 = csub<R>(w12, csub<R>(u.e[1][2], cconj<R>(u.e[2][1])));
-      M3<R> b;
-      U.load_ro(mu, site_back(g, s, c, mu), b);
-      im0 += b.e[0][0].y; im1 += b.e[1][1].y; im2 += b.e[2][2].y;
-      w01 = cadd<R>(w01, csub<R>(b.e[0][1], cconj<R>(b.e[1][0])));
-      w02 = cadd<R>(w02, csub<R>(b.e[0][2], cconj<R>(b.e[2][0])));
-      w12 = cadd<R>(w12, csub<R>(b.e[1][2], cconj<R>(b.e[2][1])));
+    R im0, im1, im2;           // Im W_ii
+    C2<R> w01, w02, w12;       // W_ij - conj(W_ji)
+    if constexpr (sizeof(R) == sizeof(double)) {
+      SiteDiv o;
+      site_divergence_fx<ROWS>(g, U, s, c, o);
+      fsum = o.f;
+      im0 = o.im0; im1 = o.im1; im2 = o.im2;
+      w01 = o.w01; w02 = o.w02; w12 = o.w12;
+    } else {
+      site_divergence<R, ROWS>(g, U, s, c, fsum, im0, im1, im2, w01, w02, w12);
     }
     const R tr = (im0 + im1 + im2) * (R)(1.0 / 3.0);
     const R a0 = im0 - tr, a1 = im1 - tr, a2 = im2 - tr;
@@ -434,12 +573,150 @@ update_kernel(Geom g, MatField<R, LROWS> U, MatField<R, GROWS> Gf, Batch B) {
   }
 }
 
+// The FP64 path of one link outside the fixed-point range.
+template <int LROWS>
+__device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatField<double, 3> Gf, int mu, int64_t s,
+                                              int64_t sf) {
+  M3<double> gx, u, h, o;
+  Gf.load_ro(0, s, gx);
+  U.load(mu, s, u);
+  Gf.load_ro(0, sf, h);
+  gauge_product<double>(gx, u, h, o);
+  U.store(mu, s, o);
+}
+
+// FP64 links: the two products in fixed point on the integer pipe
+// (lgf_fixed.cuh), row 3 of 18-real links on the FP64 pipe beside it.
+// Links whose off-diagonal entries are all below 2^-12, where FP64 rounds
+// finer than the fixed-point unit, and entries outside its range take the
+// FP64 path.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
+// end at 2.4e-15 (FP64 products: 2.6e-15).
+// Bound by instruction issue (9300 per site, 12 warps per SM at 168
+// registers).  32^4: 18-real 518 us, 12-real 626 us; with FP64 products 1176
+// and 1177 us at 95 % of the FP64 pipe.
+template <int LROWS>
+__global__ void __launch_bounds__(UPDATE_THREADS)
+update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batch B) {
+  if (batch_skip(B)) return;
+  U.p += blockIdx.z * B.s_links;
+  Gf.p += blockIdx.z * B.s_g;
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  int c[4];
+  site_coords(g, s, c);
+  uint32_t mg = 0;
+  FxC gx[2][3];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const double2 v = __ldg(&Gf.p[Gf.off(0, i, j, s)]);
+      mg = fx_max(mg, v);
+      gx[i][j] = fx_from(v);
+    }
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    int64_t sf, sb;
+    site_nbrs_sel(g, s, c, mu, sf, sb);
+    double2 u[LROWS][3], h[3][3];
+#pragma unroll
+    for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) u[i][j] = U.p[U.off(mu, i, j, s)];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) h[i][j] = __ldg(&Gf.p[Gf.off(0, i, j, sf)]);
+    uint32_t m = mg, t = 0;
+#pragma unroll
+    for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) m = fx_max(m, u[i][j]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) m = fx_max(m, h[i][j]);
+    uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
+    // T = g(x)[rows 0,1] U
+    FxC T[2][3];
+    FxC ux[3][3];
+#pragma unroll
+    for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) ux[i][j] = fx_from(u[i][j]);
+    if (LROWS == 2) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        FxAcc re = fx_zero(), im = fx_zero();
+        fx_cross_conj(re, im, ux[0][(j + 1) % 3], ux[0][(j + 2) % 3], ux[1][(j + 1) % 3], ux[1][(j + 2) % 3]);
+        ux[2][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fx_cmac(re, im, gx[i][k], fx_neg(gx[i][k].y), ux[k][j]);
+        T[i][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+      }
+    // rows 0,1 of T h^dagger
+    int64_t n[2][3][2];
+    bool big = true;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      FxC hj[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) hj[k] = fx_from(h[j][k]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fx_cmacc(re, im, T[i][k], fx_neg(T[i][k].x), hj[k]);
+        n[i][j][0] = fx_sum60(re, t);
+        n[i][j][1] = fx_sum60(im, t);
+      }
+    }
+    if (fx_bad(m, t) || w < FX_WEAK_HI) {
+      update_link_fp64<LROWS>(U, Gf, mu, s, sf);
+      continue;
+    }
+    double2 o[3][3];
+    if (LROWS == 3) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          o[i][j] = make_double2(fx_to_double_int<60>(n[i][j][0], big), fx_to_double_int<60>(n[i][j][1], big));
+    }
+    if (LROWS == 2 || !big) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          o[i][j] = make_double2(fx_to_double_fp<60>(n[i][j][0]), fx_to_double_fp<60>(n[i][j][1]));
+    }
+    if (LROWS == 3) su3_third_row<double>(o[0], o[1], o[2]);
+#pragma unroll
+    for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) U.p[U.off(mu, i, j, s)] = o[i][j];
+  }
+}
+
 template <typename R, int LROWS, int GROWS>
 cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cudaStream_t s, const Batch& B) {
   MatField<R, LROWS> U{links, g.V};
   MatField<R, GROWS> Gf{const_cast<C2<R>*>(gfield), g.V};
   const int64_t nb = (g.V + UPDATE_THREADS - 1) / UPDATE_THREADS;
-  update_kernel<R, LROWS, GROWS><<<dim3((unsigned)nb, 1, (unsigned)B.n), UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
+  const dim3 grid((unsigned)nb, 1, (unsigned)B.n);
+  if constexpr (sizeof(R) == sizeof(double)) {
+    static_assert(GROWS == 3, "FP64 lanes keep three rows of g");
+    update_fx_kernel<LROWS><<<grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
+  } else {
+    update_kernel<R, LROWS, GROWS><<<grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
+  }
   return cudaGetLastError();
 }
 

@@ -1,0 +1,93 @@
+"""The fixed-point forms of the FP64 kernels against the FP64 oracle, where
+they can go wrong: entries of exactly 0, 1, -1 and i, entries far below the
+fixed-point unit, lattices that do not fill a CTA, and values outside the
+fixed-point range (an infinite step), which take the FP64 path.
+
+Tolerances: a link of the update is two sums of three complex products and
+one FP64 rounding of entries of order one, 2^-53 + a few 2^-58 against the
+oracle's own 2^-53 per operation: 2e-15 covers both.  A divergence entry adds
+16 link entries: 4e-15.
+"""
+
+import numpy as np
+import pytest
+
+from oracle import lgf_oracle as O
+from paper_1206_0675_gb300 import fields, lgf
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _library():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    lgf.load_library()
+
+
+def permutation_links(ext, seed):
+    """Links with one entry of 1, -1, i or -i per row and column, determinant 1."""
+    rng = np.random.default_rng(seed)
+    lx, ly, lz, lt = ext
+    shape = (4, lt, lz, ly, lx)
+    U = np.zeros(shape + (3, 3), dtype=np.complex128)
+    perms = np.array([(0, 1, 2), (1, 2, 0), (2, 0, 1), (0, 2, 1), (1, 0, 2), (2, 1, 0)])
+    p = perms[rng.integers(0, 6, shape)]
+    ph = rng.integers(0, 4, shape + (3,))
+    odd = np.isin(np.arange(6), (3, 4, 5))[(p[..., None, :] == perms).all(-1).argmax(-1)]
+    ph[..., 2] = (-ph[..., 0] - ph[..., 1] + 2 * odd) % 4
+    vals = np.array([1, 1j, -1, -1j])[ph]
+    for r in range(3):
+        np.put_along_axis(U[..., r, :], p[..., r:r + 1], vals[..., r:r + 1], axis=-1)
+    return U
+
+
+def rebuilt(U):
+    """Row 3 from rows 1-2, (a x b)^*: what 12-real storage holds, and the row 3 of every updated link."""
+    V = U.copy()
+    V[..., 2, :] = np.conj(np.cross(U[..., 0, :], U[..., 1, :]))
+    return V
+
+
+def weak_links(ext, eps):
+    return fields.random_links(ext, eps, seed=4, gauge_rotate=False)
+
+
+CASES = {
+    "permutations": lambda ext: permutation_links(ext, 1),
+    "weak 1e-3": lambda ext: weak_links(ext, 1e-3),
+    "weak 1e-9": lambda ext: weak_links(ext, 1e-9),
+    "weak 1e-19": lambda ext: weak_links(ext, 1e-19),
+    "random": lambda ext: fields.random_links(ext, 0.9, seed=3),
+}
+
+
+@pytest.mark.parametrize("store12", [False, True])
+@pytest.mark.parametrize("name", list(CASES))
+@pytest.mark.parametrize("ext", [(2, 2, 2, 2), (3, 4, 6, 9), (8, 8, 4, 2)])
+def test_measure_and_step_against_oracle(ext, name, store12):
+    U = CASES[name](ext)
+    Us = rebuilt(U) if store12 else U
+    Fo, tho, Do = O.measure(Us)
+    with lgf.Lattice(ext, "fp64", store12=store12) as lat:
+        lat.set_links(U)
+        F, th = lat.measure()
+        D = lat.get_divergence()
+        lat.step(0.08)
+        g = lat.get_gauge()
+        U1 = lat.get_links()
+    assert np.max(np.abs(D - Do)) < 4e-15
+    assert abs(F - Fo) < 4e-15
+    assert abs(th - tho) < 1e-13 * tho
+    assert np.max(np.abs(U1 - rebuilt(O.apply_gauge(Us, g)))) < 2e-15
+
+
+@pytest.mark.parametrize("store12", [False, True])
+def test_infinite_step_is_reported(store12):
+    ext = (4, 4, 4, 4)
+    with lgf.Lattice(ext, "fp64", store12=store12) as lat:
+        lat.set_links(fields.random_links(ext, 0.9, seed=3))
+        lat.step(1e308)
+        with pytest.raises(lgf.LgfError) as e:
+            lat.measure()
+        assert e.value.status == lgf.LGF_E_NONFINITE
