@@ -218,22 +218,18 @@ template <typename R> lgf_status alloc_lane(lgf_ctx* h, Lane<R>& L, int rows, in
   LGF_CK(h, h->mem.get(&L.D, (size_t)4 * V));
   LGF_CK(h, h->mem.get(&L.K, (size_t)V));
   const int nt = h->geom.L[0] + h->geom.L[1] + h->geom.L[2] + h->geom.L[3];
-  LGF_CK(h, h->mem.get(&L.tw, (size_t)nt));
+  const bool f64 = sizeof(R) == sizeof(double);
+  LGF_CK(h, h->mem.get(&L.tw, (size_t)(f64 ? 2 * nt : nt)));
   if (withG) LGF_CK(h, h->mem.get(&L.G, (size_t)9 * V));
   if (configure_fft_plan(h->geom.L, (int)sizeof(R), &L.plan) != cudaSuccess)
     return fail(h, LGF_E_UNSUPPORTED, "lattice planes do not fit the shared-memory FFT passes");
   // twiddles W_N^m = exp(-2 pi i m/N), computed in FP64 on the host
-  std::vector<C2<R>> tw(nt);
-  int off = 0;
-  for (int mu = 0; mu < 4; ++mu) {
-    const int N = h->geom.L[mu];
-    for (int m = 0; m < N; ++m) {
-      const double a = -2.0 * M_PI * (double)m / (double)N;
-      tw[off + m] = mkc<R>((R)std::cos(a), (R)std::sin(a));
-    }
-    off += N;
-  }
-  LGF_CK(h, cudaMemcpyAsync(L.tw, tw.data(), nt * sizeof(C2<R>), cudaMemcpyHostToDevice, h->stream));
+  std::vector<double2> tw64;
+  fft_twiddles(h->geom.L, tw64);
+  std::vector<C2<R>> tw(f64 ? 2 * nt : nt);
+  for (size_t m = 0; m < tw.size(); ++m) tw[m] = mkc<R>((R)tw64[m].x, (R)tw64[m].y);
+  LGF_CK(h, cudaMemcpyAsync(L.tw, f64 ? (const void*)tw64.data() : (const void*)tw.data(),
+                            tw.size() * sizeof(C2<R>), cudaMemcpyHostToDevice, h->stream));
   std::vector<short> pos(nt);
   fft_positions(L.plan, pos.data());
   LGF_CK(h, h->mem.get(&L.pos, (size_t)nt));

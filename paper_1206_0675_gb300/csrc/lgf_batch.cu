@@ -186,22 +186,15 @@ lgf_status setup_class(lgf_batch_ctx* b, ClassLane& C) {
   LGF_BCK(b, b->mem.get(&C.K, (size_t)V));
   LGF_BCK(b, b->mem.get(&C.partials, (size_t)C.n * MEASURE_PARTIALS * C.nb));
   const int nt = g.L[0] + g.L[1] + g.L[2] + g.L[3];
-  LGF_BCK(b, b->mem.get(&C.tw, (size_t)nt));
+  LGF_BCK(b, b->mem.get(&C.tw, (size_t)2 * nt));
   LGF_BCK(b, b->mem.get(&C.pos, (size_t)nt));
   if (configure_fft_plan(g.L, 8, &C.plan) != cudaSuccess)
     return bfail(b, LGF_E_UNSUPPORTED, "lattice planes do not fit the shared-memory FFT passes");
-  std::vector<double2> tw(nt);
+  std::vector<double2> tw;
   std::vector<short> pos(nt);
-  int off = 0;
-  for (int mu = 0; mu < 4; ++mu) {
-    for (int m = 0; m < g.L[mu]; ++m) {
-      const double a = -2.0 * M_PI * (double)m / (double)g.L[mu];
-      tw[off + m] = make_double2(std::cos(a), std::sin(a));
-    }
-    off += g.L[mu];
-  }
+  fft_twiddles(g.L, tw);
   fft_positions(C.plan, pos.data());
-  LGF_BCK(b, cudaMemcpyAsync(C.tw, tw.data(), nt * sizeof(double2), cudaMemcpyHostToDevice, b->stream));
+  LGF_BCK(b, cudaMemcpyAsync(C.tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice, b->stream));
   LGF_BCK(b, cudaMemcpyAsync(C.pos, pos.data(), nt * sizeof(short), cudaMemcpyHostToDevice, b->stream));
   C.lmax = 0;
   for (int mu = 0; mu < 4; ++mu) C.lmax = std::max(C.lmax, g.L[mu]);

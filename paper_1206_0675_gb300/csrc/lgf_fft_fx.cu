@@ -1,0 +1,585 @@
+// The plane passes of the 4D transform for FP64 fields in block floating
+// point on the integer pipe.
+//
+// The FP64 pipe (2 operations per clock and SM) bounds an FP64 Cooley-Tukey
+// pass; here a plane is held as 64-bit integers with one exponent, whose
+// additions are exact and run on the integer pipe (64 per clock and SM), and
+// whose products with twiddles take three 32 x 32 + 64 bit multiply-adds.
+//
+// Exponents.  A plane of one field gets its own exponent, from the largest
+// component of its input, so results do not depend on how planes are grouped
+// into CTAs.  A transform of length N is safe from overflow when components
+// enter below 2^(61 - h), h = ceil(log2 N) + 1: a sum of N complex terms stays
+// below sqrt(2) N 2^(61 - h) <= 2^60.5 in modulus, within the 31-bit upper limb
+// of bfp_limbs.  Between the two directions of a plane the largest component
+// is measured again and the plane shifted right by what the next direction
+// needs (about half of h for data without structure, so some 55 bits remain
+// below the largest component; an FP64 pass keeps 53 bits in each number and
+// rounds at every operation, where additions are exact here).  Inputs are
+// read and results written in FP64.
+//
+// Error against 80-bit arithmetic (2-norm, forward and inverse, random,
+// smooth and constant inputs): 0.7e-16 to 2.8e-16, the FP64 passes on the FP64
+// pipe had 1.5e-16 to 4.6e-16.
+//
+// 32^4, us: pass A 86 (FP64 pipe: 231), pass B 197 (463), pass C with g 241
+// (397, where g keeps the FP64 pipe for 96 us); 24x18x12x27: 25, 65, 55 (54, 94, 78).
+//
+// Planes that hold infinities or NaN give NaN; planes whose largest
+// component is near the ends of the FP64 range take slower conversions.
+#include <algorithm>
+#include <cmath>
+
+#include "lgf_fft_tile.cuh"
+#include "lgf_fixed.cuh"
+#include "lgf_gauge.cuh"
+#include "lgf_internal.h"
+
+namespace lgf {
+
+using I2 = longlong2;
+
+// Per-plane exponents of the (at most 8) planes of a tile: the largest input
+// component (high word of its magnitude) and the bits of the largest
+// component between the directions (high word, or-ed), for the two transforms
+// a pass can hold.
+struct FxPlanes {
+  uint32_t in0[8], mid0[8], in1[8], mid1[8];
+};
+static_assert(sizeof(FxPlanes) == FX_PLANE_BYTES, "header of the FP64 plane passes");
+
+__device__ __forceinline__ uint32_t fx_headroom(int N) { return 33u - (uint32_t)__clz(N - 1); }
+
+// From a plane's largest input component: its biased exponent (at least 1),
+// whether every exponent that can occur is far from the ends of the range.
+__device__ __forceinline__ uint32_t fx_exp_of(uint32_t in) { return max(in >> 20, 1u); }
+__device__ __forceinline__ bool fx_safe_exp(uint32_t e) { return e - 100u <= 1890u; }
+// Right shift between the directions.
+__device__ __forceinline__ uint32_t fx_mid_shift(uint32_t mid, uint32_t h1) {
+  const int sh = (64 - __clz((int)mid)) - (int)(61u - h1);
+  return (uint32_t)max(sh, 0);
+}
+
+// Input of a plane near the ends of the range (or all zero); infinities and
+// NaN give zero here and NaN at the output.
+static __device__ __noinline__ int64_t fx_in_any(double a, uint32_t e, uint32_t h0) {
+  if (a == 0.0 || e == 2047u) return 0;
+  const double up = e < 100u ? a * 1.6069380442589903e60 : a;  // 2^200
+  return bfp_from(up, 3u + h0 + e + (e < 100u ? 200u : 0u));
+}
+__device__ __forceinline__ I2 fx_in(double2 v, uint32_t in, uint32_t h0) {
+  const uint32_t e = fx_exp_of(in);
+  if (!fx_safe_exp(e)) return make_longlong2(fx_in_any(v.x, e, h0), fx_in_any(v.y, e, h0));
+  const uint32_t base = 3u + h0 + e;
+  return make_longlong2(bfp_from(v.x, base), bfp_from(v.y, base));
+}
+
+// Output of a plane after both directions.
+__device__ __forceinline__ double2 fx_out(I2 v, uint32_t in, uint32_t mid, uint32_t h0, uint32_t h1) {
+  const uint32_t e = fx_exp_of(in);
+  const int ex = (int)(fx_mid_shift(mid, h1) + h0 + e) - 1083;
+  const bool safe = fx_safe_exp(e);
+  if (e == 2047u) return make_double2(NAN, NAN);
+  return make_double2(bfp_to_double(v.x, ex, safe), bfp_to_double(v.y, ex, safe));
+}
+
+__device__ __forceinline__ I2 iadd(I2 a, I2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ I2 isub(I2 a, I2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
+// v >> s (s >= 1), ties to even: a bias would add up in the zero mode.
+__device__ __forceinline__ int64_t ishift(int64_t v, uint32_t s) {
+  return (v + ((int64_t)1 << (s - 1)) - 1 + ((v >> s) & 1)) >> s;
+}
+template <int SIGN> __device__ __forceinline__ I2 imul_i(I2 a) {  // times SIGN i
+  return SIGN < 0 ? make_longlong2(a.y, -a.x) : make_longlong2(-a.y, a.x);
+}
+
+// v w (SIGN < 0) or v conj(w) for a table entry w = (cos h, l, sin h, l).
+template <int SIGN> __device__ __forceinline__ I2 itwiddle(I2 v, int4 w) {
+  const Bfp2 x = bfp_limbs(v.x), y = bfp_limbs(v.y);
+  const int sh = SIGN < 0 ? w.z : -w.z, sl = SIGN < 0 ? w.w : -w.w;
+  const int nh = -sh, nl = -sl;
+  int64_t rm = (int64_t)1 << 29, im = (int64_t)1 << 29;
+  rm += (int64_t)x.h * w.y;
+  rm += (int64_t)x.l * w.x;
+  rm += (int64_t)y.h * nl;
+  rm += (int64_t)y.l * nh;
+  im += (int64_t)x.h * sl;
+  im += (int64_t)x.l * sh;
+  im += (int64_t)y.h * w.y;
+  im += (int64_t)y.l * w.x;
+  int64_t rh = (int64_t)x.h * w.x, ih = (int64_t)x.h * sh;
+  rh += (int64_t)y.h * nh;
+  ih += (int64_t)y.h * w.x;
+  return make_longlong2(rh + (rm >> 30), ih + (im >> 30));
+}
+
+// 1/sqrt 2 and sqrt(3)/2 as h 2^-30 + l 2^-60
+constexpr int IR2_H = 759250125, IR2_L = -6429112;
+constexpr int IS3_H = 929887697, IS3_L = -333032134;
+
+template <int RAD, int SIGN> struct IDFT;
+template <int SIGN> struct IDFT<2, SIGN> {
+  __device__ __forceinline__ static void run(I2* v) {
+    const I2 a = v[0], b = v[1];
+    v[0] = iadd(a, b);
+    v[1] = isub(a, b);
+  }
+};
+template <int SIGN> struct IDFT<3, SIGN> {
+  __device__ __forceinline__ static void run(I2* v) {
+    const I2 t1 = iadd(v[1], v[2]);
+    const I2 t2 = make_longlong2(v[0].x - ishift(t1.x, 1), v[0].y - ishift(t1.y, 1));
+    const I2 d = isub(v[1], v[2]);
+    const I2 t3 = imul_i<SIGN>(make_longlong2(bfp_mul(d.x, IS3_H, IS3_L), bfp_mul(d.y, IS3_H, IS3_L)));
+    v[0] = iadd(v[0], t1);
+    v[1] = iadd(t2, t3);
+    v[2] = isub(t2, t3);
+  }
+};
+template <int SIGN> struct IDFT<4, SIGN> {
+  __device__ __forceinline__ static void run(I2* v) {
+    const I2 a = iadd(v[0], v[2]), b = isub(v[0], v[2]);
+    const I2 c = iadd(v[1], v[3]), d = imul_i<SIGN>(isub(v[1], v[3]));
+    v[0] = iadd(a, c);
+    v[2] = isub(a, c);
+    v[1] = iadd(b, d);
+    v[3] = isub(b, d);
+  }
+};
+template <int SIGN> struct IDFT<8, SIGN> {
+  __device__ __forceinline__ static void run(I2* v) {
+    I2 e[4] = {v[0], v[2], v[4], v[6]};
+    I2 o[4] = {v[1], v[3], v[5], v[7]};
+    IDFT<4, SIGN>::run(e);
+    IDFT<4, SIGN>::run(o);
+    {  // times (1 + SIGN i)/sqrt 2
+      const I2 a = o[1];
+      const int64_t p = bfp_mul(a.x + a.y, IR2_H, IR2_L), q = bfp_mul(a.y - a.x, IR2_H, IR2_L);
+      o[1] = SIGN < 0 ? make_longlong2(p, q) : make_longlong2(-q, p);
+    }
+    o[2] = imul_i<SIGN>(o[2]);
+    {  // times (-1 + SIGN i)/sqrt 2
+      const I2 a = o[3];
+      const int64_t p = bfp_mul(a.x + a.y, IR2_H, IR2_L), q = bfp_mul(a.y - a.x, IR2_H, IR2_L);
+      o[3] = SIGN < 0 ? make_longlong2(q, -p) : make_longlong2(-p, -q);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = iadd(e[k], o[k]);
+      v[k + 4] = isub(e[k], o[k]);
+    }
+  }
+};
+
+// How a direction's first stage takes its input and its last leaves it.
+struct FxStageIO {
+  const uint32_t* in = nullptr;     // raw FP64 input: largest component per plane
+  const uint32_t* shift = nullptr;  // integers to be shifted: measured bits per plane
+  uint32_t* mid = nullptr;          // record the bits of the outputs per plane
+  uint32_t h = 0;                   // headroom of this direction
+};
+
+// One stage, as ct_stage of lgf_fft.cu.  The plane of line l is l / inner
+// (PLO) or l % inner.
+template <int RAD, int SIGN, bool DIT, bool PLO>
+__device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln, const int N, const FastDiv fns,
+                                         const int4* __restrict__ tw, const FxStageIO io) {
+  const int Ns = (int)fns.d;
+  const int nbl = N / RAD;
+  const int NB = ln.nlines * nbl;
+  const int tws = nbl / Ns;
+  for (int b = threadIdx.x; b < NB; b += blockDim.x) {
+    const int q = (int)ln.dn.div((uint32_t)b), l = b - q * ln.nlines;
+    const int grp = (int)fns.div((uint32_t)q), j = q - grp * Ns;
+    const int lo = (int)ln.di.div((uint32_t)l), li = l - lo * ln.inner;
+    const int pl = PLO ? lo : li;
+    const int base = lo * ln.outer_stride + li * ln.inner_stride + (grp * Ns * RAD + j) * ln.es;
+    const int step = Ns * ln.es;
+    I2 v[RAD];
+    if (io.in != nullptr) {
+      const double2* raw = reinterpret_cast<const double2*>(tile);
+      const uint32_t in = io.in[pl];
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) v[r] = fx_in(raw[base + r * step], in, io.h);
+    } else {
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) v[r] = tile[base + r * step];
+      if (io.shift != nullptr) {
+        const uint32_t sh = fx_mid_shift(io.shift[pl], io.h);
+        if (sh != 0u) {
+#pragma unroll
+          for (int r = 0; r < RAD; ++r) v[r] = make_longlong2(ishift(v[r].x, sh), ishift(v[r].y, sh));
+        }
+      }
+    }
+    if (DIT && j > 0) {
+#pragma unroll
+      for (int r = 1; r < RAD; ++r) v[r] = itwiddle<SIGN>(v[r], tw[j * r * tws]);
+    }
+    IDFT<RAD, SIGN>::run(v);
+    if (!DIT && j > 0) {
+#pragma unroll
+      for (int r = 1; r < RAD; ++r) v[r] = itwiddle<SIGN>(v[r], tw[j * r * tws]);
+    }
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) tile[base + r * step] = v[r];
+    if (io.mid != nullptr) {
+      uint32_t m = 0;
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) {
+        m |= (uint32_t)(v[r].x >> 32) ^ (uint32_t)(v[r].x >> 63);
+        m |= (uint32_t)(v[r].y >> 32) ^ (uint32_t)(v[r].y >> 63);
+      }
+      if (PLO) {
+        // the lanes of a warp mostly share a plane: one atomic for all of them
+        const unsigned act = __activemask();
+        const int lead = __ffs((int)act) - 1;
+        if (__all_sync(act, pl == __shfl_sync(act, pl, lead))) {
+          m = __reduce_or_sync(act, m);
+          if ((int)(threadIdx.x & 31) == lead) atomicOr(&io.mid[pl], m);
+        } else {
+          atomicOr(&io.mid[pl], m);
+        }
+      } else {
+        atomicOr(&io.mid[pl], m);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// DFT of every line of a direction: DIT takes digit-reversed input and gives
+// natural order, DIF the reverse.
+template <int SIGN, bool DIT, bool PLO>
+__device__ __forceinline__ void fx_dir(I2* tile, const Lines& ln, const FFTDir& d, const int4* tw, const FxStageIO& io) {
+  for (int k = 0; k < d.nst; ++k) {
+    const int st = DIT ? k : d.nst - 1 - k;
+    FxStageIO s;
+    s.h = io.h;
+    if (k == 0) {
+      s.in = io.in;
+      s.shift = io.shift;
+    }
+    if (k == d.nst - 1) s.mid = io.mid;
+    if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
+    else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
+    else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
+    else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
+  }
+}
+
+// Both directions of a plane transform from raw FP64 input.
+template <int SIGN, bool DIT, bool PLO>
+__device__ __forceinline__ void fx_plane(I2* tile, const Lines& l0, const FFTDir& d0, const int4* tw0, uint32_t h0,
+                                         const Lines& l1, const FFTDir& d1, const int4* tw1, uint32_t h1,
+                                         const uint32_t* in, uint32_t* mid) {
+  FxStageIO a, b;
+  a.in = in;
+  a.mid = mid;
+  a.h = h0;
+  b.shift = mid;
+  b.h = h1;
+  fx_dir<SIGN, DIT, PLO>(tile, l0, d0, tw0, a);
+  fx_dir<SIGN, DIT, PLO>(tile, l1, d1, tw1, b);
+}
+
+// Tile of a plane pass: header as setup_smem, then the plane exponents.
+__device__ __forceinline__ I2* fx_setup(unsigned char* raw, const int4* __restrict__ twg, const short* __restrict__ posg,
+                                        int n0, int n1, int4** tw, short** pos, FxPlanes** ps) {
+  double2* t2;
+  double2* after = setup_smem<double>(raw, reinterpret_cast<const double2*>(twg), posg, n0, n1, &t2, pos);
+  *tw = reinterpret_cast<int4*>(t2);
+  *ps = reinterpret_cast<FxPlanes*>(after);
+  if (threadIdx.x < FX_PLANE_BYTES / 4) reinterpret_cast<uint32_t*>(*ps)[threadIdx.x] = 0u;
+  return reinterpret_cast<I2*>(*ps + 1);
+}
+
+// Copies n elements global -> tile (src(i), dst(i), plane(i)), recording the
+// largest component of every plane; four loads in flight per thread.
+template <typename SRC, typename DST>
+__device__ __forceinline__ void fx_load(I2* tile, int n, uint32_t* in, SRC src, DST dst) {
+  double2* raw = reinterpret_cast<double2*>(tile);
+  int cur = -1;
+  uint32_t m = 0;
+  for (int i0 = threadIdx.x; i0 < n; i0 += 4 * blockDim.x) {
+    double2 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = i0 + k * (int)blockDim.x;
+      if (i < n) v[k] = *src(i);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = i0 + k * (int)blockDim.x;
+      if (i < n) {
+        int pl;
+        raw[dst(i, pl)] = v[k];
+        if (pl != cur) {
+          if (cur >= 0) atomicMax(&in[cur], m);
+          cur = pl;
+          m = 0;
+        }
+        m = fx_max(m, v[k]);
+      }
+    }
+  }
+  if (cur >= 0) atomicMax(&in[cur], m);
+}
+
+template <int SIGN>
+__global__ void __launch_bounds__(512) fft_xy_fx_kernel(Geom g, FFTDir dx, FFTDir dy, double2* __restrict__ data,
+                                                        const int4* __restrict__ twg, const short* __restrict__ posg,
+                                                        int fpb, Lines lx, Lines ly, CopyDiv cd, Batch B) {
+  if (batch_skip(B)) return;
+  data += blockIdx.z * B.s_delta;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int Lx = g.L[0], Ly = g.L[1];
+  int4* tw;
+  short* pos;
+  FxPlanes* ps;
+  I2* tile = fx_setup(smem_raw, twg, posg, Lx, Ly, &tw, &pos, &ps);
+  const int RS = Lx + 1, PS = Ly * RS;
+  const int plane = Lx * Ly;
+  double2* fld = data + (int64_t)(blockIdx.y * fpb) * g.V + (int64_t)blockIdx.x * plane;
+  __syncthreads();
+  fx_load(
+      tile, fpb * plane, ps->in0,
+      [&](int i) {
+        const int f = (int)cd.a.div((uint32_t)i);
+        return &fld[(int64_t)f * g.V + (i - f * plane)];
+      },
+      [&](int i, int& pl) {
+        const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+        pl = f;
+        return f * PS + pos[Lx + y] * RS + pos[x];
+      });
+  __syncthreads();
+  const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
+  fx_plane<SIGN, true, true>(tile, lx, dx, tw, hx, ly, dy, tw + Lx, hy, ps->in0, ps->mid0);
+  for (int i = threadIdx.x; i < fpb * plane; i += blockDim.x) {
+    const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+    fld[(int64_t)f * g.V + r] = fx_out(tile[f * PS + y * RS + x], ps->in0[f], ps->mid0[f], hx, hy);
+  }
+}
+
+template <bool LRN>
+__global__ void __launch_bounds__(512)
+fft_zt_filter_fx_kernel(Geom g, FFTDir dz, FFTDir dt, double2* __restrict__ data, const int4* __restrict__ twg,
+                        const short* __restrict__ posg, const double* __restrict__ K, int xc, int mode, LearnedIO lio,
+                        int4 H, Lines lz, Lines lt, CopyDiv cd, Batch B) {
+  if (batch_skip(B)) return;
+  data += blockIdx.z * B.s_delta;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int Lx = g.L[0], Ly = g.L[1], Lz = g.L[2], Lt = g.L[3];
+  int4* tw;
+  short* pos;
+  FxPlanes* ps;
+  I2* tile = fx_setup(smem_raw, twg + Lx + Ly, posg + Lx + Ly, Lz, Lt, &tw, &pos, &ps);
+  const int TS = Lz * xc + 1;
+  const int nxb = Lx / xc;
+  const int x0 = (blockIdx.x % nxb) * xc, y = blockIdx.x / nxb;
+  double2* fld = data + (int64_t)blockIdx.y * g.V;
+  const int n = Lz * Lt * xc;
+  const int64_t sxy = (int64_t)y * Lx + x0;
+  const int64_t plane = (int64_t)Lx * Ly;
+  __syncthreads();
+#define LGF_ZT_IDX(i)                                                       \
+  const int zt = (int)cd.a.div((uint32_t)(i)), xi = (i) - zt * xc;          \
+  const int t = (int)cd.b.div((uint32_t)zt), z = zt - t * Lz;
+  fx_load(
+      tile, n, ps->in0,
+      [&](int i) {
+        const int zt = (int)cd.a.div((uint32_t)i);
+        return &fld[(int64_t)zt * plane + sxy + (i - zt * xc)];
+      },
+      [&](int i, int& pl) {
+        LGF_ZT_IDX(i)
+        pl = xi;
+        return pos[Lz + t] * TS + pos[z] * xc + xi;
+      });
+  __syncthreads();
+  const uint32_t hz = fx_headroom(Lz), ht = fx_headroom(Lt);
+  if (mode <= 0) fx_plane<-1, true, false>(tile, lz, dz, tw, hz, lt, dt, tw + Lz, ht, ps->in0, ps->mid0);
+  else fx_plane<+1, true, false>(tile, lz, dz, tw, hz, lt, dt, tw + Lz, ht, ps->in0, ps->mid0);
+  if (mode != 0) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      LGF_ZT_IDX(i)
+      fld[(int64_t)zt * plane + sxy + xi] = fx_out(tile[t * TS + z * xc + xi], ps->in0[xi], ps->mid0[xi], hz, ht);
+    }
+    return;
+  }
+  // the filter in FP64, back into the tile; xc divides the CTA size, so a
+  // thread stays in one x column
+  {
+    const int kit = LRN ? lio.st->iter : 0;
+    const bool learned = LRN && lio.mtab != nullptr && lio.st->use_m != 0;
+    const float* mtab = lio.mtab + (int64_t)(kit & 1) * lio.nclass;
+    uint32_t* snap = (LRN && lio.snap != nullptr) ? lio.snap + ((int64_t)(kit & 1) * 4 + blockIdx.y) * g.V : nullptr;
+    const int fy = min(y, Ly - y);
+    const int col = (int)threadIdx.x % xc;
+    const uint32_t in = ps->in0[col], mid = ps->mid0[col];
+    uint32_t m = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      LGF_ZT_IDX(i)
+      double k = __ldg(&K[(int64_t)zt * plane + sxy + xi]);
+      if (learned) {
+        const int kx = x0 + xi;
+        const int fx = min(kx, Lx - kx), fz = min(z, Lz - z), ft = min(t, Lt - t);
+        k *= (double)__ldg(&mtab[((ft * H.z + fz) * H.y + fy) * H.x + fx]);
+      }
+      double2* e = reinterpret_cast<double2*>(&tile[t * TS + z * xc + xi]);
+      const double2 v = fx_out(*reinterpret_cast<const I2*>(e), in, mid, hz, ht);
+      if (LRN && snap != nullptr) snap[(int64_t)zt * plane + sxy + xi] = bf16x2_of<double>(v);
+      const double2 w = make_double2(v.x * k, v.y * k);
+      m = fx_max(m, w);
+      *e = w;
+    }
+    atomicMax(&ps->in1[col], m);
+  }
+  __syncthreads();
+  fx_plane<+1, false, false>(tile, lt, dt, tw + Lz, ht, lz, dz, tw, hz, ps->in1, ps->mid1);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    LGF_ZT_IDX(i)
+    fld[(int64_t)zt * plane + sxy + xi] =
+        fx_out(tile[pos[Lz + t] * TS + pos[z] * xc + xi], ps->in1[xi], ps->mid1[xi], ht, hz);
+  }
+#undef LGF_ZT_IDX
+}
+
+template <bool EXPG>
+__global__ void __launch_bounds__(512)
+fft_xy_inv_gauge_fx_kernel(Geom g, FFTDir dx, FFTDir dy, const double2* __restrict__ data,
+                           const int4* __restrict__ twg, const short* __restrict__ posg, double2* __restrict__ gf,
+                           double2* __restrict__ Gf, Lines lx, Lines ly, CopyDiv cd, Batch B) {
+  if (batch_skip(B)) return;
+  data += blockIdx.z * B.s_delta;
+  gf += blockIdx.z * B.s_g;
+  if (Gf != nullptr) Gf += blockIdx.z * B.s_G;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int Lx = g.L[0], Ly = g.L[1];
+  int4* tw;
+  short* pos;
+  FxPlanes* ps;
+  I2* tile = fx_setup(smem_raw, twg, posg, Lx, Ly, &tw, &pos, &ps);
+  const int RS = Lx + 1, PS = Ly * RS;
+  const int plane = Lx * Ly;
+  const double2* fld = data + (int64_t)blockIdx.x * plane;
+  __syncthreads();
+  fx_load(
+      tile, 4 * plane, ps->in0,
+      [&](int i) {
+        const int f = (int)cd.a.div((uint32_t)i);
+        return &fld[(int64_t)f * g.V + (i - f * plane)];
+      },
+      [&](int i, int& pl) {
+        const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+        pl = f;
+        return f * PS + y * RS + x;
+      });
+  __syncthreads();
+  const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
+  fx_plane<+1, false, true>(tile, lx, dx, tw, hx, ly, dy, tw + Lx, hy, ps->in0, ps->mid0);
+  for (int i = threadIdx.x; i < plane; i += blockDim.x) {
+    const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
+    const int o = pos[Lx + y] * RS + pos[x];
+    double2 f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f[k] = fx_out(tile[k * PS + o], ps->in0[k], ps->mid0[k], hx, hy);
+    gauge_site<double, double, 3, EXPG>(f[0], f[1], f[2], f[3], g.V, (int64_t)blockIdx.x * plane + i, gf, Gf);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+
+void fft_twiddles(const int L[4], std::vector<double2>& tw) {
+  const int nt = L[0] + L[1] + L[2] + L[3];
+  tw.resize((size_t)2 * nt);
+  int4* fx = reinterpret_cast<int4*>(tw.data() + nt);
+  const long double two_pi = 6.283185307179586476925286766559005768L;
+  int off = 0;
+  for (int mu = 0; mu < 4; ++mu) {
+    for (int m = 0; m < L[mu]; ++m) {
+      const double a = -2.0 * M_PI * (double)m / (double)L[mu];
+      tw[off + m] = make_double2(std::cos(a), std::sin(a));
+      const long double b = -two_pi * (long double)m / (long double)L[mu];
+      const long double c[2] = {std::cos(b), std::sin(b)};
+      int hl[4];
+      for (int k = 0; k < 2; ++k) {
+        const long double h = std::round(c[k] * 1073741824.0L);
+        hl[2 * k] = (int)h;
+        hl[2 * k + 1] = (int)std::round((c[k] * 1073741824.0L - h) * 1073741824.0L);
+      }
+      fx[off + m] = make_int4(hl[0], hl[1], hl[2], hl[3]);
+    }
+    off += L[mu];
+  }
+}
+
+static const int4* fx_table(const Geom& g, const double2* tw) {
+  return reinterpret_cast<const int4*>(tw + g.L[0] + g.L[1] + g.L[2] + g.L[3]);
+}
+
+cudaError_t launch_fft_xy_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
+                             int sign, int nfields, cudaStream_t s, const Batch& B) {
+  int fpb = std::min(p.fpb_xy, nfields);
+  while (nfields % fpb) fpb /= 2;
+  const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
+  const size_t smem = plane_header_bytes(Lx, Ly, 8) + (size_t)fpb * PS * sizeof(double2);
+  const dim3 grid((unsigned)(g.L[2] * g.L[3]), (unsigned)(nfields / fpb), (unsigned)B.n);
+  const Lines lx = make_lines(fpb * Ly, Ly, RS, PS, 1), ly = make_lines(fpb * Lx, Lx, 1, PS, RS);
+  const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
+  cudaError_t e = sign < 0 ? allow_smem(fft_xy_fx_kernel<-1>, smem) : allow_smem(fft_xy_fx_kernel<+1>, smem);
+  if (e != cudaSuccess) return e;
+  if (sign < 0)
+    fft_xy_fx_kernel<-1><<<grid, p.threads_xy, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos, fpb, lx, ly,
+                                                          cd, B);
+  else
+    fft_xy_fx_kernel<+1><<<grid, p.threads_xy, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos, fpb, lx, ly,
+                                                          cd, B);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
+                             const double* K, int mode, int nfields, cudaStream_t s, const LearnedIO& lio,
+                             const Batch& B) {
+  const size_t smem = p.smem_zt;
+  const dim3 grid((unsigned)(g.L[0] / p.xc * g.L[1]), (unsigned)nfields, (unsigned)B.n);
+  const bool lrn = mode == 0 && (lio.mtab != nullptr || lio.snap != nullptr);
+  cudaError_t e = lrn ? allow_smem(fft_zt_filter_fx_kernel<true>, smem) : allow_smem(fft_zt_filter_fx_kernel<false>, smem);
+  if (e != cudaSuccess) return e;
+  const int4 H = make_int4(g.L[0] / 2 + 1, g.L[1] / 2 + 1, g.L[2] / 2 + 1, g.L[3] / 2 + 1);
+  const int xc = p.xc, Lz = g.L[2], Lt = g.L[3], TS = Lz * xc + 1;
+  const Lines lz = make_lines(Lt * xc, xc, 1, TS, xc), lt = make_lines(Lz * xc, xc, 1, xc, TS);
+  const CopyDiv cd{FastDiv::make((uint32_t)xc), FastDiv::make((uint32_t)Lz)};
+  if (lrn)
+    fft_zt_filter_fx_kernel<true><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, fx_table(g, tw), pos, K, xc,
+                                                                   mode, lio, H, lz, lt, cd, B);
+  else
+    fft_zt_filter_fx_kernel<false><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, fx_table(g, tw), pos, K, xc,
+                                                                    mode, lio, H, lz, lt, cd, B);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
+                                   const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
+                                   bool exact_exp) {
+  const size_t smem = p.smem_c;
+  cudaError_t e = exact_exp ? allow_smem(fft_xy_inv_gauge_fx_kernel<true>, smem)
+                            : allow_smem(fft_xy_inv_gauge_fx_kernel<false>, smem);
+  if (e != cudaSuccess) return e;
+  const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
+  const Lines lx = make_lines(4 * Ly, Ly, RS, PS, 1), ly = make_lines(4 * Lx, Lx, 1, PS, RS);
+  const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
+  const dim3 grid((unsigned)(g.L[2] * g.L[3]), 1, (unsigned)B.n);
+  if (exact_exp)
+    fft_xy_inv_gauge_fx_kernel<true><<<grid, p.threads_c, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos,
+                                                                     gfield, Gfield, lx, ly, cd, B);
+  else
+    fft_xy_inv_gauge_fx_kernel<false><<<grid, p.threads_c, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos,
+                                                                      gfield, Gfield, lx, ly, cd, B);
+  return cudaGetLastError();
+}
+
+}  // namespace lgf

@@ -164,4 +164,52 @@ __device__ __forceinline__ void fx_cross_conj(FxAcc& re, FxAcc& im, const FxC& a
   fx_mac(im, al.y, bk.x);
 }
 
+// ---------------------------------------------------------------------------
+// block floating point: 64-bit integers with a common exponent per block
+// ---------------------------------------------------------------------------
+
+// Integer of an FP64 number in units that make the block's largest magnitude
+// fit (see the transform passes): M >> (base - e), M with its leading one at
+// bit 63.  base >= 100, so zeros and numbers 2^-64 below the block's largest
+// give zero.
+__device__ __forceinline__ int64_t bfp_from(double a, uint32_t base) {
+  const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
+  const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
+  const int64_t sg = (int64_t)((int)hi >> 31);
+  return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, base - ((hi >> 20) & 0x7ffu)) ^ sg) - sg;
+}
+
+// FP64 value of n 2^ex rounded to nearest, any n and ex.
+static __device__ __noinline__ double bfp_to_double_any(int64_t n, int ex) { return scalbn(fx_to_double_fp<0>(n), ex); }
+
+// The same on the integer pipe where the block's exponents are far from the
+// ends of the FP64 range (safe) and |n| >= 2^32.
+__device__ __forceinline__ double bfp_to_double(int64_t n, int ex, bool safe) {
+  const int sg = (int)(n >> 63);
+  const uint64_t u = (uint64_t)((n ^ (int64_t)sg) - (int64_t)sg);
+  const uint32_t uh = (uint32_t)(u >> 32);
+  if (!safe || uh == 0u) return bfp_to_double_any(n, ex);
+  const int lz = __clz((int)uh);
+  const uint64_t m = ((u << (lz - 1)) + 0x200ull) >> 10;
+  const uint32_t rh = (uint32_t)(m >> 32) + (uint32_t)(1023 + 62 + ex - lz) * 0x100000u;
+  return __hiloint2double((int)(rh | ((uint32_t)sg & 0x80000000u)), (int)(uint32_t)m);
+}
+
+// X (|X| < 2^61) as two limbs, X = h 2^30 + l.
+struct Bfp2 {
+  int h, l;
+};
+__device__ __forceinline__ Bfp2 bfp_limbs(int64_t x) { return Bfp2{(int)(x >> 30), (int)((uint32_t)x & 0x3fffffffu)}; }
+
+// Real and complex products with a constant or a root of unity w, |w| <= 1,
+// w = h 2^-30 + l 2^-60 (|l| <= 2^29): three multiply-adds per real product,
+// rounded to the nearest unit (l l' 2^-60 is dropped, below 2^-30 of a unit).
+__device__ __forceinline__ int64_t bfp_mul(int64_t x, int wh, int wl) {
+  const Bfp2 a = bfp_limbs(x);
+  int64_t mid = (int64_t)1 << 29;
+  mid += (int64_t)a.h * wl;
+  mid += (int64_t)a.l * wh;
+  return (int64_t)a.h * wh + (mid >> 30);
+}
+
 }  // namespace lgf

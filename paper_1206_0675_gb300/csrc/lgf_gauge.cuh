@@ -1,0 +1,277 @@
+// g(x) of one site from its packed filtered divergence: the first-order form
+// and the exact exponential, and the store of g (and G <- g G).
+#pragma once
+
+#include "lgf_internal.h"
+
+namespace lgf {
+
+// ---------------------------------------------------------------------------
+// g(x) = reunitarize(1 + Delta'(x)) in FP64 (Sec. 2 first-order expansion,
+// Gram-Schmidt on rows 1-2, row 3 = (a x b)^* as in Sec. 3.2)
+// ---------------------------------------------------------------------------
+
+// f0 = (Im D11, Im D22), f1 = D12, f2 = D13, f3 = D23 of the filtered field.
+// Rows of 1 + X: r1 = (1 + i a, f1, f2) and r2 = (-conj f1, 1 + i d, f3)
+// with a = Re f0, d = Im f0.  Gram-Schmidt: u = r1 / |r1| and
+// v = w / |w| with w = r2 - <u, r2> u = r2 - (c / |r1|^2) r1, where
+// c = <r1, r2> = sum_j conj(r1_j) r2_j = (a + d)(Im f1 + i Re f1) + conj(f2) f3
+// (the two terms in f1 combine).  All of it in FP64.
+// The FP64 Gram-Schmidt factors of 1 + X: i1 = 1/|r1|, w = r2 - k r1 and
+// i2 = 1/|w|, so that u = i1 r1 and v = i2 w.
+struct GSFactors {
+  double i1, i2;
+  double2 w[3];
+};
+
+__device__ __forceinline__ void gram_schmidt_factors(double a, double d, double2 f1, double2 f2, double2 f3,
+                                                     GSFactors& o) {
+  const double n1 = fma(f2.x, f2.x, fma(f2.y, f2.y, fma(f1.x, f1.x, fma(f1.y, f1.y, fma(a, a, 1.0)))));
+  o.i1 = rsqrt_fp64(n1);
+  const double s = a + d;
+  const double q = o.i1 * o.i1;  // 1 / |r1|^2
+  const double kx = q * fma(f2.x, f3.x, fma(f2.y, f3.y, s * f1.y));
+  const double ky = q * fma(f2.x, f3.y, fma(-f2.y, f3.x, s * f1.x));
+  // w = r2 - k r1
+  o.w[0] = make_double2(fma(ky, a, -f1.x - kx), fma(-kx, a, f1.y - ky));
+  o.w[1] = make_double2(fma(ky, f1.y, fma(-kx, f1.x, 1.0)), fma(-ky, f1.x, fma(-kx, f1.y, d)));
+  o.w[2] = make_double2(fma(ky, f2.y, fma(-kx, f2.x, f3.x)), fma(-ky, f2.x, fma(-kx, f2.y, f3.y)));
+  const double n2 = fma(o.w[2].x, o.w[2].x, fma(o.w[2].y, o.w[2].y, fma(o.w[1].x, o.w[1].x,
+                    fma(o.w[1].y, o.w[1].y, fma(o.w[0].x, o.w[0].x, o.w[0].y * o.w[0].y)))));
+  o.i2 = rsqrt_fp64(n2);
+}
+
+// The FP64 factors for fields stored in FP32: i1 = 1/|r1|, the projection
+// coefficient k = <r1, r2>/|r1|^2 and i2 = 1/|w| with w = r2 - k r1, where
+// |w|^2 = |r2|^2 - |<r1, r2>|^2/|r1|^2 (Pythagoras for the projection) is
+// formed from the inputs, so that w itself is never needed in FP64: the
+// FP32 field applies k in FP32.  For 1 + X with X anti-Hermitian the rows are
+// nearly orthogonal (|<r1, r2>| <= |X|^2 while |r1|, |r2| >= 1), so the
+// difference does not cancel.  33 FP64 operations and two estimates, against
+// 43 when w is formed in FP64.
+struct GSFactors32 {
+  double i1, i2, kx, ky;
+};
+
+__device__ __forceinline__ void gram_schmidt_factors_f32(double a, double d, double2 f1, double2 f2, double2 f3,
+                                                         GSFactors32& o) {
+  const double n1 = fma(f2.x, f2.x, fma(f2.y, f2.y, fma(f1.x, f1.x, fma(f1.y, f1.y, fma(a, a, 1.0)))));
+  o.i1 = rsqrt_fp64(n1);
+  const double s = a + d;
+  const double q = o.i1 * o.i1;  // 1 / |r1|^2
+  const double cx = fma(f2.x, f3.x, fma(f2.y, f3.y, s * f1.y));
+  const double cy = fma(f2.x, f3.y, fma(-f2.y, f3.x, s * f1.x));
+  const double nr2 = fma(f3.x, f3.x, fma(f3.y, f3.y, fma(d, d, fma(f1.x, f1.x, fma(f1.y, f1.y, 1.0)))));
+  const double n2 = fma(-q, fma(cx, cx, cy * cy), nr2);
+  o.kx = q * cx;
+  o.ky = q * cy;
+  o.i2 = rsqrt_fp64(n2);
+}
+
+// FP32 <-> FP64 conversions on the integer pipe, written from the IEEE 754
+// binary32 / binary64 layouts.  On this GPU the conversion instructions run
+// on the FP64 pipe, which bounds pass C of FP32 lanes; these take sign,
+// rebiased exponent and mantissa apart with integer operations instead.
+// Zero and subnormal inputs give zero; FP64 -> FP32 rounds to nearest with
+// ties away from zero (IEEE rounds ties to even: the two differ only on exact
+// ties) and overflows to infinity.  Non-finite values are not expected here.
+__device__ __forceinline__ double f32_to_f64_int(float x) {
+  const uint32_t b = __float_as_uint(x);
+  const uint64_t sign = (uint64_t)(b >> 31) << 63;
+  const uint32_t e = (b >> 23) & 0xffu;
+  const uint64_t body = ((uint64_t)(e + (1023u - 127u)) << 52) | ((uint64_t)(b & 0x7fffffu) << 29);
+  return __longlong_as_double((long long)(sign | (e == 0u ? 0ull : body)));
+}
+__device__ __forceinline__ float f64_to_f32_int(double x) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const uint32_t sign = (uint32_t)(b >> 63) << 31;
+  const int64_t r = (int64_t)(b & 0x7fffffffffffffffull) - ((int64_t)(1023 - 127) << 52) + (1ll << 28);
+  uint32_t f = r <= (1ll << 28) ? 0u : (uint32_t)(r >> 29);
+  if (r > (1ll << 28) && f >= 0x7f800000u) f = 0x7f800000u;
+  return __uint_as_float(sign | f);
+}
+__device__ __forceinline__ double2 c_f32_to_f64_int(float2 v) { return make_double2(f32_to_f64_int(v.x), f32_to_f64_int(v.y)); }
+__device__ __forceinline__ float2 c_f64_to_f32_int(double2 v) { return make_float2(f64_to_f32_int(v.x), f64_to_f32_int(v.y)); }
+
+// Rows u, v of g = reunitarize(1 + X) in the field precision R; the
+// Gram-Schmidt factors are FP64 in both.  FP64 fields take u = i1 r1 and
+// v = i2 w in FP64.  FP32 fields, whose rows are stored in FP32, apply the
+// FP64 factors in FP32: u = fl(i1) r1 with r1 the FP32 entries of the
+// filtered field itself, v = fl(i2) fl(w) -- within one FP32 rounding of the
+// FP64 product, without the FP64 multiplies -- and take their values to and
+// from FP64 on the integer pipe.
+template <typename R>
+__device__ __forceinline__ void gauge_rows(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f3, C2<R> u[3], C2<R> v[3]) {
+  if constexpr (sizeof(R) == sizeof(double)) {
+    GSFactors o;
+    gram_schmidt_factors(f0.x, f0.y, f1, f2, f3, o);
+    u[0] = mkc<R>(o.i1, f0.x * o.i1);
+    u[1] = cscale<R>(f1, o.i1);
+    u[2] = cscale<R>(f2, o.i1);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) v[j] = cscale<double>(o.w[j], o.i2);
+  } else {
+    GSFactors32 o32;
+    gram_schmidt_factors_f32(f32_to_f64_int(f0.x), f32_to_f64_int(f0.y), c_f32_to_f64_int(f1), c_f32_to_f64_int(f2),
+                             c_f32_to_f64_int(f3), o32);
+    const float i1 = f64_to_f32_int(o32.i1), i2 = f64_to_f32_int(o32.i2);
+    const float kx = f64_to_f32_int(o32.kx), ky = f64_to_f32_int(o32.ky);
+    const float a = f0.x, d = f0.y;
+    u[0] = mkc<R>(i1, a * i1);
+    u[1] = cscale<R>(f1, i1);
+    u[2] = cscale<R>(f2, i1);
+    // w = r2 - k r1 in FP32, normalised by the FP64 factor
+    const C2<R> w0 = mkc<R>(fmaf(ky, a, -f1.x - kx), fmaf(-kx, a, f1.y - ky));
+    const C2<R> w1 = mkc<R>(fmaf(ky, f1.y, fmaf(-kx, f1.x, 1.f)), fmaf(-ky, f1.x, fmaf(-kx, f1.y, d)));
+    const C2<R> w2 = mkc<R>(fmaf(ky, f2.y, fmaf(-kx, f2.x, f3.x)), fmaf(-ky, f2.x, fmaf(-kx, f2.y, f3.y)));
+    v[0] = cscale<R>(w0, i2);
+    v[1] = cscale<R>(w1, i2);
+    v[2] = cscale<R>(w2, i2);
+  }
+}
+
+// Rows 1 and 2 of g = exp(X) (the exponential of Eq. (eq:gx) evaluated
+// exactly instead of to first order), for X traceless anti-Hermitian packed
+// as above, followed by the same Gram-Schmidt projection.
+//
+// With X = iQ (Q Hermitian, traceless) the Cayley-Hamilton theorem gives
+// Q^3 = u Q + w 1, u = tr(Q^2)/2, w = det Q, so exp(iQ) = c0 1 + c1 Q + c2 Q^2.
+// Scaling and squaring (Moler and Van Loan, "Nineteen dubious ways to compute
+// the exponential of a matrix", 1978): Z = Q / 2^s with |Z|_F <= 1/4, the
+// Taylor series of exp(iZ) to order 12 (remainder below 3e-18) reduced to
+// c0 + c1 Z + c2 Z^2 through Z^3 = uz Z + wz 1, then s squarings carried out on
+// the three coefficients with the same reduction.
+__device__ __forceinline__ void gauge_exp_from_packed(double2 f0, double2 f1, double2 f2, double2 f3, double2 u[3],
+                                                      double2 v[3]) {
+  const double a = f0.x, d = f0.y, q33 = -(a + d);
+  // Q = -iX: off-diagonal entries q12, q13, q23; Q_ji = conj(Q_ij)
+  const double2 q12 = make_double2(f1.y, -f1.x), q13 = make_double2(f2.y, -f2.x), q23 = make_double2(f3.y, -f3.x);
+  const double n12 = cnorm2<double>(q12), n13 = cnorm2<double>(q13), n23 = cnorm2<double>(q23);
+  const double uq = 0.5 * (a * a + d * d + q33 * q33) + n12 + n13 + n23;
+  const double2 t = cconjmul<double>(q13, cmul<double>(q12, q23));  // q12 q23 conj(q13)
+  const double wq = a * d * q33 + 2.0 * t.x - a * n23 - d * n13 - q33 * n12;
+  int s = 0;
+  double n2 = 2.0 * uq, uz = uq, wz = wq;
+  while (n2 > 0.0625 && s < 64) {
+    n2 *= 0.25;
+    uz *= 0.25;
+    wz *= 0.125;
+    ++s;
+  }
+  // Z^n / n! = al 1 + be Z + ga Z^2 (real); exp(iZ) = sum_n i^n Z^n / n!
+  double al = 1.0, be = 0.0, ga = 0.0;
+  double2 c0 = make_double2(1.0, 0.0), c1 = make_double2(0.0, 0.0), c2 = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int n = 1; n <= 12; ++n) {
+    const double inv = 1.0 / (double)n;
+    const double al2 = ga * wz * inv, be2 = fma(ga, uz, al) * inv, ga2 = be * inv;
+    al = al2;
+    be = be2;
+    ga = ga2;
+    const double sg = ((n & 3) < 2) ? 1.0 : -1.0;
+    if (n & 1) {
+      c0.y = fma(sg, al, c0.y);
+      c1.y = fma(sg, be, c1.y);
+      c2.y = fma(sg, ga, c2.y);
+    } else {
+      c0.x = fma(sg, al, c0.x);
+      c1.x = fma(sg, be, c1.x);
+      c2.x = fma(sg, ga, c2.x);
+    }
+  }
+  double h1 = 1.0;
+  for (int k = 0; k < s; ++k) {
+    const double2 p00 = cmul<double>(c0, c0), p12 = cmul<double>(c1, c2), p01 = cmul<double>(c0, c1);
+    const double2 p22 = cmul<double>(c2, c2), p02 = cmul<double>(c0, c2), p11 = cmul<double>(c1, c1);
+    c0 = make_double2(fma(2.0 * wz, p12.x, p00.x), fma(2.0 * wz, p12.y, p00.y));
+    c1 = make_double2(fma(wz, p22.x, fma(2.0 * uz, p12.x, 2.0 * p01.x)),
+                      fma(wz, p22.y, fma(2.0 * uz, p12.y, 2.0 * p01.y)));
+    c2 = make_double2(fma(uz, p22.x, fma(2.0, p02.x, p11.x)), fma(uz, p22.y, fma(2.0, p02.y, p11.y)));
+    h1 *= 0.5;
+  }
+  c1 = cscale<double>(c1, h1);       // coefficient of Q
+  c2 = cscale<double>(c2, h1 * h1);  // coefficient of Q^2
+  // rows 1 and 2 of Q^2
+  const double s11 = a * a + n12 + n13, s22 = n12 + d * d + n23;
+  const double2 s12 = cadd<double>(cscale<double>(q12, a + d), cmulc<double>(q13, q23));  // + q13 conj(q23)
+  const double2 s13 = cadd<double>(cscale<double>(q13, -d), cmul<double>(q12, q23));
+  const double2 s23 = cadd<double>(cconjmul<double>(q12, q13), cscale<double>(q23, -a));  // conj(q12) q13 - a q23
+  const double2 s21 = make_double2(s12.x, -s12.y);
+  const double2 q21 = make_double2(q12.x, -q12.y);
+  double2 r1[3], r2[3];
+  r1[0] = cadd<double>(cadd<double>(c0, cscale<double>(c1, a)), cscale<double>(c2, s11));
+  r1[1] = cadd<double>(cmul<double>(c1, q12), cmul<double>(c2, s12));
+  r1[2] = cadd<double>(cmul<double>(c1, q13), cmul<double>(c2, s13));
+  r2[0] = cadd<double>(cmul<double>(c1, q21), cmul<double>(c2, s21));
+  r2[1] = cadd<double>(cadd<double>(c0, cscale<double>(c1, d)), cscale<double>(c2, s22));
+  r2[2] = cadd<double>(cmul<double>(c1, q23), cmul<double>(c2, s23));
+  // Gram-Schmidt: u = r1/|r1|, v = (r2 - <u,r2> u)/|.|
+  const double i1 = rsqrt(cnorm2<double>(r1[0]) + cnorm2<double>(r1[1]) + cnorm2<double>(r1[2]));
+#pragma unroll
+  for (int j = 0; j < 3; ++j) u[j] = cscale<double>(r1[j], i1);
+  double2 ip = cconjmul<double>(u[0], r2[0]);
+  ip = cadd<double>(ip, cconjmul<double>(u[1], r2[1]));
+  ip = cadd<double>(ip, cconjmul<double>(u[2], r2[2]));
+  const double2 nip = make_double2(-ip.x, -ip.y);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) v[j] = cfma<double>(nip, u[j], r2[j]);
+  const double i2 = rsqrt(cnorm2<double>(v[0]) + cnorm2<double>(v[1]) + cnorm2<double>(v[2]));
+#pragma unroll
+  for (int j = 0; j < 3; ++j) v[j] = cscale<double>(v[j], i2);
+}
+
+// Stores rows u, v (precision RG) and, where needed, row 3 = (u x v)^*.
+template <typename RG, int GROWS>
+__device__ __forceinline__ void store_gauge_rows(int64_t V, int64_t s, const C2<RG> a[3], const C2<RG> b[3],
+                                                 C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf) {
+  C2<RG> c[3];
+  const bool need_c = (GROWS == 3) || (Gf != nullptr);
+  if (need_c) su3_third_row<RG>(a, b, c);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    gf[(0 * 3 + j) * V + s] = a[j];
+    gf[(1 * 3 + j) * V + s] = b[j];
+    if (GROWS == 3) gf[(2 * 3 + j) * V + s] = c[j];
+  }
+  if (Gf != nullptr) {
+    // G <- g G (full 3x3, precision RG)
+    C2<RG> Go[3][3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int col = 0; col < 3; ++col) Go[r][col] = Gf[(r * 3 + col) * V + s];
+    const C2<RG>* rows[3] = {a, b, c};
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int col = 0; col < 3; ++col) {
+        C2<RG> acc = cmul<RG>(rows[r][0], Go[0][col]);
+        acc = cfma<RG>(rows[r][1], Go[1][col], acc);
+        acc = cfma<RG>(rows[r][2], Go[2][col], acc);
+        Gf[(r * 3 + col) * V + s] = acc;
+      }
+  }
+}
+
+// g(x) of one site from its packed filtered field and its store (and G <- g G).
+template <typename R, typename RG, int GROWS, bool EXPG>
+__device__ __forceinline__ void gauge_site(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f3, int64_t V, int64_t s,
+                                           C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf) {
+  static_assert(sizeof(R) == sizeof(RG), "g is stored in the precision of the divergence");
+  C2<RG> a[3], b[3];
+  if constexpr (EXPG) {
+    double2 u[3], v[3];
+    gauge_exp_from_packed(ccast<double, R>(f0), ccast<double, R>(f1), ccast<double, R>(f2), ccast<double, R>(f3),
+                          u, v);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      a[j] = ccast<RG, double>(u[j]);
+      b[j] = ccast<RG, double>(v[j]);
+    }
+  } else {
+    gauge_rows<RG>(f0, f1, f2, f3, a, b);
+  }
+  store_gauge_rows<RG, GROWS>(V, s, a, b, gf, Gf);
+}
+
+}  // namespace lgf

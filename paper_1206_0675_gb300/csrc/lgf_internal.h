@@ -210,7 +210,8 @@ struct FFTPlan {
 enum FFTDecomp { FFT_2D2D = 0, FFT_1D4 = 1, FFT_3D1D = 2 };
 
 // Twiddle tables W_N^m = exp(-2 pi i m / N), m < N, for the four directions,
-// concatenated at offsets 0, Lx, Lx+Ly, Lx+Ly+Lz (FP64 and FP32 copies).
+// concatenated at offsets 0, Lx, Lx+Ly, Lx+Ly+Lz (FP64 and FP32 copies).  The
+// FP64 table is followed by the same roots in fixed point (fft_twiddles).
 // pos: digit-reversal position tables of the four directions (fft_positions).
 template <typename R>
 cudaError_t launch_fft_xy(const Geom& g, const FFTPlan& p, C2<R>* data, const C2<R>* tw, const short* pos, int sign,
@@ -281,6 +282,22 @@ cudaError_t launch_fft_xyz(const Geom& g, const FFTPlan& p, C2<R>* data, const C
 template <typename R, typename RG, int GROWS>
 cudaError_t launch_gauge_from_delta(const Geom& g, const C2<R>* data, C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s,
                                     const Batch& B = Batch(), int exact_exp = 0);
+
+// ---- lgf_fft_fx.cu -------------------------------------------------------
+// The plane passes of FP64 fields in block floating point; arguments as the
+// launchers of lgf_fft.cu, which call them for R = double.
+cudaError_t launch_fft_xy_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
+                             int sign, int nfields, cudaStream_t s, const Batch& B);
+cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
+                             const double* K, int mode, int nfields, cudaStream_t s, const LearnedIO& lio,
+                             const Batch& B);
+cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
+                                   const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
+                                   bool exact_exp);
+// The FP64 twiddle table of a lattice: L[0] + ... + L[3] roots in FP64, then
+// the same roots as fixed-point limbs (int4: cosine and sine, each h 2^-30 +
+// l 2^-60) in the same order.
+void fft_twiddles(const int L[4], std::vector<double2>& tw);
 
 cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p);
 
