@@ -30,7 +30,7 @@ template <typename R> struct Lane {
   C2<R>* U = nullptr;      // links [4][rows][3][V]
   C2<R>* U2 = nullptr;     // second link buffer (FP32 lanes)
   bool fused = false;      // update and measurement run as one kernel, links ping-pong between U and U2
-  C2<R>* g = nullptr;      // gauge transform of the last step [grows][3][V]
+  C2<R>* g = nullptr;      // gauge transform of the last step [grows][3][V] (FP64: fixed-point operands)
   C2<R>* D = nullptr;      // packed divergence / FFT workspace [4][V]
   R* K = nullptr;          // filter table [V]
   C2<R>* tw = nullptr;     // twiddles
@@ -598,7 +598,7 @@ lgf_status measure_current(lgf_ctx* h) {
 // FP32 -> FP64 switch: G64 = proj_SU3(G32) in FP64, U64 = G64 U0 G64^dag(x+mu).
 lgf_status switch_to_fp64(lgf_ctx* h) {
   const Geom& g = h->geom;
-  LGF_CK(h, launch_project_sites_f32_to_f64(g, h->f.G, h->d.g, h->stream));
+  LGF_CK(h, launch_project_sites_f32_to_f64(g, h->f.G, h->d.g, h->d.G, h->stream));
   if (h->d.rows == 3) {
     LGF_CK(h, (launch_links_from_aos<double, 3>(g, h->U0, h->d.U, h->stream)));
     LGF_CK(h, (launch_update<double, 3, 3>(g, h->d.U, h->d.g, h->stream)));
@@ -606,8 +606,6 @@ lgf_status switch_to_fp64(lgf_ctx* h) {
     LGF_CK(h, (launch_links_from_aos<double, 2>(g, h->U0, h->d.U, h->stream)));
     LGF_CK(h, (launch_update<double, 2, 3>(g, h->d.U, h->d.g, h->stream)));
   }
-  if (h->d.G) LGF_CK(h, cudaMemcpyAsync(h->d.G, h->d.g, sizeof(double2) * 9 * g.V, cudaMemcpyDeviceToDevice,
-                                        h->stream));
   h->phase = 64;
   lgf_status s = measure_current(h);
   return s;
@@ -823,12 +821,8 @@ lgf_status lgf_create_with_allocator(const int32_t extents[4], lgf_precision pre
     if (allocator) h->mem.user = *allocator;
     if (cudaGetDevice(&h->device) != cudaSuccess) { delete h; return LGF_E_CUDA; }
     Geom& g = h->geom;
-    g.V = 1;
-    for (int mu = 0; mu < 4; ++mu) {
-      g.L[mu] = extents[mu];
-      g.stride[mu] = g.V;
-      g.V *= extents[mu];
-    }
+    for (int mu = 0; mu < 4; ++mu) g.L[mu] = extents[mu];
+    g.finish();
     lgf_status s = LGF_OK;
     const bool store12 = (flags & LGF_STORE12) != 0;
     const bool track = (flags & LGF_TRACK_G) != 0;
@@ -1160,7 +1154,7 @@ lgf_status lgf_get_gauge(lgf_handle h, double* gout, int where) {
   const Geom& g = h->geom;
   double* dst = where == LGF_DEVICE ? gout : h->stage;
   if (h->phase == 64) {
-    LGF_CK(h, (launch_sites_to_aos<double, 3>(g, h->d.g, dst, h->stream)));
+    LGF_CK(h, launch_gauge_to_aos(g, h->d.g, dst, h->stream));
   } else if (h->f.grows == 2) {
     LGF_CK(h, (launch_sites_to_aos<float, 2>(g, h->f.g, dst, h->stream)));
   } else {

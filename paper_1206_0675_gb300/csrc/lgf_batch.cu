@@ -340,12 +340,8 @@ lgf_status lgf_batch_create(int32_t n, const int32_t* extents, lgf_precision pre
       }
       if (c == (int)b->cls.size()) {
         ClassLane C;
-        C.geom.V = 1;
-        for (int mu = 0; mu < 4; ++mu) {
-          C.geom.L[mu] = L[mu];
-          C.geom.stride[mu] = C.geom.V;
-          C.geom.V *= L[mu];
-        }
+        for (int mu = 0; mu < 4; ++mu) C.geom.L[mu] = L[mu];
+        C.geom.finish();
         b->cls.push_back(C);
       }
       b->cls_of[i] = c;

@@ -155,13 +155,26 @@ struct Geom {
   int L[4];        // Lx, Ly, Lz, Lt
   int64_t V;       // volume
   int64_t stride[4];  // 1, Lx, Lx*Ly, Lx*Ly*Lz
+  FastDiv dL[3];   // divisors Lx, Ly, Lz (extents are at most 128, so a site index has 28 bits)
+  // Volume, strides and divisors from the extents.
+  void finish() {
+    V = 1;
+    for (int mu = 0; mu < 4; ++mu) {
+      stride[mu] = V;
+      V *= L[mu];
+      if (mu < 3) dL[mu] = FastDiv::make((uint32_t)L[mu]);
+    }
+  }
 };
 
 __device__ __forceinline__ void site_coords(const Geom& g, int64_t s, int c[4]) {
-  int64_t r = s;
-  c[0] = (int)(r % g.L[0]); r /= g.L[0];
-  c[1] = (int)(r % g.L[1]); r /= g.L[1];
-  c[2] = (int)(r % g.L[2]); r /= g.L[2];
+  uint32_t r = (uint32_t)s;
+#pragma unroll
+  for (int mu = 0; mu < 3; ++mu) {
+    const uint32_t q = g.dL[mu].div(r);
+    c[mu] = (int)(r - q * g.dL[mu].d);
+    r = q;
+  }
   c[3] = (int)r;
 }
 

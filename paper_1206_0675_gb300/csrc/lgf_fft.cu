@@ -498,13 +498,16 @@ __global__ void gauge_from_delta_kernel(Geom g, const C2<R>* __restrict__ data, 
 // plan and launchers
 // ---------------------------------------------------------------------------
 
-static int radix_schedule(int N, int* radix) {
+// real_bytes 8: 16 = 4 x 4 and 128 = 8 x 4 x 4 instead of stages of 2, whose
+// index arithmetic costs the integer passes more than the larger radix saves.
+static int radix_schedule(int N, int real_bytes, int* radix) {
   int a = 0, b = 0, n = N;
   while (n % 2 == 0) { n /= 2; ++a; }
   while (n % 3 == 0) { n /= 3; ++b; }
   if (n != 1 || N < 2) return -1;
   int k = 0;
-  while (a >= 3) { radix[k++] = 8; a -= 3; }
+  while (a >= 3 && !(real_bytes == 8 && a == 4)) { radix[k++] = 8; a -= 3; }
+  if (a == 4) { radix[k++] = 4; a = 2; }
   if (a == 2) radix[k++] = 4;
   if (a == 1) radix[k++] = 2;
   while (b-- > 0) radix[k++] = 3;
@@ -577,7 +580,7 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   const size_t cb = 2 * (size_t)real_bytes;  // bytes per complex element
   for (int mu = 0; mu < 4; ++mu) {
     p->d[mu].N = L[mu];
-    p->d[mu].nst = radix_schedule(L[mu], p->d[mu].radix);
+    p->d[mu].nst = radix_schedule(L[mu], real_bytes, p->d[mu].radix);
     if (p->d[mu].nst < 0) return cudaErrorInvalidValue;
     int Ns = 1;
     for (int st = 0; st < p->d[mu].nst; ++st) {
@@ -590,24 +593,30 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   const size_t hzt = plane_header_bytes(Lz, Lt, real_bytes);
   const size_t plane_xy = (size_t)Ly * (Lx + 1) * cb;
   const size_t budget = 100 * 1024, maxsm = 220 * 1024;
-  p->fpb_xy = 4;
+  // FP64 planes (integer arithmetic, 90 to 130 registers) run best as many
+  // small CTAs, one field or one x column each: 412 us for the three passes at
+  // 32^4 against 477 us with tiles of 66 KB, and no slower at 16^4 or
+  // 24x18x12x27.  FP32 planes take up to four fields and eight columns.
+  const bool small = real_bytes == 8;
+  p->fpb_xy = small ? 1 : 4;
   while (p->fpb_xy > 1 && p->fpb_xy * plane_xy > budget) p->fpb_xy /= 2;
   if (plane_xy * p->fpb_xy + hxy > maxsm) return cudaErrorInvalidValue;
   p->smem_xy = hxy + p->fpb_xy * plane_xy;
   p->fuse_g = (4 * plane_xy + hxy <= maxsm) ? 1 : 0;
   p->smem_c = hxy + 4 * plane_xy;
   int xc = 1;
-  for (int c = 8; c >= 1; c /= 2) {
+  for (int c = small ? 1 : 8; c >= 1; c /= 2) {
     if (Lx % c) continue;
     if (hzt + (size_t)Lt * (Lz * c + 1) * cb <= budget) { xc = c; break; }
   }
-  if (xc == 1 && Lx % 2 == 0 && hzt + (size_t)Lt * (Lz * 2 + 1) * cb <= maxsm) xc = 2;
+  if (!small && xc == 1 && Lx % 2 == 0 && hzt + (size_t)Lt * (Lz * 2 + 1) * cb <= maxsm) xc = 2;
   p->xc = xc;
   p->smem_zt = hzt + (size_t)Lt * (Lz * xc + 1) * cb;
   if (p->smem_zt > maxsm) return cudaErrorInvalidValue;
-  p->threads_xy = threads_for(p->fpb_xy * Lx * Ly);
-  p->threads_zt = threads_for(Lz * Lt * xc);
-  p->threads_c = threads_for(4 * Lx * Ly);
+  const int most = real_bytes == 8 ? FX_MAX_THREADS : 512;
+  p->threads_xy = std::min(most, threads_for(p->fpb_xy * Lx * Ly));
+  p->threads_zt = std::min(most, threads_for(Lz * Lt * xc));
+  p->threads_c = std::min(most, threads_for(4 * Lx * Ly));
   configure_alt_passes(L, real_bytes, p);
   return cudaSuccess;
 }
@@ -637,7 +646,7 @@ void fft_plan_candidates(const int L[4], int real_bytes, std::vector<FFTPlan>& o
         auto thr = [&](int points) {
           int t = (points + tdiv - 1) / tdiv;
           t = ((t + 31) / 32) * 32;
-          return std::max(64, std::min(512, t));
+          return std::max(64, std::min(real_bytes == 8 ? FX_MAX_THREADS : 512, t));
         };
         p.threads_xy = thr(fpb * Lx * Ly);
         p.threads_zt = thr(Lz * Lt * xc);

@@ -22,8 +22,9 @@
 // smooth and constant inputs): 0.7e-16 to 2.8e-16, the FP64 passes on the FP64
 // pipe had 1.5e-16 to 4.6e-16.
 //
-// 32^4, us: pass A 86 (FP64 pipe: 231), pass B 197 (463), pass C with g 241
-// (397, where g keeps the FP64 pipe for 96 us); 24x18x12x27: 25, 65, 55 (54, 94, 78).
+// 32^4, us: pass A 76 (FP64 pipe: 231), pass B 160 (463), pass C with g 153 (397);
+// 24x18x12x27: 24, 41, 47 (54, 94, 78).  Bound by instruction issue (about 400
+// instructions per element of pass A, 800 of pass B) at 12 to 24 warps per SM.
 //
 // Planes that hold infinities or NaN give NaN; planes whose largest
 // component is near the ends of the FP64 range take slower conversions.
@@ -50,38 +51,76 @@ static_assert(sizeof(FxPlanes) == FX_PLANE_BYTES, "header of the FP64 plane pass
 
 __device__ __forceinline__ uint32_t fx_headroom(int N) { return 33u - (uint32_t)__clz(N - 1); }
 
-// From a plane's largest input component: its biased exponent (at least 1),
-// whether every exponent that can occur is far from the ends of the range.
-__device__ __forceinline__ uint32_t fx_exp_of(uint32_t in) { return max(in >> 20, 1u); }
-__device__ __forceinline__ bool fx_safe_exp(uint32_t e) { return e - 100u <= 1890u; }
+// The word of a plane after fx_classify: the biased exponent that its input
+// is scaled by and, above bit 16, what was done to a plane out of the ordinary:
+// scaled up or down by 2^FX_ODD_SCALE so that every exponent that can occur is
+// far from the ends of the FP64 range (all-zero planes among them), or set to
+// zero because it holds infinities or NaN.
+constexpr int FX_ODD_SCALE = 600;
+enum { FX_UP = 1, FX_DOWN = 2, FX_NONFINITE = 3 };
+__device__ __forceinline__ uint32_t fx_exp_of(uint32_t code) { return code & 0xffffu; }
+__device__ __forceinline__ uint32_t fx_classify(uint32_t in) {
+  const uint32_t e = max(in >> 20, 1u);
+  if (e < 100u) return (e + FX_ODD_SCALE) | (FX_UP << 16);
+  if (e == 2047u) return 1023u | (FX_NONFINITE << 16);
+  if (e > 1990u) return (e - FX_ODD_SCALE) | (FX_DOWN << 16);
+  return e;
+}
 // Right shift between the directions.
 __device__ __forceinline__ uint32_t fx_mid_shift(uint32_t mid, uint32_t h1) {
   const int sh = (64 - __clz((int)mid)) - (int)(61u - h1);
   return (uint32_t)max(sh, 0);
 }
 
-// Input of a plane near the ends of the range (or all zero); infinities and
-// NaN give zero here and NaN at the output.
-static __device__ __noinline__ int64_t fx_in_any(double a, uint32_t e, uint32_t h0) {
-  if (a == 0.0 || e == 2047u) return 0;
-  const double up = e < 100u ? a * 1.6069380442589903e60 : a;  // 2^200
-  return bfp_from(up, 3u + h0 + e + (e < 100u ? 200u : 0u));
-}
-__device__ __forceinline__ I2 fx_in(double2 v, uint32_t in, uint32_t h0) {
-  const uint32_t e = fx_exp_of(in);
-  if (!fx_safe_exp(e)) return make_longlong2(fx_in_any(v.x, e, h0), fx_in_any(v.y, e, h0));
-  const uint32_t base = 3u + h0 + e;
+__device__ __forceinline__ I2 fx_in(double2 v, uint32_t base) {
   return make_longlong2(bfp_from(v.x, base), bfp_from(v.y, base));
 }
 
-// Output of a plane after both directions.
-__device__ __forceinline__ double2 fx_out(I2 v, uint32_t in, uint32_t mid, uint32_t h0, uint32_t h1) {
-  const uint32_t e = fx_exp_of(in);
-  const int ex = (int)(fx_mid_shift(mid, h1) + h0 + e) - 1083;
-  const bool safe = fx_safe_exp(e);
-  if (e == 2047u) return make_double2(NAN, NAN);
-  return make_double2(bfp_to_double(v.x, ex, safe), bfp_to_double(v.y, ex, safe));
+// Exponent of a plane's integers after both directions (of the scaled plane).
+__device__ __forceinline__ int fx_out_exp(uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
+  return (int)(fx_mid_shift(mid, h1) + h0 + fx_exp_of(code)) - 1083;
 }
+// The same of the plane as it was, large where it holds infinities or NaN.
+__device__ __forceinline__ int fx_true_exp(uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
+  const int ex = fx_out_exp(code, mid, h0, h1);
+  const uint32_t k = code >> 16;
+  return k == 0u ? ex : k == FX_UP ? ex - FX_ODD_SCALE : k == FX_DOWN ? ex + FX_ODD_SCALE : 4096;
+}
+// Output of a plane after both directions.
+__device__ __forceinline__ double2 fx_out(I2 v, uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
+  const int ex = fx_out_exp(code, mid, h0, h1);
+  return make_double2(bfp_to_double(v.x, ex), bfp_to_double(v.y, ex));
+}
+// The same for any plane.
+static __device__ __noinline__ double2 fx_out_any(I2 v, uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
+  if (code >> 16 == FX_NONFINITE) return make_double2(NAN, NAN);
+  const double2 r = fx_out(v, code, mid, h0, h1);
+  const int k = code >> 16 == FX_UP ? -FX_ODD_SCALE : code >> 16 == FX_DOWN ? FX_ODD_SCALE : 0;
+  return make_double2(scalbn(r.x, k), scalbn(r.y, k));
+}
+
+// v 2^ex in units of 2^-58, rounded; ok = false unless it is below 1 in magnitude.
+__device__ __forceinline__ int64_t fx_unit58(int64_t v, int ex, bool& ok) {
+  if (ex > -62) {  // |v| 2^ex can reach 1
+    const uint64_t u = (uint64_t)(v ^ (v >> 63));
+    ok = ok && ex < 0 && shr64_clamp(u, (uint32_t)-ex) == 0;
+  }
+  const int sh = -58 - ex;
+  if (sh <= 0) return (int64_t)((uint64_t)v << (-sh & 63));
+  const int c = min(sh, 63);
+  return (v + ((int64_t)1 << (c - 1))) >> c;
+}
+
+struct FxOut {
+  __device__ __forceinline__ double2 operator()(I2 v, uint32_t c, uint32_t m, uint32_t h0, uint32_t h1) const {
+    return fx_out(v, c, m, h0, h1);
+  }
+};
+struct FxOutAny {
+  __device__ __forceinline__ double2 operator()(I2 v, uint32_t c, uint32_t m, uint32_t h0, uint32_t h1) const {
+    return fx_out_any(v, c, m, h0, h1);
+  }
+};
 
 __device__ __forceinline__ I2 iadd(I2 a, I2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ I2 isub(I2 a, I2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
@@ -98,19 +137,13 @@ template <int SIGN> __device__ __forceinline__ I2 itwiddle(I2 v, int4 w) {
   const Bfp2 x = bfp_limbs(v.x), y = bfp_limbs(v.y);
   const int sh = SIGN < 0 ? w.z : -w.z, sl = SIGN < 0 ? w.w : -w.w;
   const int nh = -sh, nl = -sl;
-  int64_t rm = (int64_t)1 << 29, im = (int64_t)1 << 29;
-  rm += (int64_t)x.h * w.y;
-  rm += (int64_t)x.l * w.x;
-  rm += (int64_t)y.h * nl;
-  rm += (int64_t)y.l * nh;
-  im += (int64_t)x.h * sl;
-  im += (int64_t)x.l * sh;
-  im += (int64_t)y.h * w.y;
-  im += (int64_t)y.l * w.x;
-  int64_t rh = (int64_t)x.h * w.x, ih = (int64_t)x.h * sh;
-  rh += (int64_t)y.h * nh;
-  ih += (int64_t)y.h * w.x;
-  return make_longlong2(rh + (rm >> 30), ih + (im >> 30));
+  const int64_t half = (int64_t)1 << 29;
+  int64_t rm = mad_wide(x.l, w.x, mad_wide(x.h, w.y, half));
+  int64_t im = mad_wide(x.l, sh, mad_wide(x.h, sl, half));
+  rm = mad_wide(y.l, nh, mad_wide(y.h, nl, rm));
+  im = mad_wide(y.l, w.x, mad_wide(y.h, w.y, im));
+  return make_longlong2(mad_wide(y.h, nh, mad_wide(x.h, w.x, rm >> 30)),
+                        mad_wide(y.h, w.x, mad_wide(x.h, sh, im >> 30)));
 }
 
 // 1/sqrt 2 and sqrt(3)/2 as h 2^-30 + l 2^-60
@@ -198,9 +231,9 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
     I2 v[RAD];
     if (io.in != nullptr) {
       const double2* raw = reinterpret_cast<const double2*>(tile);
-      const uint32_t in = io.in[pl];
+      const uint32_t sc = 3u + io.h + fx_exp_of(io.in[pl]);
 #pragma unroll
-      for (int r = 0; r < RAD; ++r) v[r] = fx_in(raw[base + r * step], in, io.h);
+      for (int r = 0; r < RAD; ++r) v[r] = fx_in(raw[base + r * step], sc);
     } else {
 #pragma unroll
       for (int r = 0; r < RAD; ++r) v[r] = tile[base + r * step];
@@ -248,39 +281,40 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
   __syncthreads();
 }
 
-// DFT of every line of a direction: DIT takes digit-reversed input and gives
-// natural order, DIF the reverse.
-template <int SIGN, bool DIT, bool PLO>
-__device__ __forceinline__ void fx_dir(I2* tile, const Lines& ln, const FFTDir& d, const int4* tw, const FxStageIO& io) {
-  for (int k = 0; k < d.nst; ++k) {
-    const int st = DIT ? k : d.nst - 1 - k;
-    FxStageIO s;
-    s.h = io.h;
-    if (k == 0) {
-      s.in = io.in;
-      s.shift = io.shift;
-    }
-    if (k == d.nst - 1) s.mid = io.mid;
-    if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
-    else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
-    else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
-    else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], tw, s);
-  }
-}
+// The two directions of a plane pass: d[0] and l[0] the first axis of the
+// plane (x or z), d[1] and l[1] the second.
+struct FxPass {
+  FFTDir d[2];
+  Lines l[2];
+};
 
-// Both directions of a plane transform from raw FP64 input.
+// Both directions of a plane transform from raw FP64 input, axis `first` and
+// then the other; DIT takes digit-reversed input and gives natural order, DIF
+// the reverse.  One loop over the directions: the stages of a radix are the
+// same code for both (the instruction cache held neither copy otherwise).
 template <int SIGN, bool DIT, bool PLO>
-__device__ __forceinline__ void fx_plane(I2* tile, const Lines& l0, const FFTDir& d0, const int4* tw0, uint32_t h0,
-                                         const Lines& l1, const FFTDir& d1, const int4* tw1, uint32_t h1,
-                                         const uint32_t* in, uint32_t* mid) {
-  FxStageIO a, b;
-  a.in = in;
-  a.mid = mid;
-  a.h = h0;
-  b.shift = mid;
-  b.h = h1;
-  fx_dir<SIGN, DIT, PLO>(tile, l0, d0, tw0, a);
-  fx_dir<SIGN, DIT, PLO>(tile, l1, d1, tw1, b);
+__device__ __forceinline__ void fx_plane(I2* tile, const FxPass& P, const int4* tw, int first, const uint32_t* in,
+                                         uint32_t* mid) {
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const int ax = first ^ k;
+    const FFTDir& d = P.d[ax];
+    const Lines& ln = P.l[ax];
+    const int4* w = ax == 0 ? tw : tw + P.d[0].N;
+    FxStageIO s;
+    s.h = fx_headroom(d.N);
+#pragma unroll 1
+    for (int i = 0; i < d.nst; ++i) {
+      const int st = DIT ? i : d.nst - 1 - i;
+      s.in = k == 0 && i == 0 ? in : nullptr;
+      s.shift = k == 1 && i == 0 ? mid : nullptr;
+      s.mid = k == 0 && i == d.nst - 1 ? mid : nullptr;
+      if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
+      else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
+      else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
+      else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
+    }
+  }
 }
 
 // Tile of a plane pass: header as setup_smem, then the plane exponents.
@@ -326,10 +360,37 @@ __device__ __forceinline__ void fx_load(I2* tile, int n, uint32_t* in, SRC src, 
   if (cur >= 0) atomicMax(&in[cur], m);
 }
 
+// After the largest components are known (behind a __syncthreads): the words of
+// the planes and, where one is out of the ordinary, its scaling in the tile.
+// Returns whether any is; ends with a __syncthreads.
+template <typename DST>
+__device__ __forceinline__ bool fx_prepare(I2* tile, int n, int nplanes, uint32_t* in, DST dst) {
+  bool odd = false;
+  if ((int)threadIdx.x < nplanes) {
+    const uint32_t code = fx_classify(in[threadIdx.x]);
+    odd = (code >> 16) != 0u;
+    in[threadIdx.x] = code;
+  }
+  odd = __syncthreads_or(odd);
+  if (odd) {
+    double2* raw = reinterpret_cast<double2*>(tile);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      int pl;
+      double2& v = raw[dst(i, pl)];
+      const uint32_t k = in[pl] >> 16;
+      if (k == FX_NONFINITE) v = make_double2(0.0, 0.0);
+      else if (k != 0u) v = make_double2(scalbn(v.x, k == FX_UP ? FX_ODD_SCALE : -FX_ODD_SCALE),
+                                         scalbn(v.y, k == FX_UP ? FX_ODD_SCALE : -FX_ODD_SCALE));
+    }
+    __syncthreads();
+  }
+  return odd;
+}
+
 template <int SIGN>
-__global__ void __launch_bounds__(512) fft_xy_fx_kernel(Geom g, FFTDir dx, FFTDir dy, double2* __restrict__ data,
-                                                        const int4* __restrict__ twg, const short* __restrict__ posg,
-                                                        int fpb, Lines lx, Lines ly, CopyDiv cd, Batch B) {
+__global__ void __launch_bounds__(FX_MAX_THREADS, 2) fft_xy_fx_kernel(Geom g, const __grid_constant__ FxPass P,
+                                                        double2* __restrict__ data, const int4* __restrict__ twg,
+                                                        const short* __restrict__ posg, int fpb, CopyDiv cd, Batch B) {
   if (batch_skip(B)) return;
   data += blockIdx.z * B.s_delta;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -342,31 +403,39 @@ __global__ void __launch_bounds__(512) fft_xy_fx_kernel(Geom g, FFTDir dx, FFTDi
   const int plane = Lx * Ly;
   double2* fld = data + (int64_t)(blockIdx.y * fpb) * g.V + (int64_t)blockIdx.x * plane;
   __syncthreads();
+  const int n = fpb * plane;
+  auto dst = [&](int i, int& pl) {
+    const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+    pl = f;
+    return f * PS + pos[Lx + y] * RS + pos[x];
+  };
   fx_load(
-      tile, fpb * plane, ps->in0,
+      tile, n, ps->in0,
       [&](int i) {
         const int f = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)f * g.V + (i - f * plane)];
       },
-      [&](int i, int& pl) {
-        const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
-        pl = f;
-        return f * PS + pos[Lx + y] * RS + pos[x];
-      });
+      dst);
   __syncthreads();
+  const bool odd = fx_prepare(tile, n, fpb, ps->in0, dst);
   const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
-  fx_plane<SIGN, true, true>(tile, lx, dx, tw, hx, ly, dy, tw + Lx, hy, ps->in0, ps->mid0);
-  for (int i = threadIdx.x; i < fpb * plane; i += blockDim.x) {
-    const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
-    fld[(int64_t)f * g.V + r] = fx_out(tile[f * PS + y * RS + x], ps->in0[f], ps->mid0[f], hx, hy);
-  }
+  fx_plane<SIGN, true, true>(tile, P, tw, 0, ps->in0, ps->mid0);
+  auto out = [&](auto convert) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+      fld[(int64_t)f * g.V + r] = convert(tile[f * PS + y * RS + x], ps->in0[f], ps->mid0[f], hx, hy);
+    }
+  };
+  if (!odd) out(FxOut());
+  else out(FxOutAny());
 }
 
-template <bool LRN>
-__global__ void __launch_bounds__(512)
-fft_zt_filter_fx_kernel(Geom g, FFTDir dz, FFTDir dt, double2* __restrict__ data, const int4* __restrict__ twg,
-                        const short* __restrict__ posg, const double* __restrict__ K, int xc, int mode, LearnedIO lio,
-                        int4 H, Lines lz, Lines lt, CopyDiv cd, Batch B) {
+// MODE as launch_fft_zt: 0 forward, filter, inverse; -1 / +1 one transform.
+template <int MODE, bool LRN>
+__global__ void __launch_bounds__(FX_MAX_THREADS, 2)
+fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __restrict__ data,
+                        const int4* __restrict__ twg, const short* __restrict__ posg, const double* __restrict__ K,
+                        int xc, LearnedIO lio, int4 H, CopyDiv cd, Batch B) {
   if (batch_skip(B)) return;
   data += blockIdx.z * B.s_delta;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -386,37 +455,42 @@ fft_zt_filter_fx_kernel(Geom g, FFTDir dz, FFTDir dt, double2* __restrict__ data
 #define LGF_ZT_IDX(i)                                                       \
   const int zt = (int)cd.a.div((uint32_t)(i)), xi = (i) - zt * xc;          \
   const int t = (int)cd.b.div((uint32_t)zt), z = zt - t * Lz;
+  auto dst = [&](int i, int& pl) {
+    LGF_ZT_IDX(i)
+    pl = xi;
+    return pos[Lz + t] * TS + pos[z] * xc + xi;
+  };
   fx_load(
       tile, n, ps->in0,
       [&](int i) {
         const int zt = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)zt * plane + sxy + (i - zt * xc)];
       },
-      [&](int i, int& pl) {
-        LGF_ZT_IDX(i)
-        pl = xi;
-        return pos[Lz + t] * TS + pos[z] * xc + xi;
-      });
+      dst);
   __syncthreads();
   const uint32_t hz = fx_headroom(Lz), ht = fx_headroom(Lt);
-  if (mode <= 0) fx_plane<-1, true, false>(tile, lz, dz, tw, hz, lt, dt, tw + Lz, ht, ps->in0, ps->mid0);
-  else fx_plane<+1, true, false>(tile, lz, dz, tw, hz, lt, dt, tw + Lz, ht, ps->in0, ps->mid0);
-  if (mode != 0) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      LGF_ZT_IDX(i)
-      fld[(int64_t)zt * plane + sxy + xi] = fx_out(tile[t * TS + z * xc + xi], ps->in0[xi], ps->mid0[xi], hz, ht);
-    }
+  bool odd = fx_prepare(tile, n, xc, ps->in0, dst);
+  fx_plane<(MODE > 0 ? +1 : -1), true, false>(tile, P, tw, 0, ps->in0, ps->mid0);
+  if (MODE != 0) {
+    auto out = [&](auto convert) {
+      for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        LGF_ZT_IDX(i)
+        fld[(int64_t)zt * plane + sxy + xi] = convert(tile[t * TS + z * xc + xi], ps->in0[xi], ps->mid0[xi], hz, ht);
+      }
+    };
+    if (!odd) out(FxOut());
+    else out(FxOutAny());
     return;
   }
   // the filter in FP64, back into the tile; xc divides the CTA size, so a
   // thread stays in one x column
-  {
+  const int col = (int)threadIdx.x % xc;
+  auto filter = [&](auto convert) {
     const int kit = LRN ? lio.st->iter : 0;
     const bool learned = LRN && lio.mtab != nullptr && lio.st->use_m != 0;
     const float* mtab = lio.mtab + (int64_t)(kit & 1) * lio.nclass;
     uint32_t* snap = (LRN && lio.snap != nullptr) ? lio.snap + ((int64_t)(kit & 1) * 4 + blockIdx.y) * g.V : nullptr;
     const int fy = min(y, Ly - y);
-    const int col = (int)threadIdx.x % xc;
     const uint32_t in = ps->in0[col], mid = ps->mid0[col];
     uint32_t m = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -428,29 +502,40 @@ fft_zt_filter_fx_kernel(Geom g, FFTDir dz, FFTDir dt, double2* __restrict__ data
         k *= (double)__ldg(&mtab[((ft * H.z + fz) * H.y + fy) * H.x + fx]);
       }
       double2* e = reinterpret_cast<double2*>(&tile[t * TS + z * xc + xi]);
-      const double2 v = fx_out(*reinterpret_cast<const I2*>(e), in, mid, hz, ht);
+      const double2 v = convert(*reinterpret_cast<const I2*>(e), in, mid, hz, ht);
       if (LRN && snap != nullptr) snap[(int64_t)zt * plane + sxy + xi] = bf16x2_of<double>(v);
       const double2 w = make_double2(v.x * k, v.y * k);
       m = fx_max(m, w);
       *e = w;
     }
     atomicMax(&ps->in1[col], m);
-  }
+  };
+  if (!odd) filter(FxOut());
+  else filter(FxOutAny());
   __syncthreads();
-  fx_plane<+1, false, false>(tile, lt, dt, tw + Lz, ht, lz, dz, tw, hz, ps->in1, ps->mid1);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  odd = fx_prepare(tile, n, xc, ps->in1, [&](int i, int& pl) {
     LGF_ZT_IDX(i)
-    fld[(int64_t)zt * plane + sxy + xi] =
-        fx_out(tile[pos[Lz + t] * TS + pos[z] * xc + xi], ps->in1[xi], ps->mid1[xi], ht, hz);
-  }
+    pl = xi;
+    return t * TS + z * xc + xi;
+  });
+  fx_plane<+1, false, false>(tile, P, tw, 1, ps->in1, ps->mid1);
+  auto out = [&](auto convert) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      LGF_ZT_IDX(i)
+      fld[(int64_t)zt * plane + sxy + xi] =
+          convert(tile[pos[Lz + t] * TS + pos[z] * xc + xi], ps->in1[xi], ps->mid1[xi], ht, hz);
+    }
+  };
+  if (!odd) out(FxOut());
+  else out(FxOutAny());
 #undef LGF_ZT_IDX
 }
 
 template <bool EXPG>
-__global__ void __launch_bounds__(512)
-fft_xy_inv_gauge_fx_kernel(Geom g, FFTDir dx, FFTDir dy, const double2* __restrict__ data,
+__global__ void __launch_bounds__(FX_MAX_THREADS)
+fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const double2* __restrict__ data,
                            const int4* __restrict__ twg, const short* __restrict__ posg, double2* __restrict__ gf,
-                           double2* __restrict__ Gf, Lines lx, Lines ly, CopyDiv cd, Batch B) {
+                           double2* __restrict__ Gf, CopyDiv cd, Batch B) {
   if (batch_skip(B)) return;
   data += blockIdx.z * B.s_delta;
   gf += blockIdx.z * B.s_g;
@@ -465,27 +550,45 @@ fft_xy_inv_gauge_fx_kernel(Geom g, FFTDir dx, FFTDir dy, const double2* __restri
   const int plane = Lx * Ly;
   const double2* fld = data + (int64_t)blockIdx.x * plane;
   __syncthreads();
+  auto dst = [&](int i, int& pl) {
+    const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
+    pl = f;
+    return f * PS + y * RS + x;
+  };
   fx_load(
       tile, 4 * plane, ps->in0,
       [&](int i) {
         const int f = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)f * g.V + (i - f * plane)];
       },
-      [&](int i, int& pl) {
-        const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
-        pl = f;
-        return f * PS + y * RS + x;
-      });
+      dst);
   __syncthreads();
+  fx_prepare(tile, 4 * plane, 4, ps->in0, dst);
   const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
-  fx_plane<+1, false, true>(tile, lx, dx, tw, hx, ly, dy, tw + Lx, hy, ps->in0, ps->mid0);
+  fx_plane<+1, false, true>(tile, P, tw, 0, ps->in0, ps->mid0);
   for (int i = threadIdx.x; i < plane; i += blockDim.x) {
     const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
     const int o = pos[Lx + y] * RS + pos[x];
+    const int64_t s = (int64_t)blockIdx.x * plane + i;
+    if (!EXPG) {
+      int64_t A[8];
+      bool ok = true;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const I2 v = tile[k * PS + o];
+        const int ex = fx_true_exp(ps->in0[k], ps->mid0[k], hx, hy);
+        A[2 * k] = fx_unit58(v.x, ex, ok);
+        A[2 * k + 1] = fx_unit58(v.y, ex, ok);
+      }
+      if (ok) {
+        gauge_site_fx(A, g.V, s, gf, Gf);
+        continue;
+      }
+    }
     double2 f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) f[k] = fx_out(tile[k * PS + o], ps->in0[k], ps->mid0[k], hx, hy);
-    gauge_site<double, double, 3, EXPG>(f[0], f[1], f[2], f[3], g.V, (int64_t)blockIdx.x * plane + i, gf, Gf);
+    for (int k = 0; k < 4; ++k) f[k] = fx_out_any(tile[k * PS + o], ps->in0[k], ps->mid0[k], hx, hy);
+    gauge_site_fp64<EXPG>(f[0], f[1], f[2], f[3], g.V, s, gf, Gf);
   }
 }
 
@@ -521,65 +624,58 @@ static const int4* fx_table(const Geom& g, const double2* tw) {
   return reinterpret_cast<const int4*>(tw + g.L[0] + g.L[1] + g.L[2] + g.L[3]);
 }
 
+// The (x, y) planes of nf fields side by side in a tile.
+static FxPass xy_pass(const FFTPlan& p, int Lx, int Ly, int nf) {
+  const int RS = Lx + 1, PS = Ly * RS;
+  return FxPass{{p.d[0], p.d[1]}, {make_lines(nf * Ly, Ly, RS, PS, 1), make_lines(nf * Lx, Lx, 1, PS, RS)}};
+}
+
+template <typename K, typename... Args>
+static cudaError_t fx_launch(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, const Args&... args) {
+  const cudaError_t e = allow_smem(kernel, smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<grid, threads, smem, s>>>(args...);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_fft_xy_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
                              int sign, int nfields, cudaStream_t s, const Batch& B) {
   int fpb = std::min(p.fpb_xy, nfields);
   while (nfields % fpb) fpb /= 2;
-  const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
-  const size_t smem = plane_header_bytes(Lx, Ly, 8) + (size_t)fpb * PS * sizeof(double2);
+  const int Lx = g.L[0], Ly = g.L[1];
+  const size_t smem = plane_header_bytes(Lx, Ly, 8) + (size_t)fpb * Ly * (Lx + 1) * sizeof(double2);
   const dim3 grid((unsigned)(g.L[2] * g.L[3]), (unsigned)(nfields / fpb), (unsigned)B.n);
-  const Lines lx = make_lines(fpb * Ly, Ly, RS, PS, 1), ly = make_lines(fpb * Lx, Lx, 1, PS, RS);
+  const FxPass P = xy_pass(p, Lx, Ly, fpb);
   const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
-  cudaError_t e = sign < 0 ? allow_smem(fft_xy_fx_kernel<-1>, smem) : allow_smem(fft_xy_fx_kernel<+1>, smem);
-  if (e != cudaSuccess) return e;
-  if (sign < 0)
-    fft_xy_fx_kernel<-1><<<grid, p.threads_xy, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos, fpb, lx, ly,
-                                                          cd, B);
-  else
-    fft_xy_fx_kernel<+1><<<grid, p.threads_xy, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos, fpb, lx, ly,
-                                                          cd, B);
-  return cudaGetLastError();
+  return fx_launch(sign < 0 ? fft_xy_fx_kernel<-1> : fft_xy_fx_kernel<+1>, grid, p.threads_xy, smem, s, g, P, data,
+                   fx_table(g, tw), pos, fpb, cd, B);
 }
 
 cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, const double2* tw, const short* pos,
                              const double* K, int mode, int nfields, cudaStream_t s, const LearnedIO& lio,
                              const Batch& B) {
-  const size_t smem = p.smem_zt;
   const dim3 grid((unsigned)(g.L[0] / p.xc * g.L[1]), (unsigned)nfields, (unsigned)B.n);
   const bool lrn = mode == 0 && (lio.mtab != nullptr || lio.snap != nullptr);
-  cudaError_t e = lrn ? allow_smem(fft_zt_filter_fx_kernel<true>, smem) : allow_smem(fft_zt_filter_fx_kernel<false>, smem);
-  if (e != cudaSuccess) return e;
   const int4 H = make_int4(g.L[0] / 2 + 1, g.L[1] / 2 + 1, g.L[2] / 2 + 1, g.L[3] / 2 + 1);
   const int xc = p.xc, Lz = g.L[2], Lt = g.L[3], TS = Lz * xc + 1;
-  const Lines lz = make_lines(Lt * xc, xc, 1, TS, xc), lt = make_lines(Lz * xc, xc, 1, xc, TS);
+  const FxPass P{{p.d[2], p.d[3]}, {make_lines(Lt * xc, xc, 1, TS, xc), make_lines(Lz * xc, xc, 1, xc, TS)}};
   const CopyDiv cd{FastDiv::make((uint32_t)xc), FastDiv::make((uint32_t)Lz)};
-  if (lrn)
-    fft_zt_filter_fx_kernel<true><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, fx_table(g, tw), pos, K, xc,
-                                                                   mode, lio, H, lz, lt, cd, B);
-  else
-    fft_zt_filter_fx_kernel<false><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, fx_table(g, tw), pos, K, xc,
-                                                                    mode, lio, H, lz, lt, cd, B);
-  return cudaGetLastError();
+  auto kernel = mode < 0   ? fft_zt_filter_fx_kernel<-1, false>
+                : mode > 0 ? fft_zt_filter_fx_kernel<+1, false>
+                : lrn      ? fft_zt_filter_fx_kernel<0, true>
+                           : fft_zt_filter_fx_kernel<0, false>;
+  return fx_launch(kernel, grid, p.threads_zt, p.smem_zt, s, g, P, data, fx_table(g, tw), pos, K, xc, lio, H, cd, B);
 }
 
 cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
                                    const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
                                    bool exact_exp) {
-  const size_t smem = p.smem_c;
-  cudaError_t e = exact_exp ? allow_smem(fft_xy_inv_gauge_fx_kernel<true>, smem)
-                            : allow_smem(fft_xy_inv_gauge_fx_kernel<false>, smem);
-  if (e != cudaSuccess) return e;
-  const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
-  const Lines lx = make_lines(4 * Ly, Ly, RS, PS, 1), ly = make_lines(4 * Lx, Lx, 1, PS, RS);
+  const int Lx = g.L[0], Ly = g.L[1];
+  const FxPass P = xy_pass(p, Lx, Ly, 4);
   const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
   const dim3 grid((unsigned)(g.L[2] * g.L[3]), 1, (unsigned)B.n);
-  if (exact_exp)
-    fft_xy_inv_gauge_fx_kernel<true><<<grid, p.threads_c, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos,
-                                                                     gfield, Gfield, lx, ly, cd, B);
-  else
-    fft_xy_inv_gauge_fx_kernel<false><<<grid, p.threads_c, smem, s>>>(g, p.d[0], p.d[1], data, fx_table(g, tw), pos,
-                                                                      gfield, Gfield, lx, ly, cd, B);
-  return cudaGetLastError();
+  return fx_launch(exact_exp ? fft_xy_inv_gauge_fx_kernel<true> : fft_xy_inv_gauge_fx_kernel<false>, grid, p.threads_c,
+                   p.smem_c, s, g, P, data, fx_table(g, tw), pos, gfield, Gfield, cd, B);
 }
 
 }  // namespace lgf

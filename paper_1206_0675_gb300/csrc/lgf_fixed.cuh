@@ -2,18 +2,20 @@
 // (elements of SU(3) matrices), on the integer pipe.
 //
 // Why: a GB300 SM issues 2 FP64 operations per clock but 64 IMAD.WIDE
-// (32 x 32 + 64 -> 64 bits), so a real multiply-add of two 59-bit fixed-point
+// (32 x 32 + 64 -> 64 bits), so a real multiply-add of two 60-bit fixed-point
 // numbers, three IMAD.WIDE, takes 3/64 clock against 1/2 clock of the FP64 pipe.
 // Its rounding is finer too: every product is kept to 2^-60 absolute, while
 // an FP64 operation on numbers of order one rounds at 2^-54 (measured on the
 // link update of random SU(3) fields: see update_kernel).
 //
-// Format: a = (H 2^29 + L) 2^-59 with |a| < FX_LIM = 1.125; H and L are
-// 32-bit signed words, |H| <= 1.125 2^30 and |L| < 2^29.  An accumulator
-// keeps two 64-bit sums, hi += H H' (unit 2^-60) and mid += H L' + L H'
-// (unit 2^-89); L L' < 2^-60 is dropped.  Six real products (one component
-// of a row times column) stay below 6 (1.125 2^30)^2 < 2^63 in hi and
-// 12 (1.125 2^30) 2^29 < 2^63 in mid, so sums never overflow whatever the
+// Format: a = (H 2^30 + L) 2^-60 with |a| < FX_LIM = 1.125; H and L are
+// 32-bit signed words, |H| <= 1.125 2^30 and |L| <= 2^29 (centred, so that what
+// is dropped has no preferred sign: a bias of a few 2^-62 per product adds up
+// over the steps of a converging field, whose theta it shows in).  An
+// accumulator keeps two 64-bit sums, hi += H H' (unit 2^-60) and mid += H L' +
+// L H' (unit 2^-90); L L' < 2^-62 is dropped.  Six real products (one
+// component of a row times column) stay below 6 (1.125 2^30)^2 < 2^63 in hi
+// and 12 (1.125 2^30) 2^29 < 2^63 in mid, so sums never overflow whatever the
 // matrices are, as long as each entry is below FX_LIM.  Callers test that
 // (fx_bad) and take an FP64 path otherwise, which also carries infinities
 // and NaN through.
@@ -54,30 +56,41 @@ __device__ __forceinline__ uint32_t shr32_clamp(uint32_t x, uint32_t s) {
   return r;
 }
 
-// Fixed point from FP64, |a| < FX_LIM; bits below 2^-59 are cut off.
+// The operand of a number in units of 2^-60.
+__device__ __forceinline__ Fx fx_operand(int64_t r60) {
+  return Fx{(int)((r60 + ((int64_t)1 << 29)) >> 30), (int)((uint32_t)r60 << 2) >> 2};
+}
+
+// Fixed point from FP64, |a| < FX_LIM; bits below 2^-60 are cut off.
 // With the leading one at bit 63 the significand M has the value
-// M 2^(e - 1086), so the magnitude in units of 2^-59 is M >> (1027 - e).
+// M 2^(e - 1086), so the magnitude in units of 2^-60 is M >> (1026 - e).
 __device__ __forceinline__ Fx fx_from(double a) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
-  const uint32_t s = 1027u - ((hi >> 20) & 0x7ffu);
-  const int sg = (int)hi >> 31;
-  const uint32_t h = shr32_clamp(mh, s - 3u);
-  const uint32_t l = (uint32_t)shr64_clamp(((uint64_t)mh << 32) | ml, s) & 0x1fffffffu;
-  return Fx{((int)h ^ sg) - sg, ((int)l ^ sg) - sg};
+  const int64_t sg = (int64_t)((int)hi >> 31);
+  return fx_operand(
+      ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, 1026u - ((hi >> 20) & 0x7ffu)) ^ sg) - sg);
 }
 __device__ __forceinline__ FxC fx_from(double2 a) { return FxC{fx_from(a.x), fx_from(a.y)}; }
 __device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }
+
+// c + a b with a 64-bit sum: one IMAD.WIDE (written out, so that sums of
+// products are not taken apart into products and 64-bit additions).
+__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c) {
+  int64_t r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
 
 // Two-part accumulator of real products.
 struct FxAcc {
   int64_t hi, mid;
 };
-__device__ __forceinline__ FxAcc fx_zero() { return FxAcc{0, (int64_t)1 << 28}; }  // rounds when mid is shifted by 29
+__device__ __forceinline__ FxAcc fx_zero() { return FxAcc{0, (int64_t)1 << 29}; }  // rounds when mid is shifted by 30
 __device__ __forceinline__ void fx_mac(FxAcc& s, Fx a, Fx b) {
-  s.hi += (int64_t)a.h * b.h;
-  s.mid += (int64_t)a.h * b.l;
-  s.mid += (int64_t)a.l * b.h;
+  s.hi = mad_wide(a.h, b.h, s.hi);
+  s.mid = mad_wide(a.h, b.l, s.mid);
+  s.mid = mad_wide(a.l, b.h, s.mid);
 }
 // s += a b and s += a conj(b) for complex numbers; na = -a where a sign is needed
 __device__ __forceinline__ void fx_cmac(FxAcc& re, FxAcc& im, const FxC& a, Fx nay, const FxC& b) {
@@ -99,16 +112,11 @@ __device__ __forceinline__ void fx_cmacc(FxAcc& re, FxAcc& im, const FxC& a, Fx 
 // bad if it reaches 2 FX_LIM.
 constexpr uint32_t FX_SUM_OFF = 0x12000000u;  // 1.125 in units of 2^-28
 __device__ __forceinline__ int64_t fx_sum60(const FxAcc& s, uint32_t& t) {
-  const int64_t r = s.hi + (s.mid >> 29);
+  const int64_t r = s.hi + (s.mid >> 30);
   t = max(t, (uint32_t)(r >> 32) + FX_SUM_OFF);
   return r;
 }
 __device__ __forceinline__ bool fx_bad(uint32_t m, uint32_t t) { return m >= FX_LIM_HI || t >= 2u * FX_SUM_OFF; }
-// The sum as an operand of the next product.
-__device__ __forceinline__ Fx fx_operand(int64_t r60) {
-  return Fx{(int)(r60 >> 30), (int)((uint32_t)(r60 >> 1) & 0x1fffffffu)};
-}
-
 // 64-bit fixed point in units of 2^-58 from FP64, |a| < 2 (zero for what lies
 // below): for sums of up to 16 entries.
 __device__ __forceinline__ int64_t fx58_from(double a) {
@@ -118,9 +126,7 @@ __device__ __forceinline__ int64_t fx58_from(double a) {
   const int64_t sg = (int64_t)((int)hi >> 31);
   return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, s) ^ sg) - sg;
 }
-__device__ __forceinline__ Fx fx_operand58(int64_t a58) {
-  return Fx{(int)(a58 >> 28), (int)((uint32_t)(a58 << 1) & 0x1fffffffu)};
-}
+__device__ __forceinline__ Fx fx_operand58(int64_t a58) { return fx_operand(a58 << 2); }
 
 // FP64 value of a 64-bit integer n times 2^-K, rounded to nearest, on the
 // FP64 pipe: the two halves are placed into the significands of doubles of
@@ -134,8 +140,8 @@ template <int K> __device__ __forceinline__ double fx_to_double_fp(int64_t n) {
   return (h - off) + l;
 }
 
-// The same on the integer pipe, for |n| >= 2^32 (ok = false below; ties go
-// away from zero): leading one to bit 62, half a unit of the last kept bit,
+// The same on the integer pipe, for |n| >= 2^32 (ok = false below): leading
+// one to bit 62, rounding of the 10 bits below the significand, ties to even,
 // then the significand's leading one and a carry add into the exponent.
 template <int K> __device__ __forceinline__ double fx_to_double_int(int64_t n, bool& ok) {
   const int sg = (int)(n >> 63);
@@ -143,7 +149,8 @@ template <int K> __device__ __forceinline__ double fx_to_double_int(int64_t n, b
   const uint32_t uh = (uint32_t)(u >> 32);
   ok = ok && uh != 0u;
   const int lz = __clz((int)uh);
-  const uint64_t m = ((u << (lz - 1)) + 0x200ull) >> 10;
+  const uint64_t v = u << (lz - 1);
+  const uint64_t m = (v + 0x1ffull + (((uint32_t)v >> 10) & 1u)) >> 10;
   const uint32_t ew = (uint32_t)(1023 + 62 - K) * 0x100000u - (uint32_t)lz * 0x100000u;
   const uint32_t rh = (uint32_t)(m >> 32) + ew;
   return __hiloint2double((int)(rh | ((uint32_t)sg & 0x80000000u)), (int)(uint32_t)m);
@@ -170,7 +177,7 @@ __device__ __forceinline__ void fx_cross_conj(FxAcc& re, FxAcc& im, const FxC& a
 
 // Integer of an FP64 number in units that make the block's largest magnitude
 // fit (see the transform passes): M >> (base - e), M with its leading one at
-// bit 63.  base >= 100, so zeros and numbers 2^-64 below the block's largest
+// bit 63.  base >= 64, so zeros and numbers 2^-64 below the block's largest
 // give zero.
 __device__ __forceinline__ int64_t bfp_from(double a, uint32_t base) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
@@ -179,16 +186,16 @@ __device__ __forceinline__ int64_t bfp_from(double a, uint32_t base) {
   return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, base - ((hi >> 20) & 0x7ffu)) ^ sg) - sg;
 }
 
-// FP64 value of n 2^ex rounded to nearest, any n and ex.
-static __device__ __noinline__ double bfp_to_double_any(int64_t n, int ex) { return scalbn(fx_to_double_fp<0>(n), ex); }
-
-// The same on the integer pipe where the block's exponents are far from the
-// ends of the FP64 range (safe) and |n| >= 2^32.
-__device__ __forceinline__ double bfp_to_double(int64_t n, int ex, bool safe) {
+// FP64 value of n 2^ex rounded to nearest, where the result is far from the
+// ends of the FP64 range or zero.
+__device__ __forceinline__ double bfp_to_double(int64_t n, int ex) {
   const int sg = (int)(n >> 63);
   const uint64_t u = (uint64_t)((n ^ (int64_t)sg) - (int64_t)sg);
   const uint32_t uh = (uint32_t)(u >> 32);
-  if (!safe || uh == 0u) return bfp_to_double_any(n, ex);
+  if (uh == 0u) {  // rare: zeros and numbers 2^-29 below the block's largest
+    const double r = fx_to_double_fp<0>(n);
+    return r == 0.0 ? r : __hiloint2double(__double2hiint(r) + ex * 0x100000, __double2loint(r));
+  }
   const int lz = __clz((int)uh);
   const uint64_t m = ((u << (lz - 1)) + 0x200ull) >> 10;
   const uint32_t rh = (uint32_t)(m >> 32) + (uint32_t)(1023 + 62 + ex - lz) * 0x100000u;
@@ -206,10 +213,66 @@ __device__ __forceinline__ Bfp2 bfp_limbs(int64_t x) { return Bfp2{(int)(x >> 30
 // rounded to the nearest unit (l l' 2^-60 is dropped, below 2^-30 of a unit).
 __device__ __forceinline__ int64_t bfp_mul(int64_t x, int wh, int wl) {
   const Bfp2 a = bfp_limbs(x);
-  int64_t mid = (int64_t)1 << 29;
-  mid += (int64_t)a.h * wl;
-  mid += (int64_t)a.l * wh;
-  return (int64_t)a.h * wh + (mid >> 30);
+  const int64_t mid = mad_wide(a.l, wh, mad_wide(a.h, wl, (int64_t)1 << 29));
+  return mad_wide(a.h, wh, mid >> 30);
+}
+
+// ---------------------------------------------------------------------------
+// g of FP64 lanes, stored as fixed-point operands
+// ---------------------------------------------------------------------------
+
+// One complex entry is four words (re h, re l, im h, im l), the 16 bytes of
+// an FP64 one, so that the update reads its operands as they are (five
+// threads read every g(x): converting FP64 entries cost the update a seventh
+// of its instructions).  The unit 2^-60 is below the noise of any g: the
+// divergence that it comes from is a sum of FP64 entries of order one.  A g
+// that is not finite is marked in its first word.
+constexpr int FX_G_NAN = (int)0x80000000u;
+
+__device__ __forceinline__ FxC fxg_unpack(int4 w) { return FxC{Fx{w.x, w.y}, Fx{w.z, w.w}}; }
+__device__ __forceinline__ int4 fxg_pack(const FxC& a) { return make_int4(a.x.h, a.x.l, a.y.h, a.y.l); }
+__device__ __forceinline__ double fx_value(Fx a) { return fx_to_double_fp<60>(((int64_t)a.h << 30) + a.l); }
+
+// g(s) in FP64 (NaN where marked).
+__device__ __forceinline__ void fxg_load(const double2* __restrict__ gf, int64_t V, int64_t s, M3<double>& M) {
+  const int4* p = reinterpret_cast<const int4*>(gf);
+  const bool bad = __ldg(&p[s]).x == FX_G_NAN;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const FxC w = fxg_unpack(__ldg(&p[e * V + s]));
+    M.e[e / 3][e % 3] = bad ? make_double2(NAN, NAN) : make_double2(fx_value(w.x), fx_value(w.y));
+  }
+}
+// The store, from FP64 rows.
+__device__ __forceinline__ void fxg_store(double2* __restrict__ gf, int64_t V, int64_t s, const double2 a[3],
+                                          const double2 b[3], const double2 c[3]) {
+  int4* p = reinterpret_cast<int4*>(gf);
+  uint32_t m = 0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) m = fx_max(fx_max(fx_max(m, a[j]), b[j]), c[j]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    int4 w = fxg_pack(fx_from(a[j]));
+    if (j == 0 && m >= FX_LIM_HI) w.x = FX_G_NAN;
+    p[j * V + s] = w;
+    p[(3 + j) * V + s] = fxg_pack(fx_from(b[j]));
+    p[(6 + j) * V + s] = fxg_pack(fx_from(c[j]));
+  }
+}
+
+// y/2 in units of 2^-60 for y = 1/sqrt(n), n in units of 2^-60 and
+// 0.2 < n < 2: the FP32 estimate, a 23-bit integer, and one third-order step
+// (e = 1 - n y0^2 below 2^-19 in magnitude, so 5 e^3 / 16 is below 2^-58 of y0;
+// see rsqrt_fp64).
+__device__ __forceinline__ int64_t fx_half_rsqrt(int64_t n) {
+  const float f = (float)(int)(n >> 30) * 9.3132257e-10f;  // 2^-30
+  const int y0 = __float2int_rn(rsqrtf(f) * 4194304.f);    // unit 2^-22
+  const int64_t t = ((int64_t)((int)(n >> 30)) * y0 << 8) + ((int64_t)((int)n & 0x3fffffff) * y0 >> 22);
+  const int64_t q = ((int64_t)((int)(t >> 30)) * y0 << 8) + ((int64_t)((int)t & 0x3fffffff) * y0 >> 22);
+  const int64_t e = ((int64_t)1 << 60) - q;
+  const int eh = (int)(e >> 20);
+  const int64_t c = (e >> 1) + (3 * ((int64_t)eh * eh) >> 23);
+  return ((int64_t)y0 << 37) + ((int64_t)((int)(c >> 20)) * y0 >> 3) + ((int64_t)((int)c & 0xfffff) * y0 >> 23);
 }
 
 }  // namespace lgf

@@ -2,6 +2,7 @@
 // and the exact exponential, and the store of g (and G <- g G).
 #pragma once
 
+#include "lgf_fixed.cuh"
 #include "lgf_internal.h"
 
 namespace lgf {
@@ -220,37 +221,46 @@ __device__ __forceinline__ void gauge_exp_from_packed(double2 f0, double2 f1, do
   for (int j = 0; j < 3; ++j) v[j] = cscale<double>(v[j], i2);
 }
 
-// Stores rows u, v (precision RG) and, where needed, row 3 = (u x v)^*.
+// G(s) <- g G(s) of one site, full 3x3 in precision RG.
+template <typename RG>
+__device__ __forceinline__ void accumulate_gauge(int64_t V, int64_t s, const C2<RG> a[3], const C2<RG> b[3],
+                                                 const C2<RG> c[3], C2<RG>* __restrict__ Gf) {
+  C2<RG> Go[3][3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int col = 0; col < 3; ++col) Go[r][col] = Gf[(r * 3 + col) * V + s];
+  const C2<RG>* rows[3] = {a, b, c};
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int col = 0; col < 3; ++col) {
+      C2<RG> acc = cmul<RG>(rows[r][0], Go[0][col]);
+      acc = cfma<RG>(rows[r][1], Go[1][col], acc);
+      acc = cfma<RG>(rows[r][2], Go[2][col], acc);
+      Gf[(r * 3 + col) * V + s] = acc;
+    }
+}
+
+// Stores rows u, v (precision RG) and, where needed, row 3 = (u x v)^*, and
+// G <- g G where tracked.  FP64 lanes keep g as fixed-point operands.
 template <typename RG, int GROWS>
 __device__ __forceinline__ void store_gauge_rows(int64_t V, int64_t s, const C2<RG> a[3], const C2<RG> b[3],
                                                  C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf) {
   C2<RG> c[3];
   const bool need_c = (GROWS == 3) || (Gf != nullptr);
   if (need_c) su3_third_row<RG>(a, b, c);
+  if constexpr (sizeof(RG) == sizeof(double)) {
+    fxg_store(gf, V, s, a, b, c);
+  } else {
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    gf[(0 * 3 + j) * V + s] = a[j];
-    gf[(1 * 3 + j) * V + s] = b[j];
-    if (GROWS == 3) gf[(2 * 3 + j) * V + s] = c[j];
+    for (int j = 0; j < 3; ++j) {
+      gf[(0 * 3 + j) * V + s] = a[j];
+      gf[(1 * 3 + j) * V + s] = b[j];
+      if (GROWS == 3) gf[(2 * 3 + j) * V + s] = c[j];
+    }
   }
-  if (Gf != nullptr) {
-    // G <- g G (full 3x3, precision RG)
-    C2<RG> Go[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int col = 0; col < 3; ++col) Go[r][col] = Gf[(r * 3 + col) * V + s];
-    const C2<RG>* rows[3] = {a, b, c};
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int col = 0; col < 3; ++col) {
-        C2<RG> acc = cmul<RG>(rows[r][0], Go[0][col]);
-        acc = cfma<RG>(rows[r][1], Go[1][col], acc);
-        acc = cfma<RG>(rows[r][2], Go[2][col], acc);
-        Gf[(r * 3 + col) * V + s] = acc;
-      }
-  }
+  if (Gf != nullptr) accumulate_gauge<RG>(V, s, a, b, c, Gf);
 }
 
 // g(x) of one site from its packed filtered field and its store (and G <- g G).
@@ -272,6 +282,147 @@ __device__ __forceinline__ void gauge_site(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f
     gauge_rows<RG>(f0, f1, f2, f3, a, b);
   }
   store_gauge_rows<RG, GROWS>(V, s, a, b, gf, Gf);
+}
+
+// The FP64 path of a site outside the fixed-point range.
+template <bool EXPG>
+static __device__ __noinline__ void gauge_site_fp64(double2 f0, double2 f1, double2 f2, double2 f3, int64_t V,
+                                                    int64_t s, double2* __restrict__ gf, double2* __restrict__ Gf) {
+  gauge_site<double, double, 3, EXPG>(f0, f1, f2, f3, V, s, gf, Gf);
+}
+
+static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, const double2* __restrict__ gf,
+                                                          double2* __restrict__ Gf) {
+  M3<double> g;
+  fxg_load(gf, V, s, g);
+  accumulate_gauge<double>(V, s, g.e[0], g.e[1], g.e[2], Gf);
+}
+
+// G(s) <- g G(s) in fixed point, for g as stored (a call: its operands would
+// otherwise crowd the registers of every pass, tracked transform or not).
+static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, const double2* __restrict__ gf,
+                                                        double2* __restrict__ Gf) {
+  const int4* p = reinterpret_cast<const int4*>(gf);
+  uint32_t m = 0, t = 0;
+  FxC G[3][3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2 v = Gf[(r * 3 + c) * V + s];
+      m = fx_max(m, v);
+      G[r][c] = fx_from(v);
+    }
+  double2 o[3][3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    FxC g[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) g[k] = fxg_unpack(p[(r * 3 + k) * V + s]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(re, im, g[k], fx_neg(g[k].y), G[k][c]);
+      bool bx = true, by = true;
+      const int64_t x = fx_sum60(re, t), y = fx_sum60(im, t);
+      o[r][c].x = fx_to_double_int<60>(x, bx);
+      o[r][c].y = fx_to_double_int<60>(y, by);
+      if (!bx) o[r][c].x = fx_to_double_fp<60>(x);
+      if (!by) o[r][c].y = fx_to_double_fp<60>(y);
+    }
+  }
+  if (fx_bad(m, t)) {
+    accumulate_gauge_fp64(V, s, gf, Gf);
+    return;
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Gf[(r * 3 + c) * V + s] = o[r][c];
+}
+
+// g = reunitarize(1 + X) of one site in fixed point: A holds the components of
+// (f0, f1, f2, f3) in units of 2^-58, each below 1 in magnitude.
+//
+// Rows are halved so that everything stays within the operand range (a
+// projection does not see the scale): with r1 = (1 + i a, f1, f2)/2 and
+// r2 = (-conj f1, 1 + i d, f3)/2, |r1|^2 and |r2|^2 lie in [1/4, 3/2); then
+// u = r1 / |r1|, w = r2 - <u, r2> u with |w| in [1/2, 5/4) (the singular
+// values of 1 + X are at least 1) and v = w / |w|; row 3 is (u x v)^*.
+// <r1, r2> = (a + d)(Im f1 + i Re f1) + conj(f2) f3 as in gram_schmidt_factors.
+// 66 real products on the integer pipe against 77 operations on the FP64 pipe.
+__device__ __forceinline__ void gauge_site_fx(const int64_t A[8], int64_t V, int64_t s, double2* __restrict__ gf,
+                                              double2* __restrict__ Gf) {
+  uint32_t t = 0;  // no sum can leave the range here
+  const int64_t half = (int64_t)1 << 58;
+  Fx f[8];  // a, d, f1, f2, f3
+#pragma unroll
+  for (int k = 0; k < 8; ++k) f[k] = fx_operand(2 * A[k]);
+  const FxC f1{f[2], f[3]}, f2{f[4], f[5]}, f3{f[6], f[7]};
+  FxAcc n = fx_zero();
+  n.hi = half;  // 1/4
+  fx_mac(n, f[0], f[0]);
+  fx_mac(n, f1.x, f1.x);
+  fx_mac(n, f1.y, f1.y);
+  fx_mac(n, f2.x, f2.x);
+  fx_mac(n, f2.y, f2.y);
+  const int64_t yh = fx_half_rsqrt(fx_sum60(n, t));
+  const Fx y = fx_operand(yh);
+  // u = 2 (y/2) r1
+  auto scaled = [&](Fx a, Fx b) {
+    FxAcc p = fx_zero();
+    fx_mac(p, a, b);
+    return 2 * fx_sum60(p, t);
+  };
+  FxC g[3][3];
+  g[0][0] = FxC{y, fx_operand(scaled(f[0], y))};
+  g[0][1] = FxC{fx_operand(scaled(f1.x, y)), fx_operand(scaled(f1.y, y))};
+  g[0][2] = FxC{fx_operand(scaled(f2.x, y)), fx_operand(scaled(f2.y, y))};
+  // <r1, r2>, then <u, r2>
+  const Fx sm = fx_operand(2 * (A[0] + A[1]));
+  FxAcc cr = fx_zero(), ci = fx_zero();
+  fx_mac(cr, sm, f1.y);
+  fx_mac(cr, f2.x, f3.x);
+  fx_mac(cr, f2.y, f3.y);
+  fx_mac(ci, sm, f1.x);
+  fx_mac(ci, f2.x, f3.y);
+  fx_mac(ci, fx_neg(f2.y), f3.x);
+  const Fx kx = fx_operand(-scaled(fx_operand(fx_sum60(cr, t)), y));
+  const Fx ky = fx_operand(-scaled(fx_operand(fx_sum60(ci, t)), y));
+  const FxC k{kx, ky};  // -<u, r2>
+  // w = r2 - <u, r2> u
+  const int64_t r2[3][2] = {{-2 * A[2], 2 * A[3]}, {2 * half, 2 * A[1]}, {2 * A[6], 2 * A[7]}};
+  FxC w[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    FxAcc re = fx_zero(), im = fx_zero();
+    re.hi = r2[j][0];
+    im.hi = r2[j][1];
+    fx_cmac(re, im, k, fx_neg(ky), g[0][j]);
+    w[j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+  }
+  n = fx_zero();
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    fx_mac(n, w[j].x, w[j].x);
+    fx_mac(n, w[j].y, w[j].y);
+  }
+  const Fx z = fx_operand(fx_half_rsqrt(fx_sum60(n, t)));
+#pragma unroll
+  for (int j = 0; j < 3; ++j) g[1][j] = FxC{fx_operand(scaled(w[j].x, z)), fx_operand(scaled(w[j].y, z))};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    FxAcc re = fx_zero(), im = fx_zero();
+    fx_cross_conj(re, im, g[0][(j + 1) % 3], g[0][(j + 2) % 3], g[1][(j + 1) % 3], g[1][(j + 2) % 3]);
+    g[2][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+  }
+  int4* p = reinterpret_cast<int4*>(gf);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) p[(r * 3 + j) * V + s] = fxg_pack(g[r][j]);
+  if (Gf != nullptr) accumulate_gauge_fx(V, s, gf, Gf);
 }
 
 }  // namespace lgf

@@ -125,6 +125,8 @@ template <typename R, int ROWS>
 cudaError_t launch_sites_to_aos(const Geom& g, const C2<R>* field, double* aos, cudaStream_t s);
 template <typename R, int ROWS>
 cudaError_t launch_sites_from_aos(const Geom& g, const double* aos, C2<R>* field, cudaStream_t s);
+// g of an FP64 lane (fixed-point operands, lgf_fixed.cuh) -> AoS.
+cudaError_t launch_gauge_to_aos(const Geom& g, const double2* gfield, double* aos, cudaStream_t s);
 // Packed divergence fields -> 3x3 anti-Hermitian matrices in the site AoS layout.
 template <typename R>
 cudaError_t launch_delta_to_aos(const Geom& g, const C2<R>* delta, double* aos, cudaStream_t s);
@@ -151,8 +153,10 @@ cudaError_t launch_reunitarize_links(const Geom& g, C2<R>* links, DevState* st, 
 cudaError_t launch_c2_f64_to_f32(const double2* in, float2* out, int64_t n, cudaStream_t s);
 cudaError_t launch_c2_f32_to_f64(const float2* in, double2* out, int64_t n, cudaStream_t s);
 
-// G64 = reunitarize(G32) in FP64 (3-row FP32 site field -> 3-row FP64 site field).
-cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* G64, cudaStream_t s);
+// reunitarize(G32) in FP64 (3-row FP32 site field) as g of the FP64 lane and,
+// where given, as the 3-row FP64 site field G64.
+cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* gfield, double2* G64,
+                                            cudaStream_t s);
 
 // Site field G <- 1.
 template <typename R, int ROWS>

@@ -578,131 +578,143 @@ template <int LROWS>
 __device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatField<double, 3> Gf, int mu, int64_t s,
                                               int64_t sf) {
   M3<double> gx, u, h, o;
-  Gf.load_ro(0, s, gx);
+  fxg_load(Gf.p, Gf.V, s, gx);
   U.load(mu, s, u);
-  Gf.load_ro(0, sf, h);
+  fxg_load(Gf.p, Gf.V, sf, h);
   gauge_product<double>(gx, u, h, o);
   U.store(mu, s, o);
 }
 
-// FP64 links: the two products in fixed point on the integer pipe
-// (lgf_fixed.cuh), row 3 of 18-real links on the FP64 pipe beside it.
+// FP64 links: the two products and row 3 in fixed point on the integer pipe
+// (lgf_fixed.cuh); g arrives as operands.
 // Links whose off-diagonal entries are all below 2^-12, where FP64 rounds
 // finer than the fixed-point unit, and entries outside its range take the
 // FP64 path.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
 // end at 2.4e-15 (FP64 products: 2.6e-15).
-// Bound by instruction issue (9300 per site, 12 warps per SM at 168
-// registers).  32^4: 18-real 518 us, 12-real 626 us; with FP64 products 1176
-// and 1177 us at 95 % of the FP64 pipe.
+// Bound by the integer pipe (2040 instructions a link, 504 of them IMAD.WIDE,
+// which run at about 30 of their 64 lanes a clock when all operands vary).
+// 32^4, us: 18-real 505, 12-real 431; with FP64 products 1176 and 1177 at 95 %
+// of the FP64 pipe.
+// One thread per link: a CTA takes 32 sites, one direction per warp, so that
+// the 24 operand loads of a link are all in flight before its arithmetic and
+// g(x) comes from L1 for three of the four warps.
 template <int LROWS>
-__global__ void __launch_bounds__(UPDATE_THREADS)
+__global__ void __launch_bounds__(UPDATE_THREADS, 6)
 update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batch B) {
   if (batch_skip(B)) return;
   U.p += blockIdx.z * B.s_links;
   Gf.p += blockIdx.z * B.s_g;
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t s = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int mu = threadIdx.x >> 5;
   if (s >= g.V) return;
   int c[4];
   site_coords(g, s, c);
-  uint32_t mg = 0;
-  FxC gx[2][3];
+  int64_t sf, sb;
+  site_nbrs_sel(g, s, c, mu, sf, sb);
+  const int4* G = reinterpret_cast<const int4*>(Gf.p);
+  double2 u[LROWS][3];
+  int4 g4[2][3], h4[3][3];
+#pragma unroll
+  for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) u[i][j] = U.p[U.off(mu, i, j, s)];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) g4[i][j] = __ldg(&G[Gf.off(0, i, j, s)]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) h4[i][j] = __ldg(&G[Gf.off(0, i, j, sf)]);
+  uint32_t m = 0, t = 0;
+#pragma unroll
+  for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) m = fx_max(m, u[i][j]);
+  const uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
+  // T = g(x)[rows 0,1] U
+  FxC T[2][3], ux[3][3];
+#pragma unroll
+  for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ux[i][j] = fx_from(u[i][j]);
+  if (LROWS == 2) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      FxAcc re = fx_zero(), im = fx_zero();
+      fx_cross_conj(re, im, ux[0][(j + 1) % 3], ux[0][(j + 2) % 3], ux[1][(j + 1) % 3], ux[1][(j + 2) % 3]);
+      ux[2][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    FxC gx[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gx[k] = fxg_unpack(g4[i][k]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(re, im, gx[k], fx_neg(gx[k].y), ux[k][j]);
+      T[i][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
+    }
+  }
+  // rows 0,1 of T h^dagger
+  int64_t n[2][3][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const double2 v = __ldg(&Gf.p[Gf.off(0, i, j, s)]);
-      mg = fx_max(mg, v);
-      gx[i][j] = fx_from(v);
+      FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmacc(re, im, T[i][k], fx_neg(T[i][k].x), fxg_unpack(h4[j][k]));
+      n[i][j][0] = fx_sum60(re, t);
+      n[i][j][1] = fx_sum60(im, t);
     }
-#pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
-    int64_t sf, sb;
-    site_nbrs_sel(g, s, c, mu, sf, sb);
-    double2 u[LROWS][3], h[3][3];
-#pragma unroll
-    for (int i = 0; i < LROWS; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) u[i][j] = U.p[U.off(mu, i, j, s)];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) h[i][j] = __ldg(&Gf.p[Gf.off(0, i, j, sf)]);
-    uint32_t m = mg, t = 0;
-#pragma unroll
-    for (int i = 0; i < LROWS; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) m = fx_max(m, u[i][j]);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) m = fx_max(m, h[i][j]);
-    uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
-    // T = g(x)[rows 0,1] U
-    FxC T[2][3];
-    FxC ux[3][3];
-#pragma unroll
-    for (int i = 0; i < LROWS; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) ux[i][j] = fx_from(u[i][j]);
-    if (LROWS == 2) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        FxAcc re = fx_zero(), im = fx_zero();
-        fx_cross_conj(re, im, ux[0][(j + 1) % 3], ux[0][(j + 2) % 3], ux[1][(j + 1) % 3], ux[1][(j + 2) % 3]);
-        ux[2][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
-      }
-    }
+  // row 3 of 18-real links: (row 1 x row 2)^*
+  int64_t n3[3][2];
+  if (LROWS == 3) {
+    FxC r[2][3];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        FxAcc re = fx_zero(), im = fx_zero();
-#pragma unroll
-        for (int k = 0; k < 3; ++k) fx_cmac(re, im, gx[i][k], fx_neg(gx[i][k].y), ux[k][j]);
-        T[i][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
-      }
-    // rows 0,1 of T h^dagger
-    int64_t n[2][3][2];
-    bool big = true;
+      for (int j = 0; j < 3; ++j) r[i][j] = FxC{fx_operand(n[i][j][0]), fx_operand(n[i][j][1])};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      FxC hj[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) hj[k] = fx_from(h[j][k]);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        FxAcc re = fx_zero(), im = fx_zero();
-#pragma unroll
-        for (int k = 0; k < 3; ++k) fx_cmacc(re, im, T[i][k], fx_neg(T[i][k].x), hj[k]);
-        n[i][j][0] = fx_sum60(re, t);
-        n[i][j][1] = fx_sum60(im, t);
-      }
+      FxAcc re = fx_zero(), im = fx_zero();
+      fx_cross_conj(re, im, r[0][(j + 1) % 3], r[0][(j + 2) % 3], r[1][(j + 1) % 3], r[1][(j + 2) % 3]);
+      n3[j][0] = fx_sum60(re, t);
+      n3[j][1] = fx_sum60(im, t);
     }
-    if (fx_bad(m, t) || w < FX_WEAK_HI) {
-      update_link_fp64<LROWS>(U, Gf, mu, s, sf);
-      continue;
+  }
+  if (fx_bad(m, t) || w < FX_WEAK_HI || g4[0][0].x == FX_G_NAN || h4[0][0].x == FX_G_NAN) {
+    update_link_fp64<LROWS>(U, Gf, mu, s, sf);
+    return;
+  }
+  bool big = true;
+  double2 o[LROWS][3];
+#pragma unroll
+  for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int64_t x = i < 2 ? n[i][j][0] : n3[j][0], y = i < 2 ? n[i][j][1] : n3[j][1];
+      // row 3 on the FP64 pipe, which is idle otherwise
+      o[i][j] = i == 2 ? make_double2(fx_to_double_fp<60>(x), fx_to_double_fp<60>(y))
+                       : make_double2(fx_to_double_int<60>(x, big), fx_to_double_int<60>(y, big));
     }
-    double2 o[3][3];
-    if (LROWS == 3) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-          o[i][j] = make_double2(fx_to_double_int<60>(n[i][j][0], big), fx_to_double_int<60>(n[i][j][1], big));
-    }
-    if (LROWS == 2 || !big) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-          o[i][j] = make_double2(fx_to_double_fp<60>(n[i][j][0]), fx_to_double_fp<60>(n[i][j][1]));
-    }
-    if (LROWS == 3) su3_third_row<double>(o[0], o[1], o[2]);
+  if (!big) {  // an entry below 2^-28, zeros among them
 #pragma unroll
     for (int i = 0; i < LROWS; ++i)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) U.p[U.off(mu, i, j, s)] = o[i][j];
+      for (int j = 0; j < 3; ++j) {
+        const int64_t x = i < 2 ? n[i][j][0] : n3[j][0], y = i < 2 ? n[i][j][1] : n3[j][1];
+        o[i][j] = make_double2(fx_to_double_fp<60>(x), fx_to_double_fp<60>(y));
+      }
   }
+#pragma unroll
+  for (int i = 0; i < LROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) U.p[U.off(mu, i, j, s)] = o[i][j];
 }
 
 template <typename R, int LROWS, int GROWS>
@@ -713,7 +725,8 @@ cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cuda
   const dim3 grid((unsigned)nb, 1, (unsigned)B.n);
   if constexpr (sizeof(R) == sizeof(double)) {
     static_assert(GROWS == 3, "FP64 lanes keep three rows of g");
-    update_fx_kernel<LROWS><<<grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
+    const dim3 fx_grid((unsigned)((g.V + 31) / 32), 1, (unsigned)B.n);
+    update_fx_kernel<LROWS><<<fx_grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
   } else {
     update_kernel<R, LROWS, GROWS><<<grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
   }
@@ -723,6 +736,15 @@ cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cuda
 // ---------------------------------------------------------------------------
 // undo of a rejected step: U_mu(x) <- g^dag(x) U_mu(x) g(x + mu^), G <- g^dag G
 // ---------------------------------------------------------------------------
+
+// g(s) of a lane as a matrix (FP64 lanes keep it as fixed-point operands).
+template <int GROWS>
+__device__ __forceinline__ void load_g(const MatField<float, GROWS>& Gf, int64_t s, M3<float>& M) {
+  Gf.load_ro(0, s, M);
+}
+__device__ __forceinline__ void load_g(const MatField<double, 3>& Gf, int64_t s, M3<double>& M) {
+  fxg_load(Gf.p, Gf.V, s, M);
+}
 
 template <typename R, int LROWS, int GROWS>
 __global__ void __launch_bounds__(UPDATE_THREADS)
@@ -735,12 +757,12 @@ revert_kernel(Geom g, MatField<R, LROWS> U, MatField<R, GROWS> Gf, MatField<R, 3
   int c[4];
   site_coords(g, s, c);
   M3<R> gx;
-  Gf.load_ro(0, s, gx);
+  load_g(Gf, s, gx);
 #pragma unroll 1
   for (int mu = 0; mu < 4; ++mu) {
     M3<R> u, h;
     U.load(mu, s, u);
-    Gf.load_ro(0, site_fwd(g, s, c, mu), h);
+    load_g(Gf, site_fwd(g, s, c, mu), h);
     // T = (g^dag U)[rows 0,1]: T_ij = sum_k conj(g_ki) U_kj
     C2<R> T[2][3];
 #pragma unroll
@@ -825,6 +847,21 @@ __global__ void to_aos_kernel(int64_t V, int nmat, MatField<R, ROWS> F, double2*
   for (int r = 0; r < 3; ++r)
 #pragma unroll
     for (int c = 0; c < 3; ++c) dst[r * 3 + c] = make_double2((double)M.e[r][c].x, (double)M.e[r][c].y);
+}
+
+__global__ void gauge_to_aos_kernel(int64_t V, const double2* __restrict__ gf, double2* __restrict__ aos) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= V) return;
+  M3<double> M;
+  fxg_load(gf, V, s, M);
+#pragma unroll
+  for (int e = 0; e < 9; ++e) aos[s * 9 + e] = M.e[e / 3][e % 3];
+}
+
+cudaError_t launch_gauge_to_aos(const Geom& g, const double2* gfield, double* aos, cudaStream_t s) {
+  gauge_to_aos_kernel<<<(unsigned)((g.V + CONV_THREADS - 1) / CONV_THREADS), CONV_THREADS, 0, s>>>(
+      g.V, gfield, reinterpret_cast<double2*>(aos));
+  return cudaGetLastError();
 }
 
 template <typename R, int ROWS>
@@ -1101,8 +1138,10 @@ cudaError_t launch_c2_f32_to_f64(const float2* in, double2* out, int64_t n, cuda
   return cudaGetLastError();
 }
 
-// Gram-Schmidt projection of rows 1-2 to SU(3) in FP64, row 3 = (a x b)^*.
-__global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, double2* __restrict__ out) {
+// Gram-Schmidt projection of rows 1-2 to SU(3) in FP64, row 3 = (a x b)^*,
+// as g of the FP64 lane and, where it tracks the transform, as its G.
+__global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, double2* __restrict__ gf,
+                                     double2* __restrict__ out) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
   double2 a[3], b[3], c[3];
@@ -1125,6 +1164,8 @@ __global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, d
 #pragma unroll
   for (int j = 0; j < 3; ++j) b[j] = cscale<double>(b[j], ib);
   su3_third_row<double>(a, b, c);
+  fxg_store(gf, V, s, a, b, c);
+  if (out == nullptr) return;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     out[(0 * 3 + j) * V + s] = a[j];
@@ -1133,8 +1174,10 @@ __global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, d
   }
 }
 
-cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* G64, cudaStream_t s) {
-  project_sites_kernel<<<(unsigned)((g.V + CONV_THREADS - 1) / CONV_THREADS), CONV_THREADS, 0, s>>>(g.V, G32, G64);
+cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* gfield, double2* G64,
+                                            cudaStream_t s) {
+  project_sites_kernel<<<(unsigned)((g.V + CONV_THREADS - 1) / CONV_THREADS), CONV_THREADS, 0, s>>>(g.V, G32, gfield,
+                                                                                                    G64);
   return cudaGetLastError();
 }
 

@@ -149,13 +149,11 @@ extern "C" lgf_status lgf_measure_static(const int32_t extents[4], const double*
                                          void* cuda_stream) {
   if (!extents || !U || !F_theta) return LGF_E_ARG;
   Geom g{};
-  g.V = 1;
   for (int mu = 0; mu < 4; ++mu) {
     if (!extent_ok(extents[mu])) return LGF_E_UNSUPPORTED;
     g.L[mu] = extents[mu];
-    g.stride[mu] = g.V;
-    g.V *= extents[mu];
   }
+  g.finish();
   if (g.V > LGF_STATIC_MAX_SITES) return LGF_E_UNSUPPORTED;  // scratch holds one partial pair per 256 sites
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return LGF_E_CUDA;
