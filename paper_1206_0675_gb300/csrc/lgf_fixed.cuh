@@ -61,18 +61,20 @@ __device__ __forceinline__ Fx fx_operand(int64_t r60) {
   return Fx{(int)((r60 + ((int64_t)1 << 29)) >> 30), (int)((uint32_t)r60 << 2) >> 2};
 }
 
-// Fixed point from FP64, |a| < FX_LIM; bits below 2^-60 are cut off.
+// Fixed point from FP64 in units of 2^-60, |a| < 2; what lies below is cut off.
 // With the leading one at bit 63 the significand M has the value
 // M 2^(e - 1086), so the magnitude in units of 2^-60 is M >> (1026 - e).
-__device__ __forceinline__ Fx fx_from(double a) {
+__device__ __forceinline__ int64_t fx60_from(double a) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
   const int64_t sg = (int64_t)((int)hi >> 31);
-  return fx_operand(
-      ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, 1026u - ((hi >> 20) & 0x7ffu)) ^ sg) - sg);
+  return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, 1026u - ((hi >> 20) & 0x7ffu)) ^ sg) - sg;
 }
+__device__ __forceinline__ Fx fx_from(double a) { return fx_operand(fx60_from(a)); }
 __device__ __forceinline__ FxC fx_from(double2 a) { return FxC{fx_from(a.x), fx_from(a.y)}; }
 __device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }
+__device__ __forceinline__ FxC fx_neg(FxC a) { return FxC{fx_neg(a.x), fx_neg(a.y)}; }
+__device__ __forceinline__ FxC fx_conj(FxC a) { return FxC{a.x, fx_neg(a.y)}; }
 
 // c + a b with a 64-bit sum: one IMAD.WIDE (written out, so that sums of
 // products are not taken apart into products and 64-bit additions).
@@ -233,15 +235,17 @@ __device__ __forceinline__ FxC fxg_unpack(int4 w) { return FxC{Fx{w.x, w.y}, Fx{
 __device__ __forceinline__ int4 fxg_pack(const FxC& a) { return make_int4(a.x.h, a.x.l, a.y.h, a.y.l); }
 __device__ __forceinline__ double fx_value(Fx a) { return fx_to_double_fp<60>(((int64_t)a.h << 30) + a.l); }
 
-// g(s) in FP64 (NaN where marked).
-__device__ __forceinline__ void fxg_load(const double2* __restrict__ gf, int64_t V, int64_t s, M3<double>& M) {
-  const int4* p = reinterpret_cast<const int4*>(gf);
-  const bool bad = __ldg(&p[s]).x == FX_G_NAN;
+// g in FP64 (NaN where marked) from its entries p[e stride].
+__device__ __forceinline__ void fxg_load(const int4* p, int64_t stride, M3<double>& M) {
+  const bool bad = p[0].x == FX_G_NAN;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    const FxC w = fxg_unpack(__ldg(&p[e * V + s]));
+    const FxC w = fxg_unpack(p[e * stride]);
     M.e[e / 3][e % 3] = bad ? make_double2(NAN, NAN) : make_double2(fx_value(w.x), fx_value(w.y));
   }
+}
+__device__ __forceinline__ void fxg_load(const double2* gf, int64_t V, int64_t s, M3<double>& M) {
+  fxg_load(reinterpret_cast<const int4*>(gf) + s, V, M);
 }
 // The store, from FP64 rows.
 __device__ __forceinline__ void fxg_store(double2* __restrict__ gf, int64_t V, int64_t s, const double2 a[3],
@@ -261,7 +265,7 @@ __device__ __forceinline__ void fxg_store(double2* __restrict__ gf, int64_t V, i
 }
 
 // y/2 in units of 2^-60 for y = 1/sqrt(n), n in units of 2^-60 and
-// 0.2 < n < 2: the FP32 estimate, a 23-bit integer, and one third-order step
+// 1/16 <= n < 2: the FP32 estimate, a 24-bit integer, and one third-order step
 // (e = 1 - n y0^2 below 2^-19 in magnitude, so 5 e^3 / 16 is below 2^-58 of y0;
 // see rsqrt_fp64).
 __device__ __forceinline__ int64_t fx_half_rsqrt(int64_t n) {
@@ -273,6 +277,46 @@ __device__ __forceinline__ int64_t fx_half_rsqrt(int64_t n) {
   const int eh = (int)(e >> 20);
   const int64_t c = (e >> 1) + (3 * ((int64_t)eh * eh) >> 23);
   return ((int64_t)y0 << 37) + ((int64_t)((int)(c >> 20)) * y0 >> 3) + ((int64_t)((int)c & 0xfffff) * y0 >> 23);
+}
+
+// ---------------------------------------------------------------------------
+// updated links
+// ---------------------------------------------------------------------------
+
+// Third row (as operands or sums) from rows that are operands.
+__device__ __forceinline__ void fx_third_row(const FxC a[3], const FxC b[3], int64_t c[3][2], uint32_t& t) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    FxAcc re = fx_zero(), im = fx_zero();
+    fx_cross_conj(re, im, a[(j + 1) % 3], a[(j + 2) % 3], b[(j + 1) % 3], b[(j + 2) % 3]);
+    c[j][0] = fx_sum60(re, t);
+    c[j][1] = fx_sum60(im, t);
+  }
+}
+
+// An updated link in FP64 from the sums of its rows 1-2 (n, units of 2^-60)
+// and, for 18-real storage, of row 3 (n3).  Row 3 converts on the FP64 pipe,
+// which is idle otherwise.
+template <int ROWS>
+__device__ __forceinline__ void fx_link_to_double(const int64_t n[2][3][2], const int64_t n3[3][2],
+                                                  double2 o[ROWS][3]) {
+  bool big = true;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      o[i][j] = make_double2(fx_to_double_int<60>(n[i][j][0], big), fx_to_double_int<60>(n[i][j][1], big));
+  if (!big) {  // an entry below 2^-28, zeros among them
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        o[i][j] = make_double2(fx_to_double_fp<60>(n[i][j][0]), fx_to_double_fp<60>(n[i][j][1]));
+  }
+  if (ROWS == 3) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) o[2][j] = make_double2(fx_to_double_fp<60>(n3[j][0]), fx_to_double_fp<60>(n3[j][1]));
+  }
 }
 
 }  // namespace lgf

@@ -291,18 +291,18 @@ static __device__ __noinline__ void gauge_site_fp64(double2 f0, double2 f1, doub
   gauge_site<double, double, 3, EXPG>(f0, f1, f2, f3, V, s, gf, Gf);
 }
 
-static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, const double2* __restrict__ gf,
-                                                          double2* __restrict__ Gf) {
+static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, const int4* __restrict__ gp,
+                                                          int64_t gstride, double2* __restrict__ Gf) {
   M3<double> g;
-  fxg_load(gf, V, s, g);
+  fxg_load(gp, gstride, g);
   accumulate_gauge<double>(V, s, g.e[0], g.e[1], g.e[2], Gf);
 }
 
-// G(s) <- g G(s) in fixed point, for g as stored (a call: its operands would
-// otherwise crowd the registers of every pass, tracked transform or not).
-static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, const double2* __restrict__ gf,
+// G(s) <- g G(s) in fixed point, for the entries gp[e gstride] of g (a call:
+// its operands would otherwise crowd the registers of every caller, tracked
+// transform or not).
+static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, const int4* gp, int64_t gstride,
                                                         double2* __restrict__ Gf) {
-  const int4* p = reinterpret_cast<const int4*>(gf);
   uint32_t m = 0, t = 0;
   FxC G[3][3];
 #pragma unroll
@@ -318,7 +318,7 @@ static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, co
   for (int r = 0; r < 3; ++r) {
     FxC g[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) g[k] = fxg_unpack(p[(r * 3 + k) * V + s]);
+    for (int k = 0; k < 3; ++k) g[k] = fxg_unpack(gp[(r * 3 + k) * gstride]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       FxAcc re = fx_zero(), im = fx_zero();
@@ -333,7 +333,7 @@ static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, co
     }
   }
   if (fx_bad(m, t)) {
-    accumulate_gauge_fp64(V, s, gf, Gf);
+    accumulate_gauge_fp64(V, s, gp, gstride, Gf);
     return;
   }
 #pragma unroll
@@ -422,7 +422,7 @@ __device__ __forceinline__ void gauge_site_fx(const int64_t A[8], int64_t V, int
   for (int r = 0; r < 3; ++r)
 #pragma unroll
     for (int j = 0; j < 3; ++j) p[(r * 3 + j) * V + s] = fxg_pack(g[r][j]);
-  if (Gf != nullptr) accumulate_gauge_fx(V, s, gf, Gf);
+  if (Gf != nullptr) accumulate_gauge_fx(V, s, p + s, V, Gf);
 }
 
 }  // namespace lgf

@@ -17,11 +17,15 @@
 // Every link joins two sites of opposite colour, so within one colour each
 // link is read and written by exactly one thread: the update is in place.
 //
-// One thread per site of the colour.  Its links are read twice (once for w,
+// FP32 links: one thread per site of the colour.  Its links are read twice (once for w,
 // once for the product, the second time from L1/L2) so that only w, the
 // running subgroup block and g stay in registers.  The site algebra runs in
 // the link precision; rows 1-2 of every product are formed and row 3 is
 // rebuilt as (a x b)^* (Sec. 3.2), as in the Fourier-accelerated update.
+#include <cmath>
+
+#include "lgf_fixed.cuh"
+#include "lgf_gauge.cuh"
 #include "lgf_internal.h"
 
 namespace lgf {
@@ -116,25 +120,22 @@ __device__ __forceinline__ int64_t or_back(const Geom& g, int64_t s, const int c
   return cm == 0 ? s + (int64_t)(L - 1) * st : s - st;
 }
 
-template <typename R, int ROWS>
-__global__ void __launch_bounds__(OR_THREADS)
-or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, const DevState* __restrict__ st,
-                     C2<R>* __restrict__ G, int parity, R omega) {
-  // fused FP32 lanes keep their current links in one of two buffers
-  const MatField<R, ROWS> U{(U1 != nullptr && st->ubuf) ? U1 : U0, g.V};
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if ((int64_t)j >= (g.V >> 1)) return;
-  // site of the colour: x = 2 xh + ((y + z + t + parity) & 1) in its (y, z, t) row
-  const uint32_t hx = (uint32_t)g.L[0] >> 1;
-  const uint32_t row = j / hx;
-  int c[4];
-  c[1] = (int)(row % (uint32_t)g.L[1]);
-  const uint32_t r2 = row / (uint32_t)g.L[1];
-  c[2] = (int)(r2 % (uint32_t)g.L[2]);
-  c[3] = (int)(r2 / (uint32_t)g.L[2]);
-  c[0] = 2 * (int)(j - row * hx) + ((c[1] + c[2] + c[3] + parity) & 1);
-  const int64_t s = (int64_t)c[0] + (int64_t)g.L[0] * row;
+// Site j of the colour: x = 2 xh + ((y + z + t + parity) & 1) in its (y, z, t)
+// row; dhx divides by Lx / 2.
+__device__ __forceinline__ int64_t or_coords(const Geom& g, const FastDiv& dhx, uint32_t j, int parity, int c[4]) {
+  const uint32_t row = dhx.div(j);
+  const uint32_t r2 = g.dL[1].div(row);
+  c[1] = (int)(row - r2 * g.dL[1].d);
+  c[3] = (int)g.dL[2].div(r2);
+  c[2] = (int)(r2 - (uint32_t)c[3] * g.dL[2].d);
+  c[0] = 2 * (int)(j - row * dhx.d) + ((c[1] + c[2] + c[3] + parity) & 1);
+  return (int64_t)c[0] + (int64_t)g.L[0] * row;
+}
 
+// One site of the colour: its hit and the products with its eight links.
+template <typename R, int ROWS>
+__device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
+                                        C2<R>* __restrict__ G, R omega) {
   // w(x) = sum_mu [U_mu(x) + U_mu^dag(x - mu^)]
   M3<R> M;
 #pragma unroll
@@ -211,11 +212,285 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 }
 
 template <typename R, int ROWS>
+__global__ void __launch_bounds__(OR_THREADS)
+or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, const DevState* __restrict__ st,
+                     C2<R>* __restrict__ G, int parity, FastDiv dhx, R omega) {
+  // fused FP32 lanes keep their current links in one of two buffers
+  const MatField<R, ROWS> U{(U1 != nullptr && st->ubuf) ? U1 : U0, g.V};
+  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if ((int64_t)j >= (g.V >> 1)) return;
+  int c[4];
+  const int64_t s = or_coords(g, dhx, j, parity, c);
+  or_site<R, ROWS>(g, U, c, s, G, omega);
+}
+
+// ---------------------------------------------------------------------------
+// FP64 links in fixed point (lgf_fixed.cuh)
+// ---------------------------------------------------------------------------
+//
+// A CTA takes 32 sites, one direction per warp: every thread converts its
+// forward and its backward link once and keeps them as operands, the four
+// warps' parts of w(x) meet in shared memory, the first warp does the hits and
+// every thread multiplies its two links.  Sites with a link outside the
+// fixed-point range or near the identity (see update_fx_kernel), or with a
+// local field too small for its direction to be resolved, are done by one
+// thread in FP64.
+// With FP64 arithmetic one thread a site kept the FP64 pipe 93 % busy (1199
+// operations a site and sweep); now the integer pipe bounds it, with 12 warps
+// per SM at 168 registers.  24^4, 18-real: 20 sweeps with set_links and get_links 15.4
+// -> 8.6 ms; error of 20 sweeps against 64 bits 2.2e-15 -> 1.7e-15.
+
+// The 64-bit sum an operand stands for (units of 2^-60).
+__device__ __forceinline__ int64_t fx_r60(Fx a) { return mad_wide(a.h, 1 << 30, (int64_t)a.l); }
+
+// 2 a (y/2) for y/2 given as an operand.
+__device__ __forceinline__ Fx fx_scaled(Fx a, Fx half_y) {
+  uint32_t t = 0;
+  FxAcc p = fx_zero();
+  fx_mac(p, a, half_y);
+  return fx_operand(2 * fx_sum60(p, t));
+}
+
+// or_subgroup in fixed point.  The block's components b0..b3 (of the local
+// field over 64, so below 1/4) are shifted up until the largest lies in
+// [1/4, 1/2): |b|^2 is in [1/16, 1).  q is scaled by 7/16, which puts |q|^2 in
+// [0.19, 1.73) for 1 <= omega < 2: w7 = 7 omega / 16 and c7 = 7 (1 - omega) / 16
+// in units of 2^-60.  ok = false where |b| / 64 is below 2^-20: too small to
+// shift up without losing its direction.
+__device__ __forceinline__ void or_subgroup_fx(const FxC& mii, const FxC& mij, const FxC& mji, const FxC& mjj, Fx w7,
+                                               int64_t c7, FxC& a, FxC& b, bool& ok) {
+  int64_t v[4] = {fx_r60(mii.x) + fx_r60(mjj.x), -(fx_r60(mij.y) + fx_r60(mji.y)), fx_r60(mji.x) - fx_r60(mij.x),
+                  fx_r60(mjj.y) - fx_r60(mii.y)};  // |b| r / |r|
+  uint64_t mag = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) mag |= (uint64_t)(v[k] ^ (v[k] >> 63));
+  const int lz = __clzll((long long)(mag | 1u));
+  ok = ok && lz <= 24;
+  const int sh = min(max(lz - 5, 0), 20);
+  uint32_t t = 0;
+  Fx r[4];
+  FxAcc n = fx_zero();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    r[k] = fx_operand(v[k] << sh);
+    fx_mac(n, r[k], r[k]);
+  }
+  const Fx yq = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t), (int64_t)1 << 56)) >> 1);  // 1 / (4 |b|)
+  Fx q[4];
+  n = fx_zero();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    FxAcc p = fx_zero();
+    fx_mac(p, r[k], yq);
+    const Fx rk = fx_operand(4 * fx_sum60(p, t));
+    p = fx_zero();
+    if (k == 0) p.hi = c7;
+    fx_mac(p, w7, rk);
+    q[k] = fx_operand(fx_sum60(p, t));
+    fx_mac(n, q[k], q[k]);
+  }
+  const Fx zh = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t), (int64_t)1 << 56)));
+  a = FxC{fx_scaled(q[0], zh), fx_scaled(q[3], zh)};
+  b = FxC{fx_scaled(q[2], zh), fx_scaled(q[1], zh)};
+}
+
+// or_rot in fixed point.
+__device__ __forceinline__ void or_rot_fx(const FxC& a, const FxC& b, FxC& xi, FxC& xj) {
+  uint32_t t = 0;
+  FxAcc ir = fx_zero(), ii = fx_zero(), jr = fx_zero(), ji = fx_zero();
+  fx_cmac(ir, ii, a, fx_neg(a.y), xi);
+  fx_cmac(ir, ii, b, fx_neg(b.y), xj);
+  const FxC ac = fx_conj(a), nbc{fx_neg(b.x), b.y};  // conj(a), -conj(b)
+  fx_cmac(jr, ji, ac, a.y, xj);
+  fx_cmac(jr, ji, nbc, fx_neg(b.y), xi);
+  xi = FxC{fx_operand(fx_sum60(ir, t)), fx_operand(fx_sum60(ii, t))};
+  xj = FxC{fx_operand(fx_sum60(jr, t)), fx_operand(fx_sum60(ji, t))};
+}
+
+// g(x) of one Cabibbo-Marinari hit, as or_site_gauge.
+__device__ __forceinline__ void or_site_gauge_fx(FxC M[3][3], Fx w7, int64_t c7, FxC gx[3][3], bool& ok) {
+  const FxC zero{{0, 0}, {0, 0}}, one{{1 << 30, 0}, {0, 0}};
+  FxC a, b;
+  or_subgroup_fx(M[0][0], M[0][1], M[1][0], M[1][1], w7, c7, a, b, ok);
+  gx[0][0] = a;
+  gx[0][1] = b;
+  gx[0][2] = zero;
+  gx[1][0] = FxC{fx_neg(b.x), b.y};
+  gx[1][1] = fx_conj(a);
+  gx[1][2] = zero;
+  gx[2][0] = zero;
+  gx[2][1] = zero;
+  gx[2][2] = one;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) or_rot_fx(a, b, M[0][c], M[1][c]);
+  or_subgroup_fx(M[0][0], M[0][2], M[2][0], M[2][2], w7, c7, a, b, ok);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) or_rot_fx(a, b, gx[0][c], gx[2][c]);
+#pragma unroll
+  for (int c = 1; c < 3; ++c) or_rot_fx(a, b, M[0][c], M[2][c]);
+  or_subgroup_fx(M[1][1], M[1][2], M[2][1], M[2][2], w7, c7, a, b, ok);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) or_rot_fx(a, b, gx[1][c], gx[2][c]);
+}
+
+template <int ROWS>
+static __device__ __noinline__ void or_site_fp64(const Geom& g, MatField<double, ROWS> U, int64_t s, double2* G,
+                                                 double omega) {
+  int c[4];
+  site_coords(g, s, c);
+  or_site<double, ROWS>(g, U, c, s, G, omega);
+}
+
+// Link (mu, s) as operands, its entries in the range tests.
+template <int ROWS>
+__device__ __forceinline__ void or_load_fx(const MatField<double, ROWS>& U, int mu, int64_t s, FxC x[3][3], uint32_t& m,
+                                           uint32_t& t, bool& weak) {
+  double2 u[ROWS][3];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[r][k] = U.p[U.off(mu, r, k, s)];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      m = fx_max(m, u[r][k]);
+      x[r][k] = fx_from(u[r][k]);
+    }
+  weak = weak || fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_WEAK_HI;
+  if (ROWS == 2) {
+    int64_t c3[3][2];
+    fx_third_row(x[0], x[1], c3, t);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[2][k] = FxC{fx_operand(c3[k][0]), fx_operand(c3[k][1])};
+  }
+}
+
+template <int ROWS>
+__device__ __forceinline__ void or_store_fx(const MatField<double, ROWS>& U, int mu, int64_t s,
+                                            const int64_t n[2][3][2]) {
+  uint32_t t = 0;
+  int64_t n3[3][2];
+  if (ROWS == 3) {
+    FxC r[2][3];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) r[i][j] = FxC{fx_operand(n[i][j][0]), fx_operand(n[i][j][1])};
+    fx_third_row(r[0], r[1], n3, t);
+  }
+  double2 o[ROWS][3];
+  fx_link_to_double<ROWS>(n, n3, o);
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) U.p[U.off(mu, i, j, s)] = o[i][j];
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(OR_THREADS, 3)
+or_half_sweep_fx_kernel(Geom g, double2* __restrict__ U0, double2* __restrict__ G, int parity, FastDiv dhx,
+                        double omega, int64_t w7, int64_t c7) {
+  __shared__ int64_t part[4][18][32];  // each direction's part of w(x), units of 2^-58
+  __shared__ int4 gs[9][32];
+  __shared__ int skip[32];
+  const MatField<double, ROWS> U{U0, g.V};
+  const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
+  const uint32_t n_sites = (uint32_t)(g.V >> 1), j = blockIdx.x * 32u + (uint32_t)lane;
+  const bool live = j < n_sites;
+  int c[4];
+  const int64_t s = or_coords(g, dhx, min(j, n_sites - 1u), parity, c);
+  const int64_t sb = or_back(g, s, c, mu);
+  if (threadIdx.x < 32) skip[lane] = 0;
+  FxC uf[3][3], ub[3][3];
+  uint32_t m = 0, t = 0;
+  bool weak = false;
+  or_load_fx<ROWS>(U, mu, s, uf, m, t, weak);
+  or_load_fx<ROWS>(U, mu, sb, ub, m, t, weak);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      part[mu][2 * (3 * r + k)][lane] = (fx_r60(uf[r][k].x) >> 2) + (fx_r60(ub[k][r].x) >> 2);
+      part[mu][2 * (3 * r + k) + 1][lane] = (fx_r60(uf[r][k].y) >> 2) - (fx_r60(ub[k][r].y) >> 2);
+    }
+  __syncthreads();
+  if (fx_bad(m, t) || weak) skip[lane] = 1;
+  if (mu == 0) {
+    FxC M[3][3], gx[3][3];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      int64_t x = 0, y = 0;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) {
+        x += part[d][2 * e][lane];
+        y += part[d][2 * e + 1][lane];
+      }
+      M[e / 3][e % 3] = FxC{fx_operand(x >> 4), fx_operand(y >> 4)};  // w / 64
+    }
+    bool ok = true;
+    or_site_gauge_fx(M, fx_operand(w7), c7, gx, ok);
+    if (!ok) skip[lane] = 1;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) gs[e][lane] = fxg_pack(gx[e / 3][e % 3]);
+  }
+  __syncthreads();
+  if (!live) return;
+  if (skip[lane]) {
+    if (mu == 0) or_site_fp64<ROWS>(g, U, s, G, omega);
+    return;
+  }
+  int64_t n[2][3][2];
+  t = 0;
+  // U_mu(x) <- g U_mu(x)
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    FxC gr[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gr[k] = fxg_unpack(gs[3 * i + k][lane]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int q = 0; q < 3; ++q) fx_cmac(re, im, gr[q], fx_neg(gr[q].y), uf[q][k]);
+      n[i][k][0] = fx_sum60(re, t);
+      n[i][k][1] = fx_sum60(im, t);
+    }
+  }
+  or_store_fx<ROWS>(U, mu, s, n);
+  // U_mu(x - mu^) <- U_mu(x - mu^) g^dag
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    FxC gr[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) gr[q] = fxg_unpack(gs[3 * k + q][lane]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+      for (int q = 0; q < 3; ++q) fx_cmacc(re, im, ub[i][q], fx_neg(ub[i][q].x), gr[q]);
+      n[i][k][0] = fx_sum60(re, t);
+      n[i][k][1] = fx_sum60(im, t);
+    }
+  }
+  or_store_fx<ROWS>(U, mu, sb, n);
+  if (G != nullptr && mu == 0) accumulate_gauge_fx(g.V, s, &gs[0][lane], 32, G);
+}
+
+template <typename R, int ROWS>
 cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* G, int parity,
                                  double omega, cudaStream_t s) {
   const int64_t n = g.V >> 1;
-  const unsigned nb = (unsigned)((n + OR_THREADS - 1) / OR_THREADS);
-  or_half_sweep_kernel<R, ROWS><<<nb, OR_THREADS, 0, s>>>(g, U0, U1, st, G, parity & 1, (R)omega);
+  const FastDiv dhx = FastDiv::make((uint32_t)g.L[0] / 2);
+  if constexpr (sizeof(R) == sizeof(double)) {
+    // FP64 lanes have one link buffer
+    const int64_t w7 = std::llround(std::ldexp(7.0 * omega, 56)), c7 = std::llround(std::ldexp(7.0 * (1.0 - omega), 56));
+    or_half_sweep_fx_kernel<ROWS><<<(unsigned)((n + 31) / 32), OR_THREADS, 0, s>>>(g, U0, G, parity & 1, dhx, omega, w7,
+                                                                                   c7);
+  } else {
+    const unsigned nb = (unsigned)((n + OR_THREADS - 1) / OR_THREADS);
+    or_half_sweep_kernel<R, ROWS><<<nb, OR_THREADS, 0, s>>>(g, U0, U1, st, G, parity & 1, dhx, (R)omega);
+  }
   return cudaGetLastError();
 }
 

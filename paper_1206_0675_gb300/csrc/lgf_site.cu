@@ -284,12 +284,11 @@ __device__ __forceinline__ void site_divergence_fx(const Geom& g, const MatField
           w[r][j] = FxC{fx_operand58(q[r][j][0]), fx_operand58(q[r][j][1])};
         }
       int64_t z[3][2];
+      fx_third_row(w[0], w[1], z, t);
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        FxAcc re = fx_zero(), im = fx_zero();
-        fx_cross_conj(re, im, w[0][(j + 1) % 3], w[0][(j + 2) % 3], w[1][(j + 1) % 3], w[1][(j + 2) % 3]);
-        z[j][0] = fx_sum60(re, t) >> 2;
-        z[j][1] = fx_sum60(im, t) >> 2;
+        z[j][0] >>= 2;
+        z[j][1] >>= 2;
       }
       f00 = fwd ? q[0][0][0] : 0;
       f11 = fwd ? q[1][1][0] : 0;
@@ -639,12 +638,10 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
 #pragma unroll
     for (int j = 0; j < 3; ++j) ux[i][j] = fx_from(u[i][j]);
   if (LROWS == 2) {
+    int64_t c3[3][2];
+    fx_third_row(ux[0], ux[1], c3, t);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      FxAcc re = fx_zero(), im = fx_zero();
-      fx_cross_conj(re, im, ux[0][(j + 1) % 3], ux[0][(j + 2) % 3], ux[1][(j + 1) % 3], ux[1][(j + 2) % 3]);
-      ux[2][j] = FxC{fx_operand(fx_sum60(re, t)), fx_operand(fx_sum60(im, t))};
-    }
+    for (int j = 0; j < 3; ++j) ux[2][j] = FxC{fx_operand(c3[j][0]), fx_operand(c3[j][1])};
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -679,38 +676,14 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) r[i][j] = FxC{fx_operand(n[i][j][0]), fx_operand(n[i][j][1])};
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      FxAcc re = fx_zero(), im = fx_zero();
-      fx_cross_conj(re, im, r[0][(j + 1) % 3], r[0][(j + 2) % 3], r[1][(j + 1) % 3], r[1][(j + 2) % 3]);
-      n3[j][0] = fx_sum60(re, t);
-      n3[j][1] = fx_sum60(im, t);
-    }
+    fx_third_row(r[0], r[1], n3, t);
   }
   if (fx_bad(m, t) || w < FX_WEAK_HI || g4[0][0].x == FX_G_NAN || h4[0][0].x == FX_G_NAN) {
     update_link_fp64<LROWS>(U, Gf, mu, s, sf);
     return;
   }
-  bool big = true;
   double2 o[LROWS][3];
-#pragma unroll
-  for (int i = 0; i < LROWS; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int64_t x = i < 2 ? n[i][j][0] : n3[j][0], y = i < 2 ? n[i][j][1] : n3[j][1];
-      // row 3 on the FP64 pipe, which is idle otherwise
-      o[i][j] = i == 2 ? make_double2(fx_to_double_fp<60>(x), fx_to_double_fp<60>(y))
-                       : make_double2(fx_to_double_int<60>(x, big), fx_to_double_int<60>(y, big));
-    }
-  if (!big) {  // an entry below 2^-28, zeros among them
-#pragma unroll
-    for (int i = 0; i < LROWS; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const int64_t x = i < 2 ? n[i][j][0] : n3[j][0], y = i < 2 ? n[i][j][1] : n3[j][1];
-        o[i][j] = make_double2(fx_to_double_fp<60>(x), fx_to_double_fp<60>(y));
-      }
-  }
+  fx_link_to_double<LROWS>(n, n3, o);
 #pragma unroll
   for (int i = 0; i < LROWS; ++i)
 #pragma unroll

@@ -149,3 +149,25 @@ def test_fft4_nonfinite_input(bad):
     assert not np.any(np.isfinite(got[2]))
     ref = fft_ref(f[[0, 1, 3]], -1)
     assert np.linalg.norm(got[[0, 1, 3]] - ref) < 1e-15 * np.linalg.norm(ref)
+
+
+# ---------------------------------------------------------------------------
+# overrelaxation
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("omega", [1.0, 1.7, 1.999])
+@pytest.mark.parametrize("name", ["random", "weak 1e-3", "weak 1e-9"])
+@pytest.mark.parametrize("ext", [(2, 2, 2, 2), (2, 2, 4, 6), (4, 6, 2, 8)])
+def test_or_sweep_against_oracle(ext, name, omega):
+    """One sweep (both colours), with and without row 3 and the transform, at site counts that end inside a CTA;
+    links within the rounding of the two sides, 1e-12 as for the other sweeps."""
+    from oracle import lgf_or_oracle as R
+    U = CASES[name](ext)
+    Uo, Go = R.or_sweep(U, omega)
+    for store12 in (False, True):
+        with lgf.Lattice(ext, "fp64", store12=store12, track_G=True) as lat:
+            lat.set_links(U)
+            lat.or_sweep(omega, 1)
+            U1, G = lat.get_links(), lat.get_transform()
+        assert np.max(np.abs(U1 - Uo)) < 1e-12
+        assert np.max(np.abs(G - Go)) < 1e-12
