@@ -334,25 +334,93 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
   return x ^ (x >> 31);
 }
 
+// Activations and their gradients are kept feature-major, [feature][sample], so
+// that every product of a layer reads both of its operands as vectors of
+// four: a thread forms a 4 x 4 tile of each 64 x 64 result from eight 16-byte
+// shared loads per 64 multiply-adds.  Rows are padded to 68 floats (rows four
+// banks apart).  The gradients of W2 and W3 stay in registers over all chunks
+// of a CTA.  110 KB, two CTAs per SM.
+constexpr int TS = 68;
 struct TrainSmem {
-  float P[MLP_NPARAM + 3];
-  float G[MLP_NPARAM + 3];
-  float X[TCH * MLP_NIN];
-  float H1[TCH * MLP_NH], H2[TCH * MLP_NH], H3[TCH * MLP_NH], D[TCH * MLP_NH];
-  float dz[TCH];
-  int idx[TCH];
+  float W2[MLP_NH * TS], W3[MLP_NH * TS];  // [out][in]
+  float W1[MLP_NH * MLP_NIN];
+  float b1[MLP_NH], b2[MLP_NH], b3[MLP_NH], w4[MLP_NH];
+  float X[MLP_NIN * TS];
+  float H1[MLP_NH * TS], H2[MLP_NH * TS], H3[MLP_NH * TS], D[MLP_NH * TS];
+  float dz[TCH], y[TCH], w[TCH];
+  float zp[4][TCH];   // parts of the output sum
+  float b4;
 };
+static_assert(sizeof(TrainSmem) <= 113 * 1024, "two CTAs of the training kernel per SM");
 
-// out[s][n] = act(sum_k in[s][k] W[n][k] + b[n]) for a chunk; W row-major [n][K].
-__device__ __forceinline__ void dense_fwd(const float* in, int K, const float* W, const float* b, float* out) {
-  for (int e = threadIdx.x; e < TCH * MLP_NH; e += blockDim.x) {
-    const int s = e / MLP_NH, n = e % MLP_NH;
-    float a = b[n];
-    const float* x = in + s * K;
-    const float* w = W + n * K;
-    for (int k = 0; k < K; ++k) a = fmaf(x[k], w[k], a);
-    out[e] = fmaxf(a, 0.f);
+__device__ __forceinline__ void ld4(const float* p, float v[4]) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void st4(float* p, const float v[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// acc[i][j] += sum_k A[r0 + i][k] B[k][c0 + j] over 64 k; rows of TS floats.
+__device__ __forceinline__ void tile_ab(const float* A, const float* B, int r0, int c0, float acc[4][4]) {
+#pragma unroll 4
+  for (int k = 0; k < MLP_NH; k += 4) {
+    float a[4][4], b[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ld4(A + (r0 + i) * TS + k, a[i]);
+      ld4(B + (k + i) * TS + c0, b[i]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i][q], b[q][j], acc[i][j]);
   }
+}
+// acc[i][j] += sum_k A[k][r0 + i] B[k][c0 + j].
+__device__ __forceinline__ void tile_atb(const float* A, const float* B, int r0, int c0, float acc[4][4]) {
+#pragma unroll 4
+  for (int k = 0; k < MLP_NH; ++k) {
+    float a[4], b[4];
+    ld4(A + k * TS + r0, a);
+    ld4(B + k * TS + c0, b);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+  }
+}
+// acc[i][j] += sum_s A[r0 + i][s] B[c0 + 16 j][s]: the columns of a thread are
+// 16 apart, so that the lanes of a warp read 16 consecutive rows of B.
+__device__ __forceinline__ void tile_abt(const float* A, const float* B, int r0, int c0, float acc[4][4]) {
+#pragma unroll 2
+  for (int s = 0; s < TCH; s += 4) {
+    float a[4][4], b[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ld4(A + (r0 + i) * TS + s, a[i]);
+      ld4(B + (c0 + 16 * i) * TS + s, b[i]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i][q], b[j][q], acc[i][j]);
+  }
+}
+__device__ __forceinline__ float row_sum(const float* row) {
+  float t[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int s = 0; s < TCH; s += 4) {
+    float v[4];
+    ld4(row + s, v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) t[j] += v[j];
+  }
+  return (t[0] + t[1]) + (t[2] + t[3]);
 }
 
 // Loss and gradient of the weighted MSE of log m against y, summed over the
@@ -360,157 +428,254 @@ __device__ __forceinline__ void dense_fwd(const float* in, int K, const float* W
 // written to part_g[blockIdx] and part_l[blockIdx] (reduced later in order).
 // Samples: idx = hash(seed, step, j) mod n for j < batch when batch > 0,
 // otherwise every sample once in order.
-__global__ void __launch_bounds__(TTH) mlp_grad_kernel(const float* __restrict__ Pg, const float* __restrict__ X,
-                                                       const float* __restrict__ Y, const float* __restrict__ Wt,
-                                                       int64_t n, int64_t batch, uint64_t seed, int step,
-                                                       float inv_sw, float* __restrict__ part_g,
-                                                       double* __restrict__ part_l) {
+__global__ void __launch_bounds__(TTH, 2) mlp_grad_kernel(const float* __restrict__ Pg, const float* __restrict__ X,
+                                                          const float* __restrict__ Y, const float* __restrict__ Wt,
+                                                          int64_t n, int64_t batch, uint64_t seed, int step,
+                                                          float inv_sw, float* __restrict__ part_g,
+                                                          double* __restrict__ part_l) {
+  static_assert(TTH == 256 && TCH == 64 && MLP_NH == 64 && MLP_NIN == 8, "thread mapping below");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  for (int i = threadIdx.x; i < MLP_NPARAM; i += blockDim.x) {
-    S.P[i] = Pg[i];
-    S.G[i] = 0.f;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < MLP_NH * MLP_NH; i += TTH) {
+    S.W2[(i >> 6) * TS + (i & 63)] = Pg[MLP_OFF_W2 + i];
+    S.W3[(i >> 6) * TS + (i & 63)] = Pg[MLP_OFF_W3 + i];
   }
-  const float* W1 = S.P + MLP_OFF_W1;
-  const float* b1 = S.P + MLP_OFF_B1;
-  const float* W2 = S.P + MLP_OFF_W2;
-  const float* b2 = S.P + MLP_OFF_B2;
-  const float* W3 = S.P + MLP_OFF_W3;
-  const float* b3 = S.P + MLP_OFF_B3;
-  const float* w4 = S.P + MLP_OFF_W4;
+  for (int i = tid; i < MLP_NH * MLP_NIN; i += TTH) S.W1[i] = Pg[MLP_OFF_W1 + i];
+  if (tid < MLP_NH) {
+    S.b1[tid] = Pg[MLP_OFF_B1 + tid];
+    S.b2[tid] = Pg[MLP_OFF_B2 + tid];
+    S.b3[tid] = Pg[MLP_OFF_B3 + tid];
+    S.w4[tid] = Pg[MLP_OFF_W4 + tid];
+  }
+  if (tid == 0) S.b4 = Pg[MLP_OFF_B4];
+  // tile of a 64 x 64 result: rows r0..r0+3, columns c0..c0+3
+  const int cx = tid & 15, r0 = 4 * (tid >> 4), c0 = 4 * cx;
+  // one sample and one quarter of the features in the output sum
+  const int sample = tid & 63, part = tid >> 6;
   const int64_t total = batch > 0 ? batch : n;
   const int64_t nchunks = (total + TCH - 1) / TCH;
+  const bool x_aligned = (reinterpret_cast<uintptr_t>(X) & 15) == 0;  // the caller's rows may start anywhere
   double lsum = 0.0;
+  float g2[4][4] = {}, g3[4][4] = {};
+  float g1[2] = {0.f, 0.f};              // W1 entries 2 tid, 2 tid + 1
+  float gb = 0.f, gw4 = 0.f, gb4 = 0.f;  // gb: b1, b2, b3 for the first three groups of 64 threads; gw4: the fourth
   __syncthreads();
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    for (int s = threadIdx.x; s < TCH; s += blockDim.x) {
-      const int64_t j = ch * TCH + s;
+    if (part < 2) {  // two threads per sample, four features each
+      const int64_t j = ch * TCH + sample;
       int64_t i = -1;
       if (j < total) i = batch > 0 ? (int64_t)(splitmix64(seed ^ splitmix64(((uint64_t)step << 32) + j)) % n) : j;
-      S.idx[s] = (int)i;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i >= 0) {
+        const float* xp = &X[i * MLP_NIN + 4 * part];
+        x = x_aligned ? *reinterpret_cast<const float4*>(xp) : make_float4(xp[0], xp[1], xp[2], xp[3]);
+      }
+      S.X[(4 * part) * TS + sample] = x.x;
+      S.X[(4 * part + 1) * TS + sample] = x.y;
+      S.X[(4 * part + 2) * TS + sample] = x.z;
+      S.X[(4 * part + 3) * TS + sample] = x.w;
+      if (part == 0) S.y[sample] = i >= 0 ? Y[i] : 0.f;
+      else S.w[sample] = i >= 0 ? Wt[i] * inv_sw : 0.f;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < TCH * MLP_NIN; e += blockDim.x) {
-      const int i = S.idx[e / MLP_NIN];
-      S.X[e] = i >= 0 ? X[(int64_t)i * MLP_NIN + e % MLP_NIN] : 0.f;
+    // layer 1
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float b = S.b1[r0 + i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = b;
     }
+#pragma unroll
+    for (int k = 0; k < MLP_NIN; ++k) {
+      float x[4];
+      ld4(&S.X[k * TS + c0], x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(S.W1[(r0 + i) * MLP_NIN + k], x[j], acc[i][j]);
+    }
+    auto relu_store = [&](float* H) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaxf(acc[i][j], 0.f);
+        st4(H + (r0 + i) * TS + c0, acc[i]);
+      }
+    };
+    auto set_bias = [&](const float* b) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = b[r0 + i];
+    };
+    relu_store(S.H1);
     __syncthreads();
-    dense_fwd(S.X, MLP_NIN, W1, b1, S.H1);
+    set_bias(S.b2);
+    tile_ab(S.W2, S.H1, r0, c0, acc);
+    relu_store(S.H2);
     __syncthreads();
-    dense_fwd(S.H1, MLP_NH, W2, b2, S.H2);
-    __syncthreads();
-    dense_fwd(S.H2, MLP_NH, W3, b3, S.H3);
+    set_bias(S.b3);
+    tile_ab(S.W3, S.H2, r0, c0, acc);
+    relu_store(S.H3);
     __syncthreads();
     // output, loss and dL/dz
-    for (int s = threadIdx.x; s < TCH; s += blockDim.x) {
-      const int i = S.idx[s];
+    {
+      float z = 0.f;
+#pragma unroll 4
+      for (int k = 16 * part; k < 16 * part + 16; ++k) z = fmaf(S.H3[k * TS + sample], S.w4[k], z);
+      S.zp[part][sample] = z;
+    }
+    __syncthreads();
+    if (part == 0) {
+      const float z = S.b4 + ((S.zp[0][sample] + S.zp[1][sample]) + (S.zp[2][sample] + S.zp[3][sample]));
+      const float w = S.w[sample];
       float dz = 0.f;
-      if (i >= 0) {
-        float z = S.P[MLP_OFF_B4];
-        for (int k = 0; k < MLP_NH; ++k) z = fmaf(S.H3[s * MLP_NH + k], w4[k], z);
+      if (ch * TCH + sample < total) {
         const float m = softplusf(z);
-        const float e = logf(m) - Y[i];
-        const float w = Wt[i] * inv_sw;
+        const float e = logf(m) - S.y[sample];
         lsum += (double)w * e * e;
         const float sig = 1.f / (1.f + expf(-z));
         dz = 2.f * w * e * sig / m;
       }
-      S.dz[s] = dz;
+      S.dz[sample] = dz;
     }
     __syncthreads();
-    // dA3 = dz w4 (H3 > 0), in place of H3 after its use for gw4
-    for (int k = threadIdx.x; k < MLP_NH; k += blockDim.x) {
-      float gw = 0.f;
-      for (int s = 0; s < TCH; ++s) gw = fmaf(S.dz[s], S.H3[s * MLP_NH + k], gw);
-      S.G[MLP_OFF_W4 + k] += gw;
-    }
-    if (threadIdx.x == 0) {
-      float gb = 0.f;
-      for (int s = 0; s < TCH; ++s) gb += S.dz[s];
-      S.G[MLP_OFF_B4] += gb;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < TCH * MLP_NH; e += blockDim.x) {
-      const int s = e / MLP_NH, k = e % MLP_NH;
-      S.H3[e] = S.H3[e] > 0.f ? S.dz[s] * w4[k] : 0.f;
-    }
-    __syncthreads();
-    // layer 3 gradients and dH2 = dA3 W3 (into D), then dA2 = dH2 (H2 > 0)
-    for (int e = threadIdx.x; e < MLP_NH * MLP_NH; e += blockDim.x) {
-      const int nn = e / MLP_NH, k = e % MLP_NH;
-      float gw = 0.f;
-      for (int s = 0; s < TCH; ++s) gw = fmaf(S.H3[s * MLP_NH + nn], S.H2[s * MLP_NH + k], gw);
-      S.G[MLP_OFF_W3 + e] += gw;
-    }
-    for (int nn = threadIdx.x; nn < MLP_NH; nn += blockDim.x) {
-      float gb = 0.f;
-      for (int s = 0; s < TCH; ++s) gb += S.H3[s * MLP_NH + nn];
-      S.G[MLP_OFF_B3 + nn] += gb;
-    }
-    for (int e = threadIdx.x; e < TCH * MLP_NH; e += blockDim.x) {
-      const int s = e / MLP_NH, k = e % MLP_NH;
-      float d = 0.f;
-      for (int nn = 0; nn < MLP_NH; ++nn) d = fmaf(S.H3[s * MLP_NH + nn], W3[nn * MLP_NH + k], d);
-      S.D[e] = S.H2[e] > 0.f ? d : 0.f;
+    // w4 and b4, then dA3 = dz w4 (H3 > 0) in place of H3
+    if (part == 3) {
+      const float* h = S.H3 + sample * TS;  // here `sample` is a feature
+      float t[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int q = 0; q < TCH; q += 4) {
+        float v[4], d[4];
+        ld4(h + q, v);
+        ld4(S.dz + q, d);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = fmaf(v[j], d[j], t[j]);
+      }
+      gw4 += (t[0] + t[1]) + (t[2] + t[3]);
+    } else if (tid == 0) {
+      gb4 += row_sum(S.dz);
     }
     __syncthreads();
-    // layer 2 gradients and dH1 = dA2 W2 (into H3), then dA1 = dH1 (H1 > 0)
-    for (int e = threadIdx.x; e < MLP_NH * MLP_NH; e += blockDim.x) {
-      const int nn = e / MLP_NH, k = e % MLP_NH;
-      float gw = 0.f;
-      for (int s = 0; s < TCH; ++s) gw = fmaf(S.D[s * MLP_NH + nn], S.H1[s * MLP_NH + k], gw);
-      S.G[MLP_OFF_W2 + e] += gw;
-    }
-    for (int nn = threadIdx.x; nn < MLP_NH; nn += blockDim.x) {
-      float gb = 0.f;
-      for (int s = 0; s < TCH; ++s) gb += S.D[s * MLP_NH + nn];
-      S.G[MLP_OFF_B2 + nn] += gb;
-    }
-    for (int e = threadIdx.x; e < TCH * MLP_NH; e += blockDim.x) {
-      const int s = e / MLP_NH, k = e % MLP_NH;
-      float d = 0.f;
-      for (int nn = 0; nn < MLP_NH; ++nn) d = fmaf(S.D[s * MLP_NH + nn], W2[nn * MLP_NH + k], d);
-      S.H3[e] = S.H1[e] > 0.f ? d : 0.f;
+    {
+      float d[4];
+      ld4(S.dz + c0, d);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float w = S.w4[r0 + i];
+        float h[4];
+        ld4(S.H3 + (r0 + i) * TS + c0, h);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) h[j] = h[j] > 0.f ? d[j] * w : 0.f;
+        st4(S.H3 + (r0 + i) * TS + c0, h);
+      }
     }
     __syncthreads();
-    // layer 1 gradients
-    for (int e = threadIdx.x; e < MLP_NH * MLP_NIN; e += blockDim.x) {
-      const int nn = e / MLP_NIN, k = e % MLP_NIN;
-      float gw = 0.f;
-      for (int s = 0; s < TCH; ++s) gw = fmaf(S.H3[s * MLP_NH + nn], S.X[s * MLP_NIN + k], gw);
-      S.G[MLP_OFF_W1 + e] += gw;
+    // a layer's gradient and dA of the layer below: D = (W^T dA) (H > 0)
+    auto backward = [&](const float* dA, const float* W, const float* H, float* Dn) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+      tile_atb(W, dA, r0, c0, acc);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float h[4];
+        ld4(H + (r0 + i) * TS + c0, h);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = h[j] > 0.f ? acc[i][j] : 0.f;
+        st4(Dn + (r0 + i) * TS + c0, acc[i]);
+      }
+    };
+    tile_abt(S.H3, S.H2, r0, cx, g3);
+    if (part == 2) gb += row_sum(S.H3 + sample * TS);
+    backward(S.H3, S.W3, S.H2, S.D);
+    __syncthreads();
+    tile_abt(S.D, S.H1, r0, cx, g2);
+    if (part == 1) gb += row_sum(S.D + sample * TS);
+    backward(S.D, S.W2, S.H1, S.H3);
+    __syncthreads();
+    // layer 1
+    {
+      const float* d = S.H3 + (tid >> 2) * TS;
+      const float* x0 = S.X + (2 * (tid & 3)) * TS;
+      float t[2][4] = {};
+#pragma unroll 4
+      for (int q = 0; q < TCH; q += 4) {
+        float v[4], a[4], b[4];
+        ld4(d + q, v);
+        ld4(x0 + q, a);
+        ld4(x0 + TS + q, b);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          t[0][j] = fmaf(v[j], a[j], t[0][j]);
+          t[1][j] = fmaf(v[j], b[j], t[1][j]);
+        }
+      }
+      g1[0] += (t[0][0] + t[0][1]) + (t[0][2] + t[0][3]);
+      g1[1] += (t[1][0] + t[1][1]) + (t[1][2] + t[1][3]);
     }
-    for (int nn = threadIdx.x; nn < MLP_NH; nn += blockDim.x) {
-      float gb = 0.f;
-      for (int s = 0; s < TCH; ++s) gb += S.H3[s * MLP_NH + nn];
-      S.G[MLP_OFF_B1 + nn] += gb;
-    }
+    if (part == 0) gb += row_sum(S.H3 + sample * TS);
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < MLP_NPARAM; i += blockDim.x) part_g[(int64_t)blockIdx.x * MLP_NPARAM + i] = S.G[i];
-  // loss partial of the CTA (fixed order: per-thread sums, then thread order)
-  __shared__ double ls[TTH];
-  ls[threadIdx.x] = lsum;
+  float* out = part_g + (int64_t)blockIdx.x * MLP_NPARAM;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      out[MLP_OFF_W2 + (r0 + i) * MLP_NH + cx + 16 * j] = g2[i][j];
+      out[MLP_OFF_W3 + (r0 + i) * MLP_NH + cx + 16 * j] = g3[i][j];
+    }
+  out[MLP_OFF_W1 + 2 * tid] = g1[0];
+  out[MLP_OFF_W1 + 2 * tid + 1] = g1[1];
+  if (part == 0) out[MLP_OFF_B1 + sample] = gb;
+  if (part == 1) out[MLP_OFF_B2 + sample] = gb;
+  if (part == 2) out[MLP_OFF_B3 + sample] = gb;
+  if (part == 3) out[MLP_OFF_W4 + sample] = gw4;
+  if (tid == 0) out[MLP_OFF_B4] = gb4;
+  // loss partial of the CTA: the first two warps hold the samples' terms
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+  __shared__ double ls[2];
+  if (tid < 64 && (tid & 31) == 0) ls[tid >> 5] = lsum;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < (int)blockDim.x; ++i) t += ls[i];
-    part_l[blockIdx.x] = t;
-  }
+  if (tid == 0) part_l[blockIdx.x] = ls[0] + ls[1];
 }
 
-__global__ void mlp_reduce_kernel(const float* __restrict__ part_g, const double* __restrict__ part_l, int nb,
-                                  float* __restrict__ grad, double* __restrict__ loss) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < MLP_NPARAM) {
-    float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part_g[(int64_t)b * MLP_NPARAM + i];
-    grad[i] = s;
-  }
-  if (i == 0 && loss) {
+// Sums the CTAs' partials in a fixed order: a CTA takes 32 parameters, its
+// eight warps an eighth of the partials each; the warp of one more CTA sums the
+// loss.
+constexpr int RED_WARPS = 8;
+__global__ void __launch_bounds__(32 * RED_WARPS) mlp_reduce_kernel(const float* __restrict__ part_g,
+                                                                    const double* __restrict__ part_l, int nb,
+                                                                    float* __restrict__ grad,
+                                                                    double* __restrict__ loss) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (warp != 0 || loss == nullptr) return;
     double t = 0.0;
-    for (int b = 0; b < nb; ++b) t += part_l[b];
-    *loss = t;
+    for (int b = lane; b < nb; b += 32) t += part_l[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) *loss = t;
+    return;
+  }
+  __shared__ float sums[RED_WARPS][32];
+  const int i = blockIdx.x * 32 + lane;
+  const int per = (nb + RED_WARPS - 1) / RED_WARPS, b0 = warp * per, b1 = min(nb, b0 + per);
+  float s = 0.f;
+  if (i < MLP_NPARAM) {
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) s += part_g[(int64_t)b * MLP_NPARAM + i];
+  }
+  sums[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && i < MLP_NPARAM) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < RED_WARPS; ++w) t += sums[w][lane];
+    grad[i] = t;
   }
 }
 
@@ -537,7 +702,7 @@ cudaError_t launch_mlp_grad(const float* P, const float* X, const float* Y, cons
   if (e != cudaSuccess) return e;
   mlp_grad_kernel<<<nblocks, TTH, smem, s>>>(P, X, Y, Wt, n, batch, seed, step, inv_sw, part_g, part_l);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  mlp_reduce_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(part_g, part_l, nblocks, grad, loss);
+  mlp_reduce_kernel<<<(MLP_NPARAM + 31) / 32 + 1, 32 * RED_WARPS, 0, s>>>(part_g, part_l, nblocks, grad, loss);
   return cudaGetLastError();
 }
 
