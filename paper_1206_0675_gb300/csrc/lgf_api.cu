@@ -537,8 +537,8 @@ template <typename R> cudaError_t enqueue_or_sweeps(lgf_ctx* h, Lane<R>& L, doub
   C2<R>* U1 = L.fused ? L.U2 : nullptr;
   for (int k = 0; k < n; ++k)
     for (int parity = 0; parity < 2; ++parity) {
-      cudaError_t e = L.rows == 3 ? launch_or_half_sweep<R, 3>(h->geom, L.U, U1, h->st, L.G, parity, omega, s)
-                                  : launch_or_half_sweep<R, 2>(h->geom, L.U, U1, h->st, L.G, parity, omega, s);
+      cudaError_t e = L.rows == 3 ? launch_or_half_sweep<R, 3>(h->geom, L.U, U1, h->st, L.g, L.G, parity, omega, s)
+                                  : launch_or_half_sweep<R, 2>(h->geom, L.U, U1, h->st, L.g, L.G, parity, omega, s);
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;

@@ -135,8 +135,8 @@ template <int SIGN> __device__ __forceinline__ I2 imul_i(I2 a) {  // times SIGN 
 // v w (SIGN < 0) or v conj(w) for a table entry w = (cos h, l, sin h, l).
 template <int SIGN> __device__ __forceinline__ I2 itwiddle(I2 v, int4 w) {
   const Bfp2 x = bfp_limbs(v.x), y = bfp_limbs(v.y);
-  const int sh = SIGN < 0 ? w.z : -w.z, sl = SIGN < 0 ? w.w : -w.w;
-  const int nh = -sh, nl = -sl;
+  const int sh = fx_opaque(SIGN < 0 ? w.z : -w.z), sl = fx_opaque(SIGN < 0 ? w.w : -w.w);
+  const int nh = fx_opaque(SIGN < 0 ? -w.z : w.z), nl = fx_opaque(SIGN < 0 ? -w.w : w.w);
   const int64_t half = (int64_t)1 << 29;
   int64_t rm = mad_wide(x.l, w.x, mad_wide(x.h, w.y, half));
   int64_t im = mad_wide(x.l, sh, mad_wide(x.h, sl, half));

@@ -30,6 +30,17 @@ constexpr uint32_t FX_LIM_HI = 0x3ff20000u;
 // high word of 2^-12: below it an FP64 rounding (2^-65) is finer than the unit
 constexpr uint32_t FX_WEAK_HI = 0x3f300000u;
 
+// c + a b with a 64-bit sum: one IMAD.WIDE.  (Both factors have to look like
+// signed 32-bit words to the compiler, which turns products with a factor of
+// known range or sign into 64 x 64 bit ones and differences: every operand
+// passes through fx_opaque.  Written in PTX the sum costs a register move per
+// product.)
+__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c) { return c + (int64_t)a * b; }
+__device__ __forceinline__ int fx_opaque(int a) {
+  asm("" : "+r"(a));
+  return a;
+}
+
 struct Fx {
   int h, l;
 };
@@ -58,7 +69,7 @@ __device__ __forceinline__ uint32_t shr32_clamp(uint32_t x, uint32_t s) {
 
 // The operand of a number in units of 2^-60.
 __device__ __forceinline__ Fx fx_operand(int64_t r60) {
-  return Fx{(int)((r60 + ((int64_t)1 << 29)) >> 30), (int)((uint32_t)r60 << 2) >> 2};
+  return Fx{fx_opaque((int)((r60 + ((int64_t)1 << 29)) >> 30)), fx_opaque((int)((uint32_t)r60 << 2) >> 2)};
 }
 
 // Fixed point from FP64 in units of 2^-60, |a| < 2; what lies below is cut off.
@@ -72,17 +83,9 @@ __device__ __forceinline__ int64_t fx60_from(double a) {
 }
 __device__ __forceinline__ Fx fx_from(double a) { return fx_operand(fx60_from(a)); }
 __device__ __forceinline__ FxC fx_from(double2 a) { return FxC{fx_from(a.x), fx_from(a.y)}; }
-__device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }
+__device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{fx_opaque(-a.h), fx_opaque(-a.l)}; }
 __device__ __forceinline__ FxC fx_neg(FxC a) { return FxC{fx_neg(a.x), fx_neg(a.y)}; }
 __device__ __forceinline__ FxC fx_conj(FxC a) { return FxC{a.x, fx_neg(a.y)}; }
-
-// c + a b with a 64-bit sum: one IMAD.WIDE (written out, so that sums of
-// products are not taken apart into products and 64-bit additions).
-__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c) {
-  int64_t r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
 
 // Two-part accumulator of real products.
 struct FxAcc {
@@ -208,7 +211,9 @@ __device__ __forceinline__ double bfp_to_double(int64_t n, int ex) {
 struct Bfp2 {
   int h, l;
 };
-__device__ __forceinline__ Bfp2 bfp_limbs(int64_t x) { return Bfp2{(int)(x >> 30), (int)((uint32_t)x & 0x3fffffffu)}; }
+__device__ __forceinline__ Bfp2 bfp_limbs(int64_t x) {
+  return Bfp2{fx_opaque((int)(x >> 30)), fx_opaque((int)((uint32_t)x & 0x3fffffffu))};
+}
 
 // Real and complex products with a constant or a root of unity w, |w| <= 1,
 // w = h 2^-30 + l 2^-60 (|l| <= 2^29): three multiply-adds per real product,

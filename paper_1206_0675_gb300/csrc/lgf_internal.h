@@ -174,11 +174,12 @@ cudaError_t launch_filter_table(const Geom& g, const double* sin2 /* 4 x Lmax: 4
 // every site x with (x + y + z + t) % 2 == parity gets g(x), and
 // U_mu(x) <- g(x) U_mu(x), U_mu(x - mu^) <- U_mu(x - mu^) g^dag(x), in place.
 // Links of precision R with ROWS stored rows; U1 != nullptr (fused lanes):
-// the current links are U1 when st->ubuf is set, else U0.  G != nullptr:
+// the current links are U1 when st->ubuf is set, else U0.  gfield: the lane's g,
+// in which FP64 lanes keep g(x) between their two kernels.  G != nullptr:
 // G(x) <- g(x) G(x) (3 rows, precision R).  Every extent must be even.
 template <typename R, int ROWS>
-cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* G, int parity,
-                                 double omega, cudaStream_t s);
+cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* gfield, C2<R>* G,
+                                 int parity, double omega, cudaStream_t s);
 
 // ---- lgf_fft.cu ---------------------------------------------------------
 // Radix schedule of one lattice direction.

@@ -132,12 +132,10 @@ __device__ __forceinline__ int64_t or_coords(const Geom& g, const FastDiv& dhx, 
   return (int64_t)c[0] + (int64_t)g.L[0] * row;
 }
 
-// One site of the colour: its hit and the products with its eight links.
+// w(x) = sum_mu [U_mu(x) + U_mu^dag(x - mu^)]
 template <typename R, int ROWS>
-__device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
-                                        C2<R>* __restrict__ G, R omega) {
-  // w(x) = sum_mu [U_mu(x) + U_mu^dag(x - mu^)]
-  M3<R> M;
+__device__ __forceinline__ void or_local_field(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
+                                               M3<R>& M) {
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -156,7 +154,14 @@ __device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& 
 #pragma unroll
       for (int k = 0; k < 3; ++k) M.e[r][k] = cadd<R>(M.e[r][k], cconj<R>(u.e[k][r]));
   }
+}
 
+// One site of the colour: its hit and the products with its eight links.
+template <typename R, int ROWS>
+__device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
+                                        C2<R>* __restrict__ G, R omega) {
+  M3<R> M;
+  or_local_field<R, ROWS>(g, U, c, s, M);
   M3<R> gx;
   or_site_gauge<R>(M, omega, gx);
 
@@ -228,17 +233,14 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // FP64 links in fixed point (lgf_fixed.cuh)
 // ---------------------------------------------------------------------------
 //
-// A CTA takes 32 sites, one direction per warp: every thread converts its
-// forward and its backward link once and keeps them as operands, the four
-// warps' parts of w(x) meet in shared memory, the first warp does the hits and
-// every thread multiplies its two links.  Sites with a link outside the
-// fixed-point range or near the identity (see update_fx_kernel), or with a
-// local field too small for its direction to be resolved, are done by one
-// thread in FP64.
-// With FP64 arithmetic one thread a site kept the FP64 pipe 93 % busy (1199
-// operations a site and sweep); now the integer pipe bounds it, with 12 warps
-// per SM at 168 registers.  24^4, 18-real: 20 sweeps with set_links and get_links 15.4
-// -> 8.6 ms; error of 20 sweeps against 64 bits 2.2e-15 -> 1.7e-15.
+// Two kernels per colour: the first forms w(x) and g(x) of the colour's sites,
+// one thread each; the second multiplies every link of the lattice by the one
+// g that touches it, one thread per link, as in update_fx_kernel.  Sites and
+// links outside the fixed-point range or near the identity, and local fields
+// too small for their direction to be resolved, are done in FP64.
+// With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
+// busy (1199 operations a site and sweep).  One fixed-point kernel with the
+// hits between two barriers left three of four warps waiting for them.
 
 // The 64-bit sum an operand stands for (units of 2^-60).
 __device__ __forceinline__ int64_t fx_r60(Fx a) { return mad_wide(a.h, 1 << 30, (int64_t)a.l); }
@@ -333,160 +335,220 @@ __device__ __forceinline__ void or_site_gauge_fx(FxC M[3][3], Fx w7, int64_t c7,
   for (int c = 0; c < 3; ++c) or_rot_fx(a, b, gx[1][c], gx[2][c]);
 }
 
+// g(x) of a site from FP64 sums, and its store.
 template <int ROWS>
-static __device__ __noinline__ void or_site_fp64(const Geom& g, MatField<double, ROWS> U, int64_t s, double2* G,
-                                                 double omega) {
+static __device__ __noinline__ void or_gauge_fp64(const Geom& g, MatField<double, ROWS> U, int64_t s,
+                                                  double2* __restrict__ gf, double omega) {
   int c[4];
   site_coords(g, s, c);
-  or_site<double, ROWS>(g, U, c, s, G, omega);
+  M3<double> M, gx;
+  or_local_field<double, ROWS>(g, U, c, s, M);
+  or_site_gauge<double>(M, omega, gx);
+  fxg_store(gf, g.V, s, gx.e[0], gx.e[1], gx.e[2]);
 }
 
-// Link (mu, s) as operands, its entries in the range tests.
 template <int ROWS>
-__device__ __forceinline__ void or_load_fx(const MatField<double, ROWS>& U, int mu, int64_t s, FxC x[3][3], uint32_t& m,
-                                           uint32_t& t, bool& weak) {
-  double2 u[ROWS][3];
+__global__ void __launch_bounds__(OR_THREADS)
+or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, double2* __restrict__ G, int parity,
+                   FastDiv dhx, double omega, int64_t w7, int64_t c7) {
+  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if ((int64_t)j >= (g.V >> 1)) return;
+  int c[4];
+  const int64_t s = or_coords(g, dhx, j, parity, c);
+  // w(x) in units of 2^-58
+  int64_t W[9][2];
 #pragma unroll
-  for (int r = 0; r < ROWS; ++r)
+  for (int e = 0; e < 9; ++e) W[e][0] = W[e][1] = 0;
+  uint32_t m = 0, t = 0, strong = 0;
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    const int mu = k >> 1;
+    const bool fwd = (k & 1) == 0;
+    const int64_t sl = fwd ? s : or_back(g, s, c, mu);
+    double2 u[ROWS][3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) u[r][k] = U.p[U.off(mu, r, k, s)];
+    for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-  for (int r = 0; r < ROWS; ++r)
+      for (int q = 0; q < 3; ++q) u[r][q] = __ldg(&U.p[U.off(mu, r, q, sl)]);
+    int64_t x[3][3][2];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        m = fx_max(m, u[r][q]);
+        x[r][q][0] = fx58_from(u[r][q].x);
+        x[r][q][1] = fx58_from(u[r][q].y);
+      }
+    strong = max(strong, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]));
+    if (ROWS == 2) {
+      FxC a[2][3];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) a[r][q] = FxC{fx_operand58(x[r][q][0]), fx_operand58(x[r][q][1])};
+      int64_t c3[3][2];
+      fx_third_row(a[0], a[1], c3, t);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        x[2][q][0] = c3[q][0] >> 2;
+        x[2][q][1] = c3[q][1] >> 2;
+      }
+    }
+    if (fwd) {
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        W[e][0] += x[e / 3][e % 3][0];
+        W[e][1] += x[e / 3][e % 3][1];
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        W[e][0] += x[e % 3][e / 3][0];
+        W[e][1] -= x[e % 3][e / 3][1];
+      }
+    }
+  }
+  FxC M[3][3], gx[3][3];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) M[e / 3][e % 3] = FxC{fx_operand(W[e][0] >> 4), fx_operand(W[e][1] >> 4)};  // w / 64
+  bool ok = !fx_bad(m, t) && strong >= FX_WEAK_HI;
+  or_site_gauge_fx(M, fx_operand(w7), c7, gx, ok);
+  if (ok) {
+    int4* p = reinterpret_cast<int4*>(gf);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) p[e * g.V + s] = fxg_pack(gx[e / 3][e % 3]);
+  } else {
+    or_gauge_fp64<ROWS>(g, U, s, gf, omega);
+  }
+  if (G != nullptr) accumulate_gauge_fx(g.V, s, reinterpret_cast<const int4*>(gf) + s, g.V, G);
+}
+
+// One link in FP64: fwd ? g U : U g^dag.
+template <int ROWS>
+static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const double2* gf, int mu, int64_t sl,
+                                                 int64_t s, bool fwd) {
+  M3<double> g, u, o;
+  fxg_load(gf, U.V, s, g);
+  U.load(mu, sl, u);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      double2 acc;
+      if (fwd) {
+        acc = cmul_fx<double>(g.e[i][0], u.e[0][k]);
+        acc = cfma<double>(g.e[i][1], u.e[1][k], acc);
+        o.e[i][k] = cfma<double>(g.e[i][2], u.e[2][k], acc);
+      } else {
+        acc = cmulc_fx<double>(u.e[i][0], g.e[k][0]);
+        acc = cfmac<double>(u.e[i][1], g.e[k][1], acc);
+        o.e[i][k] = cfmac<double>(u.e[i][2], g.e[k][2], acc);
+      }
+    }
+  su3_third_row<double>(o.e[0], o.e[1], o.e[2]);
+  U.store(mu, sl, o);
+}
+
+// A CTA takes 32 sites of the colour and half of their links: four warps, the
+// directions' forward (blockIdx.y = 0) or backward links.
+template <int ROWS>
+__global__ void __launch_bounds__(OR_THREADS, 5)
+or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__ gf, int parity, FastDiv dhx) {
+  const uint32_t j = blockIdx.x * 32u + (threadIdx.x & 31u);
+  const int mu = threadIdx.x >> 5;
+  const bool fwd = blockIdx.y == 0;
+  if ((int64_t)j >= (g.V >> 1)) return;
+  int c[4];
+  const int64_t s = or_coords(g, dhx, j, parity, c);
+  const int64_t sl = fwd ? s : or_back(g, s, c, mu);
+  const int4* p = reinterpret_cast<const int4*>(gf);
+  constexpr int UR = ROWS;
+  double2 u[UR][3];
+  int4 g4[3][3];
+#pragma unroll
+  for (int r = 0; r < UR; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[r][k] = U.p[U.off(mu, r, k, sl)];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) g4[e / 3][e % 3] = __ldg(&p[e * g.V + s]);
+  uint32_t m = 0, t = 0;
+  FxC x[3][3];
+#pragma unroll
+  for (int r = 0; r < UR; ++r)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       m = fx_max(m, u[r][k]);
       x[r][k] = fx_from(u[r][k]);
     }
-  weak = weak || fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_WEAK_HI;
-  if (ROWS == 2) {
-    int64_t c3[3][2];
-    fx_third_row(x[0], x[1], c3, t);
+  const uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
+  int64_t n[2][3][2];
+  if (fwd) {
+    if (ROWS == 2) {
+      int64_t c3[3][2];
+      fx_third_row(x[0], x[1], c3, t);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) x[2][k] = FxC{fx_operand(c3[k][0]), fx_operand(c3[k][1])};
+      for (int k = 0; k < 3; ++k) x[2][k] = FxC{fx_operand(c3[k][0]), fx_operand(c3[k][1])};
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const FxC a = fxg_unpack(g4[i][q]);
+          fx_cmac(re, im, a, fx_neg(a.y), x[q][k]);
+        }
+        n[i][k][0] = fx_sum60(re, t);
+        n[i][k][1] = fx_sum60(im, t);
+      }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        FxAcc re = fx_zero(), im = fx_zero();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) fx_cmacc(re, im, x[i][q], fx_neg(x[i][q].x), fxg_unpack(g4[k][q]));
+        n[i][k][0] = fx_sum60(re, t);
+        n[i][k][1] = fx_sum60(im, t);
+      }
   }
-}
-
-template <int ROWS>
-__device__ __forceinline__ void or_store_fx(const MatField<double, ROWS>& U, int mu, int64_t s,
-                                            const int64_t n[2][3][2]) {
-  uint32_t t = 0;
   int64_t n3[3][2];
   if (ROWS == 3) {
     FxC r[2][3];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) r[i][j] = FxC{fx_operand(n[i][j][0]), fx_operand(n[i][j][1])};
+      for (int k = 0; k < 3; ++k) r[i][k] = FxC{fx_operand(n[i][k][0]), fx_operand(n[i][k][1])};
     fx_third_row(r[0], r[1], n3, t);
+  }
+  if (fx_bad(m, t) || w < FX_WEAK_HI || g4[0][0].x == FX_G_NAN) {
+    or_link_fp64<ROWS>(U, gf, mu, sl, s, fwd);
+    return;
   }
   double2 o[ROWS][3];
   fx_link_to_double<ROWS>(n, n3, o);
 #pragma unroll
-  for (int i = 0; i < ROWS; ++i)
+  for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) U.p[U.off(mu, i, j, s)] = o[i][j];
-}
-
-template <int ROWS>
-__global__ void __launch_bounds__(OR_THREADS, 3)
-or_half_sweep_fx_kernel(Geom g, double2* __restrict__ U0, double2* __restrict__ G, int parity, FastDiv dhx,
-                        double omega, int64_t w7, int64_t c7) {
-  __shared__ int64_t part[4][18][32];  // each direction's part of w(x), units of 2^-58
-  __shared__ int4 gs[9][32];
-  __shared__ int skip[32];
-  const MatField<double, ROWS> U{U0, g.V};
-  const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
-  const uint32_t n_sites = (uint32_t)(g.V >> 1), j = blockIdx.x * 32u + (uint32_t)lane;
-  const bool live = j < n_sites;
-  int c[4];
-  const int64_t s = or_coords(g, dhx, min(j, n_sites - 1u), parity, c);
-  const int64_t sb = or_back(g, s, c, mu);
-  if (threadIdx.x < 32) skip[lane] = 0;
-  FxC uf[3][3], ub[3][3];
-  uint32_t m = 0, t = 0;
-  bool weak = false;
-  or_load_fx<ROWS>(U, mu, s, uf, m, t, weak);
-  or_load_fx<ROWS>(U, mu, sb, ub, m, t, weak);
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      part[mu][2 * (3 * r + k)][lane] = (fx_r60(uf[r][k].x) >> 2) + (fx_r60(ub[k][r].x) >> 2);
-      part[mu][2 * (3 * r + k) + 1][lane] = (fx_r60(uf[r][k].y) >> 2) - (fx_r60(ub[k][r].y) >> 2);
-    }
-  __syncthreads();
-  if (fx_bad(m, t) || weak) skip[lane] = 1;
-  if (mu == 0) {
-    FxC M[3][3], gx[3][3];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      int64_t x = 0, y = 0;
-#pragma unroll
-      for (int d = 0; d < 4; ++d) {
-        x += part[d][2 * e][lane];
-        y += part[d][2 * e + 1][lane];
-      }
-      M[e / 3][e % 3] = FxC{fx_operand(x >> 4), fx_operand(y >> 4)};  // w / 64
-    }
-    bool ok = true;
-    or_site_gauge_fx(M, fx_operand(w7), c7, gx, ok);
-    if (!ok) skip[lane] = 1;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) gs[e][lane] = fxg_pack(gx[e / 3][e % 3]);
-  }
-  __syncthreads();
-  if (!live) return;
-  if (skip[lane]) {
-    if (mu == 0) or_site_fp64<ROWS>(g, U, s, G, omega);
-    return;
-  }
-  int64_t n[2][3][2];
-  t = 0;
-  // U_mu(x) <- g U_mu(x)
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    FxC gr[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gr[k] = fxg_unpack(gs[3 * i + k][lane]);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      FxAcc re = fx_zero(), im = fx_zero();
-#pragma unroll
-      for (int q = 0; q < 3; ++q) fx_cmac(re, im, gr[q], fx_neg(gr[q].y), uf[q][k]);
-      n[i][k][0] = fx_sum60(re, t);
-      n[i][k][1] = fx_sum60(im, t);
-    }
-  }
-  or_store_fx<ROWS>(U, mu, s, n);
-  // U_mu(x - mu^) <- U_mu(x - mu^) g^dag
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    FxC gr[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) gr[q] = fxg_unpack(gs[3 * k + q][lane]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      FxAcc re = fx_zero(), im = fx_zero();
-#pragma unroll
-      for (int q = 0; q < 3; ++q) fx_cmacc(re, im, ub[i][q], fx_neg(ub[i][q].x), gr[q]);
-      n[i][k][0] = fx_sum60(re, t);
-      n[i][k][1] = fx_sum60(im, t);
-    }
-  }
-  or_store_fx<ROWS>(U, mu, sb, n);
-  if (G != nullptr && mu == 0) accumulate_gauge_fx(g.V, s, &gs[0][lane], 32, G);
+    for (int k = 0; k < 3; ++k) U.p[U.off(mu, r, k, sl)] = o[r][k];
 }
 
 template <typename R, int ROWS>
-cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* G, int parity,
-                                 double omega, cudaStream_t s) {
+cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* gfield, C2<R>* G,
+                                 int parity, double omega, cudaStream_t s) {
   const int64_t n = g.V >> 1;
   const FastDiv dhx = FastDiv::make((uint32_t)g.L[0] / 2);
   if constexpr (sizeof(R) == sizeof(double)) {
     // FP64 lanes have one link buffer
     const int64_t w7 = std::llround(std::ldexp(7.0 * omega, 56)), c7 = std::llround(std::ldexp(7.0 * (1.0 - omega), 56));
-    or_half_sweep_fx_kernel<ROWS><<<(unsigned)((n + 31) / 32), OR_THREADS, 0, s>>>(g, U0, G, parity & 1, dhx, omega, w7,
-                                                                                   c7);
+    const MatField<double, ROWS> U{U0, g.V};
+    or_gauge_fx_kernel<ROWS><<<(unsigned)((n + OR_THREADS - 1) / OR_THREADS), OR_THREADS, 0, s>>>(
+        g, U, gfield, G, parity & 1, dhx, omega, w7, c7);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    or_links_fx_kernel<ROWS><<<dim3((unsigned)((n + 31) / 32), 2), OR_THREADS, 0, s>>>(g, U, gfield, parity & 1, dhx);
   } else {
     const unsigned nb = (unsigned)((n + OR_THREADS - 1) / OR_THREADS);
     or_half_sweep_kernel<R, ROWS><<<nb, OR_THREADS, 0, s>>>(g, U0, U1, st, G, parity & 1, dhx, (R)omega);
@@ -494,13 +556,13 @@ cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevS
   return cudaGetLastError();
 }
 
-template cudaError_t launch_or_half_sweep<double, 3>(const Geom&, double2*, double2*, const DevState*, double2*, int,
+template cudaError_t launch_or_half_sweep<double, 3>(const Geom&, double2*, double2*, const DevState*, double2*, double2*, int,
                                                      double, cudaStream_t);
-template cudaError_t launch_or_half_sweep<double, 2>(const Geom&, double2*, double2*, const DevState*, double2*, int,
+template cudaError_t launch_or_half_sweep<double, 2>(const Geom&, double2*, double2*, const DevState*, double2*, double2*, int,
                                                      double, cudaStream_t);
-template cudaError_t launch_or_half_sweep<float, 3>(const Geom&, float2*, float2*, const DevState*, float2*, int,
+template cudaError_t launch_or_half_sweep<float, 3>(const Geom&, float2*, float2*, const DevState*, float2*, float2*, int,
                                                     double, cudaStream_t);
-template cudaError_t launch_or_half_sweep<float, 2>(const Geom&, float2*, float2*, const DevState*, float2*, int,
+template cudaError_t launch_or_half_sweep<float, 2>(const Geom&, float2*, float2*, const DevState*, float2*, float2*, int,
                                                     double, cudaStream_t);
 
 }  // namespace lgf

@@ -590,15 +590,15 @@ __device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatFiel
 // finer than the fixed-point unit, and entries outside its range take the
 // FP64 path.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
 // end at 2.4e-15 (FP64 products: 2.6e-15).
-// Bound by the integer pipe (2040 instructions a link, 504 of them IMAD.WIDE,
+// Bound by the integer pipe (1850 instructions a link, 504 of them IMAD.WIDE,
 // which run at about 30 of their 64 lanes a clock when all operands vary).
-// 32^4, us: 18-real 505, 12-real 431; with FP64 products 1176 and 1177 at 95 %
+// 32^4, us: 18-real 381, 12-real 346; with FP64 products 1176 and 1177 at 95 %
 // of the FP64 pipe.
 // One thread per link: a CTA takes 32 sites, one direction per warp, so that
 // the 24 operand loads of a link are all in flight before its arithmetic and
 // g(x) comes from L1 for three of the four warps.
 template <int LROWS>
-__global__ void __launch_bounds__(UPDATE_THREADS, 6)
+__global__ void __launch_bounds__(UPDATE_THREADS, 5)
 update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batch B) {
   if (batch_skip(B)) return;
   U.p += blockIdx.z * B.s_links;
