@@ -78,6 +78,24 @@ __device__ __forceinline__ double rsqrt_fp64(double x) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// FP64 <-> FP32 with IEEE rounding (to nearest, ties to even) on the integer
+// pipe: the conversion instructions share the FP64 pipe (2 per clock and SM).
+// Zeros, subnormal, infinite and NaN values take the conversion instruction.
+__device__ __forceinline__ float f64_to_f32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t mag = (hi & 0x7fffffffu) - (896u << 20);  // exponent rebiased from 1023 to 127
+  if (mag - (1u << 20) >= (253u << 20)) return (float)x;   // exponent field outside 1 to 253
+  uint32_t f = __funnelshift_l(lo, mag, 3);
+  const uint32_t rest = lo << 3;  // 29 bits below the FP32 significand
+  f += (rest > 0x80000000u || (rest == 0x80000000u && (f & 1u))) ? 1u : 0u;
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double f32_to_f64(float x) {
+  const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u >= 0x7f000000u) return (double)x;
+  return __hiloint2double((int)(((mag >> 3) + (896u << 20)) | (b & 0x80000000u)), (int)(b << 29));
+}
+
 // 3x3 complex matrix held in registers.
 template <typename R> struct M3 {
   C2<R> e[3][3];

@@ -171,3 +171,36 @@ def test_or_sweep_against_oracle(ext, name, omega):
             U1, G = lat.get_links(), lat.get_transform()
         assert np.max(np.abs(U1 - Uo)) < 1e-12
         assert np.max(np.abs(G - Go)) < 1e-12
+
+
+# ---------------------------------------------------------------------------
+# links in and out
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("where", [0, 1, 130, 2591])
+@pytest.mark.parametrize("bad", [False, True])
+def test_su3_check_accepts_and_rejects_by_its_bound(where, bad):
+    """|det U - 1| = 3 eps of one scaled matrix just below and just above 1e-10, first, last and inside a tile."""
+    ext = (3, 4, 6, 9)
+    U = fields.random_links(ext, 0.8, seed=6)
+    U.reshape(-1, 3, 3)[where] *= 1 + (3.4e-11 if bad else 3.25e-11)
+    with lgf.Lattice(ext, "fp64") as lat:
+        if bad:
+            with pytest.raises(lgf.LgfError) as e:
+                lat.set_links(U)
+            assert e.value.status == lgf.LGF_E_ARG
+        else:
+            lat.set_links(U)
+
+
+@pytest.mark.parametrize("name", ["random", "permutations", "weak 1e-40"])
+@pytest.mark.parametrize("ext", [(2, 2, 2, 2), (3, 4, 6, 9)])
+def test_links_round_trip(ext, name):
+    """FP64 links come back as they went in, FP32 links as their IEEE rounding (zeros and subnormals among them)."""
+    U = weak_links(ext, 1e-40) if name == "weak 1e-40" else CASES[name](ext)
+    with lgf.Lattice(ext, "fp64") as lat:
+        lat.set_links(U)
+        assert np.array_equal(lat.get_links(), U)
+    with lgf.Lattice(ext, "fp32") as lat:
+        lat.set_links(U)
+        assert np.array_equal(lat.get_links(), U.astype(np.complex64).astype(np.complex128))
