@@ -62,13 +62,13 @@ template <typename R> __device__ __forceinline__ float rows_defect(const C2<R> a
                fmaxf(fabsf((float)ip.x), fabsf((float)ip.y)));
 }
 
-// The links whose defect a measurement samples: every sixteenth warp of the
-// grid (warp index w with w % 16 == 0) takes direction (w / 16) % 4 of its 32
+// The links whose defect a measurement samples: every sixteenth group of 32
+// sites (group w with w % 16 == 0) takes direction (w / 16) % 4 of its 32
 // sites, i.e. one link in 64, spread over all directions (the drift the
 // guard watches is slow and lattice-wide).  The choice is uniform within a
 // warp, so the other warps skip the work entirely.
-__device__ __forceinline__ int defect_sample_mu() {
-  const unsigned w = (unsigned)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+__device__ __forceinline__ int defect_sample_mu(int64_t s) {
+  const unsigned w = (unsigned)(s >> 5);
   return (w & 15u) == 0 ? (int)((w >> 4) & 3u) : -1;
 }
 
@@ -78,8 +78,8 @@ __device__ __forceinline__ int defect_sample_mu() {
 // the batch retirement flag or the graph's WHILE condition; flip_ubuf != 0
 // also flips st->ubuf (after every CTA has read it); fp64 != 0 marks the
 // measurement as one of FP64 links in the trace flags.
-// fsum and tsum are one site's sums, already in FP64; every sum above a
-// site (warp, CTA, grid) is FP64 in a fixed order.
+// fsum and tsum are the sums over the sites a thread collected, in FP64; every
+// sum above a site (thread, warp, CTA, grid) is FP64 in a fixed order.
 __device__ __forceinline__ void measure_tail(const Geom& g, double fsum, double tsum, float dmax,
                                              double* __restrict__ partials, DevState* __restrict__ st, int count_iter,
                                              unsigned long long cond, int use_cond, bool batch, int flip_ubuf,
@@ -103,6 +103,7 @@ __device__ __forceinline__ void measure_tail(const Geom& g, double fsum, double 
   // which CTA finished last), so the result is bit-reproducible.
   double f = 0.0, t = 0.0;
   float d = 0.f;
+#pragma unroll 8
   for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
     f += __ldcg(&partials[MEASURE_PARTIALS * i]);
     t += __ldcg(&partials[MEASURE_PARTIALS * i + 1]);
@@ -182,98 +183,166 @@ __device__ __forceinline__ R delta_norm2(R a0, R a1, R a2, C2<R> d01, C2<R> d02,
   return fma((R)2, off, dia);
 }
 
-// Divergence of one site: the sums over its eight links that Delta is made of
-// (W = sum_mu [U_mu(x - mu^) - U_mu(x)]: Im W_ii and W_ij - conj(W_ji)) and
-// the Re Tr sum of its forward links, in FP64.
-struct SiteDiv {
-  double f, im0, im1, im2;
-  double2 w01, w02, w12;
+// What one link M adds to a site's sums W = sum_mu [U_mu(x - mu^) - U_mu(x)]:
+// Im M_ii and M_ij - conj(M_ji), the entries that enter the traceless
+// anti-Hermitian part, and its trace.
+template <typename R> struct LinkTerms {
+  R tr, y0, y1, y2;
+  C2<R> a01, a02, a12;
+};
+template <typename R> __device__ __forceinline__ LinkTerms<R> link_terms(const M3<R>& m) {
+  LinkTerms<R> t;
+  t.tr = m.e[0][0].x + m.e[1][1].x + m.e[2][2].x;
+  t.y0 = m.e[0][0].y;
+  t.y1 = m.e[1][1].y;
+  t.y2 = m.e[2][2].y;
+  t.a01 = csub<R>(m.e[0][1], cconj<R>(m.e[1][0]));
+  t.a02 = csub<R>(m.e[0][2], cconj<R>(m.e[2][0]));
+  t.a12 = csub<R>(m.e[1][2], cconj<R>(m.e[2][1]));
+  return t;
+}
+
+// A site's sums: F's trace sum (FP64 above one link) and W in the link precision.
+template <typename R> struct SiteSums {
+  double f;
+  R im0, im1, im2;
+  C2<R> w01, w02, w12;
+};
+template <typename R> __device__ __forceinline__ SiteSums<R> site_sums_zero() {
+  SiteSums<R> o;
+  o.f = 0;
+  o.im0 = o.im1 = o.im2 = 0;
+  o.w01 = o.w02 = o.w12 = mkc<R>(0, 0);
+  return o;
+}
+// A site's own link of a direction, and the link of it that ends in the site.
+template <typename R> __device__ __forceinline__ void add_own(SiteSums<R>& o, const LinkTerms<R>& t) {
+  o.f += (double)t.tr;
+  o.im0 -= t.y0; o.im1 -= t.y1; o.im2 -= t.y2;
+  o.w01 = csub<R>(o.w01, t.a01);
+  o.w02 = csub<R>(o.w02, t.a02);
+  o.w12 = csub<R>(o.w12, t.a12);
+}
+template <typename R> __device__ __forceinline__ void add_back(SiteSums<R>& o, const LinkTerms<R>& t) {
+  o.im0 += t.y0; o.im1 += t.y1; o.im2 += t.y2;
+  o.w01 = cadd<R>(o.w01, t.a01);
+  o.w02 = cadd<R>(o.w02, t.a02);
+  o.w12 = cadd<R>(o.w12, t.a12);
+}
+
+// Place of a thread of a measuring kernel: its site and the directions mu0 <=
+// mu < mu1 of it.  SPLIT: eight sites to a warp (a whole 128-byte line of each
+// FP64 entry), a lane per direction; lanes 0 to 7 go on with the sites' sums.
+template <bool SPLIT> struct MeasurePlace {
+  int64_t s;
+  int mu0, mu1;
+  __device__ __forceinline__ MeasurePlace() {
+    if (SPLIT) {
+      s = ((int64_t)blockIdx.x * (MEASURE_SPLIT_THREADS / 32) + (threadIdx.x >> 5)) * 8 + (threadIdx.x & 7);
+      mu0 = (threadIdx.x >> 3) & 3;
+      mu1 = mu0 + 1;
+    } else {
+      s = (int64_t)blockIdx.x * MEASURE_THREADS + threadIdx.x;
+      mu0 = 0;
+      mu1 = 4;
+    }
+  }
+  static __device__ __forceinline__ bool collects() { return !SPLIT || (threadIdx.x & 24) == 0; }
+  // the sum over the directions, in every lane of a site; all lanes of a warp call it
+  template <typename T> static __device__ __forceinline__ void join(T& v) {
+    if (SPLIT) {
+      v += __shfl_xor_sync(0xffffffffu, v, 8);
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+    }
+  }
+  static __device__ __forceinline__ void join_or(uint32_t& v) {
+    if (SPLIT) {
+      v |= __shfl_xor_sync(0xffffffffu, v, 8);
+      v |= __shfl_xor_sync(0xffffffffu, v, 16);
+    }
+  }
+  static __device__ __forceinline__ void join(SiteSums<float>& o) {
+    if (SPLIT) {
+      join(o.f);
+      join(o.im0); join(o.im1); join(o.im2);
+      join(o.w01.x); join(o.w01.y); join(o.w02.x); join(o.w02.y); join(o.w12.x); join(o.w12.y);
+    }
+  }
 };
 
-// In the link precision (FP64 sum over mu of each link's trace).
-template <typename R, int ROWS>
-__device__ __forceinline__ void site_divergence(const Geom& g, const MatField<R, ROWS>& U, int64_t s, const int c[4],
-                                                double& fsum, R& im0, R& im1, R& im2, C2<R>& w01, C2<R>& w02,
-                                                C2<R>& w12) {
-  fsum = 0;
-  im0 = im1 = im2 = 0;
-  w01 = w02 = w12 = mkc<R>(0, 0);
+// Delta of a site, stored, and its part of theta.
+template <typename R>
+__device__ __forceinline__ double store_delta(const SiteSums<R>& o, C2<R>* __restrict__ delta, int64_t V, int64_t s) {
+  const R tr = (o.im0 + o.im1 + o.im2) * (R)(1.0 / 3.0);
+  const R a0 = o.im0 - tr, a1 = o.im1 - tr, a2 = o.im2 - tr;
+  const C2<R> d01 = cscale<R>(o.w01, (R)0.5), d02 = cscale<R>(o.w02, (R)0.5), d12 = cscale<R>(o.w12, (R)0.5);
+  delta[s] = mkc<R>(a0, a1);
+  delta[V + s] = d01;
+  delta[2 * V + s] = d02;
+  delta[3 * V + s] = d12;
+  // ||Delta_A||_F^2
+  return (double)delta_norm2<R>(a0, a1, a2, d01, d02, d12);
+}
+
+// The FP64 path of a site with links outside the fixed-point range.
+template <int ROWS>
+__device__ __noinline__ void site_sums_fp64(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                            SiteSums<double>& o) {
+  int c[4];
+  site_coords(g, s, c);
+  o = site_sums_zero<double>();
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
-    M3<R> u;
+    M3<double> u, b;
     U.load_ro(mu, s, u);
-    fsum += (double)(u.e[0][0].x + u.e[1][1].x + u.e[2][2].x);
-    im0 -= u.e[0][0].y; im1 -= u.e[1][1].y; im2 -= u.e[2][2].y;
-    w01 = csub<R>(w01, csub<R>(u.e[0][1], cconj<R>(u.e[1][0])));
-    w02 = csub<R>(w02, csub<R>(u.e[0][2], cconj<R>(u.e[2][0])));
-    w12 = csub<R>(w12, csub<R>(u.e[1][2], cconj<R>(u.e[2][1])));
-    M3<R> b;
     U.load_ro(mu, site_back(g, s, c, mu), b);
-    im0 += b.e[0][0].y; im1 += b.e[1][1].y; im2 += b.e[2][2].y;
-    w01 = cadd<R>(w01, csub<R>(b.e[0][1], cconj<R>(b.e[1][0])));
-    w02 = cadd<R>(w02, csub<R>(b.e[0][2], cconj<R>(b.e[2][0])));
-    w12 = cadd<R>(w12, csub<R>(b.e[1][2], cconj<R>(b.e[2][1])));
+    add_own<double>(o, link_terms<double>(u));
+    add_back<double>(o, link_terms<double>(b));
   }
 }
 
-// The FP64 path of links outside the fixed-point range.
+// FP64 links: a site's sums over the two links of its directions mu0 <= mu < mu1 in 64-bit fixed point (unit 2^-58) on the integer
+// pipe: exact but for what lies below 2^-58 in an entry, against one FP64
+// rounding per addition (2^-54 for sums of order one).  12-real links rebuild
+// row 3 in fixed point as well.
+// t[0]: trace; t[1..3]: Im W_ii; t[4..9]: W_01, W_02, W_12; bad, strong: range
+// tests (an entry outside it; high words of the anti-symmetric real parts,
+// or-ed).
+constexpr int FX_TERMS = 10;
 template <int ROWS>
-__device__ __noinline__ void site_divergence_fp64(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
-                                                  SiteDiv& o) {
-  int c[4];
-  site_coords(g, s, c);
-  site_divergence<double, ROWS>(g, U, s, c, o.f, o.im0, o.im1, o.im2, o.w01, o.w02, o.w12);
-}
-
-// FP64 links, summed in 64-bit fixed point (unit 2^-58) on the integer pipe:
-// 132 entries of eight links enter the sums, exactly but for what lies below
-// 2^-58 in an entry, against one FP64 rounding per addition (2^-54 for sums
-// of order one).  12-real links rebuild row 3 in fixed point as well.
-// Where the anti-symmetric real parts of all eight links are below 2^-12 (a
-// field near the identity), FP64 sums are relative to numbers that small and
-// round finer than 2^-58: that site takes the FP64 path, as do entries
-// outside the fixed-point range.
-// Bound by the ALU pipe (65 % busy in ncu) beside HBM (41 %).  32^4: 18-real
-// 195 us (FP64 sums on the FP64 pipe: 355 us), 12-real 314 us (665 us).
-template <int ROWS>
-__device__ __forceinline__ void site_divergence_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
-                                                   const int c[4], SiteDiv& o) {
-  int64_t f = 0, i0 = 0, i1 = 0, i2 = 0, x01 = 0, y01 = 0, x02 = 0, y02 = 0, x12 = 0, y12 = 0;
-  uint32_t m = 0, t = 0, w = 0;
+__device__ __forceinline__ void site_terms_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                              const int c[4], int mu0, int mu1, int64_t t[FX_TERMS], uint32_t& bad,
+                                              uint32_t& strong) {
+  uint32_t m = 0, big = 0;
 #pragma unroll 1
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 2 * mu0; k < 2 * mu1; ++k) {
     const int mu = k >> 1;
+    const bool own = (k & 1) == 0;
     int64_t sf, sb;
     site_nbrs_sel(g, s, c, mu, sf, sb);
-    const bool fwd = (k & 1) == 0;  // the site's own link, else the one that ends in it
-    const int64_t sl = fwd ? s : sb;
-    double2 e[3][3];
+    double2 e[ROWS][3];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        e[r][j] = __ldg(&U.p[U.off(mu, r, j, sl)]);
+        e[r][j] = __ldg(&U.p[U.off(mu, r, j, own ? s : sb)]);
         m = fx_max(m, e[r][j]);
       }
-    int64_t f00, f11, f22, d0, d1, d2, ax, ay, bx, by, cx, cy;
-    d0 = fx58_from(e[0][0].y);
-    d1 = fx58_from(e[1][1].y);
+    int64_t x[FX_TERMS];
+    x[0] = 0;
+    x[1] = fx58_from(e[0][0].y);
+    x[2] = fx58_from(e[1][1].y);
     if (ROWS == 3) {
-      f00 = f11 = f22 = 0;
-      if (fwd) {
-        f00 = fx58_from(e[0][0].x);
-        f11 = fx58_from(e[1][1].x);
-        f22 = fx58_from(e[2][2].x);
-      }
-      d2 = fx58_from(e[2][2].y);
-      ax = fx58_from(e[0][1].x) - fx58_from(e[1][0].x);
-      ay = fx58_from(e[0][1].y) + fx58_from(e[1][0].y);
-      bx = fx58_from(e[0][2].x) - fx58_from(e[2][0].x);
-      by = fx58_from(e[0][2].y) + fx58_from(e[2][0].y);
-      cx = fx58_from(e[1][2].x) - fx58_from(e[2][1].x);
-      cy = fx58_from(e[1][2].y) + fx58_from(e[2][1].y);
+      if (own) x[0] = fx58_from(e[0][0].x) + fx58_from(e[1][1].x) + fx58_from(e[ROWS - 1][2].x);
+      x[3] = fx58_from(e[ROWS - 1][2].y);
+      x[4] = fx58_from(e[0][1].x) - fx58_from(e[1][0].x);
+      x[5] = fx58_from(e[0][1].y) + fx58_from(e[1][0].y);
+      x[6] = fx58_from(e[0][2].x) - fx58_from(e[ROWS - 1][0].x);
+      x[7] = fx58_from(e[0][2].y) + fx58_from(e[ROWS - 1][0].y);
+      x[8] = fx58_from(e[1][2].x) - fx58_from(e[ROWS - 1][1].x);
+      x[9] = fx58_from(e[1][2].y) + fx58_from(e[ROWS - 1][1].y);
     } else {
-      int64_t q[2][3][2];
+      int64_t q[2][3][2], z[3][2];
       FxC w[2][3];
 #pragma unroll
       for (int r = 0; r < 2; ++r)
@@ -283,51 +352,61 @@ __device__ __forceinline__ void site_divergence_fx(const Geom& g, const MatField
           q[r][j][1] = fx58_from(e[r][j].y);
           w[r][j] = FxC{fx_operand58(q[r][j][0]), fx_operand58(q[r][j][1])};
         }
-      int64_t z[3][2];
-      fx_third_row(w[0], w[1], z, t);
+      fx_third_row(w[0], w[1], z, big);
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         z[j][0] >>= 2;
         z[j][1] >>= 2;
       }
-      f00 = fwd ? q[0][0][0] : 0;
-      f11 = fwd ? q[1][1][0] : 0;
-      f22 = fwd ? z[2][0] : 0;
-      d2 = z[2][1];
-      ax = q[0][1][0] - q[1][0][0];
-      ay = q[0][1][1] + q[1][0][1];
-      bx = q[0][2][0] - z[0][0];
-      by = q[0][2][1] + z[0][1];
-      cx = q[1][2][0] - z[1][0];
-      cy = q[1][2][1] + z[1][1];
+      if (own) x[0] = q[0][0][0] + q[1][1][0] + z[2][0];
+      x[3] = z[2][1];
+      x[4] = q[0][1][0] - q[1][0][0];
+      x[5] = q[0][1][1] + q[1][0][1];
+      x[6] = q[0][2][0] - z[0][0];
+      x[7] = q[0][2][1] + z[0][1];
+      x[8] = q[1][2][0] - z[1][0];
+      x[9] = q[1][2][1] + z[1][1];
     }
-    w |= (uint32_t)(ax >> 32) ^ (uint32_t)(ax >> 63);
-    w |= (uint32_t)(bx >> 32) ^ (uint32_t)(bx >> 63);
-    w |= (uint32_t)(cx >> 32) ^ (uint32_t)(cx >> 63);
-    if (fwd) {
-      f += f00 + f11 + f22;
-      i0 -= d0; i1 -= d1; i2 -= d2;
-      x01 -= ax; y01 -= ay; x02 -= bx; y02 -= by; x12 -= cx; y12 -= cy;
+#pragma unroll
+    for (int i = 4; i < FX_TERMS; i += 2) strong |= (uint32_t)(x[i] >> 32) ^ (uint32_t)(x[i] >> 63);
+    t[0] += x[0];
+    if (own) {
+#pragma unroll
+      for (int i = 1; i < FX_TERMS; ++i) t[i] -= x[i];
     } else {
-      i0 += d0; i1 += d1; i2 += d2;
-      x01 += ax; y01 += ay; x02 += bx; y02 += by; x12 += cx; y12 += cy;
+#pragma unroll
+      for (int i = 1; i < FX_TERMS; ++i) t[i] += x[i];
     }
   }
-  if (fx_bad(m, t) || w < (1u << (58 - 12 - 32))) {
-    site_divergence_fp64<ROWS>(g, U, s, o);
-    return;
-  }
-  o.f = fx_to_double_fp<58>(f);
-  o.im0 = fx_to_double_fp<58>(i0);
-  o.im1 = fx_to_double_fp<58>(i1);
-  o.im2 = fx_to_double_fp<58>(i2);
-  o.w01 = make_double2(fx_to_double_fp<58>(x01), fx_to_double_fp<58>(y01));
-  o.w02 = make_double2(fx_to_double_fp<58>(x02), fx_to_double_fp<58>(y02));
-  o.w12 = make_double2(fx_to_double_fp<58>(x12), fx_to_double_fp<58>(y12));
+  bad = fx_bad(m, big);
 }
 
-template <typename R, int ROWS>
-__global__ void __launch_bounds__(MEASURE_THREADS)
+// A site's sums from its directions' terms t.  Where the anti-symmetric real
+// parts of all eight links are below 2^-12 (a field near the identity), FP64
+// sums are relative to numbers that small and round finer than 2^-58: that site
+// takes the FP64 path, as do entries outside the fixed-point range.
+template <int ROWS>
+__device__ __forceinline__ void site_sums_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                             const int64_t t[FX_TERMS], bool bad, uint32_t strong,
+                                             SiteSums<double>& o) {
+  if (bad || strong < (1u << (58 - 12 - 32))) {
+    site_sums_fp64<ROWS>(g, U, s, o);
+    return;
+  }
+  o.f = fx_to_double_fp<58>(t[0]);
+  o.im0 = fx_to_double_fp<58>(t[1]);
+  o.im1 = fx_to_double_fp<58>(t[2]);
+  o.im2 = fx_to_double_fp<58>(t[3]);
+  o.w01 = make_double2(fx_to_double_fp<58>(t[4]), fx_to_double_fp<58>(t[5]));
+  o.w02 = make_double2(fx_to_double_fp<58>(t[6]), fx_to_double_fp<58>(t[7]));
+  o.w12 = make_double2(fx_to_double_fp<58>(t[8]), fx_to_double_fp<58>(t[9]));
+}
+
+// FP64 links are bound by the ALU pipe (65 % busy in ncu) beside HBM (41 %).
+// 32^4: 18-real 197 us (FP64 sums on the FP64 pipe: 355 us), 12-real 271 us
+// (665 us).
+template <typename R, int ROWS, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS)
 measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt, C2<R>* __restrict__ delta,
                double* __restrict__ partials, DevState* __restrict__ st, int count_iter, unsigned long long cond,
                int use_cond, int only_if_revert, Batch B, unsigned long long cond_undo) {
@@ -342,42 +421,51 @@ measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt,
   }
   if (only_if_revert && !st->revert) return;
   if (links_alt != nullptr && st->ubuf) U.p = const_cast<C2<R>*>(links_alt);  // ping-pong links of a fused lane
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const MeasurePlace<SPLIT> p;
+  const bool in = p.s < g.V;
   // Re Tr of one link in the link precision; every sum above one link (the
   // site's F and theta terms, warp, CTA and grid sums) in FP64
   double fsum = 0, tsum = 0;
-  if (s < g.V) {
-    int c[4];
-    site_coords(g, s, c);
-    // W = sum_mu [U_mu(x - mu^) - U_mu(x)]; only the entries that enter its
-    // traceless anti-Hermitian part are accumulated.
-    R im0, im1, im2;           // Im W_ii
-    C2<R> w01, w02, w12;       // W_ij - conj(W_ji)
-    if constexpr (sizeof(R) == sizeof(double)) {
-      SiteDiv o;
-      site_divergence_fx<ROWS>(g, U, s, c, o);
-      fsum = o.f;
-      im0 = o.im0; im1 = o.im1; im2 = o.im2;
-      w01 = o.w01; w02 = o.w02; w12 = o.w12;
-    } else {
-      site_divergence<R, ROWS>(g, U, s, c, fsum, im0, im1, im2, w01, w02, w12);
-    }
-    const R tr = (im0 + im1 + im2) * (R)(1.0 / 3.0);
-    const R a0 = im0 - tr, a1 = im1 - tr, a2 = im2 - tr;
-    const C2<R> d01 = cscale<R>(w01, (R)0.5), d02 = cscale<R>(w02, (R)0.5), d12 = cscale<R>(w12, (R)0.5);
-    delta[s] = mkc<R>(a0, a1);
-    delta[g.V + s] = d01;
-    delta[2 * g.V + s] = d02;
-    delta[3 * g.V + s] = d12;
-    // ||Delta_A||_F^2
-    tsum = (double)delta_norm2<R>(a0, a1, a2, d01, d02, d12);
-  }
   float dmax = 0.f;
-  const int dmu = defect_sample_mu();
-  if (dmu >= 0 && s < g.V) {
-    C2<R> rows[2][3];
-    U.load_rows01_ro(dmu, s, rows);
-    dmax = rows_defect<R>(rows[0], rows[1]);
+  int c[4];
+  if (in) site_coords(g, p.s, c);
+  // W = sum_mu [U_mu(x - mu^) - U_mu(x)]; only the entries that enter its
+  // traceless anti-Hermitian part are accumulated.
+  SiteSums<R> o = site_sums_zero<R>();
+  if constexpr (sizeof(R) == sizeof(double)) {
+    int64_t t[FX_TERMS] = {};
+    uint32_t bad = 0, strong = 0;
+    if (in) site_terms_fx<ROWS>(g, U, p.s, c, p.mu0, p.mu1, t, bad, strong);
+#pragma unroll
+    for (int i = 0; i < FX_TERMS; ++i) p.join(t[i]);
+    p.join_or(bad);
+    p.join_or(strong);
+    if (in && p.collects()) site_sums_fx<ROWS>(g, U, p.s, t, bad != 0, strong, o);
+  } else {
+    if (in) {
+#pragma unroll
+      for (int k = 0; k < (SPLIT ? 1 : 4); ++k) {
+        const int mu = p.mu0 + k;
+        int64_t sf, sb;
+        site_nbrs_sel(g, p.s, c, mu, sf, sb);
+        M3<R> u, b;
+        U.load_ro(mu, p.s, u);
+        add_own<R>(o, link_terms<R>(u));
+        U.load_ro(mu, sb, b);
+        add_back<R>(o, link_terms<R>(b));
+      }
+    }
+    p.join(o);
+  }
+  if (in && p.collects()) {
+    fsum = o.f;
+    tsum = store_delta<R>(o, delta, g.V, p.s);
+    const int dmu = defect_sample_mu(p.s);
+    if (dmu >= 0) {
+      C2<R> rows[2][3];
+      U.load_rows01_ro(dmu, p.s, rows);
+      dmax = rows_defect<R>(rows[0], rows[1]);
+    }
   }
   measure_tail(g, fsum, tsum, dmax, partials, st, count_iter, cond, use_cond, batch, 0, sizeof(R) == 8, cond_undo);
 }
@@ -387,10 +475,14 @@ cudaError_t launch_measure(const Geom& g, const C2<R>* links, C2<R>* delta, doub
                            int count_iter, unsigned long long cond_handle, int use_cond, cudaStream_t s,
                            int only_if_revert, const Batch& B, const C2<R>* links_alt,
                            unsigned long long cond_undo) {
-  MatField<R, ROWS> U{const_cast<C2<R>*>(links), g.V};
-  const int64_t nb = measure_blocks(g.V);
-  measure_kernel<R, ROWS><<<dim3((unsigned)nb, 1, (unsigned)B.n), MEASURE_THREADS, 0, s>>>(
-      g, U, links_alt, delta, partials, st, count_iter, cond_handle, use_cond, only_if_revert, B, cond_undo);
+  const MatField<R, ROWS> U{const_cast<C2<R>*>(links), g.V};
+  const dim3 grid((unsigned)measure_blocks(g.V), 1, (unsigned)B.n);
+  if (measure_split(g.V))
+    measure_kernel<R, ROWS, true><<<grid, MEASURE_SPLIT_THREADS, 0, s>>>(
+        g, U, links_alt, delta, partials, st, count_iter, cond_handle, use_cond, only_if_revert, B, cond_undo);
+  else
+    measure_kernel<R, ROWS, false><<<grid, MEASURE_THREADS, 0, s>>>(
+        g, U, links_alt, delta, partials, st, count_iter, cond_handle, use_cond, only_if_revert, B, cond_undo);
   return cudaGetLastError();
 }
 
@@ -423,74 +515,54 @@ __device__ __forceinline__ void gauge_product(const M3<R>& gl, const M3<R>& u, c
   su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
 }
 
-// Contribution of one link M to W = sum_mu [U_mu(x - mu^) - U_mu(x)]: the
-// entries that enter its traceless anti-Hermitian part, with sign sg.
-template <typename R>
-__device__ __forceinline__ void add_antiherm(const M3<R>& m, R sg, R& im0, R& im1, R& im2, C2<R>& w01, C2<R>& w02,
-                                             C2<R>& w12) {
-  im0 += sg * m.e[0][0].y;
-  im1 += sg * m.e[1][1].y;
-  im2 += sg * m.e[2][2].y;
-  const C2<R> a = csub<R>(m.e[0][1], cconj<R>(m.e[1][0]));
-  const C2<R> b = csub<R>(m.e[0][2], cconj<R>(m.e[2][0]));
-  const C2<R> c = csub<R>(m.e[1][2], cconj<R>(m.e[2][1]));
-  w01 = mkc<R>(w01.x + sg * a.x, w01.y + sg * a.y);
-  w02 = mkc<R>(w02.x + sg * b.x, w02.y + sg * b.y);
-  w12 = mkc<R>(w12.x + sg * c.x, w12.y + sg * c.y);
-}
-
-template <typename R, int LROWS, int GROWS>
-__global__ void __launch_bounds__(MEASURE_THREADS, 3)
+template <typename R, int LROWS, int GROWS, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS, 3)
 update_measure_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, MatField<R, GROWS> Gf,
                       C2<R>* __restrict__ delta, double* __restrict__ partials, DevState* __restrict__ st,
                       unsigned long long cond, int use_cond, unsigned long long cond_undo) {
   const int cur = st->ubuf;
   const MatField<R, LROWS> Us{cur ? U1 : U0, g.V}, Ud{cur ? U0 : U1, g.V};
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const MeasurePlace<SPLIT> p;
+  const bool in = p.s < g.V;
   double fsum = 0, tsum = 0;  // as in measure_kernel: FP64 above one link
   float dmax = 0.f;
-  const int dmu = defect_sample_mu();
-  if (s < g.V) {
+  SiteSums<R> o = site_sums_zero<R>();
+  const int dmu = defect_sample_mu(p.s);
+  if (in) {
     int c[4];
-    site_coords(g, s, c);
+    site_coords(g, p.s, c);
     M3<R> gx;
-    Gf.load_ro(0, s, gx);
-    R im0 = 0, im1 = 0, im2 = 0;
-    C2<R> w01 = mkc<R>(0, 0), w02 = mkc<R>(0, 0), w12 = mkc<R>(0, 0);
+    Gf.load_ro(0, p.s, gx);
 #pragma unroll 1
-    for (int mu = 0; mu < 4; ++mu) {
-      M3<R> u, h, o;
-      Us.load_ro(mu, s, u);
-      Gf.load_ro(0, site_fwd(g, s, c, mu), h);
-      gauge_product<R>(gx, u, h, o);
-      Ud.store(mu, s, o);
-      fsum += (double)(o.e[0][0].x + o.e[1][1].x + o.e[2][2].x);
-      add_antiherm<R>(o, (R)-1, im0, im1, im2, w01, w02, w12);
-      const int64_t sb = site_back(g, s, c, mu);
-      M3<R> b, gb, ob;
+    for (int mu = p.mu0; mu < p.mu1; ++mu) {
+      M3<R> u, h, w;
+      Us.load_ro(mu, p.s, u);
+      Gf.load_ro(0, site_fwd(g, p.s, c, mu), h);
+      gauge_product<R>(gx, u, h, w);
+      Ud.store(mu, p.s, w);
+      add_own<R>(o, link_terms<R>(w));
+      const int64_t sb = site_back(g, p.s, c, mu);
+      M3<R> b, gb, wb;
       Us.load_ro(mu, sb, b);
       Gf.load_ro(0, sb, gb);
-      gauge_product<R>(gb, b, gx, ob);
-      add_antiherm<R>(ob, (R)1, im0, im1, im2, w01, w02, w12);
+      gauge_product<R>(gb, b, gx, wb);
+      add_back<R>(o, link_terms<R>(wb));
     }
-    const R tr = (im0 + im1 + im2) * (R)(1.0 / 3.0);
-    const R a0 = im0 - tr, a1 = im1 - tr, a2 = im2 - tr;
-    const C2<R> d01 = cscale<R>(w01, (R)0.5), d02 = cscale<R>(w02, (R)0.5), d12 = cscale<R>(w12, (R)0.5);
-    delta[s] = mkc<R>(a0, a1);
-    delta[g.V + s] = d01;
-    delta[2 * g.V + s] = d02;
-    delta[3 * g.V + s] = d12;
-    tsum = (double)delta_norm2<R>(a0, a1, a2, d01, d02, d12);
-    if (dmu >= 0) {
+    if (dmu >= p.mu0 && dmu < p.mu1) {
       // the sampled link as this thread stored it above (plain loads see the
       // thread's own stores; keeping the rows in registers instead spilled)
       C2<R> rows[2][3];
 #pragma unroll
       for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) rows[r][c] = Ud.p[Ud.off(dmu, r, c, s)];
+        for (int j = 0; j < 3; ++j) rows[r][j] = Ud.p[Ud.off(dmu, r, j, p.s)];
       dmax = rows_defect<R>(rows[0], rows[1]);
     }
+  }
+  p.join(o);
+  if (in && p.collects()) {
+    fsum = o.f;
+    tsum = store_delta<R>(o, delta, g.V, p.s);
   }
   measure_tail(g, fsum, tsum, dmax, partials, st, 1, cond, use_cond, false, 1, sizeof(R) == 8, cond_undo);
 }
@@ -500,9 +572,13 @@ cudaError_t launch_update_measure(const Geom& g, C2<R>* U0, C2<R>* U1, const C2<
                                   double* partials, DevState* st, unsigned long long cond, int use_cond,
                                   cudaStream_t s, unsigned long long cond_undo) {
   MatField<R, GROWS> Gf{const_cast<C2<R>*>(gfield), g.V};
-  const int64_t nb = measure_blocks(g.V);
-  update_measure_kernel<R, LROWS, GROWS><<<(unsigned)nb, MEASURE_THREADS, 0, s>>>(g, U0, U1, Gf, delta, partials,
-                                                                                  st, cond, use_cond, cond_undo);
+  const unsigned nb = (unsigned)measure_blocks(g.V);
+  if (measure_split(g.V))
+    update_measure_kernel<R, LROWS, GROWS, true><<<nb, MEASURE_SPLIT_THREADS, 0, s>>>(g, U0, U1, Gf, delta, partials,
+                                                                                      st, cond, use_cond, cond_undo);
+  else
+    update_measure_kernel<R, LROWS, GROWS, false><<<nb, MEASURE_THREADS, 0, s>>>(g, U0, U1, Gf, delta, partials, st,
+                                                                                 cond, use_cond, cond_undo);
   return cudaGetLastError();
 }
 
