@@ -49,7 +49,8 @@ __device__ __forceinline__ void gram_schmidt_factors(double a, double d, double2
 // FP32 field applies k in FP32.  For 1 + X with X anti-Hermitian the rows are
 // nearly orthogonal (|<r1, r2>| <= |X|^2 while |r1|, |r2| >= 1), so the
 // difference does not cancel.  33 FP64 operations and two estimates, against
-// 43 when w is formed in FP64.
+// 43 when w is formed in FP64.  Taken by entries outside the range of the
+// FP32 pairs below.
 struct GSFactors32 {
   double i1, i2, kx, ky;
 };
@@ -70,9 +71,7 @@ __device__ __forceinline__ void gram_schmidt_factors_f32(double a, double d, dou
 }
 
 // FP32 <-> FP64 conversions on the integer pipe, written from the IEEE 754
-// binary32 / binary64 layouts.  On this GPU the conversion instructions run
-// on the FP64 pipe, which bounds pass C of FP32 lanes; these take sign,
-// rebiased exponent and mantissa apart with integer operations instead.
+// binary32 / binary64 layouts: sign, rebiased exponent and mantissa apart.
 // Zero and subnormal inputs give zero; FP64 -> FP32 rounds to nearest with
 // ties away from zero (IEEE rounds ties to even: the two differ only on exact
 // ties) and overflows to infinity.  Non-finite values are not expected here.
@@ -94,13 +93,96 @@ __device__ __forceinline__ float f64_to_f32_int(double x) {
 __device__ __forceinline__ double2 c_f32_to_f64_int(float2 v) { return make_double2(f32_to_f64_int(v.x), f32_to_f64_int(v.y)); }
 __device__ __forceinline__ float2 c_f64_to_f32_int(double2 v) { return make_float2(f64_to_f32_int(v.x), f64_to_f32_int(v.y)); }
 
-// Rows u, v of g = reunitarize(1 + X) in the field precision R; the
-// Gram-Schmidt factors are FP64 in both.  FP64 fields take u = i1 r1 and
-// v = i2 w in FP64.  FP32 fields, whose rows are stored in FP32, apply the
-// FP64 factors in FP32: u = fl(i1) r1 with r1 the FP32 entries of the
-// filtered field itself, v = fl(i2) fl(w) -- within one FP32 rounding of the
-// FP64 product, without the FP64 multiplies -- and take their values to and
-// from FP64 on the integer pipe.
+// The same factors in FP32 pairs h + l (|l| <= ulp(h)/2: 48 bits) on the FP32
+// pipe, which has 64 times the FP64 rate: error-free products (FMA) and sums
+// (Knuth, The Art of Computer Programming 2, 4.2.2), about 200 FP32 operations.
+// Each factor is within 2^-35 of its exact value before it is rounded to FP32.
+struct Pair32 {
+  float h, l;
+};
+__device__ __forceinline__ Pair32 two_prod(float a, float b) {
+  const float h = __fmul_rn(a, b);
+  return Pair32{h, __fmaf_rn(a, b, -h)};
+}
+__device__ __forceinline__ Pair32 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return Pair32{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair32 pair_add(Pair32 a, Pair32 b) {
+  const Pair32 s = two_sum(a.h, b.h);
+  return Pair32{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ Pair32 pair_norm(Pair32 a) {  // |a.h| >= |a.l|
+  const float h = __fadd_rn(a.h, a.l);
+  return Pair32{h, __fsub_rn(a.l, __fsub_rn(h, a.h))};
+}
+// 1 / sqrt(n), n >= 1: a Newton step on the estimate, with its residual exact to 2^-44.
+__device__ __forceinline__ Pair32 pair_rsqrt(Pair32 n) {
+  const float y = rsqrtf(n.h);
+  const Pair32 p = two_prod(y, y);
+  const float r = fmaf(-n.l, p.h, fmaf(-n.h, p.l, fmaf(-n.h, p.h, 1.f)));
+  const float yr = y * r;
+  return Pair32{y, fmaf(0.375f * r, yr, 0.5f * yr)};
+}
+
+struct GSFactorsOut {
+  float i1, i2, kx, ky;
+};
+// Entries beyond this, and NaN, take FP64 (squares of squares stay far from overflow below it).
+constexpr float GS_PAIR_MAX = 4096.f;
+static __device__ __noinline__ GSFactorsOut gram_schmidt_fp64_call(float2 f0, float2 f1, float2 f2, float2 f3) {
+  GSFactors32 o;
+  gram_schmidt_factors_f32(f32_to_f64_int(f0.x), f32_to_f64_int(f0.y), c_f32_to_f64_int(f1), c_f32_to_f64_int(f2),
+                           c_f32_to_f64_int(f3), o);
+  return GSFactorsOut{f64_to_f32_int(o.i1), f64_to_f32_int(o.i2), f64_to_f32_int(o.kx), f64_to_f32_int(o.ky)};
+}
+__device__ __forceinline__ GSFactorsOut gram_schmidt_pair(float2 f0, float2 f1, float2 f2, float2 f3) {
+  auto mag = [](float x) { return __float_as_uint(x) & 0x7fffffffu; };
+  const uint32_t m = max(max(max(mag(f0.x), mag(f0.y)), max(mag(f1.x), mag(f1.y))),
+                         max(max(mag(f2.x), mag(f2.y)), max(mag(f3.x), mag(f3.y))));
+  if (m > __float_as_uint(GS_PAIR_MAX)) return gram_schmidt_fp64_call(f0, f1, f2, f3);
+  const float a = f0.x, d = f0.y;
+  const Pair32 n11 = pair_add(two_prod(f1.x, f1.x), two_prod(f1.y, f1.y));
+  const Pair32 n22 = pair_add(two_prod(f2.x, f2.x), two_prod(f2.y, f2.y));
+  const Pair32 n33 = pair_add(two_prod(f3.x, f3.x), two_prod(f3.y, f3.y));
+  // |r1|^2 and |r2|^2
+  const Pair32 n1 = pair_norm(pair_add(Pair32{1.f, 0.f}, pair_add(two_prod(a, a), pair_add(n11, n22))));
+  const Pair32 nr2 = pair_add(Pair32{1.f, 0.f}, pair_add(two_prod(d, d), pair_add(n11, n33)));
+  const Pair32 i1 = pair_rsqrt(n1);
+  Pair32 q = two_prod(i1.h, i1.h);  // 1 / |r1|^2
+  q.l = fmaf(2.f * i1.h, i1.l, q.l);
+  const Pair32 s = two_sum(a, d);
+  auto times_s = [&](float x) {
+    Pair32 p = two_prod(s.h, x);
+    p.l = fmaf(s.l, x, p.l);
+    return p;
+  };
+  const Pair32 cx = pair_norm(pair_add(times_s(f1.y), pair_add(two_prod(f2.y, f3.y), two_prod(f2.x, f3.x))));
+  const Pair32 cy = pair_norm(pair_add(times_s(f1.x), pair_add(two_prod(-f2.y, f3.x), two_prod(f2.x, f3.y))));
+  auto square = [](Pair32 x) {
+    Pair32 p = two_prod(x.h, x.h);
+    p.l = fmaf(2.f * x.h, x.l, p.l);
+    return p;
+  };
+  const Pair32 c2 = pair_norm(pair_add(square(cx), square(cy)));
+  Pair32 t = two_prod(-q.h, c2.h);
+  t.l = fmaf(-q.h, c2.l, fmaf(-q.l, c2.h, t.l));
+  const Pair32 i2 = pair_rsqrt(pair_norm(pair_add(nr2, t)));
+  GSFactorsOut o;
+  o.i1 = i1.h + i1.l;
+  o.i2 = i2.h + i2.l;
+  o.kx = fmaf(q.h, cx.h, fmaf(q.h, cx.l, q.l * cx.h));
+  o.ky = fmaf(q.h, cy.h, fmaf(q.h, cy.l, q.l * cy.h));
+  return o;
+}
+
+// Rows u, v of g = reunitarize(1 + X) in the field precision R.  FP64 fields
+// take u = i1 r1 and v = i2 w in FP64.  FP32 fields, whose rows are stored in
+// FP32, round their factors to FP32: u = fl(i1) r1 with r1 the FP32 entries of
+// the filtered field itself, v = fl(i2) fl(w) -- within one FP32 rounding of
+// the product of the exact factors.  Pass C with those factors in FP64 sat on
+// the FP64 pipe (82 % busy): in pairs 84 -> 48 us at 32^4, 754 -> 461 us at
+// 48^3x96 (12-real FP32 links).
 template <typename R>
 __device__ __forceinline__ void gauge_rows(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f3, C2<R> u[3], C2<R> v[3]) {
   if constexpr (sizeof(R) == sizeof(double)) {
@@ -112,11 +194,8 @@ __device__ __forceinline__ void gauge_rows(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f
 #pragma unroll
     for (int j = 0; j < 3; ++j) v[j] = cscale<double>(o.w[j], o.i2);
   } else {
-    GSFactors32 o32;
-    gram_schmidt_factors_f32(f32_to_f64_int(f0.x), f32_to_f64_int(f0.y), c_f32_to_f64_int(f1), c_f32_to_f64_int(f2),
-                             c_f32_to_f64_int(f3), o32);
-    const float i1 = f64_to_f32_int(o32.i1), i2 = f64_to_f32_int(o32.i2);
-    const float kx = f64_to_f32_int(o32.kx), ky = f64_to_f32_int(o32.ky);
+    const GSFactorsOut o32 = gram_schmidt_pair(f0, f1, f2, f3);
+    const float i1 = o32.i1, i2 = o32.i2, kx = o32.kx, ky = o32.ky;
     const float a = f0.x, d = f0.y;
     u[0] = mkc<R>(i1, a * i1);
     u[1] = cscale<R>(f1, i1);

@@ -204,3 +204,30 @@ def test_links_round_trip(ext, name):
     with lgf.Lattice(ext, "fp32") as lat:
         lat.set_links(U)
         assert np.array_equal(lat.get_links(), U.astype(np.complex64).astype(np.complex128))
+
+
+# ---------------------------------------------------------------------------
+# Gram-Schmidt of FP32 lanes in FP32 pairs
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("alpha", [1e-6, 0.08, 3.0, 3e3, 3e7])
+def test_fp32_gauge_against_oracle(alpha):
+    """g(x) of one FP32 step; alpha = 3e3 puts sites on both sides of the pairs' range, 3e7 all beyond it.
+
+    Tolerance: the filtered field is known to about 1e-6 of its size (FP32
+    divergence and transforms), which row 2 minus its projection on row 1
+    amplifies by |r2| / |w|; 5e-6 of that covers the rounding of g as well.
+    """
+    ext = (3, 4, 6, 9)
+    U = fields.random_links(ext, 0.9, seed=3)
+    D, K = O.divergence(U), O.fa_filter(ext, alpha)
+    go = O.gauge_transform_from_divergence(D, K)
+    M = O.ifft4(O.fft4(D) * K[..., None, None]) + np.eye(3)
+    r1, r2 = M[..., 0, :], M[..., 1, :]
+    ip = np.sum(np.conj(go[..., 0, :]) * r2, axis=-1)
+    kappa = np.linalg.norm(r2, axis=-1) / np.linalg.norm(r2 - ip[..., None] * go[..., 0, :], axis=-1)
+    with lgf.Lattice(ext, "fp32") as lat:
+        lat.set_links(U)
+        lat.step(alpha)
+        g = lat.get_gauge()
+    assert np.all(np.abs(g - go).max(axis=(-1, -2)) < 5e-6 * kappa)
