@@ -8,10 +8,16 @@
 //   pass C : inverse DFT over (x, y), then g(x) = reunitarize(1 + Delta'(x))
 //            in FP64, optionally G <- g G                           [k5 fused]
 //
-// Each 1D transform is an in-place mixed-radix (2, 3, 4, 8) Cooley-Tukey FFT
+// Each 1D transform is an in-place mixed-radix (2, 3, 4, 6, 8) Cooley-Tukey FFT
 // in shared memory (see ct_stage).  Consecutive threads work on neighbouring
 // lines and every line stride is padded by one element, so the butterflies'
 // shared-memory accesses are free of bank conflicts in every direction.
+//
+// FP64 fields take the integer passes of lgf_fft_fx.cu, FP32 fields the passes
+// on pairs of lgf_fft_pair.cu; the scalar passes here remain for the FP32
+// planes that leave nothing to pair (an odd x extent, planes of which one fills
+// the shared memory, transforms without the filter) and for the other
+// decompositions.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -66,6 +72,19 @@ template <typename R, int SIGN> struct DFT<R, 4, SIGN> {
     v[2] = csub<R>(a, c);
     v[1] = cadd<R>(b, d);
     v[3] = csub<R>(b, d);
+  }
+};
+
+// 2 x 3 without twiddles (Good's mapping): input (3 n1 + 2 n2) mod 6, output
+// (3 k1 + 4 k2) mod 6.
+template <typename R, int SIGN> struct DFT<R, 6, SIGN> {
+  __device__ __forceinline__ static void run(C2<R>* v) {
+    C2<R> s[3] = {cadd<R>(v[0], v[3]), cadd<R>(v[2], v[5]), cadd<R>(v[4], v[1])};
+    C2<R> d[3] = {csub<R>(v[0], v[3]), csub<R>(v[2], v[5]), csub<R>(v[4], v[1])};
+    DFT<R, 3, SIGN>::run(s);
+    DFT<R, 3, SIGN>::run(d);
+    v[0] = s[0]; v[4] = s[1]; v[2] = s[2];
+    v[3] = d[0]; v[1] = d[1]; v[5] = d[2];
   }
 };
 
@@ -152,6 +171,7 @@ __device__ __forceinline__ void ct_stage_any(C2<R>* tile, const Lines& ln, int N
                                              const C2<R>* tw) {
   if (rad == 8) ct_stage<R, 8, SIGN, DIT>(tile, ln, N, fns, tw);
   else if (rad == 4) ct_stage<R, 4, SIGN, DIT>(tile, ln, N, fns, tw);
+  else if (sizeof(R) == sizeof(float) && rad == 6) ct_stage<R, 6, SIGN, DIT>(tile, ln, N, fns, tw);
   else if (rad == 3) ct_stage<R, 3, SIGN, DIT>(tile, ln, N, fns, tw);
   else ct_stage<R, 2, SIGN, DIT>(tile, ln, N, fns, tw);
 }
@@ -447,39 +467,6 @@ __global__ void __launch_bounds__(512) fft_xyz_kernel(Geom g, FFTDir dx, FFTDir 
 // inverse (x, y) plane pass with g(x)
 // ---------------------------------------------------------------------------
 
-template <typename R, typename RG, int GROWS, bool EXPG>
-__global__ void __launch_bounds__(512) fft_xy_inv_gauge_kernel(Geom g, FFTDir dx, FFTDir dy, const C2<R>* __restrict__ data,
-                                        const C2<R>* __restrict__ twg, const short* __restrict__ posg,
-                                        C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf, Lines lx, Lines ly,
-                                        CopyDiv cd, Batch B) {
-  if (batch_skip(B)) return;
-  data += blockIdx.z * B.s_delta;
-  gf += blockIdx.z * B.s_g;
-  if (Gf != nullptr) Gf += blockIdx.z * B.s_G;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int Lx = g.L[0], Ly = g.L[1];
-  C2<R>* tw;
-  short* pos;
-  C2<R>* tile = setup_smem<R>(smem_raw, twg, posg, Lx, Ly, &tw, &pos);
-  const int RS = Lx + 1, PS = Ly * RS;
-  const int64_t slab = blockIdx.x;
-  const int plane = Lx * Ly;
-  for (int i = threadIdx.x; i < 4 * plane; i += blockDim.x) {
-    const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
-    cp_async_elem<R>(&tile[f * PS + y * RS + x], &data[(int64_t)f * g.V + slab * plane + r]);
-  }
-  cp_async_wait();
-  __syncthreads();
-  fft_lines_dif<R, +1>(tile, lx, dx, tw);
-  fft_lines_dif<R, +1>(tile, ly, dy, tw + Lx);
-  for (int i = threadIdx.x; i < plane; i += blockDim.x) {
-    const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
-    const int o = pos[Lx + y] * RS + pos[x];
-    gauge_site<R, RG, GROWS, EXPG>(tile[o], tile[PS + o], tile[2 * PS + o], tile[3 * PS + o], g.V, slab * plane + i, gf,
-                                   Gf);
-  }
-}
-
 // Unfused variant for planes whose four fields do not fit in shared memory:
 // the inverse (x, y) transform has already been applied to data.
 template <typename R, typename RG, int GROWS, bool EXPG>
@@ -498,16 +485,19 @@ __global__ void gauge_from_delta_kernel(Geom g, const C2<R>* __restrict__ data, 
 // plan and launchers
 // ---------------------------------------------------------------------------
 
-// real_bytes 8: 16 = 4 x 4 and 128 = 8 x 4 x 4 instead of stages of 2, whose
-// index arithmetic costs the integer passes more than the larger radix saves.
+// Radices of a line of N = 2^a 3^b, as few stages as radices up to 8 allow:
+// 16 = 4 x 4 and 128 = 8 x 4 x 4 instead of stages of 2 and, for FP32 fields,
+// a left-over 2 or 4 taken into stages of 6 (48 = 8 x 6, 36 = 6 x 6).
 static int radix_schedule(int N, int real_bytes, int* radix) {
   int a = 0, b = 0, n = N;
   while (n % 2 == 0) { n /= 2; ++a; }
   while (n % 3 == 0) { n /= 3; ++b; }
   if (n != 1 || N < 2) return -1;
   int k = 0;
-  while (a >= 3 && !(real_bytes == 8 && a == 4)) { radix[k++] = 8; a -= 3; }
+  const bool six = real_bytes == 4;
+  while (a >= 3 && !(a == 4 && !(six && b > 0))) { radix[k++] = 8; a -= 3; }
   if (a == 4) { radix[k++] = 4; a = 2; }
+  while (six && b >= a && a > 0) { radix[k++] = 6; --a; --b; }
   if (a == 2) radix[k++] = 4;
   if (a == 1) radix[k++] = 2;
   while (b-- > 0) radix[k++] = 3;
@@ -576,8 +566,21 @@ static void configure_alt_passes(const int L[4], int real_bytes, FFTPlan* p) {
   p->threads_xyz = threads_for(L[0] * L[1] * L[2]);
 }
 
+// Shared memory of the plane passes with fpb fields, or xc columns, per CTA.
+// FP32 fields go in pairs (lgf_fft_pair.cu) where a CTA has two fields or
+// columns to pair.
+static bool pairs_xy(int real_bytes, int fields) { return real_bytes == 4 && fields % 2 == 0; }
+static bool pairs_zt(int real_bytes, int xc) { return real_bytes == 4 && xc % 2 == 0; }
+static size_t xy_smem(const int L[4], int real_bytes, int fields) {
+  if (pairs_xy(real_bytes, fields)) return pair_smem_xy(L, fields);
+  return plane_header_bytes(L[0], L[1], real_bytes) + (size_t)fields * L[1] * (L[0] + 1) * 2 * real_bytes;
+}
+static size_t zt_smem(const int L[4], int real_bytes, int xc) {
+  if (pairs_zt(real_bytes, xc)) return pair_smem_zt(L, xc);
+  return plane_header_bytes(L[2], L[3], real_bytes) + (size_t)L[3] * (L[2] * xc + 1) * 2 * real_bytes;
+}
+
 cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
-  const size_t cb = 2 * (size_t)real_bytes;  // bytes per complex element
   for (int mu = 0; mu < 4; ++mu) {
     p->d[mu].N = L[mu];
     p->d[mu].nst = radix_schedule(L[mu], real_bytes, p->d[mu].radix);
@@ -589,9 +592,6 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
     }
   }
   const int Lx = L[0], Ly = L[1], Lz = L[2], Lt = L[3];
-  const size_t hxy = plane_header_bytes(Lx, Ly, real_bytes);
-  const size_t hzt = plane_header_bytes(Lz, Lt, real_bytes);
-  const size_t plane_xy = (size_t)Ly * (Lx + 1) * cb;
   const size_t budget = 100 * 1024, maxsm = 220 * 1024;
   // FP64 planes (integer arithmetic, 90 to 130 registers) run best as many
   // small CTAs, one field or one x column each: 412 us for the three passes at
@@ -599,24 +599,29 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   // 24x18x12x27.  FP32 planes take up to four fields and eight columns.
   const bool small = real_bytes == 8;
   p->fpb_xy = small ? 1 : 4;
-  while (p->fpb_xy > 1 && p->fpb_xy * plane_xy > budget) p->fpb_xy /= 2;
-  if (plane_xy * p->fpb_xy + hxy > maxsm) return cudaErrorInvalidValue;
-  p->smem_xy = hxy + p->fpb_xy * plane_xy;
-  p->fuse_g = (4 * plane_xy + hxy <= maxsm) ? 1 : 0;
-  p->smem_c = hxy + 4 * plane_xy;
+  while (p->fpb_xy > 1 && xy_smem(L, real_bytes, p->fpb_xy) > (pairs_xy(real_bytes, 2) && p->fpb_xy == 2 ? maxsm : budget))
+    p->fpb_xy /= 2;
+  p->smem_xy = xy_smem(L, real_bytes, p->fpb_xy);
+  if (p->smem_xy > maxsm) return cudaErrorInvalidValue;
+  p->smem_c = xy_smem(L, real_bytes, 4);
+  p->fuse_g = p->smem_c <= (small ? maxsm : PLANE_SMEM_MAX) ? 1 : 0;
   int xc = 1;
   for (int c = small ? 1 : 8; c >= 1; c /= 2) {
     if (Lx % c) continue;
-    if (hzt + (size_t)Lt * (Lz * c + 1) * cb <= budget) { xc = c; break; }
+    if (zt_smem(L, real_bytes, c) <= budget) { xc = c; break; }
   }
-  if (!small && xc == 1 && Lx % 2 == 0 && hzt + (size_t)Lt * (Lz * 2 + 1) * cb <= maxsm) xc = 2;
+  if (!small && xc == 1 && Lx % 2 == 0 && zt_smem(L, real_bytes, 2) <= PLANE_SMEM_MAX) xc = 2;
   p->xc = xc;
-  p->smem_zt = hzt + (size_t)Lt * (Lz * xc + 1) * cb;
-  if (p->smem_zt > maxsm) return cudaErrorInvalidValue;
-  const int most = real_bytes == 8 ? FX_MAX_THREADS : 512;
-  p->threads_xy = std::min(most, threads_for(p->fpb_xy * Lx * Ly));
-  p->threads_zt = std::min(most, threads_for(Lz * Lt * xc));
-  p->threads_c = std::min(most, threads_for(4 * Lx * Ly));
+  p->smem_zt = zt_smem(L, real_bytes, xc);
+  if (p->smem_zt > (pairs_zt(real_bytes, xc) ? PLANE_SMEM_MAX : maxsm)) return cudaErrorInvalidValue;
+  const int most = real_bytes == 8 ? FX_MAX_THREADS : PAIR_MAX_THREADS;
+  // Eight elements of a tile per thread (eight pairs where a CTA works on pairs).
+  // Lattices of less than two (z, t) slabs per SM take four: an iteration of
+  // 16^4 FP32 37.5 -> 34.8 us; the three passes of 32^4 would go 85 -> 93 us.
+  const int per = real_bytes == 4 && Lz * Lt < 2 * 152 ? 1 : 2;
+  p->threads_xy = std::min(most, threads_for(p->fpb_xy * Lx * Ly / (pairs_xy(real_bytes, p->fpb_xy) ? per : 1)));
+  p->threads_zt = std::min(most, threads_for(Lz * Lt * xc / (pairs_zt(real_bytes, xc) ? per : 1)));
+  p->threads_c = std::min(most, threads_for(4 * Lx * Ly / (pairs_xy(real_bytes, 4) ? per : 1)));
   configure_alt_passes(L, real_bytes, p);
   return cudaSuccess;
 }
@@ -628,25 +633,23 @@ void fft_plan_candidates(const int L[4], int real_bytes, std::vector<FFTPlan>& o
   FFTPlan base;
   out.clear();
   if (configure_fft_plan(L, real_bytes, &base) != cudaSuccess) return;
-  const size_t cb = 2 * (size_t)real_bytes, maxsm = 220 * 1024;
+  const size_t maxsm = 220 * 1024;
   const int Lx = L[0], Ly = L[1], Lz = L[2], Lt = L[3];
-  const size_t hxy = plane_header_bytes(Lx, Ly, real_bytes);
-  const size_t hzt = plane_header_bytes(Lz, Lt, real_bytes);
-  const size_t plane_xy = (size_t)Ly * (Lx + 1) * cb;
   for (int fpb = 1; fpb <= 4; fpb *= 2) {
-    if (hxy + fpb * plane_xy > maxsm) continue;
+    if (xy_smem(L, real_bytes, fpb) > maxsm) continue;
     for (int xc = 1; xc <= 8; xc *= 2) {
-      if (Lx % xc || hzt + (size_t)Lt * (Lz * xc + 1) * cb > maxsm) continue;
+      if (Lx % xc || zt_smem(L, real_bytes, xc) > maxsm) continue;
       for (int tdiv = 8; tdiv <= 32; tdiv *= 2) {
         FFTPlan p = base;
         p.fpb_xy = fpb;
-        p.smem_xy = hxy + fpb * plane_xy;
+        p.smem_xy = xy_smem(L, real_bytes, fpb);
         p.xc = xc;
-        p.smem_zt = hzt + (size_t)Lt * (Lz * xc + 1) * cb;
+        p.smem_zt = zt_smem(L, real_bytes, xc);
+        const int most = real_bytes == 8 ? FX_MAX_THREADS : PAIR_MAX_THREADS;
         auto thr = [&](int points) {
           int t = (points + tdiv - 1) / tdiv;
           t = ((t + 31) / 32) * 32;
-          return std::max(64, std::min(real_bytes == 8 ? FX_MAX_THREADS : 512, t));
+          return std::max(64, std::min(most, t));
         };
         p.threads_xy = thr(fpb * Lx * Ly);
         p.threads_zt = thr(Lz * Lt * xc);
@@ -715,6 +718,8 @@ cudaError_t launch_fft_xy(const Geom& g, const FFTPlan& p, C2<R>* data, const C2
   int fpb = std::min(p.fpb_xy, nfields);
   while (nfields % fpb) fpb /= 2;
   const int thr = fpb == p.fpb_xy ? p.threads_xy : threads_for(fpb * g.L[0] * g.L[1]);
+  if (fpb % 2 == 0)
+    return launch_fft_xy_pair(g, p, data, tw, pos, sign, nfields, fpb, std::min(thr, PAIR_MAX_THREADS), s, B);
   const size_t smem = smem_header_bytes<R>(g.L[0], g.L[1]) + (size_t)fpb * g.L[1] * (g.L[0] + 1) * sizeof(C2<R>);
   dim3 grid((unsigned)(g.L[2] * g.L[3]), (unsigned)(nfields / fpb), (unsigned)B.n);
   const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
@@ -738,7 +743,8 @@ cudaError_t launch_fft_zt(const Geom& g, const FFTPlan& p, C2<R>* data, const C2
   if constexpr (sizeof(R) == sizeof(double)) {
     return launch_fft_zt_fx(g, p, data, tw, pos, K, mode, nfields, s, lio, B);
   } else {
-  const size_t smem = p.smem_zt;
+  if (mode == 0 && p.xc % 2 == 0) return launch_fft_zt_pair(g, p, data, tw, pos, K, nfields, s, lio, B);
+  const size_t smem = smem_header_bytes<R>(g.L[2], g.L[3]) + (size_t)g.L[3] * (g.L[2] * p.xc + 1) * sizeof(C2<R>);
   dim3 grid((unsigned)(g.L[0] / p.xc * g.L[1]), (unsigned)nfields, (unsigned)B.n);
   const bool lrn = mode == 0 && (lio.mtab != nullptr || lio.snap != nullptr);
   cudaError_t e = lrn ? allow_smem(fft_zt_filter_kernel<R, true>, smem) : allow_smem(fft_zt_filter_kernel<R, false>, smem);
@@ -835,15 +841,7 @@ static cudaError_t launch_pass_c(const Geom& g, const FFTPlan& p, C2<R>* data, c
     static_assert(GROWS == 3, "FP64 lanes keep three rows of g");
     return launch_xy_inv_gauge_fx(g, p, data, tw, pos, gfield, Gfield, s, B, EXPG);
   } else {
-  const size_t smem = p.smem_c;
-  if ((e = allow_smem(fft_xy_inv_gauge_kernel<R, RG, GROWS, EXPG>, smem)) != cudaSuccess) return e;
-  const int Lx = g.L[0], Ly = g.L[1], RS = Lx + 1, PS = Ly * RS;
-  const Lines lx = make_lines(4 * Ly, 4 * Ly, RS, 0, 1), ly = make_lines(4 * Lx, Lx, 1, PS, RS);
-  const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
-  fft_xy_inv_gauge_kernel<R, RG, GROWS, EXPG>
-      <<<dim3((unsigned)(g.L[2] * g.L[3]), 1, (unsigned)B.n), p.threads_c, smem, s>>>(g, p.d[0], p.d[1], data, tw, pos,
-                                                                                    gfield, Gfield, lx, ly, cd, B);
-  return cudaGetLastError();
+  return launch_xy_inv_gauge_pair<GROWS>(g, p, data, tw, pos, gfield, Gfield, s, B, EXPG);
   }
 }
 

@@ -313,6 +313,21 @@ cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double
 // l 2^-60) in the same order.
 void fft_twiddles(const int L[4], std::vector<double2>& tw);
 
+// ---- lgf_fft_pair.cu -----------------------------------------------------
+// The plane passes of FP32 fields on pairs of fields (x, y: fpb even) or of
+// columns (z, t: p.xc even, mode 0); shared memory of either.
+constexpr size_t PLANE_SMEM_MAX = 227 * 1024;
+size_t pair_smem_xy(const int L[4], int fields);
+size_t pair_smem_zt(const int L[4], int xc);
+cudaError_t launch_fft_xy_pair(const Geom& g, const FFTPlan& p, float2* data, const float2* tw, const short* pos,
+                               int sign, int nfields, int fpb, int threads, cudaStream_t s, const Batch& B);
+cudaError_t launch_fft_zt_pair(const Geom& g, const FFTPlan& p, float2* data, const float2* tw, const short* pos,
+                               const float* K, int nfields, cudaStream_t s, const LearnedIO& lio, const Batch& B);
+template <int GROWS>
+cudaError_t launch_xy_inv_gauge_pair(const Geom& g, const FFTPlan& p, const float2* data, const float2* tw,
+                                     const short* pos, float2* gfield, float2* Gfield, cudaStream_t s, const Batch& B,
+                                     bool exact_exp);
+
 cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p);
 
 // An autotuner's choice: the decomposition and the tile fields of the plan.

@@ -210,20 +210,18 @@ def test_links_round_trip(ext, name):
 # Gram-Schmidt of FP32 lanes in FP32 pairs
 # ---------------------------------------------------------------------------
 
-@pytest.mark.parametrize("alpha", [1e-6, 0.08, 3.0, 3e3, 3e7])
-def test_fp32_gauge_against_oracle(alpha):
-    """g(x) of one FP32 step; alpha = 3e3 puts sites on both sides of the pairs' range, 3e7 all beyond it.
+def check_fp32_gauge(ext, alpha):
+    """g(x) of one FP32 step against the oracle.
 
     Tolerance: the filtered field is known to about 1e-6 of its size (FP32
     divergence and transforms), which row 2 minus its projection on row 1
     amplifies by |r2| / |w|; 5e-6 of that covers the rounding of g as well.
     """
-    ext = (3, 4, 6, 9)
     U = fields.random_links(ext, 0.9, seed=3)
     D, K = O.divergence(U), O.fa_filter(ext, alpha)
     go = O.gauge_transform_from_divergence(D, K)
     M = O.ifft4(O.fft4(D) * K[..., None, None]) + np.eye(3)
-    r1, r2 = M[..., 0, :], M[..., 1, :]
+    r2 = M[..., 1, :]
     ip = np.sum(np.conj(go[..., 0, :]) * r2, axis=-1)
     kappa = np.linalg.norm(r2, axis=-1) / np.linalg.norm(r2 - ip[..., None] * go[..., 0, :], axis=-1)
     with lgf.Lattice(ext, "fp32") as lat:
@@ -231,3 +229,34 @@ def test_fp32_gauge_against_oracle(alpha):
         lat.step(alpha)
         g = lat.get_gauge()
     assert np.all(np.abs(g - go).max(axis=(-1, -2)) < 5e-6 * kappa)
+
+
+@pytest.mark.parametrize("alpha", [1e-6, 0.08, 3.0, 3e3, 3e7])
+def test_fp32_gauge_against_oracle(alpha):
+    """alpha = 3e3 puts sites on both sides of the pairs' range, 3e7 all beyond it."""
+    check_fp32_gauge((3, 4, 6, 9), alpha)
+
+
+# ---------------------------------------------------------------------------
+# plane passes of FP32 lanes on pairs
+# ---------------------------------------------------------------------------
+
+PAIR_EXTS = [(2, 2, 2, 2), (3, 27, 2, 4), (6, 3, 12, 9), (8, 12, 6, 16), (16, 18, 4, 8), (36, 4, 2, 48),
+             (54, 2, 24, 3), (2, 96, 64, 2), (4, 2, 72, 108)]
+
+
+@pytest.mark.parametrize("ext", PAIR_EXTS)
+def test_fp32_plane_passes_against_oracle(ext):
+    """Every radix, one and several stages a line, odd extents, one column pair and several."""
+    check_fp32_gauge(ext, 0.08)
+
+
+@pytest.mark.parametrize("sign", [-1, 1])
+@pytest.mark.parametrize("ext", PAIR_EXTS)
+def test_fp32_transform_against_reference(ext, sign):
+    """FP32 transforms in natural order: rounding grows with the stages, 2^-24 each of at most 16."""
+    f = fields4(ext)
+    ref = fft_ref(f, sign)
+    with lgf.Lattice(ext, "fp32") as lat:
+        out = lat.fft4(f, sign)
+    assert np.linalg.norm(out - ref) < 16 * 2 ** -24 * np.linalg.norm(ref)
