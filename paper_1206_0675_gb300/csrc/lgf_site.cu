@@ -23,27 +23,63 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block reduction of two sums (FP64, fixed order) and a maximum (FP32: the
-// link defect is compared with bounds far above FP32 resolution, and FP32
-// max and shuffles keep the FP64 pipe free); result valid in thread 0.
+// Sum of a warp's FP64 values on the integer pipe: an FP64 addition holds its
+// scheduler's FP64 pipe for 64 cycles, and five of them per value and warp were
+// half of what the measurement of FP32 links spent.  The significands, aligned
+// to the largest exponent of the warp with five bits below it, add exactly; what
+// an alignment drops is below 2^-58 of the largest value, 32 of them below the
+// 2^-53 of one FP64 rounding.  warp_align and warp_value frame the additions:
+// q 2^(e - 1080) is the sum.
+__device__ __forceinline__ int64_t warp_align(double v, uint32_t& e) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), field = (hi >> 20) & 0x7ffu;
+  const uint32_t ex = max(field, 1u);
+  e = __reduce_max_sync(0xffffffffu, ex);
+  const uint64_t m = ((uint64_t)((hi & 0xfffffu) | (field ? 0x100000u : 0u)) << 32) | lo;
+  const int64_t q = (int64_t)((m << 5) >> min(e - ex, 63u));
+  return (int32_t)hi < 0 ? -q : q;
+}
+__device__ __forceinline__ double warp_value(int64_t q, uint32_t e) {
+  const double d = (double)q;
+  const int hi = __double2hiint(d), ex = ((hi >> 20) & 0x7ff) + (int)e - 1080;
+  if (q == 0) return 0.0;
+  if (ex < 1 || ex > 2046) return d * 0x1p-57 * __hiloint2double((int)(e << 20), 0);
+  return __hiloint2double(hi + (((int)e - 1080) << 20), __double2loint(d));
+}
+
+// Block reduction of two sums (fixed order) and a maximum of values >= 0 (FP32:
+// the link defect is compared with bounds far above FP32 resolution; a NaN
+// counts as 0); result valid in thread 0.  At most 16 warps.
 __device__ __forceinline__ void block_reduce3(double& a, double& b, float& m) {
-  __shared__ double sa[32], sb[32];
-  __shared__ float sm[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  a = warp_sum(a);
-  b = warp_sum(b);
+  __shared__ double sums[2][16];
+  __shared__ uint32_t sm[16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  uint32_t ea, eb;
+  int64_t qa = warp_align(a, ea), qb = warp_align(b, eb);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
-  if (lane == 0) { sa[warp] = a; sb[warp] = b; sm[warp] = m; }
+  for (int o = 16; o > 0; o >>= 1) {
+    qa += __shfl_xor_sync(0xffffffffu, qa, o);
+    qb += __shfl_xor_sync(0xffffffffu, qb, o);
+  }
+  if (max(ea, eb) == 2047u) {  // infinities and NaN
+    a = warp_sum(a);
+    b = __shfl_sync(0xffffffffu, warp_sum(b), 0);
+    if (lane < 2) sums[lane][warp] = lane == 0 ? a : b;
+  } else {
+    const double v = warp_value(lane == 0 ? qa : qb, lane == 0 ? ea : eb);
+    if (lane < 2) sums[lane][warp] = v;
+  }
+  const uint32_t mw = __reduce_max_sync(0xffffffffu, m > 0.f ? __float_as_uint(m) : 0u);
+  if (lane == 0) sm[warp] = mw;
   __syncthreads();
   if (warp == 0) {
-    a = lane < nw ? sa[lane] : 0.0;
-    b = lane < nw ? sb[lane] : 0.0;
-    m = lane < nw ? sm[lane] : 0.f;
-    a = warp_sum(a);
-    b = warp_sum(b);
+    const int w = lane & 15;
+    double v = w < nw ? sums[lane >> 4][w] : 0.0;
+    m = __uint_as_float(__reduce_max_sync(0xffffffffu, w < nw ? sm[w] : 0u));
+    if (nw > 8) v += __shfl_xor_sync(0xffffffffu, v, 8);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    a = v;
+    b = __shfl_sync(0xffffffffu, v, 16);
   }
   __syncthreads();
 }
@@ -202,22 +238,31 @@ template <typename R> __device__ __forceinline__ LinkTerms<R> link_terms(const M
   return t;
 }
 
-// A site's sums: F's trace sum (FP64 above one link) and W in the link precision.
+// A site's sums: F's trace sum (FP32 links: as a pair f + fl, exact to 2^-46
+// for the four traces it adds) and W in the link precision.
 template <typename R> struct SiteSums {
-  double f;
+  R f, fl;
   R im0, im1, im2;
   C2<R> w01, w02, w12;
 };
+__device__ __forceinline__ double sum_f(const SiteSums<double>& o) { return o.f; }
+__device__ __forceinline__ double sum_f(const SiteSums<float>& o) { return f32_to_f64(o.f) + f32_to_f64(o.fl); }
+__device__ __forceinline__ void add_f(SiteSums<double>& o, double x) { o.f += x; }
+__device__ __forceinline__ void add_f(SiteSums<float>& o, float x) {
+  const float s = __fadd_rn(o.f, x), t = __fsub_rn(s, o.f);
+  o.fl += __fadd_rn(__fsub_rn(o.f, __fsub_rn(s, t)), __fsub_rn(x, t));
+  o.f = s;
+}
 template <typename R> __device__ __forceinline__ SiteSums<R> site_sums_zero() {
   SiteSums<R> o;
-  o.f = 0;
+  o.f = o.fl = 0;
   o.im0 = o.im1 = o.im2 = 0;
   o.w01 = o.w02 = o.w12 = mkc<R>(0, 0);
   return o;
 }
 // A site's own link of a direction, and the link of it that ends in the site.
 template <typename R> __device__ __forceinline__ void add_own(SiteSums<R>& o, const LinkTerms<R>& t) {
-  o.f += (double)t.tr;
+  add_f(o, t.tr);
   o.im0 -= t.y0; o.im1 -= t.y1; o.im2 -= t.y2;
   o.w01 = csub<R>(o.w01, t.a01);
   o.w02 = csub<R>(o.w02, t.a02);
@@ -263,7 +308,12 @@ template <bool SPLIT> struct MeasurePlace {
   }
   static __device__ __forceinline__ void join(SiteSums<float>& o) {
     if (SPLIT) {
-      join(o.f);
+#pragma unroll
+      for (int h = 8; h <= 16; h *= 2) {
+        const float f = __shfl_xor_sync(0xffffffffu, o.f, h), fl = __shfl_xor_sync(0xffffffffu, o.fl, h);
+        add_f(o, f);
+        o.fl += fl;
+      }
       join(o.im0); join(o.im1); join(o.im2);
       join(o.w01.x); join(o.w01.y); join(o.w02.x); join(o.w02.y); join(o.w12.x); join(o.w12.y);
     }
@@ -281,7 +331,9 @@ __device__ __forceinline__ double store_delta(const SiteSums<R>& o, C2<R>* __res
   delta[2 * V + s] = d02;
   delta[3 * V + s] = d12;
   // ||Delta_A||_F^2
-  return (double)delta_norm2<R>(a0, a1, a2, d01, d02, d12);
+  const R n = delta_norm2<R>(a0, a1, a2, d01, d02, d12);
+  if constexpr (sizeof(R) == sizeof(float)) return f32_to_f64(n);
+  else return n;
 }
 
 // The FP64 path of a site with links outside the fixed-point range.
@@ -406,7 +458,8 @@ __device__ __forceinline__ void site_sums_fx(const Geom& g, const MatField<doubl
 // 32^4: 18-real 197 us (FP64 sums on the FP64 pipe: 355 us), 12-real 271 us
 // (665 us).
 template <typename R, int ROWS, bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS)
+__global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS,
+                                  SPLIT ? 1 : sizeof(R) == sizeof(float) ? 5 : ROWS == 3 ? 3 : 2)
 measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt, C2<R>* __restrict__ delta,
                double* __restrict__ partials, DevState* __restrict__ st, int count_iter, unsigned long long cond,
                int use_cond, int only_if_revert, Batch B, unsigned long long cond_undo) {
@@ -458,7 +511,7 @@ measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt,
     p.join(o);
   }
   if (in && p.collects()) {
-    fsum = o.f;
+    fsum = sum_f(o);
     tsum = store_delta<R>(o, delta, g.V, p.s);
     const int dmu = defect_sample_mu(p.s);
     if (dmu >= 0) {
@@ -561,7 +614,7 @@ update_measure_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, Ma
   }
   p.join(o);
   if (in && p.collects()) {
-    fsum = o.f;
+    fsum = sum_f(o);
     tsum = store_delta<R>(o, delta, g.V, p.s);
   }
   measure_tail(g, fsum, tsum, dmax, partials, st, 1, cond, use_cond, false, 1, sizeof(R) == 8, cond_undo);
