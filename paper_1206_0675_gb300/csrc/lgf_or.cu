@@ -17,11 +17,15 @@
 // Every link joins two sites of opposite colour, so within one colour each
 // link is read and written by exactly one thread: the update is in place.
 //
-// FP32 links: one thread per site of the colour.  Its links are read twice (once for w,
-// once for the product, the second time from L1/L2) so that only w, the
-// running subgroup block and g stay in registers.  The site algebra runs in
-// the link precision; rows 1-2 of every product are formed and row 3 is
-// rebuilt as (a x b)^* (Sec. 3.2), as in the Fourier-accelerated update.
+// FP32 links: one thread per site of the colour, its eight links loaded at once
+// (48 loads in flight) and kept in registers from w to the products, at 168
+// registers and 12 warps per SM.  Reading them one by one, and again for the
+// products, left the warps waiting for loads (14 of 19 cycles between
+// instructions): 32^4 12-real 188 -> 148 us a sweep (118 us for its bytes at
+// 6.8 TB/s), 18-real 295 -> 273 us, 16^4 12-real 20.4 -> 16.4 us; at 128
+// registers 210 us, at 255 170 us.  The site algebra runs in the link
+// precision; rows 1-2 of every product are formed and row 3 is rebuilt as
+// (a x b)^* (Sec. 3.2), as in the Fourier-accelerated update.
 #include <cmath>
 
 #include "lgf_fixed.cuh"
@@ -132,6 +136,28 @@ __device__ __forceinline__ int64_t or_coords(const Geom& g, const FastDiv& dhx, 
   return (int64_t)c[0] + (int64_t)g.L[0] * row;
 }
 
+// The stored rows of a matrix.
+template <typename R, int ROWS> struct Rows {
+  C2<R> e[ROWS][3];
+  // rows 1 to 3, the third rebuilt where it is not stored
+  __device__ __forceinline__ void full(C2<R> (&o)[3][3]) const {
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) o[i][j] = e[i][j];
+    if (ROWS == 2) su3_third_row<R>(o[0], o[1], o[2]);
+  }
+};
+template <typename R, int ROWS>
+__device__ __forceinline__ Rows<R, ROWS> load_rows(const MatField<R, ROWS>& F, int m, int64_t s) {
+  Rows<R, ROWS> v;
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) v.e[r][j] = F.p[F.off(m, r, j, s)];
+  return v;
+}
+
 // w(x) = sum_mu [U_mu(x) + U_mu^dag(x - mu^)]
 template <typename R, int ROWS>
 __device__ __forceinline__ void or_local_field(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
@@ -156,47 +182,69 @@ __device__ __forceinline__ void or_local_field(const Geom& g, const MatField<R, 
   }
 }
 
-// One site of the colour: its hit and the products with its eight links.
+// One site of the colour: its hit and the products with its eight links, which
+// stay in registers from one use to the other (of the links that end in the
+// site, rows 1 and 2).
 template <typename R, int ROWS>
 __device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
                                         C2<R>* __restrict__ G, R omega) {
+  Rows<R, ROWS> u[4], b[4];
+  uint32_t sb[4];  // site indices have 28 bits
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    sb[mu] = (uint32_t)or_back(g, s, c, mu);
+    u[mu] = load_rows(U, mu, s);
+    b[mu] = load_rows(U, mu, sb[mu]);
+  }
   M3<R> M;
-  or_local_field<R, ROWS>(g, U, c, s, M);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) M.e[r][k] = mkc<R>(0, 0);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    C2<R> f[3][3];
+    u[mu].full(f);
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) M.e[r][k] = cadd<R>(M.e[r][k], f[r][k]);
+    b[mu].full(f);
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) M.e[r][k] = cadd<R>(M.e[r][k], cconj<R>(f[k][r]));
+  }
   M3<R> gx;
   or_site_gauge<R>(M, omega, gx);
 
-#pragma unroll 1
+#pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     // U_mu(x) <- g U_mu(x): rows 0, 1 by products, row 2 = (row0 x row1)^*
-    M3<R> u, o;
-    U.load(mu, s, u);
+    C2<R> f[3][3];
+    M3<R> o;
+    u[mu].full(f);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        C2<R> acc = cmul_fx<R>(gx.e[i][0], u.e[0][k]);
-        acc = cfma<R>(gx.e[i][1], u.e[1][k], acc);
-        o.e[i][k] = cfma<R>(gx.e[i][2], u.e[2][k], acc);
+        C2<R> acc = cmul_fx<R>(gx.e[i][0], f[0][k]);
+        acc = cfma<R>(gx.e[i][1], f[1][k], acc);
+        o.e[i][k] = cfma<R>(gx.e[i][2], f[2][k], acc);
       }
     su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
     U.store(mu, s, o);
     // U_mu(x - mu^) <- U_mu(x - mu^) g^dag: rows 0, 1 of the old link suffice
-    const int64_t sb = or_back(g, s, c, mu);
-    C2<R> v[2][3];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) v[i][k] = U.p[U.off(mu, i, k, sb)];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        C2<R> acc = cmulc_fx<R>(v[i][0], gx.e[k][0]);
-        acc = cfmac<R>(v[i][1], gx.e[k][1], acc);
-        o.e[i][k] = cfmac<R>(v[i][2], gx.e[k][2], acc);
+        C2<R> acc = cmulc_fx<R>(b[mu].e[i][0], gx.e[k][0]);
+        acc = cfmac<R>(b[mu].e[i][1], gx.e[k][1], acc);
+        o.e[i][k] = cfmac<R>(b[mu].e[i][2], gx.e[k][2], acc);
       }
     su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
-    U.store(mu, sb, o);
+    U.store(mu, sb[mu], o);
   }
 
   if (G != nullptr) {
@@ -217,7 +265,7 @@ __device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& 
 }
 
 template <typename R, int ROWS>
-__global__ void __launch_bounds__(OR_THREADS)
+__global__ void __launch_bounds__(OR_THREADS, 3)
 or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, const DevState* __restrict__ st,
                      C2<R>* __restrict__ G, int parity, FastDiv dhx, R omega) {
   // fused FP32 lanes keep their current links in one of two buffers
