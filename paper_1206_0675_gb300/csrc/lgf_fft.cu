@@ -622,6 +622,15 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   p->threads_xy = std::min(most, threads_for(p->fpb_xy * Lx * Ly / (pairs_xy(real_bytes, p->fpb_xy) ? per : 1)));
   p->threads_zt = std::min(most, threads_for(Lz * Lt * xc / (pairs_zt(real_bytes, xc) ? per : 1)));
   p->threads_c = std::min(most, threads_for(4 * Lx * Ly / (pairs_xy(real_bytes, 4) ? per : 1)));
+  if (small && p->fuse_g) {
+    // pass C of FP64 planes: as many CTAs as fit an SM's shared memory share its
+    // FX_C_THREADS threads (80 registers each).  32^4: three CTAs of 256 110 us,
+    // one of 384 threads at 168 registers 150 us, three of 128 126 us;
+    // 24x18x12x27 45 -> 31 us.
+    const int ctas = std::max(1, (int)(PLANE_SMEM_MAX / (p->smem_c + 1024)));
+    p->threads_c = std::min((4 * Lx * Ly / 8 + 31) / 32 * 32, std::max(128, FX_C_THREADS / ctas / 32 * 32));
+    p->threads_c = std::max(64, p->threads_c);
+  }
   configure_alt_passes(L, real_bytes, p);
   return cudaSuccess;
 }
@@ -653,7 +662,7 @@ void fft_plan_candidates(const int L[4], int real_bytes, std::vector<FFTPlan>& o
         };
         p.threads_xy = thr(fpb * Lx * Ly);
         p.threads_zt = thr(Lz * Lt * xc);
-        p.threads_c = thr(4 * Lx * Ly);
+        p.threads_c = real_bytes == 8 && tdiv == 8 ? base.threads_c : thr(4 * Lx * Ly);
         out.push_back(p);
       }
     }

@@ -22,9 +22,11 @@
 // smooth and constant inputs): 0.7e-16 to 2.8e-16, the FP64 passes on the FP64
 // pipe had 1.5e-16 to 4.6e-16.
 //
-// 32^4, us: pass A 76 (FP64 pipe: 231), pass B 160 (463), pass C with g 153 (397);
-// 24x18x12x27: 24, 41, 47 (54, 94, 78).  Bound by instruction issue (about 400
-// instructions per element of pass A, 800 of pass B) at 12 to 24 warps per SM.
+// 32^4, us: pass A 72 (FP64 pipe: 231), pass B 160 (463), pass C with g 111 (397);
+// 24x18x12x27: 23, 40, 32 (54, 94, 78).  Bound by instruction issue (about 400
+// instructions per element of pass A, 800 of pass B) at 24 warps per SM, 80
+// registers a thread (pass B at 96: 151 us at 32^4, but 53 at 24x18x12x27; at
+// 64: 177).
 //
 // Planes that hold infinities or NaN give NaN; planes whose largest
 // component is near the ends of the FP64 range take slower conversions.
@@ -532,7 +534,7 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
 }
 
 template <bool EXPG>
-__global__ void __launch_bounds__(FX_MAX_THREADS)
+__global__ void __launch_bounds__(FX_C_THREADS)
 fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const double2* __restrict__ data,
                            const int4* __restrict__ twg, const short* __restrict__ posg, double2* __restrict__ gf,
                            double2* __restrict__ Gf, CopyDiv cd, Batch B) {
