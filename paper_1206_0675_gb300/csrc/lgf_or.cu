@@ -289,6 +289,9 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 394 (724), 32^4 1151 (2142),
+// 16^4 79 (168), 8^4 37 (93); 12-real 32^4 883 (2311).  The CTAs per SM are the
+// best of 3 to 7 for each kernel and storage (links of 18 reals at 5: 1201 us).
 
 // The 64-bit sum an operand stands for (units of 2^-60).
 __device__ __forceinline__ int64_t fx_r60(Fx a) { return mad_wide(a.h, 1 << 30, (int64_t)a.l); }
@@ -396,7 +399,7 @@ static __device__ __noinline__ void or_gauge_fp64(const Geom& g, MatField<double
 }
 
 template <int ROWS>
-__global__ void __launch_bounds__(OR_THREADS)
+__global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 5 : 4)
 or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, double2* __restrict__ G, int parity,
                    FastDiv dhx, double omega, int64_t w7, int64_t c7) {
   const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -500,7 +503,7 @@ static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const
 // A CTA takes 32 sites of the colour and half of their links: four warps, the
 // directions' forward (blockIdx.y = 0) or backward links.
 template <int ROWS>
-__global__ void __launch_bounds__(OR_THREADS, 5)
+__global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 4 : 5)
 or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__ gf, int parity, FastDiv dhx) {
   const uint32_t j = blockIdx.x * 32u + (threadIdx.x & 31u);
   const int mu = threadIdx.x >> 5;
