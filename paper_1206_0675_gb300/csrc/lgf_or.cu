@@ -289,8 +289,8 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
-// A sweep, us (FP64 arithmetic before): 18-real 24^4 394 (724), 32^4 1151 (2142),
-// 16^4 79 (168), 8^4 37 (93); 12-real 32^4 883 (2311).  The CTAs per SM are the
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 333 (724), 32^4 960 (2142),
+// 16^4 78 (168), 8^4 37 (93); 12-real 32^4 774 (2311).  The CTAs per SM are the
 // best of 3 to 7 for each kernel and storage (links of 18 reals at 5: 1201 us).
 
 // The 64-bit sum an operand stands for (units of 2^-60).
@@ -501,13 +501,17 @@ static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const
 }
 
 // A CTA takes 32 sites of the colour and half of their links: four warps, the
-// directions' forward (blockIdx.y = 0) or backward links.
+// directions' forward (even blockIdx.x) or backward links.  The sites of a colour
+// use half of every 32-byte sector; the other half belongs to backward links of
+// neighbouring rows, so the two kinds alternate and the sector is still in L2
+// (all forward links first: 77 % of the DRAM bandwidth, 394 against 333 us a
+// sweep of 24^4).
 template <int ROWS>
 __global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 4 : 5)
 or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__ gf, int parity, FastDiv dhx) {
-  const uint32_t j = blockIdx.x * 32u + (threadIdx.x & 31u);
+  const uint32_t j = (blockIdx.x >> 1) * 32u + (threadIdx.x & 31u);
   const int mu = threadIdx.x >> 5;
-  const bool fwd = blockIdx.y == 0;
+  const bool fwd = (blockIdx.x & 1u) == 0;
   if ((int64_t)j >= (g.V >> 1)) return;
   int c[4];
   const int64_t s = or_coords(g, dhx, j, parity, c);
@@ -599,7 +603,7 @@ cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevS
         g, U, gfield, G, parity & 1, dhx, omega, w7, c7);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    or_links_fx_kernel<ROWS><<<dim3((unsigned)((n + 31) / 32), 2), OR_THREADS, 0, s>>>(g, U, gfield, parity & 1, dhx);
+    or_links_fx_kernel<ROWS><<<2 * (unsigned)((n + 31) / 32), OR_THREADS, 0, s>>>(g, U, gfield, parity & 1, dhx);
   } else {
     const unsigned nb = (unsigned)((n + OR_THREADS - 1) / OR_THREADS);
     or_half_sweep_kernel<R, ROWS><<<nb, OR_THREADS, 0, s>>>(g, U0, U1, st, G, parity & 1, dhx, (R)omega);
