@@ -289,9 +289,10 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
-// A sweep, us (FP64 arithmetic before): 18-real 24^4 333 (724), 32^4 960 (2142),
-// 16^4 78 (168), 8^4 37 (93); 12-real 32^4 774 (2311).  The CTAs per SM are the
-// best of 3 to 7 for each kernel and storage (links of 18 reals at 5: 1201 us).
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 324 (724), 32^4 933 (2142),
+// 16^4 78 (168), 8^4 37 (93); 12-real 32^4 771 (2311).  The CTAs per SM are the
+// best of 3 to 6 for each kernel and storage (links of 18 reals at 4: 960 us, at 3:
+// 1056).
 
 // The 64-bit sum an operand stands for (units of 2^-60).
 __device__ __forceinline__ int64_t fx_r60(Fx a) { return mad_wide(a.h, 1 << 30, (int64_t)a.l); }
@@ -504,10 +505,10 @@ static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const
 // directions' forward (even blockIdx.x) or backward links.  The sites of a colour
 // use half of every 32-byte sector; the other half belongs to backward links of
 // neighbouring rows, so the two kinds alternate and the sector is still in L2
-// (all forward links first: 77 % of the DRAM bandwidth, 394 against 333 us a
+// (all forward links first: 77 % of the DRAM bandwidth, 394 against 324 us a
 // sweep of 24^4).
 template <int ROWS>
-__global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 4 : 5)
+__global__ void __launch_bounds__(OR_THREADS, 5)
 or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__ gf, int parity, FastDiv dhx) {
   const uint32_t j = (blockIdx.x >> 1) * 32u + (threadIdx.x & 31u);
   const int mu = threadIdx.x >> 5;
