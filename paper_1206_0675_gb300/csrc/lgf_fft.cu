@@ -6,7 +6,7 @@
 //   pass B : forward DFT over (z, t), multiply by the momentum filter,
 //            inverse DFT over (z, t)                                [k4 fused]
 //   pass C : inverse DFT over (x, y), then g(x) = reunitarize(1 + Delta'(x))
-//            in FP64, optionally G <- g G                           [k5 fused]
+//            (lgf_gauge.cuh), optionally G <- g G                   [k5 fused]
 //
 // Each 1D transform is an in-place mixed-radix (2, 3, 4, 6, 8) Cooley-Tukey FFT
 // in shared memory (see ct_stage).  Consecutive threads work on neighbouring

@@ -68,7 +68,8 @@ __device__ __forceinline__ bool batch_skip(const Batch& b) { return b.st != null
 // a thread per site leaves most schedulers without a warp and its chain of
 // eight links is what takes the time.  8^4: 22.6 -> 15.8 us with FP64 links,
 // 16.4 -> 12.5 us fused with the update of FP32 links; 16^4: 28.2 -> 32.4 us,
-// 20.1 -> 23.2 us (the lanes' sums have to be added).
+// 20.1 -> 23.2 us (the lanes' sums have to be added).  With the warps' sums on the
+// integer pipe the 8^4 figures are 14.6 and 11.6 us.
 constexpr int MEASURE_THREADS = 256, MEASURE_SPLIT_THREADS = 128;
 inline bool measure_split(int64_t V) { return V < 152 * 128; }
 inline int64_t measure_blocks(int64_t V) {
@@ -271,7 +272,7 @@ template <typename R>
 cudaError_t launch_fft_zt(const Geom& g, const FFTPlan& p, C2<R>* data, const C2<R>* tw, const short* pos,
                           const R* K, int mode, int nfields, cudaStream_t s, const LearnedIO& lio = LearnedIO(),
                           const Batch& B = Batch());
-// Inverse (x,y) transform fused with g(x) = reunitarize(1 + Delta'(x)) in FP64
+// Inverse (x,y) transform fused with g(x) = reunitarize(1 + Delta'(x)) (lgf_gauge.cuh)
 // (exact_exp != 0: g(x) = reunitarize(exp(Delta'(x)))); g stored with GROWS
 // rows in precision RG; optional G <- g G (precision RG with 3 rows).
 template <typename R, typename RG, int GROWS>

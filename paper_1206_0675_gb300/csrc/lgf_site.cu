@@ -3,8 +3,9 @@
 //                (arXiv:1206.0675 Sec. 2 and kernel k2 of Sec. 3.2),
 //   * update   : U_mu(x) -> g(x) U_mu(x) g^dagger(x + mu^) (Sec. 2 eq. 2, kernel k6),
 //   * layout conversion, SU(3) validation, the momentum filter table (k1).
-// One thread per lattice site; link arrays are structure-of-arrays so that a
-// warp touches 32 consecutive sites of one matrix element per load.
+// One thread per lattice site, or per link in the update of FP64 links; link
+// arrays are structure-of-arrays so that a warp touches 32 consecutive sites of
+// one matrix element per load.
 #include <algorithm>
 #include <cmath>
 
@@ -454,8 +455,9 @@ __device__ __forceinline__ void site_sums_fx(const Geom& g, const MatField<doubl
   o.w12 = make_double2(fx_to_double_fp<58>(t[8]), fx_to_double_fp<58>(t[9]));
 }
 
-// FP64 links are bound by the ALU pipe (65 % busy in ncu) beside HBM (41 %).
-// 32^4: 18-real 197 us (FP64 sums on the FP64 pipe: 355 us), 12-real 271 us
+// FP64 links are bound by the ALU pipe (66 % busy in ncu) beside HBM (40 %) and
+// the FP64 pipe (41 %: the sites' conversions and norms).
+// 32^4: 18-real 195 us (FP64 sums on the FP64 pipe: 355 us), 12-real 265 us
 // (665 us).
 template <typename R, int ROWS, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS,
