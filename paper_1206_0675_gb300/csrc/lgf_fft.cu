@@ -611,6 +611,11 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
     if (zt_smem(L, real_bytes, c) <= budget) { xc = c; break; }
   }
   if (!small && xc == 1 && Lx % 2 == 0 && zt_smem(L, real_bytes, 2) <= PLANE_SMEM_MAX) xc = 2;
+  // Where only two columns leave room for a second CTA on an SM (runs of 16 bytes,
+  // half of each sector), four in one CTA of PAIR_ZT_THREADS.  Pass B, us: 48^3x96
+  // 507 -> 461, 64^4 777 -> 651, 16^2x64x96 108 -> 84, 24^2x72x54 127 -> 110.
+  const bool alone = !small && xc == 2 && Lx % 4 == 0 && zt_smem(L, real_bytes, 4) <= PLANE_SMEM_MAX;
+  if (alone) xc = 4;
   p->xc = xc;
   p->smem_zt = zt_smem(L, real_bytes, xc);
   if (p->smem_zt > (pairs_zt(real_bytes, xc) ? PLANE_SMEM_MAX : maxsm)) return cudaErrorInvalidValue;
@@ -622,6 +627,7 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   p->threads_xy = std::min(most, threads_for(p->fpb_xy * Lx * Ly / (pairs_xy(real_bytes, p->fpb_xy) ? per : 1)));
   p->threads_zt = std::min(most, threads_for(Lz * Lt * xc / (pairs_zt(real_bytes, xc) ? per : 1)));
   p->threads_c = std::min(most, threads_for(4 * Lx * Ly / (pairs_xy(real_bytes, 4) ? per : 1)));
+  if (alone) p->threads_zt = std::min(PAIR_ZT_THREADS, (Lz * Lt * xc / 16 + 31) / 32 * 32);
   if (small && p->fuse_g) {
     // pass C of FP64 planes: as many CTAs as fit an SM's shared memory share its
     // FX_C_THREADS threads (80 registers each).  32^4: three CTAs of 256 110 us,
@@ -755,6 +761,7 @@ cudaError_t launch_fft_zt(const Geom& g, const FFTPlan& p, C2<R>* data, const C2
   if (mode == 0 && p.xc % 2 == 0) return launch_fft_zt_pair(g, p, data, tw, pos, K, nfields, s, lio, B);
   const size_t smem = smem_header_bytes<R>(g.L[2], g.L[3]) + (size_t)g.L[3] * (g.L[2] * p.xc + 1) * sizeof(C2<R>);
   dim3 grid((unsigned)(g.L[0] / p.xc * g.L[1]), (unsigned)nfields, (unsigned)B.n);
+  const int threads = std::min(p.threads_zt, 512);  // a plan for pairs can have more
   const bool lrn = mode == 0 && (lio.mtab != nullptr || lio.snap != nullptr);
   cudaError_t e = lrn ? allow_smem(fft_zt_filter_kernel<R, true>, smem) : allow_smem(fft_zt_filter_kernel<R, false>, smem);
   if (e != cudaSuccess) return e;
@@ -763,10 +770,10 @@ cudaError_t launch_fft_zt(const Geom& g, const FFTPlan& p, C2<R>* data, const C2
   const Lines lz = make_lines(Lt * xc, xc, 1, TS, xc), lt = make_lines(Lz * xc, Lz * xc, 1, 0, TS);
   const CopyDiv cd{FastDiv::make((uint32_t)xc), FastDiv::make((uint32_t)Lz)};
   if (lrn)
-    fft_zt_filter_kernel<R, true><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, tw, pos, K, p.xc, mode, lio,
+    fft_zt_filter_kernel<R, true><<<grid, threads, smem, s>>>(g, p.d[2], p.d[3], data, tw, pos, K, p.xc, mode, lio,
                                                                    H, lz, lt, cd, B);
   else
-    fft_zt_filter_kernel<R, false><<<grid, p.threads_zt, smem, s>>>(g, p.d[2], p.d[3], data, tw, pos, K, p.xc, mode,
+    fft_zt_filter_kernel<R, false><<<grid, threads, smem, s>>>(g, p.d[2], p.d[3], data, tw, pos, K, p.xc, mode,
                                                                     lio, H, lz, lt, cd, B);
   return cudaGetLastError();
   }

@@ -14,11 +14,12 @@
 // instructions an element.  A, B, C of 12-real FP32 links, us, scalar -> pairs:
 //   16^4       9, 14, 10 -> 8.4, 10.1, 10.1
 //   32^4      33, 63, 48 -> 24, 37, 31
-//   48^3x96   308, 794, 461 -> 167, 506, 246
+//   48^3x96   308, 794, 461 -> 167, 461, 246
 // Floors (bytes once at 6.8 TB/s): 10, 10, 12 us at 32^4; 100, 100, 125 us at
 // 48^3x96.  What is left is latency: planes of 75 KB leave two CTAs of 384
 // threads on an SM, so registers are held to 80 (at 102, one CTA of 512: 277,
-// 623, 341 us), and pass B of 48^3x96 reads and writes runs of 16 bytes.
+// 623, 341 us); pass B of 48^3x96 takes four columns in one CTA of 768 threads
+// (runs of 32 bytes; two columns in two CTAs of 384: 507 us).
 #include "lgf_fft_tile.cuh"
 #include "lgf_gauge.cuh"
 #include "lgf_internal.h"
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(PAIR_MAX_THREADS, 2) fft_xy_pair_kernel(Geom g
 static int zt_row(int Lz, int xcp) { return xcp == 1 ? Lz | 1 : Lz * xcp + (((xcp - Lz * xcp) % 8) + 8) % 8; }
 
 template <bool LRN>
-__global__ void __launch_bounds__(PAIR_MAX_THREADS, 2) fft_zt_pair_kernel(Geom g, FFTDir dz, FFTDir dt, float2* __restrict__ data,
+__global__ void __launch_bounds__(PAIR_ZT_THREADS) fft_zt_pair_kernel(Geom g, FFTDir dz, FFTDir dt, float2* __restrict__ data,
                                                           const float2* __restrict__ twg,
                                                           const short* __restrict__ posg,
                                                           const float* __restrict__ K, int xcp, int TS, LearnedIO lio,

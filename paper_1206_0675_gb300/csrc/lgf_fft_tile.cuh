@@ -43,7 +43,8 @@ template <typename R> __host__ __device__ inline size_t smem_header_bytes(int n0
 constexpr size_t FX_PLANE_BYTES = 128;
 constexpr int FX_MAX_THREADS = 384;  // CTA size limit of the FP64 plane passes
 constexpr int FX_C_THREADS = 768;    // and of the one with g(x): threads per SM at 80 registers
-constexpr int PAIR_MAX_THREADS = 384;  // and of the FP32 passes on pairs
+constexpr int PAIR_MAX_THREADS = 384;  // and of the FP32 passes on pairs,
+constexpr int PAIR_ZT_THREADS = 768;   // of the (z, t) pass where a tile fills an SM
 inline size_t plane_header_bytes(int n0, int n1, int real_bytes) {
   return real_bytes == 8 ? smem_header_bytes<double>(n0, n1) + FX_PLANE_BYTES : smem_header_bytes<float>(n0, n1);
 }

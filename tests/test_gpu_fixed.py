@@ -242,7 +242,7 @@ def test_fp32_gauge_against_oracle(alpha):
 # ---------------------------------------------------------------------------
 
 PAIR_EXTS = [(2, 2, 2, 2), (3, 27, 2, 4), (6, 3, 12, 9), (8, 12, 6, 16), (16, 18, 4, 8), (36, 4, 2, 48),
-             (54, 2, 24, 3), (2, 96, 64, 2), (4, 2, 72, 108)]
+             (54, 2, 24, 3), (2, 96, 64, 2), (4, 2, 72, 108), (4, 2, 48, 96)]
 
 
 @pytest.mark.parametrize("ext", PAIR_EXTS)
