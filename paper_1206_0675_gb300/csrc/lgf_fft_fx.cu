@@ -18,12 +18,17 @@
 // rounds at every operation, where additions are exact here).  Inputs are
 // read and results written in FP64.
 //
-// Error against 80-bit arithmetic (2-norm, forward and inverse, random,
-// smooth and constant inputs): 0.7e-16 to 2.8e-16, the FP64 passes on the FP64
-// pipe had 1.5e-16 to 4.6e-16.
+// Error against extended precision: of the transform (2-norm, forward and
+// inverse, random, smooth and constant inputs) 0.7e-16 to 2.8e-16, of the passes
+// on the FP64 pipe 1.5e-16 to 4.6e-16; of g(x), where the filter weights the
+// lowest modes most (rms): planes of 16 x 16 0.7e-16 (1.1e-16), 32 x 32 1.2e-16
+// (1.9e-16), 48 x 48 2.1e-16 (3.0e-16), 64 x 64 5.1e-16 (7.0e-16), 128 x 2 with
+// 96 x 2 1.2e-15 (1.2e-15), 81 x 81 1.6e-15 (0.9e-15).  For that every rounding
+// is centred: inputs are rounded, halves go to even, and products carry the mean
+// of what they drop.
 //
-// 32^4, us: pass A 72 (FP64 pipe: 231), pass B 160 (463), pass C with g 111 (397);
-// 24x18x12x27: 23, 40, 32 (54, 94, 78).  Bound by instruction issue (about 400
+// 32^4, us: pass A 74 (FP64 pipe: 231), pass B 165 (463), pass C with g 113 (397);
+// 24x18x12x27: 24, 41, 33 (54, 94, 78).  Bound by instruction issue (about 400
 // instructions per element of pass A, 800 of pass B) at 24 warps per SM, 80
 // registers a thread (pass B at 96: 151 us at 32^4, but 53 at 24x18x12x27; at
 // 64: 177).
@@ -139,9 +144,9 @@ template <int SIGN> __device__ __forceinline__ I2 itwiddle(I2 v, int4 w) {
   const Bfp2 x = bfp_limbs(v.x), y = bfp_limbs(v.y);
   const int sh = fx_opaque(SIGN < 0 ? w.z : -w.z), sl = fx_opaque(SIGN < 0 ? w.w : -w.w);
   const int nh = fx_opaque(SIGN < 0 ? -w.z : w.z), nl = fx_opaque(SIGN < 0 ? -w.w : w.w);
-  const int64_t half = (int64_t)1 << 29;
-  int64_t rm = mad_wide(x.l, w.x, mad_wide(x.h, w.y, half));
-  int64_t im = mad_wide(x.l, sh, mad_wide(x.h, sl, half));
+  const int64_t half = (int64_t)1 << 29;  // and the mean of the products of low limbs (bfp_mul)
+  int64_t rm = mad_wide(x.l, w.x, mad_wide(x.h, w.y, half + ((w.y + nl) >> 1)));
+  int64_t im = mad_wide(x.l, sh, mad_wide(x.h, sl, half + ((sl + w.y) >> 1)));
   rm = mad_wide(y.l, nh, mad_wide(y.h, nl, rm));
   im = mad_wide(y.l, w.x, mad_wide(y.h, w.y, im));
   return make_longlong2(mad_wide(y.h, nh, mad_wide(x.h, w.x, rm >> 30)),

@@ -181,14 +181,14 @@ __device__ __forceinline__ void fx_cross_conj(FxAcc& re, FxAcc& im, const FxC& a
 // ---------------------------------------------------------------------------
 
 // Integer of an FP64 number in units that make the block's largest magnitude
-// fit (see the transform passes): M >> (base - e), M with its leading one at
-// bit 63.  base >= 64, so zeros and numbers 2^-64 below the block's largest
-// give zero.
+// fit (see the transform passes): M >> (base - e), rounded, M with its leading
+// one at bit 63.  base > 64, so zeros and numbers 2^-64 below the block's
+// largest give zero.
 __device__ __forceinline__ int64_t bfp_from(double a, uint32_t base) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
   const int64_t sg = (int64_t)((int)hi >> 31);
-  return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, base - ((hi >> 20) & 0x7ffu)) ^ sg) - sg;
+  return ((int64_t)((shr64_clamp(((uint64_t)mh << 32) | ml, base - 1u - ((hi >> 20) & 0x7ffu)) + 1u) >> 1) ^ sg) - sg;
 }
 
 // FP64 value of n 2^ex rounded to nearest, where the result is far from the
@@ -217,10 +217,13 @@ __device__ __forceinline__ Bfp2 bfp_limbs(int64_t x) {
 
 // Real and complex products with a constant or a root of unity w, |w| <= 1,
 // w = h 2^-30 + l 2^-60 (|l| <= 2^29): three multiply-adds per real product,
-// rounded to the nearest unit (l l' 2^-60 is dropped, below 2^-30 of a unit).
+// rounded to the nearest unit.  Of l l' 2^-60, up to half a unit, the mean over
+// the low limbs l of x, l' 2^-31, goes in with the rounding: dropped, it adds the
+// same to every product with one root, and a line of 81 (four stages with
+// sqrt(3)/2) gathered 30 times the error of one of 64 in its low modes.
 __device__ __forceinline__ int64_t bfp_mul(int64_t x, int wh, int wl) {
   const Bfp2 a = bfp_limbs(x);
-  const int64_t mid = mad_wide(a.l, wh, mad_wide(a.h, wl, (int64_t)1 << 29));
+  const int64_t mid = mad_wide(a.l, wh, mad_wide(a.h, wl, ((int64_t)1 << 29) + (wl >> 1)));
   return mad_wide(a.h, wh, mid >> 30);
 }
 
