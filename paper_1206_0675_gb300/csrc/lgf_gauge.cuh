@@ -379,9 +379,13 @@ static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, 
 
 // G(s) <- g G(s) in fixed point, for the entries gp[e gstride] of g (a call:
 // its operands would otherwise crowd the registers of every caller, tracked
-// transform or not).
+// transform or not).  A marked g (not finite) goes to FP64: its mark is no operand.
 static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, const int4* gp, int64_t gstride,
                                                         double2* __restrict__ Gf) {
+  if (gp[0].x == FX_G_NAN) {
+    accumulate_gauge_fp64(V, s, gp, gstride, Gf);
+    return;
+  }
   uint32_t m = 0, t = 0;
   FxC G[3][3];
 #pragma unroll
