@@ -46,11 +46,11 @@ __device__ __forceinline__ void gram_schmidt_factors(double a, double d, double2
 // coefficient k = <r1, r2>/|r1|^2 and i2 = 1/|w| with w = r2 - k r1, where
 // |w|^2 = |r2|^2 - |<r1, r2>|^2/|r1|^2 (Pythagoras for the projection) is
 // formed from the inputs, so that w itself is never needed in FP64: the
-// FP32 field applies k in FP32.  For 1 + X with X anti-Hermitian the rows are
-// nearly orthogonal (|<r1, r2>| <= |X|^2 while |r1|, |r2| >= 1), so the
-// difference does not cancel.  33 FP64 operations and two estimates, against
-// 43 when w is formed in FP64.  Taken by entries outside the range of the
-// FP32 pairs below.
+// FP32 field applies k in FP32.  The singular values of 1 + X, X anti-Hermitian,
+// are at least 1, so |w| >= 1 while |r2|^2 <= 1 + 5 max|X|^2: the difference
+// loses no bits for |X| < 1 and up to log2 of that ratio where large rows are
+// nearly dependent.  33 FP64 operations and two estimates, against 43 when w
+// is formed in FP64.  Taken by entries outside the range of the FP32 pairs below.
 struct GSFactors32 {
   double i1, i2, kx, ky;
 };
@@ -96,7 +96,10 @@ __device__ __forceinline__ float2 c_f64_to_f32_int(double2 v) { return make_floa
 // The same factors in FP32 pairs h + l (|l| <= ulp(h)/2: 48 bits) on the FP32
 // pipe, which has 64 times the FP64 rate: error-free products (FMA) and sums
 // (Knuth, The Art of Computer Programming 2, 4.2.2), about 200 FP32 operations.
-// Each factor is within 2^-35 of its exact value before it is rounded to FP32.
+// Each factor is within 2^-35 of its exact value before it is rounded to FP32:
+// for |X| <= GS_PAIR_MAX, over rows made to be nearly dependent, i1 within
+// 2^-44.7 and i2, whose difference cancels there, 2^-43.7 at |X| <= 1, 2^-37.7
+// at 8, 2^-35.6 at 16, 2^-33.2 at 32, 2^-20 at 4096.
 struct Pair32 {
   float h, l;
 };
@@ -128,8 +131,8 @@ __device__ __forceinline__ Pair32 pair_rsqrt(Pair32 n) {
 struct GSFactorsOut {
   float i1, i2, kx, ky;
 };
-// Entries beyond this, and NaN, take FP64 (squares of squares stay far from overflow below it).
-constexpr float GS_PAIR_MAX = 4096.f;
+// Entries beyond this, and NaN, take FP64.
+constexpr float GS_PAIR_MAX = 16.f;
 static __device__ __noinline__ GSFactorsOut gram_schmidt_fp64_call(float2 f0, float2 f1, float2 f2, float2 f3) {
   GSFactors32 o;
   gram_schmidt_factors_f32(f32_to_f64_int(f0.x), f32_to_f64_int(f0.y), c_f32_to_f64_int(f1), c_f32_to_f64_int(f2),
@@ -200,7 +203,7 @@ __device__ __forceinline__ void gauge_rows(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f
     u[0] = mkc<R>(i1, a * i1);
     u[1] = cscale<R>(f1, i1);
     u[2] = cscale<R>(f2, i1);
-    // w = r2 - k r1 in FP32, normalised by the FP64 factor
+    // w = r2 - k r1 in FP32
     const C2<R> w0 = mkc<R>(fmaf(ky, a, -f1.x - kx), fmaf(-kx, a, f1.y - ky));
     const C2<R> w1 = mkc<R>(fmaf(ky, f1.y, fmaf(-kx, f1.x, 1.f)), fmaf(-ky, f1.x, fmaf(-kx, f1.y, d)));
     const C2<R> w2 = mkc<R>(fmaf(ky, f2.y, fmaf(-kx, f2.x, f3.x)), fmaf(-ky, f2.x, fmaf(-kx, f2.y, f3.y)));

@@ -38,6 +38,23 @@ extern "C" int probe_accumulate(const double* rows, double* G) {
   cudaFree(d);
   return (int)e;
 }
+// factors (i1, i2, kx, ky) of n sites from X = (f0, f1, f2, f3)
+__global__ void factors(const float2* X, float4* out, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const GSFactorsOut o = gram_schmidt_pair(X[4 * i], X[4 * i + 1], X[4 * i + 2], X[4 * i + 3]);
+  out[i] = make_float4(o.i1, o.i2, o.kx, o.ky);
+}
+extern "C" int probe_factors(const float* X, float* out, int n) {
+  float2* d;
+  cudaMalloc(&d, (size_t)n * 48);
+  cudaMemcpy(d, X, (size_t)n * 32, cudaMemcpyHostToDevice);
+  float4* o = reinterpret_cast<float4*>(d + (size_t)4 * n);
+  factors<<<(n + 127) / 128, 128>>>(d, o, n);
+  const cudaError_t e = cudaMemcpy(out, o, (size_t)n * 16, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return (int)e;
+}
 """
 
 
@@ -75,3 +92,33 @@ def test_transform_of_a_finite_g(probe):
     want = g @ G
     assert probe.probe_accumulate(ptr(np.ascontiguousarray(g)), ptr(G)) == 0
     assert np.max(np.abs(G - want)) < 2e-15
+
+
+# ---------------------------------------------------------------------------
+# Gram-Schmidt factors of FP32 lanes on nearly dependent rows
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("A", [0.5, 4.0, 15.9, 16.1, 300.0, 4000.0])
+def test_factors_of_nearly_dependent_rows(probe, A):
+    """r1 = lambda r2 up to terms of order one, for entries up to A: i1 and i2 are the exact factors rounded once to
+    FP32 (2^-24) after an error of 2^-35 (pairs) or 2^-53 |r2|^2 / |w|^2 < 2^-26 (FP64, entries up to 4000)."""
+    n, rng = 20000, np.random.default_rng(5)
+    z = lambda: rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    lam = rng.uniform(0.2, 1, n) * np.exp(2j * np.pi * rng.uniform(0, 1, n))
+    lam[:n // 4] = np.exp(0.5j * np.pi * rng.integers(0, 4, n // 4))
+    d = A * rng.uniform(0.5, 1, n) * rng.choice([-1, 1], n)
+    f3 = A * rng.choice([0, 0.1, 0.7], n) * np.exp(2j * np.pi * rng.uniform(0, 1, n))
+    f1 = 1j * lam * d + rng.choice([0, 0.3], n) * z()
+    f2 = lam * f3 + rng.choice([0, 0.3], n) * z()
+    X = np.stack([np.abs(lam) ** 2 * d, d, f1.real, f1.imag, f2.real, f2.imag, f3.real, f3.imag], axis=1)
+    X = np.ascontiguousarray(np.clip(X, -A, A).astype(np.float32))
+    out = np.empty((n, 4), dtype=np.float32)
+    assert probe.probe_factors(ptr(X), ptr(out), n) == 0
+    a, d, f1, f2, f3 = (x.astype(np.clongdouble) for x in
+                        (X[:, 0], X[:, 1], X[:, 2] + 1j * X[:, 3].astype(np.clongdouble),
+                         X[:, 4] + 1j * X[:, 5].astype(np.clongdouble), X[:, 6] + 1j * X[:, 7].astype(np.clongdouble)))
+    r1, r2 = np.stack([1 + 1j * a, f1, f2]), np.stack([-np.conj(f1), 1 + 1j * d, f3])
+    n1 = np.sum(np.abs(r1) ** 2, axis=0)
+    w = r2 - np.sum(np.conj(r1) * r2, axis=0) / n1 * r1
+    for got, want in ((out[:, 0], 1 / np.sqrt(n1)), (out[:, 1], 1 / np.sqrt(np.sum(np.abs(w) ** 2, axis=0)))):
+        assert np.max(np.abs(got / want - 1)) < 1.25 * 2.0 ** -24
