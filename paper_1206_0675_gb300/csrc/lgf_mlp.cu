@@ -572,7 +572,21 @@ __global__ void __launch_bounds__(TTH, 2) mlp_grad_kernel(const float* __restric
       }
     }
     __syncthreads();
-    // a layer's gradient and dA of the layer below: D = (W^T dA) (H > 0)
+    // a layer's gradient: the 64 samples of a chunk in sums of their own, which
+    // are then added to those of the chunks before (one chain over all samples
+    // of a CTA would gather its rounding error with their number)
+    auto weight_grad = [&](const float* dA, const float* H, float (&g)[4][4]) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+      tile_abt(dA, H, r0, cx, acc);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[i][j] += acc[i][j];
+    };
+    // dA of the layer below: D = (W^T dA) (H > 0)
     auto backward = [&](const float* dA, const float* W, const float* H, float* Dn) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -588,11 +602,11 @@ __global__ void __launch_bounds__(TTH, 2) mlp_grad_kernel(const float* __restric
         st4(Dn + (r0 + i) * TS + c0, acc[i]);
       }
     };
-    tile_abt(S.H3, S.H2, r0, cx, g3);
+    weight_grad(S.H3, S.H2, g3);
     if (part == 2) gb += row_sum(S.H3 + sample * TS);
     backward(S.H3, S.W3, S.H2, S.D);
     __syncthreads();
-    tile_abt(S.D, S.H1, r0, cx, g2);
+    weight_grad(S.D, S.H1, g2);
     if (part == 1) gb += row_sum(S.D + sample * TS);
     backward(S.D, S.W2, S.H1, S.H3);
     __syncthreads();

@@ -1,5 +1,5 @@
-"""Fixed-point forms of the FP64 kernels at the ends of their range: values that
-are not finite, fields near the identity, nearly dependent rows, long lines."""
+"""Kernels at the ends of their range: values that are not finite, fields near
+the identity, nearly dependent rows, long lines, long sums."""
 
 import ctypes
 import subprocess
@@ -122,3 +122,26 @@ def test_factors_of_nearly_dependent_rows(probe, A):
     w = r2 - np.sum(np.conj(r1) * r2, axis=0) / n1 * r1
     for got, want in ((out[:, 0], 1 / np.sqrt(n1)), (out[:, 1], 1 / np.sqrt(np.sum(np.abs(w) ** 2, axis=0)))):
         assert np.max(np.abs(got / want - 1)) < 1.25 * 2.0 ** -24
+
+
+# ---------------------------------------------------------------------------
+# gradient of the network over many chunks of samples
+# ---------------------------------------------------------------------------
+
+def test_network_gradient_of_many_equal_samples():
+    """2^21 equal samples give the gradient of one.  Equal terms make every rounding of a sum push the same way: a
+    sum of 64 samples, of up to 108 chunks, of 38 CTAs and of 8 parts is off by at most half of 2^-24 per term."""
+    import torch
+    n, rng = 1 << 21, np.random.default_rng(3)
+    P = torch.from_numpy(np.ascontiguousarray(0.3 * rng.standard_normal(lgf.LGF_MLP_NPARAM), dtype=np.float32)).cuda()
+    x = torch.from_numpy(rng.uniform(0.5, 1.5, (1, 8)).astype(np.float32)).cuda()
+    grads = []
+    for m in (1, n):
+        X, Y, W = x.expand(m, 8).contiguous(), torch.full((m,), 0.7, device="cuda"), torch.ones(m, device="cuda")
+        g = torch.empty(lgf.LGF_MLP_NPARAM, device="cuda")
+        torch.cuda.synchronize()
+        lgf.lgf_mlp_loss_grad(P.data_ptr(), X.data_ptr(), Y.data_ptr(), W.data_ptr(), m, g.data_ptr())
+        grads.append(g.cpu().numpy().astype(np.float64))
+    one, many = grads
+    assert np.count_nonzero(one) > 1000
+    assert np.all(np.abs(many - one) <= 0.5 * (64 + 108 + 38 + 8) * 2.0 ** -24 * np.abs(one))
