@@ -641,35 +641,40 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   return cudaSuccess;
 }
 
-// Candidate plans for the autotuner: every fields-per-CTA count of the (x,y)
-// passes, every x-column count of the (z,t) pass that fits shared memory,
-// and three CTA sizes (8, 16 or 32 elements per thread) for each.
+// Candidate plans for the autotuner: the built-in plan, then every
+// fields-per-CTA count of the (x,y) passes, every x-column count of the (z,t)
+// pass that fits shared memory, and three CTA sizes (8, 16 or 32 elements per
+// thread) for each, within the limits of configure_fft_plan.
 void fft_plan_candidates(const int L[4], int real_bytes, std::vector<FFTPlan>& out) {
   FFTPlan base;
   out.clear();
   if (configure_fft_plan(L, real_bytes, &base) != cudaSuccess) return;
+  out.push_back(base);
+  const TuneChoice built_in = tune_choice_of(base, FFT_2D2D);
   const size_t maxsm = 220 * 1024;
   const int Lx = L[0], Ly = L[1], Lz = L[2], Lt = L[3];
   for (int fpb = 1; fpb <= 4; fpb *= 2) {
     if (xy_smem(L, real_bytes, fpb) > maxsm) continue;
     for (int xc = 1; xc <= 8; xc *= 2) {
-      if (Lx % xc || zt_smem(L, real_bytes, xc) > maxsm) continue;
+      const size_t zt = Lx % xc ? 0 : zt_smem(L, real_bytes, xc);
+      if (zt == 0 || zt > (pairs_zt(real_bytes, xc) ? PLANE_SMEM_MAX : maxsm)) continue;
+      const int most = real_bytes == 8 ? FX_MAX_THREADS : PAIR_MAX_THREADS;
+      const int most_zt = pairs_zt(real_bytes, xc) && zt > PLANE_SMEM_MAX / 2 ? PAIR_ZT_THREADS : most;
       for (int tdiv = 8; tdiv <= 32; tdiv *= 2) {
         FFTPlan p = base;
         p.fpb_xy = fpb;
         p.smem_xy = xy_smem(L, real_bytes, fpb);
         p.xc = xc;
-        p.smem_zt = zt_smem(L, real_bytes, xc);
-        const int most = real_bytes == 8 ? FX_MAX_THREADS : PAIR_MAX_THREADS;
-        auto thr = [&](int points) {
+        p.smem_zt = zt;
+        auto thr = [&](int points, int limit) {
           int t = (points + tdiv - 1) / tdiv;
           t = ((t + 31) / 32) * 32;
-          return std::max(64, std::min(most, t));
+          return std::max(64, std::min(limit, t));
         };
-        p.threads_xy = thr(fpb * Lx * Ly);
-        p.threads_zt = thr(Lz * Lt * xc);
-        p.threads_c = real_bytes == 8 && tdiv == 8 ? base.threads_c : thr(4 * Lx * Ly);
-        out.push_back(p);
+        p.threads_xy = thr(fpb * Lx * Ly, most);
+        p.threads_zt = thr(Lz * Lt * xc, most_zt);
+        p.threads_c = real_bytes == 8 && tdiv == 8 ? base.threads_c : thr(4 * Lx * Ly, most);
+        if (!tune_choice_matches(p, built_in)) out.push_back(p);
       }
     }
   }

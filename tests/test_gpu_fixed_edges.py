@@ -145,3 +145,21 @@ def test_network_gradient_of_many_equal_samples():
     one, many = grads
     assert np.count_nonzero(one) > 1000
     assert np.all(np.abs(many - one) <= 0.5 * (64 + 108 + 38 + 8) * 2.0 ** -24 * np.abs(one))
+
+
+# ---------------------------------------------------------------------------
+# plans
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("ext, xc, threads", [((4, 2, 48, 96), 4, 768), ((2, 2, 128, 108), 2, 384),
+                                              ((8, 12, 8, 6), 8, 64)])
+def test_autotune_times_the_built_in_plan(ext, xc, threads):
+    """The first trial is the plan an untuned handle runs: four x columns in one CTA that fills an SM, one tile
+    between 220 and 227 KB, and an ordinary lattice."""
+    with lgf.Lattice(ext, "fp32") as lat:
+        lat.set_links(fields.random_links(ext, 0.8, seed=2))
+        rep = lat.autotune()["fp32"]
+    first = rep["candidates"][0]
+    assert first["decomposition"] == "2d2d"
+    assert (first["x_columns_zt"], first["threads"][1]) == (xc, threads)
+    assert rep["candidates"][rep["chosen"]]["ms"] <= first["ms"]
