@@ -227,7 +227,7 @@ template <typename R> lgf_status alloc_lane(lgf_ctx* h, Lane<R>& L, int rows, in
     return fail(h, LGF_E_UNSUPPORTED, "lattice planes do not fit the shared-memory FFT passes");
   // twiddles W_N^m = exp(-2 pi i m/N), computed in FP64 on the host
   std::vector<double2> tw64;
-  fft_twiddles(h->geom.L, tw64);
+  fft_twiddles(h->geom.L, f64, tw64);
   std::vector<C2<R>> tw(f64 ? 2 * nt : nt);
   for (size_t m = 0; m < tw.size(); ++m) tw[m] = mkc<R>((R)tw64[m].x, (R)tw64[m].y);
   LGF_CK(h, cudaMemcpyAsync(L.tw, f64 ? (const void*)tw64.data() : (const void*)tw.data(),

@@ -192,7 +192,7 @@ lgf_status setup_class(lgf_batch_ctx* b, ClassLane& C) {
     return bfail(b, LGF_E_UNSUPPORTED, "lattice planes do not fit the shared-memory FFT passes");
   std::vector<double2> tw;
   std::vector<short> pos(nt);
-  fft_twiddles(g.L, tw);
+  fft_twiddles(g.L, true, tw);
   fft_positions(C.plan, pos.data());
   LGF_BCK(b, cudaMemcpyAsync(C.tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice, b->stream));
   LGF_BCK(b, cudaMemcpyAsync(C.pos, pos.data(), nt * sizeof(short), cudaMemcpyHostToDevice, b->stream));

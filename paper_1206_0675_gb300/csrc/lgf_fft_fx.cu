@@ -42,6 +42,7 @@
 #include "lgf_fixed.cuh"
 #include "lgf_gauge.cuh"
 #include "lgf_internal.h"
+#include "lgf_roots.h"
 
 namespace lgf {
 
@@ -603,26 +604,16 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
 // launchers
 // ---------------------------------------------------------------------------
 
-void fft_twiddles(const int L[4], std::vector<double2>& tw) {
+void fft_twiddles(const int L[4], bool fixed, std::vector<double2>& tw) {
   const int nt = L[0] + L[1] + L[2] + L[3];
-  tw.resize((size_t)2 * nt);
-  int4* fx = reinterpret_cast<int4*>(tw.data() + nt);
-  const long double two_pi = 6.283185307179586476925286766559005768L;
+  tw.resize((size_t)(fixed ? 2 * nt : nt));
   int off = 0;
   for (int mu = 0; mu < 4; ++mu) {
     for (int m = 0; m < L[mu]; ++m) {
       const double a = -2.0 * M_PI * (double)m / (double)L[mu];
       tw[off + m] = make_double2(std::cos(a), std::sin(a));
-      const long double b = -two_pi * (long double)m / (long double)L[mu];
-      const long double c[2] = {std::cos(b), std::sin(b)};
-      int hl[4];
-      for (int k = 0; k < 2; ++k) {
-        const long double h = std::round(c[k] * 1073741824.0L);
-        hl[2 * k] = (int)h;
-        hl[2 * k + 1] = (int)std::round((c[k] * 1073741824.0L - h) * 1073741824.0L);
-      }
-      fx[off + m] = make_int4(hl[0], hl[1], hl[2], hl[3]);
     }
+    if (fixed) fixed_roots(L[mu], reinterpret_cast<int*>(tw.data() + nt + off));
     off += L[mu];
   }
 }

@@ -309,10 +309,10 @@ cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, con
 cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
                                    const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
                                    bool exact_exp);
-// The FP64 twiddle table of a lattice: L[0] + ... + L[3] roots in FP64, then
-// the same roots as fixed-point limbs (int4: cosine and sine, each h 2^-30 +
-// l 2^-60) in the same order.
-void fft_twiddles(const int L[4], std::vector<double2>& tw);
+// The twiddle table of a lattice: L[0] + ... + L[3] roots in FP64 and, for FP64
+// lanes (fixed), the same roots as fixed-point limbs (int4: cosine and sine, each
+// h 2^-30 + l 2^-60) in the same order.
+void fft_twiddles(const int L[4], bool fixed, std::vector<double2>& tw);
 
 // ---- lgf_fft_pair.cu -----------------------------------------------------
 // The plane passes of FP32 fields on pairs of fields (x, y: fpb even) or of
