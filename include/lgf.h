@@ -24,7 +24,12 @@
  *   history buffers registered with lgf_set_trace.  The library owns its
  *   device workspace (allocated in lgf_create, freed in lgf_destroy), taken
  *   from CUDA's stream-ordered allocator or from a caller-supplied allocator
- *   (lgf_create_with_allocator).
+ *   (lgf_create_with_allocator).  The network functions (lgf_mlp_loss_grad,
+ *   lgf_mlp_train) take no handle: their scratch comes from a memory pool of
+ *   the library, one per device and process, safe with several threads and
+ *   streams.  It keeps up to 64 MB between calls, which lgf_destroy and
+ *   lgf_batch_destroy of any handle on the device give back, and otherwise the
+ *   end of the process.
  * Streams: all device work of a handle runs on the stream given to
  *   lgf_create (NULL = the legacy default stream), except that lgf_set_links
  *   from host memory checks the copied pieces on a second, internal stream

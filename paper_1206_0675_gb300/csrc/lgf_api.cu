@@ -8,7 +8,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
-#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -722,43 +721,51 @@ template <typename R> lgf_status step_lane(lgf_ctx* h, Lane<R>& L, double alpha)
 // system then, and the next call's kernels waited for it to be mapped again).
 // Four blocks of the default pool were 200 of the 340 us that lgf_mlp_loss_grad of
 // 65536 samples took; it takes 138 us (64 samples: 253 -> 47 us).  lgf_destroy
-// gives back what is kept.  Where the pool cannot be had the block comes from
+// and lgf_batch_destroy give back what is kept.  Where the pool cannot be had the block comes from
 // the default pool.
 constexpr uint64_t MLP_POOL_KEEP = 64u << 20;  // the pool grows by 32 MB at a time
+constexpr int MLP_POOL_DEVICES = 64;            // devices beyond these use the default pool
 std::mutex g_mlp_pool_mutex;
-std::map<int, cudaMemPool_t> g_mlp_pools;
+cudaMemPool_t g_mlp_pools[MLP_POOL_DEVICES];  // a plain array: nothing here throws through the C entries
 
 cudaError_t mlp_malloc(void** p, size_t bytes, cudaStream_t s) {
   int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) {
+  if (cudaGetDevice(&dev) == cudaSuccess && dev < MLP_POOL_DEVICES) {
     std::lock_guard<std::mutex> lock(g_mlp_pool_mutex);
-    auto it = g_mlp_pools.find(dev);
-    if (it == g_mlp_pools.end()) {
+    cudaMemPool_t& pool = g_mlp_pools[dev];
+    if (!pool) {
       cudaMemPoolProps props{};
       props.allocType = cudaMemAllocationTypePinned;
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
-      cudaMemPool_t pool = nullptr;
       uint64_t keep = MLP_POOL_KEEP;
-      if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
-          cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
-        it = g_mlp_pools.emplace(dev, pool).first;
+      if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        pool = nullptr;
+      } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        pool = nullptr;
+      }
     }
-    if (it != g_mlp_pools.end()) {
-      const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, it->second, s);
+    if (pool) {
+      const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
       if (e == cudaSuccess || e == cudaErrorMemoryAllocation) return e;
-      g_mlp_pools.erase(it);  // the device was reset
+      pool = nullptr;  // the device was reset, and the pool with it
     }
     cudaGetLastError();
   }
   return cudaMallocAsync(p, bytes, s);
 }
 
-void mlp_pool_trim(int dev) {
+}  // namespace
+
+// Gives back what the pool of the network functions keeps on a device.
+void lgf::mlp_pool_trim(int dev) {
+  if (dev < 0 || dev >= MLP_POOL_DEVICES) return;
   std::lock_guard<std::mutex> lock(g_mlp_pool_mutex);
-  auto it = g_mlp_pools.find(dev);
-  if (it != g_mlp_pools.end() && cudaMemPoolTrimTo(it->second, 0) != cudaSuccess) cudaGetLastError();
+  if (g_mlp_pools[dev] && cudaMemPoolTrimTo(g_mlp_pools[dev], 0) != cudaSuccess) cudaGetLastError();
 }
+
+namespace {
 
 struct MlpScratch {
   float* part_g = nullptr;

@@ -307,6 +307,7 @@ lgf_status lgf_batch_destroy(lgf_batch b) {
   cudaStreamSynchronize(b->stream);
   if (b->st_host) cudaFreeHost(b->st_host);
   if (b->defect_host) cudaFreeHost(b->defect_host);
+  mlp_pool_trim(b->device);
   delete b;
   return LGF_OK;
 }

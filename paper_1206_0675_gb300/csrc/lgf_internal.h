@@ -191,6 +191,10 @@ template <typename R, int ROWS>
 cudaError_t launch_or_half_sweep(const Geom& g, C2<R>* U0, C2<R>* U1, const DevState* st, C2<R>* gfield, C2<R>* G,
                                  int parity, double omega, cudaStream_t s);
 
+// ---- lgf_api.cu ---------------------------------------------------------
+// Gives back the device memory that the network functions' pool keeps.
+void mlp_pool_trim(int dev);
+
 // ---- lgf_fft.cu ---------------------------------------------------------
 // Radix schedule of one lattice direction.
 struct FFTDir {

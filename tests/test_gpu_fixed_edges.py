@@ -163,3 +163,27 @@ def test_autotune_times_the_built_in_plan(ext, xc, threads):
     assert first["decomposition"] == "2d2d"
     assert (first["x_columns_zt"], first["threads"][1]) == (xc, threads)
     assert rep["candidates"][rep["chosen"]]["ms"] <= first["ms"]
+
+
+# ---------------------------------------------------------------------------
+# scratch of the network functions
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("make", [lambda: lgf.Lattice((4, 4, 4, 4), "fp64"), lambda: lgf.Batch([(4, 4, 4, 4)])])
+def test_closing_a_handle_gives_back_the_network_scratch(make):
+    import torch
+    n, dev = 4096, "cuda"
+    P, X = torch.zeros(lgf.LGF_MLP_NPARAM, device=dev), torch.ones(n, 8, device=dev)
+    Y, W, g = torch.zeros(n, device=dev), torch.ones(n, device=dev), torch.empty(lgf.LGF_MLP_NPARAM, device=dev)
+    torch.cuda.synchronize()
+    args = [t.data_ptr() for t in (P, X, Y, W)] + [n, g.data_ptr()]
+    lgf.lgf_mlp_loss_grad(*args)  # its code is loaded
+    with lgf.Batch([(4, 4, 4, 4)]):
+        pass
+    lgf.Lattice((4, 4, 4, 4), "fp64").close()
+    before = torch.cuda.mem_get_info()[0]
+    lgf.lgf_mlp_loss_grad(*args)
+    kept = before - torch.cuda.mem_get_info()[0]
+    assert 0 < kept <= 64 << 20
+    make().close()
+    assert torch.cuda.mem_get_info()[0] == before
