@@ -11,8 +11,8 @@
 // into CTAs.  A transform of length N is safe from overflow when components
 // enter below 2^(61 - h), h = ceil(log2 N) + 1: a sum of N complex terms stays
 // below sqrt(2) N 2^(61 - h) <= 2^60.5 in modulus, within the 31-bit upper limb
-// of bfp_limbs.  Between the two directions of a plane the largest component
-// is measured again and the plane shifted right by what the next direction
+// of bfp_limbs.  Between the two directions of a plane, and within one of more
+// than 64 elements, the largest component is measured again and the plane shifted right by what the next direction
 // needs (about half of h for data without structure, so some 55 bits remain
 // below the largest component; an FP64 pass keeps 53 bits in each number and
 // rounds at every operation, where additions are exact here).  Inputs are
@@ -22,10 +22,9 @@
 // inverse, random, smooth and constant inputs) 0.7e-16 to 2.8e-16, of the passes
 // on the FP64 pipe 1.5e-16 to 4.6e-16; of g(x), where the filter weights the
 // lowest modes most (rms): planes of 16 x 16 0.7e-16 (1.1e-16), 32 x 32 1.2e-16
-// (1.9e-16), 48 x 48 2.1e-16 (3.0e-16), 64 x 64 5.1e-16 (7.0e-16), 128 x 2 with
-// 96 x 2 1.2e-15 (1.2e-15), 81 x 81 1.6e-15 (0.9e-15).  For that every rounding
-// is centred: inputs are rounded, halves go to even, and products carry the mean
-// of what they drop.
+// (1.9e-16), 48 x 48 2.1e-16 (3.0e-16), 64 x 64 5.1e-16 (7.0e-16); longer lines at
+// FxCut.  For that every rounding is centred: inputs are rounded, halves go to
+// even, and products carry the mean of what they drop.
 //
 // 32^4, us: pass A 74 (FP64 pipe: 231), pass B 165 (463), pass C with g 113 (397);
 // 24x18x12x27: 24, 41, 33 (54, 94, 78).  Bound by instruction issue (about 400
@@ -48,12 +47,15 @@ namespace lgf {
 
 using I2 = longlong2;
 
-// Per-plane exponents of the (at most 8) planes of a tile: the largest input
-// component (high word of its magnitude) and the bits of the largest
-// component between the directions (high word, or-ed), for the two transforms
-// a pass can hold.
-struct FxPlanes {
-  uint32_t in0[8], mid0[8], in1[8], mid1[8];
+// Per-plane exponents of the (at most 8) planes of a tile, for one transform:
+// the largest input component (high word of its magnitude, then the words of
+// fx_classify and fx_finish) and, where the plane is measured again (FxCut),
+// the bits of its largest component (high word, or-ed).
+struct FxTransform {
+  uint32_t in[8], mid[3][8];
+};
+struct FxPlanes {  // a pass holds up to two transforms
+  FxTransform t[2];
 };
 static_assert(sizeof(FxPlanes) == FX_PLANE_BYTES, "header of the FP64 plane passes");
 
@@ -80,30 +82,57 @@ __device__ __forceinline__ uint32_t fx_mid_shift(uint32_t mid, uint32_t h1) {
   return (uint32_t)max(sh, 0);
 }
 
+// Where the stages of a direction are cut in two, so that the plane is
+// measured, and shifted by no more than it needs, between them as well: lines
+// of more than 64, whose 8 bits of headroom leave 53 for the largest
+// component.  Cut, they enter with 56 or more.  The radices are 8|9, 9|9, 8|12,
+// 12|9 and 8|16 for 72 to 128 (decimation in time; in frequency the reverse).
+// g(x) of one step, rms in 1e-16, uncut -> cut (passes on the FP64 pipe): planes
+// of 72 x 72 10.5 -> 3.1 (8.0), 81 x 81 16.5 -> 5.1 (9.3), 96 x 72 13.7 -> 5.5
+// (11.9), 128 x 54 15.2 -> 9.5 (14.7), (z, t) planes of 128 x 81 11.9 -> 5.8 (9.6).
+constexpr int FX_CUT_ABOVE = 64;
+struct FxCut {
+  int first;        // stages before the cut (all of them where there is none)
+  uint32_t h0, h1;  // headroom of the two parts
+};
+template <bool DIT> __device__ __forceinline__ FxCut fx_cut(const FFTDir& d) {
+  if (d.N <= FX_CUT_ABOVE) return FxCut{d.nst, fx_headroom(d.N), 0u};
+  const int q = (int)d.ns[d.nst - 2].d;  // the product of all radices but the last two
+  const uint32_t ha = fx_headroom(q), hb = fx_headroom(d.N / q);
+  return DIT ? FxCut{d.nst - 2, ha, hb} : FxCut{2, hb, ha};
+}
+
 __device__ __forceinline__ I2 fx_in(double2 v, uint32_t base) {
   return make_longlong2(bfp_from(v.x, base), bfp_from(v.y, base));
 }
 
-// Exponent of a plane's integers after both directions (of the scaled plane).
-__device__ __forceinline__ int fx_out_exp(uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
-  return (int)(fx_mid_shift(mid, h1) + h0 + fx_exp_of(code)) - 1083;
+// The word of a plane after its transform: the exponent of its integers (of the
+// scaled plane) and the class of fx_classify.  c0 and c1 are the cuts of its two
+// directions; a part that is not there has no shift.
+__device__ __forceinline__ uint32_t fx_finish(const FxTransform* t, int pl, const FxCut& c0, const FxCut& c1) {
+  const uint32_t code = t->in[pl];
+  uint32_t sh = fx_mid_shift(t->mid[1][pl], c1.h0);
+  if (c0.h1 != 0u) sh += fx_mid_shift(t->mid[0][pl], c0.h1);
+  if (c1.h1 != 0u) sh += fx_mid_shift(t->mid[2][pl], c1.h1);
+  return (code & 0xffff0000u) | (sh + c0.h0 + fx_exp_of(code) - 1083u + 4096u);
 }
-// The same of the plane as it was, large where it holds infinities or NaN.
-__device__ __forceinline__ int fx_true_exp(uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
-  const int ex = fx_out_exp(code, mid, h0, h1);
-  const uint32_t k = code >> 16;
+__device__ __forceinline__ int fx_out_exp(uint32_t word) { return (int)(word & 0xffffu) - 4096; }
+// The exponent of the plane as it was, large where it holds infinities or NaN.
+__device__ __forceinline__ int fx_true_exp(uint32_t word) {
+  const int ex = fx_out_exp(word);
+  const uint32_t k = word >> 16;
   return k == 0u ? ex : k == FX_UP ? ex - FX_ODD_SCALE : k == FX_DOWN ? ex + FX_ODD_SCALE : 4096;
 }
 // Output of a plane after both directions.
-__device__ __forceinline__ double2 fx_out(I2 v, uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
-  const int ex = fx_out_exp(code, mid, h0, h1);
+__device__ __forceinline__ double2 fx_out(I2 v, uint32_t word) {
+  const int ex = fx_out_exp(word);
   return make_double2(bfp_to_double(v.x, ex), bfp_to_double(v.y, ex));
 }
 // The same for any plane.
-static __device__ __noinline__ double2 fx_out_any(I2 v, uint32_t code, uint32_t mid, uint32_t h0, uint32_t h1) {
-  if (code >> 16 == FX_NONFINITE) return make_double2(NAN, NAN);
-  const double2 r = fx_out(v, code, mid, h0, h1);
-  const int k = code >> 16 == FX_UP ? -FX_ODD_SCALE : code >> 16 == FX_DOWN ? FX_ODD_SCALE : 0;
+static __device__ __noinline__ double2 fx_out_any(I2 v, uint32_t word) {
+  if (word >> 16 == FX_NONFINITE) return make_double2(NAN, NAN);
+  const double2 r = fx_out(v, word);
+  const int k = word >> 16 == FX_UP ? -FX_ODD_SCALE : word >> 16 == FX_DOWN ? FX_ODD_SCALE : 0;
   return make_double2(scalbn(r.x, k), scalbn(r.y, k));
 }
 
@@ -120,14 +149,10 @@ __device__ __forceinline__ int64_t fx_unit58(int64_t v, int ex, bool& ok) {
 }
 
 struct FxOut {
-  __device__ __forceinline__ double2 operator()(I2 v, uint32_t c, uint32_t m, uint32_t h0, uint32_t h1) const {
-    return fx_out(v, c, m, h0, h1);
-  }
+  __device__ __forceinline__ double2 operator()(I2 v, uint32_t word) const { return fx_out(v, word); }
 };
 struct FxOutAny {
-  __device__ __forceinline__ double2 operator()(I2 v, uint32_t c, uint32_t m, uint32_t h0, uint32_t h1) const {
-    return fx_out_any(v, c, m, h0, h1);
-  }
+  __device__ __forceinline__ double2 operator()(I2 v, uint32_t word) const { return fx_out_any(v, word); }
 };
 
 __device__ __forceinline__ I2 iadd(I2 a, I2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
@@ -214,10 +239,11 @@ template <int SIGN> struct IDFT<8, SIGN> {
 
 // How a direction's first stage takes its input and its last leaves it.
 struct FxStageIO {
-  const uint32_t* in = nullptr;     // raw FP64 input: largest component per plane
-  const uint32_t* shift = nullptr;  // integers to be shifted: measured bits per plane
-  uint32_t* mid = nullptr;          // record the bits of the outputs per plane
-  uint32_t h = 0;                   // headroom of this direction
+  FxTransform* t;
+  uint32_t h;     // headroom of this part of the direction
+  bool raw;       // raw FP64 input, scaled by t->in
+  int shift;      // >= 0: integers to be shifted by what t->mid[shift] measured
+  int mid;        // >= 0: record the bits of the outputs in t->mid[mid]
 };
 
 // One stage, as ct_stage of lgf_fft.cu.  The plane of line l is l / inner
@@ -237,16 +263,16 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
     const int base = lo * ln.outer_stride + li * ln.inner_stride + (grp * Ns * RAD + j) * ln.es;
     const int step = Ns * ln.es;
     I2 v[RAD];
-    if (io.in != nullptr) {
+    if (io.raw) {
       const double2* raw = reinterpret_cast<const double2*>(tile);
-      const uint32_t sc = 3u + io.h + fx_exp_of(io.in[pl]);
+      const uint32_t sc = 3u + io.h + fx_exp_of(io.t->in[pl]);
 #pragma unroll
       for (int r = 0; r < RAD; ++r) v[r] = fx_in(raw[base + r * step], sc);
     } else {
 #pragma unroll
       for (int r = 0; r < RAD; ++r) v[r] = tile[base + r * step];
-      if (io.shift != nullptr) {
-        const uint32_t sh = fx_mid_shift(io.shift[pl], io.h);
+      if (io.shift >= 0) {
+        const uint32_t sh = fx_mid_shift(io.t->mid[io.shift][pl], io.h);
         if (sh != 0u) {
 #pragma unroll
           for (int r = 0; r < RAD; ++r) v[r] = make_longlong2(ishift(v[r].x, sh), ishift(v[r].y, sh));
@@ -264,7 +290,8 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
     }
 #pragma unroll
     for (int r = 0; r < RAD; ++r) tile[base + r * step] = v[r];
-    if (io.mid != nullptr) {
+    if (io.mid >= 0) {
+      uint32_t* mid = io.t->mid[io.mid];
       uint32_t m = 0;
 #pragma unroll
       for (int r = 0; r < RAD; ++r) {
@@ -277,12 +304,12 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
         const int lead = __ffs((int)act) - 1;
         if (__all_sync(act, pl == __shfl_sync(act, pl, lead))) {
           m = __reduce_or_sync(act, m);
-          if ((int)(threadIdx.x & 31) == lead) atomicOr(&io.mid[pl], m);
+          if ((int)(threadIdx.x & 31) == lead) atomicOr(&mid[pl], m);
         } else {
-          atomicOr(&io.mid[pl], m);
+          atomicOr(&mid[pl], m);
         }
       } else {
-        atomicOr(&io.mid[pl], m);
+        atomicOr(&mid[pl], m);
       }
     }
   }
@@ -300,27 +327,41 @@ struct FxPass {
 // then the other; DIT takes digit-reversed input and gives natural order, DIF
 // the reverse.  One loop over the directions: the stages of a radix are the
 // same code for both (the instruction cache held neither copy otherwise).
+// Leaves the word of each plane (fx_finish) in t->in; ends with a __syncthreads.
 template <int SIGN, bool DIT, bool PLO>
-__device__ __forceinline__ void fx_plane(I2* tile, const FxPass& P, const int4* tw, int first, const uint32_t* in,
-                                         uint32_t* mid) {
+__device__ __forceinline__ void fx_plane(I2* tile, const FxPass& P, const int4* tw, int first, int nplanes,
+                                         FxTransform* t) {
 #pragma unroll 1
   for (int k = 0; k < 2; ++k) {
     const int ax = first ^ k;
     const FFTDir& d = P.d[ax];
     const Lines& ln = P.l[ax];
     const int4* w = ax == 0 ? tw : tw + P.d[0].N;
+    const FxCut cut = fx_cut<DIT>(d);
     FxStageIO s;
-    s.h = fx_headroom(d.N);
+    s.t = t;
+    s.h = cut.h0;
+    s.raw = k == 0;
+    s.shift = k == 0 ? -1 : 1;
 #pragma unroll 1
     for (int i = 0; i < d.nst; ++i) {
       const int st = DIT ? i : d.nst - 1 - i;
-      s.in = k == 0 && i == 0 ? in : nullptr;
-      s.shift = k == 1 && i == 0 ? mid : nullptr;
-      s.mid = k == 0 && i == d.nst - 1 ? mid : nullptr;
+      s.mid = -1;
+      if (i == d.nst - 1) s.mid = k == 0 ? 1 : -1;
+      else if (i == cut.first - 1) s.mid = 2 * k;
+      // every measurement is complete before the last stage
+      if (k == 1 && i == d.nst - 1 && (int)threadIdx.x < nplanes)
+        t->in[threadIdx.x] = fx_finish(t, threadIdx.x, fx_cut<DIT>(P.d[first]), cut);
       if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
       else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
       else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
       else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
+      s.raw = false;
+      s.shift = -1;
+      if (i == cut.first - 1) {
+        s.shift = 2 * k;
+        s.h = cut.h1;
+      }
     }
   }
 }
@@ -418,20 +459,19 @@ __global__ void __launch_bounds__(FX_MAX_THREADS, 2) fft_xy_fx_kernel(Geom g, co
     return f * PS + pos[Lx + y] * RS + pos[x];
   };
   fx_load(
-      tile, n, ps->in0,
+      tile, n, ps->t[0].in,
       [&](int i) {
         const int f = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)f * g.V + (i - f * plane)];
       },
       dst);
   __syncthreads();
-  const bool odd = fx_prepare(tile, n, fpb, ps->in0, dst);
-  const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
-  fx_plane<SIGN, true, true>(tile, P, tw, 0, ps->in0, ps->mid0);
+  const bool odd = fx_prepare(tile, n, fpb, ps->t[0].in, dst);
+  fx_plane<SIGN, true, true>(tile, P, tw, 0, fpb, &ps->t[0]);
   auto out = [&](auto convert) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
-      fld[(int64_t)f * g.V + r] = convert(tile[f * PS + y * RS + x], ps->in0[f], ps->mid0[f], hx, hy);
+      fld[(int64_t)f * g.V + r] = convert(tile[f * PS + y * RS + x], ps->t[0].in[f]);
     }
   };
   if (!odd) out(FxOut());
@@ -469,21 +509,20 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
     return pos[Lz + t] * TS + pos[z] * xc + xi;
   };
   fx_load(
-      tile, n, ps->in0,
+      tile, n, ps->t[0].in,
       [&](int i) {
         const int zt = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)zt * plane + sxy + (i - zt * xc)];
       },
       dst);
   __syncthreads();
-  const uint32_t hz = fx_headroom(Lz), ht = fx_headroom(Lt);
-  bool odd = fx_prepare(tile, n, xc, ps->in0, dst);
-  fx_plane<(MODE > 0 ? +1 : -1), true, false>(tile, P, tw, 0, ps->in0, ps->mid0);
+  bool odd = fx_prepare(tile, n, xc, ps->t[0].in, dst);
+  fx_plane<(MODE > 0 ? +1 : -1), true, false>(tile, P, tw, 0, xc, &ps->t[0]);
   if (MODE != 0) {
     auto out = [&](auto convert) {
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
         LGF_ZT_IDX(i)
-        fld[(int64_t)zt * plane + sxy + xi] = convert(tile[t * TS + z * xc + xi], ps->in0[xi], ps->mid0[xi], hz, ht);
+        fld[(int64_t)zt * plane + sxy + xi] = convert(tile[t * TS + z * xc + xi], ps->t[0].in[xi]);
       }
     };
     if (!odd) out(FxOut());
@@ -499,7 +538,7 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
     const float* mtab = lio.mtab + (int64_t)(kit & 1) * lio.nclass;
     uint32_t* snap = (LRN && lio.snap != nullptr) ? lio.snap + ((int64_t)(kit & 1) * 4 + blockIdx.y) * g.V : nullptr;
     const int fy = min(y, Ly - y);
-    const uint32_t in = ps->in0[col], mid = ps->mid0[col];
+    const uint32_t word = ps->t[0].in[col];
     uint32_t m = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       LGF_ZT_IDX(i)
@@ -510,28 +549,28 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
         k *= (double)__ldg(&mtab[((ft * H.z + fz) * H.y + fy) * H.x + fx]);
       }
       double2* e = reinterpret_cast<double2*>(&tile[t * TS + z * xc + xi]);
-      const double2 v = convert(*reinterpret_cast<const I2*>(e), in, mid, hz, ht);
+      const double2 v = convert(*reinterpret_cast<const I2*>(e), word);
       if (LRN && snap != nullptr) snap[(int64_t)zt * plane + sxy + xi] = bf16x2_of<double>(v);
       const double2 w = make_double2(v.x * k, v.y * k);
       m = fx_max(m, w);
       *e = w;
     }
-    atomicMax(&ps->in1[col], m);
+    atomicMax(&ps->t[1].in[col], m);
   };
   if (!odd) filter(FxOut());
   else filter(FxOutAny());
   __syncthreads();
-  odd = fx_prepare(tile, n, xc, ps->in1, [&](int i, int& pl) {
+  odd = fx_prepare(tile, n, xc, ps->t[1].in, [&](int i, int& pl) {
     LGF_ZT_IDX(i)
     pl = xi;
     return t * TS + z * xc + xi;
   });
-  fx_plane<+1, false, false>(tile, P, tw, 1, ps->in1, ps->mid1);
+  fx_plane<+1, false, false>(tile, P, tw, 1, xc, &ps->t[1]);
   auto out = [&](auto convert) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       LGF_ZT_IDX(i)
       fld[(int64_t)zt * plane + sxy + xi] =
-          convert(tile[pos[Lz + t] * TS + pos[z] * xc + xi], ps->in1[xi], ps->mid1[xi], ht, hz);
+          convert(tile[pos[Lz + t] * TS + pos[z] * xc + xi], ps->t[1].in[xi]);
     }
   };
   if (!odd) out(FxOut());
@@ -564,16 +603,15 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
     return f * PS + y * RS + x;
   };
   fx_load(
-      tile, 4 * plane, ps->in0,
+      tile, 4 * plane, ps->t[0].in,
       [&](int i) {
         const int f = (int)cd.a.div((uint32_t)i);
         return &fld[(int64_t)f * g.V + (i - f * plane)];
       },
       dst);
   __syncthreads();
-  fx_prepare(tile, 4 * plane, 4, ps->in0, dst);
-  const uint32_t hx = fx_headroom(Lx), hy = fx_headroom(Ly);
-  fx_plane<+1, false, true>(tile, P, tw, 0, ps->in0, ps->mid0);
+  fx_prepare(tile, 4 * plane, 4, ps->t[0].in, dst);
+  fx_plane<+1, false, true>(tile, P, tw, 0, 4, &ps->t[0]);
   for (int i = threadIdx.x; i < plane; i += blockDim.x) {
     const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
     const int o = pos[Lx + y] * RS + pos[x];
@@ -584,7 +622,7 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const I2 v = tile[k * PS + o];
-        const int ex = fx_true_exp(ps->in0[k], ps->mid0[k], hx, hy);
+        const int ex = fx_true_exp(ps->t[0].in[k]);
         A[2 * k] = fx_unit58(v.x, ex, ok);
         A[2 * k + 1] = fx_unit58(v.y, ex, ok);
       }
@@ -595,7 +633,7 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
     }
     double2 f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) f[k] = fx_out_any(tile[k * PS + o], ps->in0[k], ps->mid0[k], hx, hy);
+    for (int k = 0; k < 4; ++k) f[k] = fx_out_any(tile[k * PS + o], ps->t[0].in[k]);
     gauge_site_fp64<EXPG>(f[0], f[1], f[2], f[3], g.V, s, gf, Gf);
   }
 }

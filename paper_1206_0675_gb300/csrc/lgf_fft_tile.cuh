@@ -40,7 +40,7 @@ template <typename R> __host__ __device__ inline size_t smem_header_bytes(int n0
 
 // Header of a plane pass: twiddles and position tables and, for FP64 fields,
 // the block exponents of its planes (FxPlanes of lgf_fft_fx.cu).
-constexpr size_t FX_PLANE_BYTES = 128;
+constexpr size_t FX_PLANE_BYTES = 256;
 constexpr int FX_MAX_THREADS = 384;  // CTA size limit of the FP64 plane passes
 constexpr int FX_C_THREADS = 768;    // and of the one with g(x): threads per SM at 80 registers
 constexpr int PAIR_MAX_THREADS = 384;  // and of the FP32 passes on pairs,
