@@ -111,6 +111,12 @@ __device__ __forceinline__ void fx_cmacc(FxAcc& re, FxAcc& im, const FxC& a, Fx 
   fx_mac(im, nax, b.y);
 }
 
+// Twice and four times a sum, rounded to 2^-60 after the multiplication.
+__device__ __forceinline__ FxAcc fx_zero_x2() { return FxAcc{0, (int64_t)1 << 28}; }
+__device__ __forceinline__ int64_t fx_sum60_x2(const FxAcc& s) { return 2 * s.hi + (s.mid >> 29); }
+__device__ __forceinline__ FxAcc fx_zero_x4() { return FxAcc{0, (int64_t)1 << 27}; }
+__device__ __forceinline__ int64_t fx_sum60_x4(const FxAcc& s) { return 4 * s.hi + (s.mid >> 28); }
+
 // An accumulated sum r in units of 2^-60, and its test against FX_LIM: sums
 // over rows and columns of matrices that are far from unitary can exceed it
 // although every entry passed fx_max.  t collects the largest r + FX_LIM;
@@ -122,15 +128,16 @@ __device__ __forceinline__ int64_t fx_sum60(const FxAcc& s, uint32_t& t) {
   return r;
 }
 __device__ __forceinline__ bool fx_bad(uint32_t m, uint32_t t) { return m >= FX_LIM_HI || t >= 2u * FX_SUM_OFF; }
-// 64-bit fixed point in units of 2^-58 from FP64, |a| < 2 (zero for what lies
-// below): for sums of up to 16 entries.
-__device__ __forceinline__ int64_t fx58_from(double a) {
+// 64-bit fixed point in units of 2^-K from FP64, |a| < 2 (zero for what lies
+// below): 2^-58 for sums of up to 16 entries, 2^-59 for sums of up to 8.
+template <int K> __device__ __forceinline__ int64_t fxk_from(double a) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
-  const uint32_t s = 1028u - ((hi >> 20) & 0x7ffu);
+  const uint32_t s = 1086u - K - ((hi >> 20) & 0x7ffu);
   const int64_t sg = (int64_t)((int)hi >> 31);
   return ((int64_t)shr64_clamp(((uint64_t)mh << 32) | ml, s) ^ sg) - sg;
 }
+__device__ __forceinline__ int64_t fx58_from(double a) { return fxk_from<58>(a); }
 __device__ __forceinline__ Fx fx_operand58(int64_t a58) { return fx_operand(a58 << 2); }
 
 // FP64 value of a 64-bit integer n times 2^-K, rounded to nearest, on the

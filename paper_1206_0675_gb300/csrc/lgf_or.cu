@@ -289,63 +289,71 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
-// A sweep, us (FP64 arithmetic before): 18-real 24^4 324 (724), 32^4 933 (2142),
-// 16^4 78 (168), 8^4 37 (93); 12-real 32^4 771 (2311).  The CTAs per SM are the
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 334 (724), 32^4 958 (2142),
+// 16^4 79 (168), 8^4 38 (93); 12-real 32^4 797 (2311).  theta of 8^4 levels off
+// (omega = 1.7) at 1.1e-32 (FP64: 1.2e-31) for eps = 0.5, 3.4e-33 (2.8e-32) for 0.25,
+// 3e-33 (6e-33) for 0.12; with operands of w / 64 and of r in [1/4, 1/2) it was
+// 2e-31 for all of them, and a sweep 2 % shorter.  The CTAs per SM are the
 // best of 3 to 6 for each kernel and storage (links of 18 reals at 4: 960 us, at 3:
 // 1056).
 
 // The 64-bit sum an operand stands for (units of 2^-60).
 __device__ __forceinline__ int64_t fx_r60(Fx a) { return mad_wide(a.h, 1 << 30, (int64_t)a.l); }
 
-// 2 a (y/2) for y/2 given as an operand.
-__device__ __forceinline__ Fx fx_scaled(Fx a, Fx half_y) {
-  uint32_t t = 0;
-  FxAcc p = fx_zero();
-  fx_mac(p, a, half_y);
-  return fx_operand(2 * fx_sum60(p, t));
+// Leading zeros of the largest magnitude of four integers.
+__device__ __forceinline__ int fx_lz4(const int64_t v[4]) {
+  uint64_t mag = 1u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) mag |= (uint64_t)(v[k] < 0 ? -v[k] : v[k]);
+  return __clzll((long long)mag);
 }
 
-// or_subgroup in fixed point.  The block's components b0..b3 (of the local
-// field over 64, so below 1/4) are shifted up until the largest lies in
-// [1/4, 1/2): |b|^2 is in [1/16, 1).  q is scaled by 7/16, which puts |q|^2 in
-// [0.19, 1.73) for 1 <= omega < 2: w7 = 7 omega / 16 and c7 = 7 (1 - omega) / 16
-// in units of 2^-60.  ok = false where |b| / 64 is below 2^-20: too small to
-// shift up without losing its direction.
-__device__ __forceinline__ void or_subgroup_fx(const FxC& mii, const FxC& mij, const FxC& mji, const FxC& mjj, Fx w7,
-                                               int64_t c7, FxC& a, FxC& b, bool& ok) {
-  int64_t v[4] = {fx_r60(mii.x) + fx_r60(mjj.x), -(fx_r60(mij.y) + fx_r60(mji.y)), fx_r60(mji.x) - fx_r60(mij.x),
-                  fx_r60(mjj.y) - fx_r60(mii.y)};  // |b| r / |r|
-  uint64_t mag = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) mag |= (uint64_t)(v[k] ^ (v[k] >> 63));
-  const int lz = __clzll((long long)(mag | 1u));
-  ok = ok && lz <= 24;
-  const int sh = min(max(lz - 5, 0), 20);
+// v / |v| of four integers of any common scale, lz = fx_lz4(v).  The components
+// are shifted until the largest lies in [1/2, 1), where an operand is finest:
+// |v|^2 is then in [1/4, 4) and 1 / (2 |v|) in (1/4, 1].  Every rounding here
+// turns g(x), and theta of a converged field is the square of that.
+__device__ __forceinline__ void fx_unit4(const int64_t v[4], int lz, Fx u[4]) {
   uint32_t t = 0;
   Fx r[4];
   FxAcc n = fx_zero();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    r[k] = fx_operand(v[k] << sh);
+    r[k] = fx_operand(lz >= 4 ? v[k] << (lz - 4) : (v[k] + ((int64_t)1 << (3 - lz))) >> (4 - lz));
     fx_mac(n, r[k], r[k]);
   }
-  const Fx yq = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t), (int64_t)1 << 56)) >> 1);  // 1 / (4 |b|)
-  Fx q[4];
-  n = fx_zero();
+  const Fx y = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t) >> 2, (int64_t)1 << 56)) >> 1);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    FxAcc p = fx_zero();
-    fx_mac(p, r[k], yq);
-    const Fx rk = fx_operand(4 * fx_sum60(p, t));
-    p = fx_zero();
-    if (k == 0) p.hi = c7;
-    fx_mac(p, w7, rk);
-    q[k] = fx_operand(fx_sum60(p, t));
-    fx_mac(n, q[k], q[k]);
+    FxAcc p = fx_zero_x2();
+    fx_mac(p, r[k], y);
+    u[k] = fx_operand(fx_sum60_x2(p));
   }
-  const Fx zh = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t), (int64_t)1 << 56)));
-  a = FxC{fx_scaled(q[0], zh), fx_scaled(q[3], zh)};
-  b = FxC{fx_scaled(q[2], zh), fx_scaled(q[1], zh)};
+}
+
+// or_subgroup in fixed point, on blocks of the local field over 16 (components
+// up to 9/16, their sums up to 9/8).  q is scaled by 7/16, which puts |q| in
+// [0.43, 1.32) for 1 <= omega < 2: w7 = 7 omega / 16 and c7 = 7 (1 - omega) / 16
+// in units of 2^-60.  ok = false where no component of b / 16 reaches 2^-21
+// (|b| < 2^-17): too small for its direction to be resolved in units of 2^-60.
+__device__ __forceinline__ void or_subgroup_fx(const FxC& mii, const FxC& mij, const FxC& mji, const FxC& mjj, Fx w7,
+                                               int64_t c7, FxC& a, FxC& b, bool& ok) {
+  const int64_t v[4] = {fx_r60(mii.x) + fx_r60(mjj.x), -(fx_r60(mij.y) + fx_r60(mji.y)),
+                        fx_r60(mji.x) - fx_r60(mij.x), fx_r60(mjj.y) - fx_r60(mii.y)};  // |b| r / |r|
+  const int lz = fx_lz4(v);
+  ok = ok && lz <= 24;
+  Fx r[4];
+  fx_unit4(v, lz, r);
+  int64_t q[4];  // units of 2^-62
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    FxAcc p = fx_zero_x4();
+    if (k == 0) p.hi = c7;
+    fx_mac(p, w7, r[k]);
+    q[k] = fx_sum60_x4(p);
+  }
+  fx_unit4(q, fx_lz4(q), r);
+  a = FxC{r[0], r[3]};
+  b = FxC{r[2], r[1]};
 }
 
 // or_rot in fixed point.
@@ -407,7 +415,7 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
   if ((int64_t)j >= (g.V >> 1)) return;
   int c[4];
   const int64_t s = or_coords(g, dhx, j, parity, c);
-  // w(x) in units of 2^-58
+  // w(x) in units of 2^-59
   int64_t W[9][2];
 #pragma unroll
   for (int e = 0; e < 9; ++e) W[e][0] = W[e][1] = 0;
@@ -428,8 +436,8 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         m = fx_max(m, u[r][q]);
-        x[r][q][0] = fx58_from(u[r][q].x);
-        x[r][q][1] = fx58_from(u[r][q].y);
+        x[r][q][0] = fxk_from<59>(u[r][q].x);
+        x[r][q][1] = fxk_from<59>(u[r][q].y);
       }
     strong = max(strong, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]));
     if (ROWS == 2) {
@@ -437,13 +445,13 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
 #pragma unroll
       for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) a[r][q] = FxC{fx_operand58(x[r][q][0]), fx_operand58(x[r][q][1])};
+        for (int q = 0; q < 3; ++q) a[r][q] = FxC{fx_operand(2 * x[r][q][0]), fx_operand(2 * x[r][q][1])};
       int64_t c3[3][2];
       fx_third_row(a[0], a[1], c3, t);
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        x[2][q][0] = c3[q][0] >> 2;
-        x[2][q][1] = c3[q][1] >> 2;
+        x[2][q][0] = c3[q][0] >> 1;
+        x[2][q][1] = c3[q][1] >> 1;
       }
     }
     if (fwd) {
@@ -462,7 +470,7 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
   }
   FxC M[3][3], gx[3][3];
 #pragma unroll
-  for (int e = 0; e < 9; ++e) M[e / 3][e % 3] = FxC{fx_operand(W[e][0] >> 4), fx_operand(W[e][1] >> 4)};  // w / 64
+  for (int e = 0; e < 9; ++e) M[e / 3][e % 3] = FxC{fx_operand((W[e][0] + 4) >> 3), fx_operand((W[e][1] + 4) >> 3)};  // w / 16
   bool ok = !fx_bad(m, t) && strong >= FX_WEAK_HI;
   or_site_gauge_fx(M, fx_operand(w7), c7, gx, ok);
   if (ok) {

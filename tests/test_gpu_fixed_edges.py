@@ -22,7 +22,7 @@ def _library():
 
 # Device functions that no entry point reaches by themselves, as a small library of their own.
 PROBE = r"""
-#include "lgf_gauge.cuh"
+#include "lgf_or.cu"
 using namespace lgf;
 // G of one site after g with the given FP64 rows (stored as a lane stores them)
 __global__ void accumulate(const double2* rows, double2* gf, double2* G) {
@@ -53,6 +53,29 @@ extern "C" int probe_factors(const float* X, float* out, int n) {
   float4* o = reinterpret_cast<float4*>(d + (size_t)4 * n);
   factors<<<(n + 127) / 128, 128>>>(d, o, n);
   const cudaError_t e = cudaMemcpy(out, o, (size_t)n * 16, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return (int)e;
+}
+// a, b of the SU(2) hits on n blocks (of the local field over 16), and whether they are resolved
+__global__ void hits(const double2* B, double2* out, int* ok, int n, double omega) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  FxC m[4], a, b;
+  for (int k = 0; k < 4; ++k) m[k] = fx_from(B[4 * i + k]);
+  const int64_t w7 = llrint(ldexp(7.0 * omega, 56)), c7 = llrint(ldexp(7.0 * (1.0 - omega), 56));
+  bool good = true;
+  or_subgroup_fx(m[0], m[1], m[2], m[3], fx_operand(w7), c7, a, b, good);
+  out[2 * i] = make_double2(fx_value(a.x), fx_value(a.y));
+  out[2 * i + 1] = make_double2(fx_value(b.x), fx_value(b.y));
+  ok[i] = good;
+}
+extern "C" int probe_hits(const double* B, double* out, int* ok, int n, double omega) {
+  double2* d;
+  cudaMalloc(&d, (size_t)n * 7 * sizeof(double2));
+  cudaMemcpy(d, B, (size_t)n * 64, cudaMemcpyHostToDevice);
+  hits<<<(n + 127) / 128, 128>>>(d, d + 4 * n, reinterpret_cast<int*>(d + 6 * n), n, omega);
+  cudaMemcpy(out, d + 4 * n, (size_t)n * 32, cudaMemcpyDeviceToHost);
+  const cudaError_t e = cudaMemcpy(ok, d + 6 * n, (size_t)n * 4, cudaMemcpyDeviceToHost);
   cudaFree(d);
   return (int)e;
 }
@@ -211,3 +234,49 @@ def test_long_lines_are_no_further_off_than_fp64(ext, fp64):
         lat.step(0.08)
         g = lat.get_gauge()
     assert np.sqrt(np.mean(np.abs(g - go) ** 2)) < 1.05 * fp64
+
+
+# ---------------------------------------------------------------------------
+# hits of overrelaxation
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("omega", [1.0, 1.7, 1.999])
+@pytest.mark.parametrize("size", [1.0, 0.3, 1e-3, 2.0 ** -20, 2.0 ** -21, 2.0 ** -22, 2.0 ** -40, 0.0])
+def test_hits_down_to_where_their_direction_is_lost(probe, size, omega):
+    """r^omega of blocks whose largest component is `size`: seven roundings of 2^-61 or less turn it, 2^-57 in all
+    for the worst.  Below 2^-21 the site is handed to FP64."""
+    n, rng = 2000, np.random.default_rng(8)
+    v = rng.standard_normal((n, 4))
+    v[:8] = np.concatenate([np.eye(4), -np.eye(4)])
+    v = np.rint(v / np.max(np.abs(v), axis=1, keepdims=True) * size * 2.0 ** 59) * 2.0 ** -59
+    B = np.zeros((n, 4), dtype=np.complex128)      # b0 .. b3 as sums of two entries each
+    B[:, 0] = v[:, 0] / 2 + 1j * v[:, 3] / 2
+    B[:, 3] = v[:, 0] / 2 - 1j * v[:, 3] / 2
+    B[:, 1] = v[:, 2] / 2 + 1j * v[:, 1] / 2
+    B[:, 2] = -v[:, 2] / 2 + 1j * v[:, 1] / 2
+    out, ok = np.empty((n, 2), dtype=np.complex128), np.empty(n, dtype=np.int32)
+    assert probe.probe_hits(ptr(B), ptr(out), ptr(ok), n, ctypes.c_double(omega)) == 0
+    assert np.all(ok == (size >= 2.0 ** -21))
+    if size < 2.0 ** -21:
+        return
+    r = np.stack([v[:, 0], -v[:, 1], -v[:, 2], -v[:, 3]], axis=1).astype(np.longdouble)
+    r /= np.sqrt(np.sum(r * r, axis=1, keepdims=True))
+    q = omega * r + np.array([1 - omega, 0, 0, 0])
+    q /= np.sqrt(np.sum(q * q, axis=1, keepdims=True))
+    got = np.stack([out[:, 0].real, out[:, 1].imag, out[:, 1].real, out[:, 0].imag], axis=1)
+    assert np.max(np.abs(got - q)) < 2.0 ** -53 + 2.0 ** -57
+
+
+@pytest.mark.parametrize("store12", [False, True])
+@pytest.mark.parametrize("eps, fp64", [(0.25, 2.8e-32), (0.5, 1.15e-31)])
+def test_or_converges_as_far_as_fp64(eps, fp64, store12):
+    """theta of 8^4 levels off no higher than it did with hits in FP64 arithmetic (within 10 %)."""
+    ext = (8, 8, 8, 8)
+    with lgf.Lattice(ext, "fp64", store12=store12) as lat:
+        lat.set_links(fields.random_links(ext, eps, seed=4))
+        lat.or_sweep(1.7, 1500)
+        theta = []
+        for _ in range(15):
+            lat.or_sweep(1.7, 1)
+            theta.append(lat.measure()[1])
+    assert np.median(theta) < 1.1 * fp64
