@@ -31,7 +31,7 @@ template <typename R> struct Lane {
   C2<R>* U = nullptr;      // links [4][rows][3][V]
   C2<R>* U2 = nullptr;     // second link buffer (FP32 lanes)
   bool fused = false;      // update and measurement run as one kernel, links ping-pong between U and U2
-  C2<R>* g = nullptr;      // gauge transform of the last step [grows][3][V] (FP64: fixed-point operands)
+  C2<R>* g = nullptr;      // gauge transform of the last step [grows][3][V] (FP64: lgf_fixed.cuh)
   C2<R>* D = nullptr;      // packed divergence / FFT workspace [4][V]
   R* K = nullptr;          // filter table [V]
   C2<R>* tw = nullptr;     // twiddles
@@ -375,8 +375,8 @@ template <typename R> cudaError_t enqueue_alt_fft(lgf_ctx* h, Lane<R>& L, int k,
     case K_F3: return launch_fft_xyz<R>(g, L.plan, L.D, L.tw, L.pos, -1, 4, s);
     case K_I3: return launch_fft_xyz<R>(g, L.plan, L.D, L.tw, L.pos, +1, 4, s);
     default:
-      if (L.grows == 3) return launch_gauge_from_delta<R, R, 3>(g, L.D, L.g, L.G, s, Batch(), exact_exp(h));
-      return launch_gauge_from_delta<R, R, 2>(g, L.D, L.g, L.G, s, Batch(), exact_exp(h));
+      if (L.grows == 3) return launch_gauge_from_delta<R, R, 3>(g, L.D, L.g, L.G, h->st, s, Batch(), exact_exp(h));
+      return launch_gauge_from_delta<R, R, 2>(g, L.D, L.g, L.G, h->st, s, Batch(), exact_exp(h));
   }
 }
 
@@ -393,10 +393,11 @@ template <> cudaError_t enqueue_kernel<double>(lgf_ctx* h, Lane<double>& L, int 
     case K_A: return launch_fft_xy<double>(g, L.plan, L.D, L.tw, L.pos, -1, 4, s);
     case K_B: return launch_fft_zt<double>(g, L.plan, L.D, L.tw, L.pos, L.K, 0, 4, s, learned_io(h, L));
     case K_C:
-      return launch_fft_xy_inv_gauge<double, double, 3>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, s, Batch(),
+      return launch_fft_xy_inv_gauge<double, double, 3>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, h->st, s, Batch(),
                                                         exact_exp(h));
     case K_UPD:
-      return L.rows == 3 ? launch_update<double, 3, 3>(g, L.U, L.g, s) : launch_update<double, 2, 3>(g, L.U, L.g, s);
+      return L.rows == 3 ? launch_update<double, 3, 3>(g, L.U, L.g, h->st, s)
+                         : launch_update<double, 2, 3>(g, L.U, L.g, h->st, s);
     case K_MEAS: return enqueue_measure<double>(h, L, 1, cond, use_cond, s, 0, cond_undo);
     case K_REVERT:
       return L.rows == 3 ? launch_revert<double, 3, 3>(g, L.U, L.g, L.G, h->st, s, L.U2)
@@ -414,11 +415,13 @@ template <> cudaError_t enqueue_kernel<float>(lgf_ctx* h, Lane<float>& L, int k,
     case K_A: return launch_fft_xy<float>(g, L.plan, L.D, L.tw, L.pos, -1, 4, s);
     case K_B: return launch_fft_zt<float>(g, L.plan, L.D, L.tw, L.pos, L.K, 0, 4, s, learned_io(h, L));
     case K_C:
-      return L.grows == 2 ? launch_fft_xy_inv_gauge<float, float, 2>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, s,
-                                                                     Batch(), exact_exp(h))
-                          : launch_fft_xy_inv_gauge<float, float, 3>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, s,
-                                                                     Batch(), exact_exp(h));
-    case K_UPD: return L.grows == 2 ? launch_update<float, 2, 2>(g, L.U, L.g, s) : launch_update<float, 3, 3>(g, L.U, L.g, s);
+      return L.grows == 2 ? launch_fft_xy_inv_gauge<float, float, 2>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, h->st,
+                                                                     s, Batch(), exact_exp(h))
+                          : launch_fft_xy_inv_gauge<float, float, 3>(g, L.plan, L.D, L.tw, L.pos, L.g, L.G, h->st,
+                                                                     s, Batch(), exact_exp(h));
+    case K_UPD:
+      return L.grows == 2 ? launch_update<float, 2, 2>(g, L.U, L.g, h->st, s)
+                          : launch_update<float, 3, 3>(g, L.U, L.g, h->st, s);
     case K_UM:
       return L.grows == 2
                  ? launch_update_measure<float, 2, 2>(g, L.U, L.U2, L.g, L.D, h->partials, h->st, cond, use_cond, s,
@@ -599,13 +602,13 @@ lgf_status measure_current(lgf_ctx* h) {
 // FP32 -> FP64 switch: G64 = proj_SU3(G32) in FP64, U64 = G64 U0 G64^dag(x+mu).
 lgf_status switch_to_fp64(lgf_ctx* h) {
   const Geom& g = h->geom;
-  LGF_CK(h, launch_project_sites_f32_to_f64(g, h->f.G, h->d.g, h->d.G, h->stream));
+  LGF_CK(h, launch_project_sites_f32_to_f64(g, h->f.G, h->U0, h->d.g, h->d.G, h->stream));
   if (h->d.rows == 3) {
     LGF_CK(h, (launch_links_from_aos<double, 3>(g, h->U0, h->d.U, h->stream)));
-    LGF_CK(h, (launch_update<double, 3, 3>(g, h->d.U, h->d.g, h->stream)));
+    LGF_CK(h, (launch_update<double, 3, 3>(g, h->d.U, h->d.g, h->st, h->stream)));
   } else {
     LGF_CK(h, (launch_links_from_aos<double, 2>(g, h->U0, h->d.U, h->stream)));
-    LGF_CK(h, (launch_update<double, 2, 3>(g, h->d.U, h->d.g, h->stream)));
+    LGF_CK(h, (launch_update<double, 2, 3>(g, h->d.U, h->d.g, h->st, h->stream)));
   }
   h->phase = 64;
   lgf_status s = measure_current(h);

@@ -131,7 +131,7 @@ cudaError_t time_plan(ClassLane& C, const FFTPlan& p, cudaStream_t s, float* ms_
     if (e == cudaSuccess) e = launch_fft_xy<double>(C.geom, p, C.D, C.tw, C.pos, -1, 4, s, B);
     if (e == cudaSuccess) e = launch_fft_zt<double>(C.geom, p, C.D, C.tw, C.pos, C.K, 0, 4, s, LearnedIO(), B);
     if (e == cudaSuccess)
-      e = launch_fft_xy_inv_gauge<double, double, 3>(C.geom, p, C.D, C.tw, C.pos, C.g, nullptr, s, B);
+      e = launch_fft_xy_inv_gauge<double, double, 3>(C.geom, p, C.D, C.tw, C.pos, C.g, nullptr, nullptr, s, B);
     if (e == cudaSuccess) e = cudaEventRecord(e1, s);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -229,10 +229,10 @@ cudaError_t enqueue_class_body(ClassLane& C, cudaStream_t s) {
   if ((e = launch_fft_xy<double>(C.geom, C.plan, C.D, C.tw, C.pos, -1, 4, s, C.B)) != cudaSuccess) return e;
   if ((e = launch_fft_zt<double>(C.geom, C.plan, C.D, C.tw, C.pos, C.K, 0, 4, s, LearnedIO(), C.B)) != cudaSuccess)
     return e;
-  if ((e = launch_fft_xy_inv_gauge<double, double, 3>(C.geom, C.plan, C.D, C.tw, C.pos, C.g, nullptr, s, C.B)) !=
-      cudaSuccess)
+  if ((e = launch_fft_xy_inv_gauge<double, double, 3>(C.geom, C.plan, C.D, C.tw, C.pos, C.g, nullptr, nullptr, s,
+                                                      C.B)) != cudaSuccess)
     return e;
-  if ((e = launch_update<double, 3, 3>(C.geom, C.U, C.g, s, C.B)) != cudaSuccess) return e;
+  if ((e = launch_update<double, 3, 3>(C.geom, C.U, C.g, nullptr, s, C.B)) != cudaSuccess) return e;
   return launch_measure<double, 3>(C.geom, C.U, C.D, C.partials, nullptr, 1, 0, 0, s, 0, C.B);
 }
 

@@ -139,7 +139,13 @@ template <typename R, int ROWS> struct MatField {
       for (int c = 0; c < 3; ++c) M.e[r][c] = __ldg(&p[off(m, r, c, s)]);
     if (ROWS == 2) su3_third_row<R>(M.e[0], M.e[1], M.e[2]);
   }
-  // rows 0..1 only (never reconstructs)
+  // rows 0..1 only (never reconstructs); plain and read-only loads
+  __device__ __forceinline__ void load_rows01(int m, int64_t s, C2<R> (*rows)[3]) const {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) rows[r][c] = p[off(m, r, c, s)];
+  }
   __device__ __forceinline__ void load_rows01_ro(int m, int64_t s, C2<R> rows[2][3]) const {
 #pragma unroll
     for (int r = 0; r < 2; ++r)

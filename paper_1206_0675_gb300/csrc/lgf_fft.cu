@@ -471,14 +471,15 @@ __global__ void __launch_bounds__(512) fft_xyz_kernel(Geom g, FFTDir dx, FFTDir 
 // the inverse (x, y) transform has already been applied to data.
 template <typename R, typename RG, int GROWS, bool EXPG>
 __global__ void gauge_from_delta_kernel(Geom g, const C2<R>* __restrict__ data, C2<RG>* __restrict__ gf,
-                                        C2<RG>* __restrict__ Gf, Batch B) {
+                                        C2<RG>* __restrict__ Gf, const DevState* __restrict__ st, Batch B) {
   if (batch_skip(B)) return;
   data += blockIdx.z * B.s_delta;
   gf += blockIdx.z * B.s_g;
   if (Gf != nullptr) Gf += blockIdx.z * B.s_G;
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
-  gauge_site<R, RG, GROWS, EXPG>(data[s], data[g.V + s], data[2 * g.V + s], data[3 * g.V + s], g.V, s, gf, Gf);
+  gauge_site<R, RG, GROWS, EXPG>(data[s], data[g.V + s], data[2 * g.V + s], data[3 * g.V + s], g.V, s, gf, Gf,
+                                 near_identity(st, B));
 }
 
 // ---------------------------------------------------------------------------
@@ -838,29 +839,29 @@ cudaError_t launch_fft_xyz(const Geom& g, const FFTPlan& p, C2<R>* data, const C
 }
 
 template <typename R, typename RG, int GROWS>
-cudaError_t launch_gauge_from_delta(const Geom& g, const C2<R>* data, C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s,
-                                    const Batch& B, int exact_exp) {
+cudaError_t launch_gauge_from_delta(const Geom& g, const C2<R>* data, C2<RG>* gfield, C2<RG>* Gfield,
+                                    const DevState* st, cudaStream_t s, const Batch& B, int exact_exp) {
   const dim3 grid((unsigned)((g.V + 127) / 128), 1, (unsigned)B.n);
   if (exact_exp)
-    gauge_from_delta_kernel<R, RG, GROWS, true><<<grid, 128, 0, s>>>(g, data, gfield, Gfield, B);
+    gauge_from_delta_kernel<R, RG, GROWS, true><<<grid, 128, 0, s>>>(g, data, gfield, Gfield, st, B);
   else
-    gauge_from_delta_kernel<R, RG, GROWS, false><<<grid, 128, 0, s>>>(g, data, gfield, Gfield, B);
+    gauge_from_delta_kernel<R, RG, GROWS, false><<<grid, 128, 0, s>>>(g, data, gfield, Gfield, st, B);
   return cudaGetLastError();
 }
 
 template <typename R, typename RG, int GROWS, bool EXPG>
 static cudaError_t launch_pass_c(const Geom& g, const FFTPlan& p, C2<R>* data, const C2<R>* tw, const short* pos,
-                                 C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s, const Batch& B) {
+                                 C2<RG>* gfield, C2<RG>* Gfield, const DevState* st, cudaStream_t s, const Batch& B) {
   cudaError_t e;
   if (!p.fuse_g) {
     if ((e = launch_fft_xy<R>(g, p, data, tw, pos, +1, 4, s, B)) != cudaSuccess) return e;
     gauge_from_delta_kernel<R, RG, GROWS, EXPG><<<dim3((unsigned)((g.V + 127) / 128), 1, (unsigned)B.n), 128, 0, s>>>(
-        g, data, gfield, Gfield, B);
+        g, data, gfield, Gfield, st, B);
     return cudaGetLastError();
   }
   if constexpr (sizeof(R) == sizeof(double)) {
     static_assert(GROWS == 3, "FP64 lanes keep three rows of g");
-    return launch_xy_inv_gauge_fx(g, p, data, tw, pos, gfield, Gfield, s, B, EXPG);
+    return launch_xy_inv_gauge_fx(g, p, data, tw, pos, gfield, Gfield, st, s, B, EXPG);
   } else {
   return launch_xy_inv_gauge_pair<GROWS>(g, p, data, tw, pos, gfield, Gfield, s, B, EXPG);
   }
@@ -868,9 +869,10 @@ static cudaError_t launch_pass_c(const Geom& g, const FFTPlan& p, C2<R>* data, c
 
 template <typename R, typename RG, int GROWS>
 cudaError_t launch_fft_xy_inv_gauge(const Geom& g, const FFTPlan& p, C2<R>* data, const C2<R>* tw, const short* pos,
-                                    C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s, const Batch& B, int exact_exp) {
-  return exact_exp ? launch_pass_c<R, RG, GROWS, true>(g, p, data, tw, pos, gfield, Gfield, s, B)
-                   : launch_pass_c<R, RG, GROWS, false>(g, p, data, tw, pos, gfield, Gfield, s, B);
+                                    C2<RG>* gfield, C2<RG>* Gfield, const DevState* st, cudaStream_t s,
+                                    const Batch& B, int exact_exp) {
+  return exact_exp ? launch_pass_c<R, RG, GROWS, true>(g, p, data, tw, pos, gfield, Gfield, st, s, B)
+                   : launch_pass_c<R, RG, GROWS, false>(g, p, data, tw, pos, gfield, Gfield, st, s, B);
 }
 
 template cudaError_t launch_fft_xy<double>(const Geom&, const FFTPlan&, C2<double>*, const C2<double>*, const short*,
@@ -883,14 +885,14 @@ template cudaError_t launch_fft_zt<float>(const Geom&, const FFTPlan&, C2<float>
                                           const float*, int, int, cudaStream_t, const LearnedIO&, const Batch&);
 #define LGF_INST_C(R, RG, GR)                                                                                    \
   template cudaError_t launch_fft_xy_inv_gauge<R, RG, GR>(const Geom&, const FFTPlan&, C2<R>*, const C2<R>*,      \
-                                                          const short*, C2<RG>*, C2<RG>*, cudaStream_t, const Batch&, \
-                                                          int);
+                                                          const short*, C2<RG>*, C2<RG>*, const DevState*,        \
+                                                          cudaStream_t, const Batch&, int);
 LGF_INST_C(double, double, 3)
 LGF_INST_C(float, float, 2)
 LGF_INST_C(float, float, 3)
 #define LGF_INST_G(R, RG, GR)                                                                                   \
   template cudaError_t launch_gauge_from_delta<R, RG, GR>(const Geom&, const C2<R>*, C2<RG>*, C2<RG>*,         \
-                                                          cudaStream_t, const Batch&, int);
+                                                          const DevState*, cudaStream_t, const Batch&, int);
 LGF_INST_G(double, double, 3)
 LGF_INST_G(double, double, 2)
 LGF_INST_G(float, float, 2)

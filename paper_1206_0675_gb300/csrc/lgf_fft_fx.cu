@@ -582,8 +582,9 @@ template <bool EXPG>
 __global__ void __launch_bounds__(FX_C_THREADS)
 fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const double2* __restrict__ data,
                            const int4* __restrict__ twg, const short* __restrict__ posg, double2* __restrict__ gf,
-                           double2* __restrict__ Gf, CopyDiv cd, Batch B) {
+                           double2* __restrict__ Gf, const DevState* __restrict__ st, CopyDiv cd, Batch B) {
   if (batch_skip(B)) return;
+  const bool near_id = near_identity(st, B);
   data += blockIdx.z * B.s_delta;
   gf += blockIdx.z * B.s_g;
   if (Gf != nullptr) Gf += blockIdx.z * B.s_G;
@@ -616,7 +617,7 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
     const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
     const int o = pos[Lx + y] * RS + pos[x];
     const int64_t s = (int64_t)blockIdx.x * plane + i;
-    if (!EXPG) {
+    if (!EXPG && !near_id) {
       int64_t A[8];
       bool ok = true;
 #pragma unroll
@@ -634,7 +635,7 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
     double2 f[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) f[k] = fx_out_any(tile[k * PS + o], ps->t[0].in[k]);
-    gauge_site_fp64<EXPG>(f[0], f[1], f[2], f[3], g.V, s, gf, Gf);
+    gauge_site_fp64<EXPG>(f[0], f[1], f[2], f[3], g.V, s, gf, Gf, near_id);
   }
 }
 
@@ -704,14 +705,14 @@ cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, con
 }
 
 cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
-                                   const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
-                                   bool exact_exp) {
+                                   const short* pos, double2* gfield, double2* Gfield, const DevState* st,
+                                   cudaStream_t s, const Batch& B, bool exact_exp) {
   const int Lx = g.L[0], Ly = g.L[1];
   const FxPass P = xy_pass(p, Lx, Ly, 4);
   const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
   const dim3 grid((unsigned)(g.L[2] * g.L[3]), 1, (unsigned)B.n);
   return fx_launch(exact_exp ? fft_xy_inv_gauge_fx_kernel<true> : fft_xy_inv_gauge_fx_kernel<false>, grid, p.threads_c,
-                   p.smem_c, s, g, P, data, fx_table(g, tw), pos, gfield, Gfield, cd, B);
+                   p.smem_c, s, g, P, data, fx_table(g, tw), pos, gfield, Gfield, st, cd, B);
 }
 
 }  // namespace lgf

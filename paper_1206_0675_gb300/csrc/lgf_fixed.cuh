@@ -27,8 +27,18 @@ namespace lgf {
 
 // high word of 1.125
 constexpr uint32_t FX_LIM_HI = 0x3ff20000u;
-// high word of 2^-12: below it an FP64 rounding (2^-65) is finer than the unit
-constexpr uint32_t FX_WEAK_HI = 0x3f300000u;
+// Links near the identity: FP64 rounds small entries finer than the fixed-point
+// unit, so theta of a converged field of links 1 + O(eps) falls with eps^2 in
+// FP64, and levels off in fixed point.  Where all off-diagonal entries of a link
+// (01, 02, 12) are below these, its warp takes FP64 as a whole (a warp would do
+// both otherwise), decided before any arithmetic.
+// High word of 2^-5: in the measurement and the hits, whose sums of links have
+// the unit 2^-58 or 2^-59.  theta of 8^4 levels off (fixed point / FP64) at
+// 1.7e-33 / 1.4e-33 for eps = 0.06, of whose warps 98 % are below the line, and at
+// 1.1e-33 / 5.4e-33 for 0.12, of whose warps 12 % are; 0.1 % are for eps = 0.3.
+constexpr uint32_t FX_NEAR_HI = 0x3fa00000u;
+// High word of 2^-7: in the products of single links, unit 2^-60.
+constexpr uint32_t FX_WEAK_HI = 0x3f800000u;
 
 // c + a b with a 64-bit sum: one IMAD.WIDE.  (Both factors have to look like
 // signed 32-bit words to the compiler, which turns products with a factor of
@@ -238,44 +248,75 @@ __device__ __forceinline__ int64_t bfp_mul(int64_t x, int wh, int wl) {
 // g of FP64 lanes, stored as fixed-point operands
 // ---------------------------------------------------------------------------
 
-// One complex entry is four words (re h, re l, im h, im l), the 16 bytes of
-// an FP64 one, so that the update reads its operands as they are (five
-// threads read every g(x): converting FP64 entries cost the update a seventh
-// of its instructions).  The unit 2^-60 is below the noise of any g: the
-// divergence that it comes from is a sum of FP64 entries of order one.  A g
-// that is not finite is marked in its first word.
-constexpr int FX_G_NAN = (int)0x80000000u;
-
+// One complex entry is 16 bytes, and the nine entries of a site have one of two
+// forms.  Operands: four words (re h, re l, im h, im l), so that the update reads
+// them as they are (five threads read every g(x): converting FP64 entries cost
+// the update a seventh of its instructions).  FP64 numbers (re, im): where the
+// field is near the identity (DevState::near_id) -- g - 1 is then small and the
+// unit 2^-60 is far above what FP64 keeps of it -- and where g is not finite.
+// The forms are told apart by the second word of the first entry: l of an
+// operand lies in [-2^29, 2^29), the high word of an FP64 number does not
+// unless its magnitude is below 2^-511 (of a positive one) or from 2^513 (of a
+// negative one), which the store replaces.
+__device__ __forceinline__ bool fxg_is_fp64(int4 first) {
+  return (uint32_t)first.y + 0x20000000u >= 0x40000000u;
+}
 __device__ __forceinline__ FxC fxg_unpack(int4 w) { return FxC{Fx{w.x, w.y}, Fx{w.z, w.w}}; }
 __device__ __forceinline__ int4 fxg_pack(const FxC& a) { return make_int4(a.x.h, a.x.l, a.y.h, a.y.l); }
+__device__ __forceinline__ double2 fxg_fp64(int4 w) {
+  return make_double2(__hiloint2double(w.y, w.x), __hiloint2double(w.w, w.z));
+}
+__device__ __forceinline__ int4 fxg_of_fp64(double2 v) {
+  return make_int4(__double2loint(v.x), __double2hiint(v.x), __double2loint(v.y), __double2hiint(v.y));
+}
 __device__ __forceinline__ double fx_value(Fx a) { return fx_to_double_fp<60>(((int64_t)a.h << 30) + a.l); }
 
-// g in FP64 (NaN where marked) from its entries p[e stride].
+// g in FP64 from its entries p[e stride].
 __device__ __forceinline__ void fxg_load(const int4* p, int64_t stride, M3<double>& M) {
-  const bool bad = p[0].x == FX_G_NAN;
+  if (fxg_is_fp64(p[0])) {
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const FxC w = fxg_unpack(p[e * stride]);
-    M.e[e / 3][e % 3] = bad ? make_double2(NAN, NAN) : make_double2(fx_value(w.x), fx_value(w.y));
+    for (int e = 0; e < 9; ++e) M.e[e / 3][e % 3] = fxg_fp64(p[e * stride]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const FxC w = fxg_unpack(p[e * stride]);
+      M.e[e / 3][e % 3] = make_double2(fx_value(w.x), fx_value(w.y));
+    }
   }
 }
 __device__ __forceinline__ void fxg_load(const double2* gf, int64_t V, int64_t s, M3<double>& M) {
   fxg_load(reinterpret_cast<const int4*>(gf) + s, V, M);
 }
-// The store, from FP64 rows.
+// The stores, from FP64 rows: as FP64 numbers, and as operands (NaN in all
+// entries where one is outside their range).
+__device__ __forceinline__ void fxg_store_fp64(double2* __restrict__ gf, int64_t V, int64_t s, const double2 a[3],
+                                               const double2 b[3], const double2 c[3]) {
+  int4* p = reinterpret_cast<int4*>(gf);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    int4 w = fxg_of_fp64(a[j]);
+    if (j == 0 && !fxg_is_fp64(w)) {
+      w.y = w.y >= 0 ? 0x20b00000 : 0x7ff80000;  // 2^-500 for 0, NaN for what is not finite
+      w.x = 0;
+    }
+    p[j * V + s] = w;
+    p[(3 + j) * V + s] = fxg_of_fp64(b[j]);
+    p[(6 + j) * V + s] = fxg_of_fp64(c[j]);
+  }
+}
 __device__ __forceinline__ void fxg_store(double2* __restrict__ gf, int64_t V, int64_t s, const double2 a[3],
                                           const double2 b[3], const double2 c[3]) {
   int4* p = reinterpret_cast<int4*>(gf);
   uint32_t m = 0;
 #pragma unroll
   for (int j = 0; j < 3; ++j) m = fx_max(fx_max(fx_max(m, a[j]), b[j]), c[j]);
+  const bool bad = m >= FX_LIM_HI;
+  const int4 nan = make_int4(0, 0x7ff80000, 0, 0x7ff80000);
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    int4 w = fxg_pack(fx_from(a[j]));
-    if (j == 0 && m >= FX_LIM_HI) w.x = FX_G_NAN;
-    p[j * V + s] = w;
-    p[(3 + j) * V + s] = fxg_pack(fx_from(b[j]));
-    p[(6 + j) * V + s] = fxg_pack(fx_from(c[j]));
+    p[j * V + s] = bad ? nan : fxg_pack(fx_from(a[j]));
+    p[(3 + j) * V + s] = bad ? nan : fxg_pack(fx_from(b[j]));
+    p[(6 + j) * V + s] = bad ? nan : fxg_pack(fx_from(c[j]));
   }
 }
 

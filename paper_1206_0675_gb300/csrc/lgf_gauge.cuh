@@ -325,15 +325,17 @@ __device__ __forceinline__ void accumulate_gauge(int64_t V, int64_t s, const C2<
 }
 
 // Stores rows u, v (precision RG) and, where needed, row 3 = (u x v)^*, and
-// G <- g G where tracked.  FP64 lanes keep g as fixed-point operands.
+// G <- g G where tracked.  FP64 lanes keep g as fixed-point operands, and as FP64
+// numbers where the field is near the identity (near_id).
 template <typename RG, int GROWS>
 __device__ __forceinline__ void store_gauge_rows(int64_t V, int64_t s, const C2<RG> a[3], const C2<RG> b[3],
-                                                 C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf) {
+                                                 C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf, bool near_id) {
   C2<RG> c[3];
   const bool need_c = (GROWS == 3) || (Gf != nullptr);
   if (need_c) su3_third_row<RG>(a, b, c);
   if constexpr (sizeof(RG) == sizeof(double)) {
-    fxg_store(gf, V, s, a, b, c);
+    if (near_id) fxg_store_fp64(gf, V, s, a, b, c);
+    else fxg_store(gf, V, s, a, b, c);
   } else {
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -348,7 +350,7 @@ __device__ __forceinline__ void store_gauge_rows(int64_t V, int64_t s, const C2<
 // g(x) of one site from its packed filtered field and its store (and G <- g G).
 template <typename R, typename RG, int GROWS, bool EXPG>
 __device__ __forceinline__ void gauge_site(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f3, int64_t V, int64_t s,
-                                           C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf) {
+                                           C2<RG>* __restrict__ gf, C2<RG>* __restrict__ Gf, bool near_id = false) {
   static_assert(sizeof(R) == sizeof(RG), "g is stored in the precision of the divergence");
   C2<RG> a[3], b[3];
   if constexpr (EXPG) {
@@ -363,14 +365,15 @@ __device__ __forceinline__ void gauge_site(C2<R> f0, C2<R> f1, C2<R> f2, C2<R> f
   } else {
     gauge_rows<RG>(f0, f1, f2, f3, a, b);
   }
-  store_gauge_rows<RG, GROWS>(V, s, a, b, gf, Gf);
+  store_gauge_rows<RG, GROWS>(V, s, a, b, gf, Gf, near_id);
 }
 
-// The FP64 path of a site outside the fixed-point range.
+// The FP64 path of a site: outside the fixed-point range, or near the identity.
 template <bool EXPG>
 static __device__ __noinline__ void gauge_site_fp64(double2 f0, double2 f1, double2 f2, double2 f3, int64_t V,
-                                                    int64_t s, double2* __restrict__ gf, double2* __restrict__ Gf) {
-  gauge_site<double, double, 3, EXPG>(f0, f1, f2, f3, V, s, gf, Gf);
+                                                    int64_t s, double2* __restrict__ gf, double2* __restrict__ Gf,
+                                                    bool near_id) {
+  gauge_site<double, double, 3, EXPG>(f0, f1, f2, f3, V, s, gf, Gf, near_id);
 }
 
 static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, const int4* __restrict__ gp,
@@ -382,10 +385,10 @@ static __device__ __noinline__ void accumulate_gauge_fp64(int64_t V, int64_t s, 
 
 // G(s) <- g G(s) in fixed point, for the entries gp[e gstride] of g (a call:
 // its operands would otherwise crowd the registers of every caller, tracked
-// transform or not).  A marked g (not finite) goes to FP64: its mark is no operand.
+// transform or not).  A g kept as FP64 numbers takes the FP64 product.
 static __device__ __noinline__ void accumulate_gauge_fx(int64_t V, int64_t s, const int4* gp, int64_t gstride,
                                                         double2* __restrict__ Gf) {
-  if (gp[0].x == FX_G_NAN) {
+  if (fxg_is_fp64(gp[0])) {
     accumulate_gauge_fp64(V, s, gp, gstride, Gf);
     return;
   }

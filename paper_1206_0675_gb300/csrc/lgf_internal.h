@@ -24,7 +24,7 @@ struct DevState {
   int iter;          // link updates performed since the counter was reset
   int max_iter;      // loop stops when iter reaches it
   int status;        // 0 ok, 1 non-finite F or theta, 2 timeout
-  unsigned int ticket;  // CTA completion counter of the measurement reduction
+  int near_id;       // FP64 lanes: most warps of the last measurement found links near the identity
   int hist_cap;      // capacity of the history buffers (0 = none)
   int done;          // batch mode: this configuration has retired (theta < tol or iter >= max_iter)
   int use_m;         // the running step multiplies the filter by the learned table
@@ -40,6 +40,7 @@ struct DevState {
   int* flag_hist;      // flags of measurement number i (TRACE_* bits) if i < hist_cap
   double* defect_hist; // defect of measurement number i if i < hist_cap
   int snaps;           // learned handles: steps whose Fourier-space divergence snapshot is kept
+  unsigned long long ticket;  // the measurement's CTAs that are done and, from bit 32, their warps near the identity
 };
 
 enum { ST_OK = 0, ST_NONFINITE = 1, ST_DEFECT = 3 };
@@ -62,6 +63,11 @@ struct Batch {
 };
 
 __device__ __forceinline__ bool batch_skip(const Batch& b) { return b.st != nullptr && b.st[blockIdx.z].done; }
+// DevState::near_id of the configuration (false where there is no state).
+__device__ __forceinline__ bool near_identity(const DevState* st, const Batch& b) {
+  if (b.st != nullptr) st = b.st + blockIdx.z;
+  return st != nullptr && st->near_id != 0;
+}
 
 // The measuring kernels take a thread per site, or a lane per direction of a
 // site (eight sites to a warp) on lattices of less than 128 sites per SM, where
@@ -119,8 +125,10 @@ cudaError_t launch_revert(const Geom& g, C2<R>* links, const C2<R>* gfield, C2<R
 
 // U_mu(x) <- g(x) U_mu(x) g^dagger(x + mu^) in place (Sec. 2 eq. 2; kernel k6).
 // Links in precision R with LROWS stored rows; g in precision R with GROWS rows.
+// st (B.st in batch mode): its near_id sends FP64 links to FP64 arithmetic.
 template <typename R, int LROWS, int GROWS>
-cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cudaStream_t s, const Batch& B = Batch());
+cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, const DevState* st, cudaStream_t s,
+                          const Batch& B = Batch());
 
 // Graph condition of a batch: true while any of the n configurations is active.
 cudaError_t launch_batch_condition(const DevState* st, int n, unsigned long long cond, cudaStream_t s);
@@ -163,10 +171,11 @@ cudaError_t launch_reunitarize_links(const Geom& g, C2<R>* links, DevState* st, 
 cudaError_t launch_c2_f64_to_f32(const double2* in, float2* out, int64_t n, cudaStream_t s);
 cudaError_t launch_c2_f32_to_f64(const float2* in, double2* out, int64_t n, cudaStream_t s);
 
-// reunitarize(G32) in FP64 (3-row FP32 site field) as g of the FP64 lane and,
-// where given, as the 3-row FP64 site field G64.
-cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* gfield, double2* G64,
-                                            cudaStream_t s);
+// reunitarize(G32) in FP64 (3-row FP32 site field) as g of the FP64 lane, which
+// is to transform `links` (user layout), and, where given, as the 3-row FP64 site
+// field G64.
+cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, const double* links, double2* gfield,
+                                            double2* G64, cudaStream_t s);
 
 // Site field G <- 1.
 template <typename R, int ROWS>
@@ -278,11 +287,13 @@ cudaError_t launch_fft_zt(const Geom& g, const FFTPlan& p, C2<R>* data, const C2
                           const Batch& B = Batch());
 // Inverse (x,y) transform fused with g(x) = reunitarize(1 + Delta'(x)) (lgf_gauge.cuh)
 // (exact_exp != 0: g(x) = reunitarize(exp(Delta'(x)))); g stored with GROWS
-// rows in precision RG; optional G <- g G (precision RG with 3 rows).
+// rows in precision RG; optional G <- g G (precision RG with 3 rows).  st (B.st
+// in batch mode): whose near_id says which form g of an FP64 lane takes
+// (lgf_fixed.cuh).
 template <typename R, typename RG, int GROWS>
 cudaError_t launch_fft_xy_inv_gauge(const Geom& g, const FFTPlan& p, C2<R>* data, const C2<R>* tw, const short* pos,
-                                    C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s, const Batch& B = Batch(),
-                                    int exact_exp = 0);
+                                    C2<RG>* gfield, C2<RG>* Gfield, const DevState* st, cudaStream_t s,
+                                    const Batch& B = Batch(), int exact_exp = 0);
 
 // 1D pass along mu (0..3) over nfields fields: mode -1 forward, +1 inverse,
 // 0 forward, multiply by K (and by the learned table when lio.mtab is given
@@ -299,8 +310,8 @@ cudaError_t launch_fft_xyz(const Geom& g, const FFTPlan& p, C2<R>* data, const C
 // g(x) from the filtered field in natural order (after an inverse transform
 // that is not fused with g); same storage conventions as launch_fft_xy_inv_gauge.
 template <typename R, typename RG, int GROWS>
-cudaError_t launch_gauge_from_delta(const Geom& g, const C2<R>* data, C2<RG>* gfield, C2<RG>* Gfield, cudaStream_t s,
-                                    const Batch& B = Batch(), int exact_exp = 0);
+cudaError_t launch_gauge_from_delta(const Geom& g, const C2<R>* data, C2<RG>* gfield, C2<RG>* Gfield,
+                                    const DevState* st, cudaStream_t s, const Batch& B = Batch(), int exact_exp = 0);
 
 // ---- lgf_fft_fx.cu -------------------------------------------------------
 // The plane passes of FP64 fields in block floating point; arguments as the
@@ -311,8 +322,8 @@ cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, con
                              const double* K, int mode, int nfields, cudaStream_t s, const LearnedIO& lio,
                              const Batch& B);
 cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double2* data, const double2* tw,
-                                   const short* pos, double2* gfield, double2* Gfield, cudaStream_t s, const Batch& B,
-                                   bool exact_exp);
+                                   const short* pos, double2* gfield, double2* Gfield, const DevState* st,
+                                   cudaStream_t s, const Batch& B, bool exact_exp);
 // The twiddle table of a lattice: L[0] + ... + L[3] roots in FP64 and, for FP64
 // lanes (fixed), the same roots as fixed-point limbs (int4: cosine and sine, each
 // h 2^-30 + l 2^-60) in the same order.

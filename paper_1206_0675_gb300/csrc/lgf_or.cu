@@ -283,14 +283,14 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 //
 // Two kernels per colour: the first forms w(x) and g(x) of the colour's sites,
 // one thread each; the second multiplies every link of the lattice by the one
-// g that touches it, one thread per link, as in update_fx_kernel.  Sites and
-// links outside the fixed-point range or near the identity, and local fields
-// too small for their direction to be resolved, are done in FP64.
+// g that touches it, one thread per link, as in update_fx_kernel.  Warps with
+// links near the identity, sites and links outside the fixed-point range, and
+// local fields too small for their direction to be resolved are done in FP64.
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
-// A sweep, us (FP64 arithmetic before): 18-real 24^4 334 (724), 32^4 958 (2142),
-// 16^4 79 (168), 8^4 38 (93); 12-real 32^4 797 (2311).  theta of 8^4 levels off
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 335 (724), 32^4 964 (2142),
+// 16^4 79 (168), 8^4 38 (93); 12-real 32^4 811 (2311).  theta of 8^4 levels off
 // (omega = 1.7) at 1.1e-32 (FP64: 1.2e-31) for eps = 0.5, 3.4e-33 (2.8e-32) for 0.25,
 // 3e-33 (6e-33) for 0.12; with operands of w / 64 and of r in [1/4, 1/2) it was
 // 2e-31 for all of them, and a sweep 2 % shorter.  The CTAs per SM are the
@@ -404,22 +404,23 @@ static __device__ __noinline__ void or_gauge_fp64(const Geom& g, MatField<double
   M3<double> M, gx;
   or_local_field<double, ROWS>(g, U, c, s, M);
   or_site_gauge<double>(M, omega, gx);
-  fxg_store(gf, g.V, s, gx.e[0], gx.e[1], gx.e[2]);
+  fxg_store_fp64(gf, g.V, s, gx.e[0], gx.e[1], gx.e[2]);
 }
 
 template <int ROWS>
 __global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 5 : 4)
 or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, double2* __restrict__ G, int parity,
                    FastDiv dhx, double omega, int64_t w7, int64_t c7) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if ((int64_t)j >= (g.V >> 1)) return;
+  const uint32_t j0 = blockIdx.x * blockDim.x + threadIdx.x, n = (uint32_t)(g.V >> 1);
+  const bool in = j0 < n;
   int c[4];
-  const int64_t s = or_coords(g, dhx, j, parity, c);
+  const int64_t s = or_coords(g, dhx, in ? j0 : n - 1, parity, c);  // lanes past the end follow their warp
   // w(x) in units of 2^-59
   int64_t W[9][2];
 #pragma unroll
   for (int e = 0; e < 9; ++e) W[e][0] = W[e][1] = 0;
-  uint32_t m = 0, t = 0, strong = 0;
+  uint32_t m = 0, t = 0;
+  bool near_id = false;
 #pragma unroll 1
   for (int k = 0; k < 8; ++k) {
     const int mu = k >> 1;
@@ -430,6 +431,10 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
     for (int r = 0; r < ROWS; ++r)
 #pragma unroll
       for (int q = 0; q < 3; ++q) u[r][q] = __ldg(&U.p[U.off(mu, r, q, sl)]);
+    if (k == 0 && __any_sync(0xffffffffu, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_NEAR_HI)) {
+      near_id = true;
+      break;
+    }
     int64_t x[3][3][2];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
@@ -439,7 +444,6 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
         x[r][q][0] = fxk_from<59>(u[r][q].x);
         x[r][q][1] = fxk_from<59>(u[r][q].y);
       }
-    strong = max(strong, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]));
     if (ROWS == 2) {
       FxC a[2][3];
 #pragma unroll
@@ -468,11 +472,18 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
       }
     }
   }
+  if (near_id) {
+    if (!in) return;
+    or_gauge_fp64<ROWS>(g, U, s, gf, omega);
+    if (G != nullptr) accumulate_gauge_fp64(g.V, s, reinterpret_cast<const int4*>(gf) + s, g.V, G);
+    return;
+  }
   FxC M[3][3], gx[3][3];
 #pragma unroll
   for (int e = 0; e < 9; ++e) M[e / 3][e % 3] = FxC{fx_operand((W[e][0] + 4) >> 3), fx_operand((W[e][1] + 4) >> 3)};  // w / 16
-  bool ok = !fx_bad(m, t) && strong >= FX_WEAK_HI;
+  bool ok = !fx_bad(m, t);
   or_site_gauge_fx(M, fx_operand(w7), c7, gx, ok);
+  if (!in) return;
   if (ok) {
     int4* p = reinterpret_cast<int4*>(gf);
 #pragma unroll
@@ -483,28 +494,33 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
   if (G != nullptr) accumulate_gauge_fx(g.V, s, reinterpret_cast<const int4*>(gf) + s, g.V, G);
 }
 
-// One link in FP64: fwd ? g U : U g^dag.
+// One link in FP64: fwd ? g U : U g^dag (of which rows 1-2 of the old link suffice).
 template <int ROWS>
 static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const double2* gf, int mu, int64_t sl,
                                                  int64_t s, bool fwd) {
   M3<double> g, u, o;
   fxg_load(gf, U.V, s, g);
-  U.load(mu, sl, u);
+  if (fwd) {
+    U.load(mu, sl, u);
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      double2 acc;
-      if (fwd) {
-        acc = cmul_fx<double>(g.e[i][0], u.e[0][k]);
+      for (int k = 0; k < 3; ++k) {
+        double2 acc = cmul_fx<double>(g.e[i][0], u.e[0][k]);
         acc = cfma<double>(g.e[i][1], u.e[1][k], acc);
         o.e[i][k] = cfma<double>(g.e[i][2], u.e[2][k], acc);
-      } else {
-        acc = cmulc_fx<double>(u.e[i][0], g.e[k][0]);
+      }
+  } else {
+    U.load_rows01(mu, sl, u.e);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        double2 acc = cmulc_fx<double>(u.e[i][0], g.e[k][0]);
         acc = cfmac<double>(u.e[i][1], g.e[k][1], acc);
         o.e[i][k] = cfmac<double>(u.e[i][2], g.e[k][2], acc);
       }
-    }
+  }
   su3_third_row<double>(o.e[0], o.e[1], o.e[2]);
   U.store(mu, sl, o);
 }
@@ -518,12 +534,12 @@ static __device__ __noinline__ void or_link_fp64(MatField<double, ROWS> U, const
 template <int ROWS>
 __global__ void __launch_bounds__(OR_THREADS, 5)
 or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__ gf, int parity, FastDiv dhx) {
-  const uint32_t j = (blockIdx.x >> 1) * 32u + (threadIdx.x & 31u);
+  const uint32_t j0 = (blockIdx.x >> 1) * 32u + (threadIdx.x & 31u), nc = (uint32_t)(g.V >> 1);
+  const bool in = j0 < nc;
   const int mu = threadIdx.x >> 5;
   const bool fwd = (blockIdx.x & 1u) == 0;
-  if ((int64_t)j >= (g.V >> 1)) return;
   int c[4];
-  const int64_t s = or_coords(g, dhx, j, parity, c);
+  const int64_t s = or_coords(g, dhx, in ? j0 : nc - 1, parity, c);  // lanes past the end follow their warp
   const int64_t sl = fwd ? s : or_back(g, s, c, mu);
   const int4* p = reinterpret_cast<const int4*>(gf);
   constexpr int UR = ROWS;
@@ -535,6 +551,11 @@ or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__
     for (int k = 0; k < 3; ++k) u[r][k] = U.p[U.off(mu, r, k, sl)];
 #pragma unroll
   for (int e = 0; e < 9; ++e) g4[e / 3][e % 3] = __ldg(&p[e * g.V + s]);
+  // as the hits' own test, so that most g in FP64 meet links that take FP64
+  if (__any_sync(0xffffffffu, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_NEAR_HI)) {
+    if (in) or_link_fp64<ROWS>(U, gf, mu, sl, s, fwd);
+    return;
+  }
   uint32_t m = 0, t = 0;
   FxC x[3][3];
 #pragma unroll
@@ -544,7 +565,6 @@ or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__
       m = fx_max(m, u[r][k]);
       x[r][k] = fx_from(u[r][k]);
     }
-  const uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
   int64_t n[2][3][2];
   if (fwd) {
     if (ROWS == 2) {
@@ -587,7 +607,8 @@ or_links_fx_kernel(Geom g, MatField<double, ROWS> U, const double2* __restrict__
       for (int k = 0; k < 3; ++k) r[i][k] = FxC{fx_operand(n[i][k][0]), fx_operand(n[i][k][1])};
     fx_third_row(r[0], r[1], n3, t);
   }
-  if (fx_bad(m, t) || w < FX_WEAK_HI || g4[0][0].x == FX_G_NAN) {
+  if (!in) return;
+  if (fx_bad(m, t) || fxg_is_fp64(g4[0][0])) {
     or_link_fp64<ROWS>(U, gf, mu, sl, s, fwd);
     return;
   }

@@ -49,10 +49,11 @@ __device__ __forceinline__ double warp_value(int64_t q, uint32_t e) {
 
 // Block reduction of two sums (fixed order) and a maximum of values >= 0 (FP32:
 // the link defect is compared with bounds far above FP32 resolution; a NaN
-// counts as 0); result valid in thread 0.  At most 16 warps.
-__device__ __forceinline__ void block_reduce3(double& a, double& b, float& m) {
+// counts as 0), and of the warps' counts k; result valid in thread 0.  At most
+// 16 warps.
+__device__ __forceinline__ void block_reduce3(double& a, double& b, float& m, uint32_t& k) {
   __shared__ double sums[2][16];
-  __shared__ uint32_t sm[16];
+  __shared__ uint32_t sm[16], sk[16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t ea, eb;
   int64_t qa = warp_align(a, ea), qb = warp_align(b, eb);
@@ -70,12 +71,16 @@ __device__ __forceinline__ void block_reduce3(double& a, double& b, float& m) {
     if (lane < 2) sums[lane][warp] = v;
   }
   const uint32_t mw = __reduce_max_sync(0xffffffffu, m > 0.f ? __float_as_uint(m) : 0u);
-  if (lane == 0) sm[warp] = mw;
+  if (lane == 0) {
+    sm[warp] = mw;
+    sk[warp] = k;
+  }
   __syncthreads();
   if (warp == 0) {
     const int w = lane & 15;
     double v = w < nw ? sums[lane >> 4][w] : 0.0;
     m = __uint_as_float(__reduce_max_sync(0xffffffffu, w < nw ? sm[w] : 0u));
+    k = __reduce_add_sync(0xffffffffu, lane < nw ? sk[lane] : 0u);
     if (nw > 8) v += __shfl_xor_sync(0xffffffffu, v, 8);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -116,22 +121,27 @@ __device__ __forceinline__ int defect_sample_mu(int64_t s) {
 // also flips st->ubuf (after every CTA has read it); fp64 != 0 marks the
 // measurement as one of FP64 links in the trace flags.
 // fsum and tsum are the sums over the sites a thread collected, in FP64; every
-// sum above a site (thread, warp, CTA, grid) is FP64 in a fixed order.
+// sum above a site (thread, warp, CTA, grid) is FP64 in a fixed order.  near_id:
+// the warp's links are near the identity (FP64 links, the same in every lane);
+// st->near_id is set where more than half of the warps' are.
 __device__ __forceinline__ void measure_tail(const Geom& g, double fsum, double tsum, float dmax,
                                              double* __restrict__ partials, DevState* __restrict__ st, int count_iter,
                                              unsigned long long cond, int use_cond, bool batch, int flip_ubuf,
-                                             int fp64, unsigned long long cond_undo) {
+                                             int fp64, unsigned long long cond_undo, bool near_id) {
   double fb = fsum, tb = tsum;
   float db = dmax;
-  block_reduce3(fb, tb, db);
+  uint32_t kb = near_id ? 1u : 0u;
+  block_reduce3(fb, tb, db, kb);
+  __shared__ uint32_t near_warps;
   __shared__ int is_last;
   if (threadIdx.x == 0) {
     partials[MEASURE_PARTIALS * blockIdx.x] = fb;
     partials[MEASURE_PARTIALS * blockIdx.x + 1] = tb;
     partials[MEASURE_PARTIALS * blockIdx.x + 2] = (double)db;
     __threadfence();
-    const unsigned int t = atomicAdd(&st->ticket, 1u);
-    is_last = (t == gridDim.x - 1);
+    const unsigned long long t = atomicAdd(&st->ticket, 1ull | ((unsigned long long)kb << 32));
+    is_last = ((uint32_t)t == gridDim.x - 1);
+    near_warps = (uint32_t)(t >> 32) + kb;
   }
   __syncthreads();
   if (!is_last) return;
@@ -146,7 +156,7 @@ __device__ __forceinline__ void measure_tail(const Geom& g, double fsum, double 
     t += __ldcg(&partials[MEASURE_PARTIALS * i + 1]);
     d = fmaxf(d, (float)__ldcg(&partials[MEASURE_PARTIALS * i + 2]));
   }
-  block_reduce3(f, t, d);
+  block_reduce3(f, t, d, kb);
   if (threadIdx.x == 0) {
     const double Vd = (double)g.V;
     const double F = f / (12.0 * Vd);
@@ -193,7 +203,8 @@ __device__ __forceinline__ void measure_tail(const Geom& g, double fsum, double 
     if (!finite) st->status = ST_NONFINITE;
     else if (!sound) st->status = ST_DEFECT;
     if (flip_ubuf) st->ubuf ^= 1;
-    st->ticket = 0u;
+    st->ticket = 0ull;
+    st->near_id = 2u * near_warps > gridDim.x * (blockDim.x >> 5) ? 1 : 0;
     if (batch) st->done = !(finite && th >= st->tol && it < st->max_iter);
     if (use_cond) {
       cudaGraphConditionalHandle h = (cudaGraphConditionalHandle)cond;
@@ -319,6 +330,12 @@ template <bool SPLIT> struct MeasurePlace {
       join(o.w01.x); join(o.w01.y); join(o.w02.x); join(o.w02.y); join(o.w12.x); join(o.w12.y);
     }
   }
+  static __device__ __forceinline__ void join(SiteSums<double>& o) {
+    if (SPLIT) {
+      join(o.f); join(o.im0); join(o.im1); join(o.im2);
+      join(o.w01.x); join(o.w01.y); join(o.w02.x); join(o.w02.y); join(o.w12.x); join(o.w12.y);
+    }
+  }
 };
 
 // Delta of a site, stored, and its part of theta.
@@ -337,18 +354,22 @@ __device__ __forceinline__ double store_delta(const SiteSums<R>& o, C2<R>* __res
   else return n;
 }
 
-// The FP64 path of a site with links outside the fixed-point range.
-template <int ROWS>
-__device__ __noinline__ void site_sums_fp64(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+// A site's sums over its directions mu0 <= mu < mu0 + NMU in FP64: links near the
+// identity and entries outside the fixed-point range.
+template <int ROWS, int NMU>
+__device__ __noinline__ void site_sums_fp64(const Geom& g, const MatField<double, ROWS>& U, int64_t s, int mu0,
                                             SiteSums<double>& o) {
   int c[4];
   site_coords(g, s, c);
   o = site_sums_zero<double>();
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
+  for (int k = 0; k < NMU; ++k) {
+    const int mu = mu0 + k;
+    int64_t sf, sb;
+    site_nbrs_sel(g, s, c, mu, sf, sb);
     M3<double> u, b;
     U.load_ro(mu, s, u);
-    U.load_ro(mu, site_back(g, s, c, mu), b);
+    U.load_ro(mu, sb, b);
     add_own<double>(o, link_terms<double>(u));
     add_back<double>(o, link_terms<double>(b));
   }
@@ -358,14 +379,13 @@ __device__ __noinline__ void site_sums_fp64(const Geom& g, const MatField<double
 // pipe: exact but for what lies below 2^-58 in an entry, against one FP64
 // rounding per addition (2^-54 for sums of order one).  12-real links rebuild
 // row 3 in fixed point as well.
-// t[0]: trace; t[1..3]: Im W_ii; t[4..9]: W_01, W_02, W_12; bad, strong: range
-// tests (an entry outside it; high words of the anti-symmetric real parts,
-// or-ed).
+// t[0]: trace; t[1..3]: Im W_ii; t[4..9]: W_01, W_02, W_12; bad: an entry outside
+// the range.  Returns false, for the whole warp, where the site's own link of
+// direction mu0 is near the identity in any lane (FX_NEAR_HI).
 constexpr int FX_TERMS = 10;
 template <int ROWS>
-__device__ __forceinline__ void site_terms_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
-                                              const int c[4], int mu0, int mu1, int64_t t[FX_TERMS], uint32_t& bad,
-                                              uint32_t& strong) {
+__device__ __forceinline__ bool site_terms_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
+                                              const int c[4], int mu0, int mu1, int64_t t[FX_TERMS], uint32_t& bad) {
   uint32_t m = 0, big = 0;
 #pragma unroll 1
   for (int k = 2 * mu0; k < 2 * mu1; ++k) {
@@ -381,6 +401,9 @@ __device__ __forceinline__ void site_terms_fx(const Geom& g, const MatField<doub
         e[r][j] = __ldg(&U.p[U.off(mu, r, j, own ? s : sb)]);
         m = fx_max(m, e[r][j]);
       }
+    if (k == 2 * mu0 &&
+        __any_sync(0xffffffffu, fx_max(fx_max(fx_max(0u, e[0][1]), e[0][2]), e[1][2]) < FX_NEAR_HI))
+      return false;
     int64_t x[FX_TERMS];
     x[0] = 0;
     x[1] = fx58_from(e[0][0].y);
@@ -420,8 +443,6 @@ __device__ __forceinline__ void site_terms_fx(const Geom& g, const MatField<doub
       x[8] = q[1][2][0] - z[1][0];
       x[9] = q[1][2][1] + z[1][1];
     }
-#pragma unroll
-    for (int i = 4; i < FX_TERMS; i += 2) strong |= (uint32_t)(x[i] >> 32) ^ (uint32_t)(x[i] >> 63);
     t[0] += x[0];
     if (own) {
 #pragma unroll
@@ -432,18 +453,16 @@ __device__ __forceinline__ void site_terms_fx(const Geom& g, const MatField<doub
     }
   }
   bad = fx_bad(m, big);
+  return true;
 }
 
-// A site's sums from its directions' terms t.  Where the anti-symmetric real
-// parts of all eight links are below 2^-12 (a field near the identity), FP64
-// sums are relative to numbers that small and round finer than 2^-58: that site
-// takes the FP64 path, as do entries outside the fixed-point range.
+// A site's sums from its directions' terms t; entries outside the fixed-point
+// range take the FP64 path.
 template <int ROWS>
 __device__ __forceinline__ void site_sums_fx(const Geom& g, const MatField<double, ROWS>& U, int64_t s,
-                                             const int64_t t[FX_TERMS], bool bad, uint32_t strong,
-                                             SiteSums<double>& o) {
-  if (bad || strong < (1u << (58 - 12 - 32))) {
-    site_sums_fp64<ROWS>(g, U, s, o);
+                                             const int64_t t[FX_TERMS], bool bad, SiteSums<double>& o) {
+  if (bad) {
+    site_sums_fp64<ROWS, 4>(g, U, s, 0, o);
     return;
   }
   o.f = fx_to_double_fp<58>(t[0]);
@@ -457,8 +476,8 @@ __device__ __forceinline__ void site_sums_fx(const Geom& g, const MatField<doubl
 
 // FP64 links are bound by the ALU pipe (66 % busy in ncu) beside HBM (40 %) and
 // the FP64 pipe (41 %: the sites' conversions and norms).
-// 32^4: 18-real 195 us (FP64 sums on the FP64 pipe: 355 us), 12-real 265 us
-// (665 us).
+// 32^4: 18-real 194 us (FP64 sums on the FP64 pipe: 355 us), 12-real 272 us
+// (665 us); fields near the identity, whose warps take FP64 sums, 344 and 656 us.
 template <typename R, int ROWS, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? MEASURE_SPLIT_THREADS : MEASURE_THREADS,
                                   SPLIT ? 1 : sizeof(R) == sizeof(float) ? 5 : ROWS == 3 ? 3 : 2)
@@ -483,19 +502,25 @@ measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt,
   double fsum = 0, tsum = 0;
   float dmax = 0.f;
   int c[4];
-  if (in) site_coords(g, p.s, c);
+  const int64_t sc = in ? p.s : g.V - 1;  // lanes past the end follow their warp
+  site_coords(g, sc, c);
+  bool near_id = false;
   // W = sum_mu [U_mu(x - mu^) - U_mu(x)]; only the entries that enter its
   // traceless anti-Hermitian part are accumulated.
   SiteSums<R> o = site_sums_zero<R>();
   if constexpr (sizeof(R) == sizeof(double)) {
     int64_t t[FX_TERMS] = {};
-    uint32_t bad = 0, strong = 0;
-    if (in) site_terms_fx<ROWS>(g, U, p.s, c, p.mu0, p.mu1, t, bad, strong);
+    uint32_t bad = 0;
+    near_id = !site_terms_fx<ROWS>(g, U, sc, c, p.mu0, p.mu1, t, bad);
+    if (!near_id) {
 #pragma unroll
-    for (int i = 0; i < FX_TERMS; ++i) p.join(t[i]);
-    p.join_or(bad);
-    p.join_or(strong);
-    if (in && p.collects()) site_sums_fx<ROWS>(g, U, p.s, t, bad != 0, strong, o);
+      for (int i = 0; i < FX_TERMS; ++i) p.join(t[i]);
+      p.join_or(bad);
+      if (in && p.collects()) site_sums_fx<ROWS>(g, U, p.s, t, bad != 0, o);
+    } else {
+      site_sums_fp64<ROWS, SPLIT ? 1 : 4>(g, U, sc, p.mu0, o);
+      p.join(o);
+    }
   } else {
     if (in) {
 #pragma unroll
@@ -522,7 +547,8 @@ measure_kernel(Geom g, MatField<R, ROWS> U, const C2<R>* __restrict__ links_alt,
       dmax = rows_defect<R>(rows[0], rows[1]);
     }
   }
-  measure_tail(g, fsum, tsum, dmax, partials, st, count_iter, cond, use_cond, batch, 0, sizeof(R) == 8, cond_undo);
+  measure_tail(g, fsum, tsum, dmax, partials, st, count_iter, cond, use_cond, batch, 0, sizeof(R) == 8, cond_undo,
+               near_id);
 }
 
 template <typename R, int ROWS>
@@ -619,7 +645,7 @@ update_measure_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, Ma
     fsum = sum_f(o);
     tsum = store_delta<R>(o, delta, g.V, p.s);
   }
-  measure_tail(g, fsum, tsum, dmax, partials, st, 1, cond, use_cond, false, 1, sizeof(R) == 8, cond_undo);
+  measure_tail(g, fsum, tsum, dmax, partials, st, 1, cond, use_cond, false, 1, sizeof(R) == 8, cond_undo, false);
 }
 
 template <typename R, int LROWS, int GROWS>
@@ -703,7 +729,7 @@ update_kernel(Geom g, MatField<R, LROWS> U, MatField<R, GROWS> Gf, Batch B) {
   }
 }
 
-// The FP64 path of one link outside the fixed-point range.
+// The FP64 path of one link: near the identity, or outside the fixed-point range.
 template <int LROWS>
 __device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatField<double, 3> Gf, int mu, int64_t s,
                                               int64_t sf) {
@@ -717,26 +743,31 @@ __device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatFiel
 
 // FP64 links: the two products and row 3 in fixed point on the integer pipe
 // (lgf_fixed.cuh); g arrives as operands.
-// Links whose off-diagonal entries are all below 2^-12, where FP64 rounds
-// finer than the fixed-point unit, and entries outside its range take the
-// FP64 path.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
+// Fields near the identity (DevState::near_id) and warps with such links
+// (FX_WEAK_HI) take FP64 before any arithmetic; links that meet a g in FP64 or
+// have entries outside the fixed-point range take it after.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
 // end at 2.4e-15 (FP64 products: 2.6e-15).
 // Bound by the integer pipe (1850 instructions a link, 504 of them IMAD.WIDE,
 // which run at about 30 of their 64 lanes a clock when all operands vary).
-// 32^4, us: 18-real 381, 12-real 346; with FP64 products 1176 and 1177 at 95 %
-// of the FP64 pipe.
+// 32^4, us: 18-real 379, 12-real 338; with FP64 products 1176 and 1177 at 95 %
+// of the FP64 pipe (fields near the identity: 1191 and 1182).
 // One thread per link: a CTA takes 32 sites, one direction per warp, so that
-// the 24 operand loads of a link are all in flight before its arithmetic and
-// g(x) comes from L1 for three of the four warps.
+// the operand loads of a link are all in flight before its arithmetic and g(x)
+// comes from L1 for three of the four warps.  The test for links near the
+// identity stands between the loads of the link and those of g: after both it
+// held all 24 in registers (393 us), and the CTAs of an SM hide the wait.
 template <int LROWS>
 __global__ void __launch_bounds__(UPDATE_THREADS, 5)
-update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batch B) {
+update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, const DevState* __restrict__ st,
+                 Batch B) {
   if (batch_skip(B)) return;
+  const bool near_id = near_identity(st, B);
   U.p += blockIdx.z * B.s_links;
   Gf.p += blockIdx.z * B.s_g;
-  const int64_t s = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int64_t s0 = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int64_t s = min(s0, g.V - 1);  // lanes past the end follow their warp
+  const bool in = s0 < g.V;
   const int mu = threadIdx.x >> 5;
-  if (s >= g.V) return;
   int c[4];
   site_coords(g, s, c);
   int64_t sf, sb;
@@ -748,6 +779,11 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
   for (int i = 0; i < LROWS; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) u[i][j] = U.p[U.off(mu, i, j, s)];
+  if (__any_sync(0xffffffffu,
+                 near_id || fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_WEAK_HI)) {
+    if (in) update_link_fp64<LROWS>(U, Gf, mu, s, sf);
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -761,7 +797,6 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
   for (int i = 0; i < LROWS; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) m = fx_max(m, u[i][j]);
-  const uint32_t w = fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]);
   // T = g(x)[rows 0,1] U
   FxC T[2][3], ux[3][3];
 #pragma unroll
@@ -809,7 +844,8 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
       for (int j = 0; j < 3; ++j) r[i][j] = FxC{fx_operand(n[i][j][0]), fx_operand(n[i][j][1])};
     fx_third_row(r[0], r[1], n3, t);
   }
-  if (fx_bad(m, t) || w < FX_WEAK_HI || g4[0][0].x == FX_G_NAN || h4[0][0].x == FX_G_NAN) {
+  if (!in) return;
+  if (fx_bad(m, t) || fxg_is_fp64(g4[0][0]) || fxg_is_fp64(h4[0][0])) {
     update_link_fp64<LROWS>(U, Gf, mu, s, sf);
     return;
   }
@@ -822,7 +858,8 @@ update_fx_kernel(Geom g, MatField<double, LROWS> U, MatField<double, 3> Gf, Batc
 }
 
 template <typename R, int LROWS, int GROWS>
-cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cudaStream_t s, const Batch& B) {
+cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, const DevState* st, cudaStream_t s,
+                          const Batch& B) {
   MatField<R, LROWS> U{links, g.V};
   MatField<R, GROWS> Gf{const_cast<C2<R>*>(gfield), g.V};
   const int64_t nb = (g.V + UPDATE_THREADS - 1) / UPDATE_THREADS;
@@ -830,7 +867,7 @@ cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cuda
   if constexpr (sizeof(R) == sizeof(double)) {
     static_assert(GROWS == 3, "FP64 lanes keep three rows of g");
     const dim3 fx_grid((unsigned)((g.V + 31) / 32), 1, (unsigned)B.n);
-    update_fx_kernel<LROWS><<<fx_grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
+    update_fx_kernel<LROWS><<<fx_grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, st, B);
   } else {
     update_kernel<R, LROWS, GROWS><<<grid, UPDATE_THREADS, 0, s>>>(g, U, Gf, B);
   }
@@ -841,7 +878,7 @@ cudaError_t launch_update(const Geom& g, C2<R>* links, const C2<R>* gfield, cuda
 // undo of a rejected step: U_mu(x) <- g^dag(x) U_mu(x) g(x + mu^), G <- g^dag G
 // ---------------------------------------------------------------------------
 
-// g(s) of a lane as a matrix (FP64 lanes keep it as fixed-point operands).
+// g(s) of a lane as a matrix (lgf_fixed.cuh has the forms of FP64 lanes).
 template <int GROWS>
 __device__ __forceinline__ void load_g(const MatField<float, GROWS>& Gf, int64_t s, M3<float>& M) {
   Gf.load_ro(0, s, M);
@@ -1348,9 +1385,11 @@ cudaError_t launch_c2_f32_to_f64(const float2* in, double2* out, int64_t n, cuda
 }
 
 // Gram-Schmidt projection of rows 1-2 to SU(3) in FP64, row 3 = (a x b)^*,
-// as g of the FP64 lane and, where it tracks the transform, as its G.
-__global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, double2* __restrict__ gf,
-                                     double2* __restrict__ out) {
+// as g of the FP64 lane and, where it tracks the transform, as its G.  links: the
+// input links (user layout) that g is about to transform; near the identity it
+// is kept in FP64.
+__global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, const double2* __restrict__ links,
+                                     double2* __restrict__ gf, double2* __restrict__ out) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
   double2 a[3], b[3], c[3];
@@ -1373,7 +1412,14 @@ __global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, d
 #pragma unroll
   for (int j = 0; j < 3; ++j) b[j] = cscale<double>(b[j], ib);
   su3_third_row<double>(a, b, c);
-  fxg_store(gf, V, s, a, b, c);
+  bool near_id = false;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const double2* u = links + (mu * V + s) * 9;
+    near_id = near_id || fx_max(fx_max(fx_max(0u, __ldg(u + 1)), __ldg(u + 2)), __ldg(u + 5)) < FX_NEAR_HI;
+  }
+  if (near_id) fxg_store_fp64(gf, V, s, a, b, c);
+  else fxg_store(gf, V, s, a, b, c);
   if (out == nullptr) return;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
@@ -1383,10 +1429,10 @@ __global__ void project_sites_kernel(int64_t V, const float2* __restrict__ in, d
   }
 }
 
-cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, double2* gfield, double2* G64,
-                                            cudaStream_t s) {
-  project_sites_kernel<<<(unsigned)((g.V + CONV_THREADS - 1) / CONV_THREADS), CONV_THREADS, 0, s>>>(g.V, G32, gfield,
-                                                                                                    G64);
+cudaError_t launch_project_sites_f32_to_f64(const Geom& g, const float2* G32, const double* links, double2* gfield,
+                                            double2* G64, cudaStream_t s) {
+  project_sites_kernel<<<(unsigned)((g.V + CONV_THREADS - 1) / CONV_THREADS), CONV_THREADS, 0, s>>>(
+      g.V, G32, reinterpret_cast<const double2*>(links), gfield, G64);
   return cudaGetLastError();
 }
 
@@ -1418,10 +1464,14 @@ template cudaError_t launch_revert<float, 2, 2>(const Geom&, C2<float>*, const C
                                                  const DevState*, cudaStream_t, C2<float>*);
 template cudaError_t launch_revert<float, 3, 3>(const Geom&, C2<float>*, const C2<float>*, C2<float>*,
                                                  const DevState*, cudaStream_t, C2<float>*);
-template cudaError_t launch_update<double, 3, 3>(const Geom&, C2<double>*, const C2<double>*, cudaStream_t, const Batch&);
-template cudaError_t launch_update<double, 2, 3>(const Geom&, C2<double>*, const C2<double>*, cudaStream_t, const Batch&);
-template cudaError_t launch_update<float, 2, 2>(const Geom&, C2<float>*, const C2<float>*, cudaStream_t, const Batch&);
-template cudaError_t launch_update<float, 3, 3>(const Geom&, C2<float>*, const C2<float>*, cudaStream_t, const Batch&);
+template cudaError_t launch_update<double, 3, 3>(const Geom&, C2<double>*, const C2<double>*, const DevState*,
+                                                 cudaStream_t, const Batch&);
+template cudaError_t launch_update<double, 2, 3>(const Geom&, C2<double>*, const C2<double>*, const DevState*,
+                                                 cudaStream_t, const Batch&);
+template cudaError_t launch_update<float, 2, 2>(const Geom&, C2<float>*, const C2<float>*, const DevState*,
+                                                 cudaStream_t, const Batch&);
+template cudaError_t launch_update<float, 3, 3>(const Geom&, C2<float>*, const C2<float>*, const DevState*,
+                                                 cudaStream_t, const Batch&);
 #define LGF_INST_UM(R, LR, GR)                                                                                     \
   template cudaError_t launch_update_measure<R, LR, GR>(const Geom&, C2<R>*, C2<R>*, const C2<R>*, C2<R>*, double*, \
                                                         DevState*, unsigned long long, int, cudaStream_t,          \

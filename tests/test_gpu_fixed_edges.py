@@ -280,3 +280,127 @@ def test_or_converges_as_far_as_fp64(eps, fp64, store12):
             lat.or_sweep(1.7, 1)
             theta.append(lat.measure()[1])
     assert np.median(theta) < 1.1 * fp64
+
+
+# ---------------------------------------------------------------------------
+# fields near the identity
+# ---------------------------------------------------------------------------
+
+def near(ext, eps, seed=4):
+    return fields.random_links(ext, eps, seed=seed, gauge_rotate=False)
+
+
+def floor_of_fix(ext, U, **kw):
+    """theta after 250 steps, the median of the last 50."""
+    decomposition = kw.pop("decomposition", None)
+    with lgf.Lattice(ext, "fp64", **kw) as lat:
+        if decomposition:
+            lat.set_fft_decomposition(decomposition)
+        lat.set_links(U)
+        _, T = lat.set_trace(260)
+        lat.fix(0.0, 250, 0.08)
+    return np.median(T[200:250])
+
+
+FORMS = [dict(), dict(store12=True), dict(exact_exp=True), dict(decomposition="1d4"), dict(track_G=True)]
+
+
+@pytest.mark.parametrize("kw", FORMS, ids=lambda kw: "-".join(kw) or "plain")
+@pytest.mark.parametrize("eps, fp64", [(1e-9, 3.9e-49), (1e-5, 3.8e-41), (1e-3, 3.9e-37), (0.03, 3.5e-34),
+                                       (0.06, 1.4e-33), (0.12, 5.4e-33)])
+def test_fix_near_the_identity_converges_as_far_as_fp64(eps, fp64, kw):
+    """theta of 8^4 levels off no higher (10 %) than it does with every product and g in FP64 arithmetic."""
+    ext = (8, 8, 8, 8)
+    assert floor_of_fix(ext, near(ext, eps), **kw) < 1.1 * fp64
+
+
+@pytest.mark.parametrize("store12", [False, True])
+@pytest.mark.parametrize("eps, fp64", [(1e-9, 4.2e-49), (1e-5, 4.1e-41), (1e-3, 4.2e-37), (0.03, 3.9e-34),
+                                       (0.06, 1.56e-33), (0.12, 6.3e-33)])
+def test_or_near_the_identity_converges_as_far_as_fp64(eps, fp64, store12):
+    ext = (8, 8, 8, 8)
+    with lgf.Lattice(ext, "fp64", store12=store12) as lat:
+        lat.set_links(near(ext, eps))
+        lat.or_sweep(1.7, 1200)
+        theta = []
+        for _ in range(9):
+            lat.or_sweep(1.7, 1)
+            theta.append(lat.measure()[1])
+    assert np.median(theta) < 1.1 * fp64
+
+
+@pytest.mark.parametrize("ext", [(2, 2, 2, 2), (3, 4, 6, 9), (8, 8, 8, 8)])
+@pytest.mark.parametrize("eps", [1e-9, 1e-4])
+def test_gauge_near_the_identity_keeps_its_digits(eps, ext):
+    """g - 1 of one step, of the size of eps, to the relative error of FP64 sums (1e-12 of its largest entry)."""
+    U = near(ext, eps)
+    D = O.divergence(U)
+    go = O.gauge_transform_from_divergence(D, O.fa_filter(ext, 0.08))
+    with lgf.Lattice(ext, "fp64") as lat:
+        lat.set_links(U)
+        lat.step(0.08)
+        g = lat.get_gauge()
+    off = ~np.eye(3, dtype=bool)
+    assert np.max(np.abs(g - go)[..., off]) < 1e-12 * np.max(np.abs(go)[..., off])
+
+
+PATCHES = {
+    # warps of one kind, warps of both, single links
+    "half": lambda x, y, z, t, mu: t < 1,
+    "stripes": lambda x, y, z, t, mu: (x + y + z + t) % 2 == 0,
+    "links": lambda x, y, z, t, mu: (x + 3 * y + 5 * z + 7 * t + mu) % 7 == 0,
+}
+
+
+@pytest.mark.parametrize("store12", [False, True])
+@pytest.mark.parametrize("name", list(PATCHES))
+@pytest.mark.parametrize("ext", [(2, 2, 2, 2), (6, 4, 2, 8), (8, 8, 6, 4), (32, 24, 6, 8)])
+def test_fields_partly_near_the_identity(ext, name, store12):
+    """Rough links with patches of links 1 + O(1e-6): measurement, step, transform and sweep against the oracle, with
+    the bounds of the rough links (test_gpu_fixed.py)."""
+    from oracle import lgf_or_oracle as R
+    lx, ly, lz, lt = ext
+    t, z, y, x = np.meshgrid(*(np.arange(n) for n in (lt, lz, ly, lx)), indexing="ij")
+    U, W = fields.random_links(ext, 0.9, seed=3), near(ext, 1e-6)
+    for mu in range(4):
+        U[mu] = np.where(PATCHES[name](x, y, z, t, mu)[..., None, None], W[mu], U[mu])
+    Us = U.copy()
+    if store12:
+        Us[..., 2, :] = np.conj(np.cross(U[..., 0, :], U[..., 1, :]))
+    Fo, tho, Do = O.measure(Us)
+    with lgf.Lattice(ext, "fp64", store12=store12, track_G=True) as lat:
+        lat.set_links(U)
+        F, th = lat.measure()
+        D = lat.get_divergence()
+        lat.step(0.08)
+        g, U1, G1 = lat.get_gauge(), lat.get_links(), lat.get_transform()
+        lat.set_links(U)
+        lat.or_sweep(1.7, 1)
+        U2, G2 = lat.get_links(), lat.get_transform()
+    assert np.max(np.abs(D - Do)) < 4e-15 and abs(F - Fo) < 4e-15 and abs(th - tho) < 1e-13 * tho
+    want = O.apply_gauge(Us, g)
+    want[..., 2, :] = np.conj(np.cross(want[..., 0, :], want[..., 1, :]))
+    assert np.max(np.abs(U1 - want)) < 2e-15
+    assert np.max(np.abs(G1 - g)) < 2e-15
+    Uo, Go = R.or_sweep(U, 1.7)
+    assert np.max(np.abs(U2 - Uo)) < 1e-12 and np.max(np.abs(G2 - Go)) < 1e-12
+
+
+def test_batch_and_mixed_near_the_identity():
+    """A batch takes the steps of single handles to theta < 1e-38, and a mixed fix reaches it too."""
+    exts = [(4, 4, 4, 4), (3, 4, 6, 9), (4, 4, 4, 4)]
+    Us = [near(e, eps, seed=i) for i, (e, eps) in enumerate(zip(exts, (1e-5, 1e-5, 3e-6)))]
+    with lgf.Batch(exts) as b:
+        for i, U in enumerate(Us):
+            b.set_links(i, U)
+        it, F, th, conv = b.fix(1e-38, 400)
+        links = [b.get_links(i) for i in range(3)]
+    assert conv
+    for i, (e, U) in enumerate(zip(exts, Us)):
+        with lgf.Lattice(e, "fp64") as lat:
+            lat.set_links(U)
+            it1, F1, th1, conv1 = lat.fix(1e-38, 400, 0.08)
+            assert conv1 and it1 == it[i] and np.array_equal(lat.get_links(), links[i])
+        with lgf.Lattice(e, "mixed", store12=True) as lat:
+            lat.set_links(U)
+            assert lat.fix(1e-38, 400, 0.08)[3]
