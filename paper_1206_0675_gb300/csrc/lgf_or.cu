@@ -17,15 +17,17 @@
 // Every link joins two sites of opposite colour, so within one colour each
 // link is read and written by exactly one thread: the update is in place.
 //
-// FP32 links: one thread per site of the colour, its eight links loaded at once
-// (48 loads in flight) and kept in registers from w to the products, at 168
-// registers and 12 warps per SM.  Reading them one by one, and again for the
-// products, left the warps waiting for loads (14 of 19 cycles between
-// instructions): 32^4 12-real 188 -> 148 us a sweep (118 us for its bytes at
-// 6.8 TB/s), 18-real 295 -> 273 us, 16^4 12-real 20.4 -> 16.4 us; at 128
-// registers 210 us, at 255 170 us.  The site algebra runs in the link
-// precision; rows 1-2 of every product are formed and row 3 is rebuilt as
-// (a x b)^* (Sec. 3.2), as in the Fourier-accelerated update.
+// FP32 links: one thread per site of the colour.  12-real links: its eight links
+// loaded at once (48 loads in flight) and kept in registers from w to the
+// products, at 168 registers and 12 warps per SM.  Reading them one by one, and
+// again for the products, left the warps waiting for loads (14 of 19 cycles
+// between instructions): 32^4 188 -> 148 us a sweep (118 us for its bytes at
+// 6.8 TB/s), 16^4 20.4 -> 16.4 us; at 128 registers 210 us, at 255 170 us.  18-real
+// links do not fit 168 registers (284 bytes of spills), so theirs are read again,
+// at 82 registers: 32^4 267 us against 275 kept, 24^4 87 against 91, 16^3x32 41
+// against 45.  The site algebra runs in the link precision; rows 1-2 of every
+// product are formed and row 3 is rebuilt as (a x b)^* (Sec. 3.2), as in the
+// Fourier-accelerated update.
 #include <cmath>
 
 #include "lgf_fixed.cuh"
@@ -182,6 +184,56 @@ __device__ __forceinline__ void or_local_field(const Geom& g, const MatField<R, 
   }
 }
 
+// U_mu(x) <- g U_mu(x): rows 0, 1 by products, row 2 = (row0 x row1)^*
+template <typename R, int ROWS>
+__device__ __forceinline__ void or_own_link(const MatField<R, ROWS>& U, int mu, int64_t s, const M3<R>& gx,
+                                            const C2<R> (&f)[3][3]) {
+  M3<R> o;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      C2<R> acc = cmul_fx<R>(gx.e[i][0], f[0][k]);
+      acc = cfma<R>(gx.e[i][1], f[1][k], acc);
+      o.e[i][k] = cfma<R>(gx.e[i][2], f[2][k], acc);
+    }
+  su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
+  U.store(mu, s, o);
+}
+// U_mu(x - mu^) <- U_mu(x - mu^) g^dag: rows 0, 1 of the old link suffice
+template <typename R, int ROWS>
+__device__ __forceinline__ void or_back_link(const MatField<R, ROWS>& U, int mu, int64_t sb, const M3<R>& gx,
+                                             const C2<R> (*b)[3]) {
+  M3<R> o;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      C2<R> acc = cmulc_fx<R>(b[i][0], gx.e[k][0]);
+      acc = cfmac<R>(b[i][1], gx.e[k][1], acc);
+      o.e[i][k] = cfmac<R>(b[i][2], gx.e[k][2], acc);
+    }
+  su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
+  U.store(mu, sb, o);
+}
+// G(x) <- g(x) G(x), full 3x3
+template <typename R>
+__device__ __forceinline__ void or_transform(C2<R>* __restrict__ G, int64_t V, int64_t s, const M3<R>& gx) {
+  if (G == nullptr) return;
+  const MatField<R, 3> Gf{G, V};
+  M3<R> Go, Gn;
+  Gf.load(0, s, Go);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      C2<R> acc = cmul<R>(gx.e[i][0], Go.e[0][k]);
+      acc = cfma<R>(gx.e[i][1], Go.e[1][k], acc);
+      Gn.e[i][k] = cfma<R>(gx.e[i][2], Go.e[2][k], acc);
+    }
+  Gf.store(0, s, Gn);
+}
+
 // One site of the colour: its hit and the products with its eight links, which
 // stay in registers from one use to the other (of the links that end in the
 // site, rows 1 and 2).
@@ -217,55 +269,38 @@ __device__ __forceinline__ void or_site(const Geom& g, const MatField<R, ROWS>& 
   }
   M3<R> gx;
   or_site_gauge<R>(M, omega, gx);
-
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
-    // U_mu(x) <- g U_mu(x): rows 0, 1 by products, row 2 = (row0 x row1)^*
     C2<R> f[3][3];
-    M3<R> o;
     u[mu].full(f);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        C2<R> acc = cmul_fx<R>(gx.e[i][0], f[0][k]);
-        acc = cfma<R>(gx.e[i][1], f[1][k], acc);
-        o.e[i][k] = cfma<R>(gx.e[i][2], f[2][k], acc);
-      }
-    su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
-    U.store(mu, s, o);
-    // U_mu(x - mu^) <- U_mu(x - mu^) g^dag: rows 0, 1 of the old link suffice
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        C2<R> acc = cmulc_fx<R>(b[mu].e[i][0], gx.e[k][0]);
-        acc = cfmac<R>(b[mu].e[i][1], gx.e[k][1], acc);
-        o.e[i][k] = cfmac<R>(b[mu].e[i][2], gx.e[k][2], acc);
-      }
-    su3_third_row<R>(o.e[0], o.e[1], o.e[2]);
-    U.store(mu, sb[mu], o);
+    or_own_link<R, ROWS>(U, mu, s, gx, f);
+    or_back_link<R, ROWS>(U, mu, sb[mu], gx, b[mu].e);
   }
+  or_transform<R>(G, g.V, s, gx);
+}
 
-  if (G != nullptr) {
-    // G(x) <- g(x) G(x), full 3x3
-    const MatField<R, 3> Gf{G, g.V};
-    M3<R> Go, Gn;
-    Gf.load(0, s, Go);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        C2<R> acc = cmul<R>(gx.e[i][0], Go.e[0][k]);
-        acc = cfma<R>(gx.e[i][1], Go.e[1][k], acc);
-        Gn.e[i][k] = cfma<R>(gx.e[i][2], Go.e[2][k], acc);
-      }
-    Gf.store(0, s, Gn);
+// The same with the links read again for the products (18-real links).
+template <typename R, int ROWS>
+__device__ __forceinline__ void or_site_reread(const Geom& g, const MatField<R, ROWS>& U, const int c[4], int64_t s,
+                                               C2<R>* __restrict__ G, R omega) {
+  M3<R> M, gx;
+  or_local_field<R, ROWS>(g, U, c, s, M);
+  or_site_gauge<R>(M, omega, gx);
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    M3<R> u;
+    U.load(mu, s, u);
+    or_own_link<R, ROWS>(U, mu, s, gx, u.e);
+    const int64_t sb = or_back(g, s, c, mu);
+    C2<R> b[2][3];
+    U.load_rows01(mu, sb, b);
+    or_back_link<R, ROWS>(U, mu, sb, gx, b);
   }
+  or_transform<R>(G, g.V, s, gx);
 }
 
 template <typename R, int ROWS>
-__global__ void __launch_bounds__(OR_THREADS, 3)
+__global__ void __launch_bounds__(OR_THREADS, ROWS == 3 ? 4 : 3)
 or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, const DevState* __restrict__ st,
                      C2<R>* __restrict__ G, int parity, FastDiv dhx, R omega) {
   // fused FP32 lanes keep their current links in one of two buffers
@@ -274,7 +309,8 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
   if ((int64_t)j >= (g.V >> 1)) return;
   int c[4];
   const int64_t s = or_coords(g, dhx, j, parity, c);
-  or_site<R, ROWS>(g, U, c, s, G, omega);
+  if (ROWS == 3) or_site_reread<R, ROWS>(g, U, c, s, G, omega);
+  else or_site<R, ROWS>(g, U, c, s, G, omega);
 }
 
 // ---------------------------------------------------------------------------
