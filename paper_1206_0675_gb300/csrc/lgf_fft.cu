@@ -602,10 +602,15 @@ cudaError_t configure_fft_plan(const int L[4], int real_bytes, FFTPlan* p) {
   p->fpb_xy = small ? 1 : 4;
   while (p->fpb_xy > 1 && xy_smem(L, real_bytes, p->fpb_xy) > (pairs_xy(real_bytes, 2) && p->fpb_xy == 2 ? maxsm : budget))
     p->fpb_xy /= 2;
-  p->smem_xy = xy_smem(L, real_bytes, p->fpb_xy);
-  if (p->smem_xy > maxsm) return cudaErrorInvalidValue;
   p->smem_c = xy_smem(L, real_bytes, 4);
   p->fuse_g = p->smem_c <= (small ? maxsm : PLANE_SMEM_MAX) ? 1 : 0;
+  // Planes too large for a fused pass C on few slabs: a field per CTA in the
+  // scalar pass, twice as many CTAs.  The three passes, us, pairs -> fields:
+  // 96x96x2x4 57 -> 53, 96x96x4x4 64 -> 58, but 96x96x4x8 65 -> 71.
+  if (!small && !p->fuse_g && p->fpb_xy == 2 && 4 * Lz * Lt <= 152 / 2 && xy_smem(L, real_bytes, 1) <= budget)
+    p->fpb_xy = 1;
+  p->smem_xy = xy_smem(L, real_bytes, p->fpb_xy);
+  if (p->smem_xy > maxsm) return cudaErrorInvalidValue;
   int xc = 1;
   for (int c = small ? 1 : 8; c >= 1; c /= 2) {
     if (Lx % c) continue;
