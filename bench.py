@@ -56,29 +56,31 @@ KERNELS_PER_STEP = {"2d2d": 5, "1d4": 10, "3d1d": 6}
 
 # DRAM bytes (read + write) per launch of the FP64 update kernel at 32^4 from
 # one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum), valid only
-# while the kernel's source text and the shared device header are unchanged
-# (sha256 prefixes); reported as null otherwise.
+# while the kernel's source text and the device headers it is made of are
+# unchanged (sha256 prefixes); reported as null otherwise.
 NCU_TRAFFIC = {
-    "update": {"bytes": 763.063552e6 + 580.143872e6, "source": "update_fx", "kernel_sha": "0a23c84ccdd434a2",
-               "common_sha": "841b0ff160dd5c05"},
+    "update": {"bytes": 764.0768e6 + 588.313856e6, "source": "update_fx", "sha": "f1bcc85b01aa0595"},
 }
 
 
 def kernel_source_sha(name):
-    """sha256 prefix of a kernel's definition text in lgf_site.cu and of lgf_common.cuh."""
+    """sha256 prefix of a kernel's definition text in lgf_site.cu, of lgf_common.cuh and of lgf_fixed.cuh."""
     import hashlib
-    src = open(os.path.join(ROOT, "paper_1206_0675_gb300/csrc/lgf_site.cu")).read()
+    csrc = os.path.join(ROOT, "paper_1206_0675_gb300", "csrc")
+    src = open(os.path.join(csrc, "lgf_site.cu")).read()
     a = src.index(f"{name}_kernel(Geom")
     b = src.index("cudaError_t launch_", a)
-    common = open(os.path.join(ROOT, "paper_1206_0675_gb300/csrc/lgf_common.cuh"), "rb").read()
-    return hashlib.sha256(src[a:b].encode()).hexdigest()[:16], hashlib.sha256(common).hexdigest()[:16]
+    h = hashlib.sha256(src[a:b].encode())
+    for header in ("lgf_common.cuh", "lgf_fixed.cuh"):
+        h.update(open(os.path.join(csrc, header), "rb").read())
+    return h.hexdigest()[:16]
 
 
 def ncu_traffic(kernel):
     rec = NCU_TRAFFIC.get(kernel)
     if rec is None or rec["bytes"] is None:
         return None
-    if kernel_source_sha(rec["source"]) != (rec["kernel_sha"], rec["common_sha"]):
+    if kernel_source_sha(rec["source"]) != rec["sha"]:
         return None
     return rec["bytes"]
 
