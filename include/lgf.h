@@ -78,8 +78,8 @@ typedef enum {
 } lgf_status;
 
 typedef enum {
-  LGF_FP64 = 0,   /* FP64 links, FFTs and updates throughout */
-  LGF_FP32 = 1,   /* FP32 links, Delta and FFTs; FP64 reductions and reunitarisation */
+  LGF_FP64 = 0,   /* FP64 links; divergence, FFTs, g and updates to FP64 accuracy or better */
+  LGF_FP32 = 1,   /* FP32 links, Delta and FFTs; FP64 reductions, reunitarisation factors to 2^-35 */
   LGF_MIXED = 2   /* FP32 phase until theta < switch level, then FP64 rebuilt from the FP64 input */
 } lgf_precision;
 
@@ -443,8 +443,9 @@ lgf_status lgf_get_phase(lgf_handle h, int32_t* bits);
  * memory where they measure -- e.g. a host application whose device memory
  * is owned entirely by its own pool allocator, or monitoring code between
  * the steps of a time-critical loop, where cudaMalloc/cudaFree could fail or
- * synchronise the device.  The computation is the one lgf_measure and
- * lgf_get_divergence perform, without a handle.
+ * synchronise the device.  The quantities are those of lgf_measure and
+ * lgf_get_divergence, without a handle and summed in FP64 throughout (FP64
+ * handles sum links in fixed point: the results agree to rounding).
  * extents: {Lx, Ly, Lz, Lt}, each 2^a 3^b in [2, 128], and at most
  *   LGF_STATIC_MAX_SITES sites in total (else LGF_E_UNSUPPORTED; nothing is
  *   launched).

@@ -27,9 +27,10 @@
 // even, and products carry the mean of what they drop.
 //
 // 32^4, us: pass A 74 (FP64 pipe: 231), pass B 165 (463), pass C with g 113 (397);
-// 24x18x12x27: 24, 41, 33 (54, 94, 78).  Bound by instruction issue (about 400
-// instructions per element of pass A, 800 of pass B) at 24 warps per SM, 80
-// registers a thread (pass B at 96: 151 us at 32^4, but 53 at 24x18x12x27; at
+// 24x18x12x27: 24, 41, 33 (54, 94, 78).  Bound by latency: about 400 instructions
+// per element of pass A, 800 of pass B, at 1.9 to 2.1 a clock and SM of the 4 it
+// can issue; the 13 to 20 warps that are active wait on fixed latencies and on
+// memory.  80 registers a thread (pass B at 96: 151 us at 32^4, but 53 at 24x18x12x27; at
 // 64: 177).
 //
 // Planes that hold infinities or NaN give NaN; planes whose largest

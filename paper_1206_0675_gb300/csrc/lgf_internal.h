@@ -75,7 +75,10 @@ __device__ __forceinline__ bool near_identity(const DevState* st, const Batch& b
 // eight links is what takes the time.  8^4: 22.6 -> 15.8 us with FP64 links,
 // 16.4 -> 12.5 us fused with the update of FP32 links; 16^4: 28.2 -> 32.4 us,
 // 20.1 -> 23.2 us (the lanes' sums have to be added).  With the warps' sums on the
-// integer pipe the 8^4 figures are 14.6 and 11.6 us.
+// integer pipe the 8^4 figures are 14.6 and 11.6 us.  V is that of one lattice,
+// also in a batch: sixteen 8^4 of a launch, which fill the GPU as one 16^4 does,
+// would gain the 4 us of 16^4 with a thread per site, but then a batch would add in
+// another order than single handles, whose results it has bit for bit.
 constexpr int MEASURE_THREADS = 256, MEASURE_SPLIT_THREADS = 128;
 inline bool measure_split(int64_t V) { return V < 152 * 128; }
 inline int64_t measure_blocks(int64_t V) {

@@ -747,7 +747,7 @@ __device__ __noinline__ void update_link_fp64(MatField<double, LROWS> U, MatFiel
 // (FX_WEAK_HI) take FP64 before any arithmetic; links that meet a g in FP64 or
 // have entries outside the fixed-point range take it after.  Error of one update against 64 bits at 32^4, eps = 1: 20 steps
 // end at 2.4e-15 (FP64 products: 2.6e-15).
-// Bound by the integer pipe (1850 instructions a link, 504 of them IMAD.WIDE,
+// Bound by the integer pipe (1780 instructions a link, 504 of them IMAD.WIDE,
 // which run at about 30 of their 64 lanes a clock when all operands vary).
 // 32^4, us: 18-real 379, 12-real 338; with FP64 products 1176 and 1177 at 95 %
 // of the FP64 pipe (fields near the identity: 1191 and 1182).

@@ -57,8 +57,8 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
   __syncthreads();
 }
 
-// The same arithmetic as the handle path's measurement, reading the FP64
-// user layout U[mu][t][z][y][x][3][3][2] directly and writing Delta_A in the
+// The measurement of the handle path in FP64 sums (FP64 lanes sum links in fixed
+// point, so the two agree to rounding), reading the FP64 user layout U[mu][t][z][y][x][3][3][2] directly and writing Delta_A in the
 // site layout D[t][z][y][x][3][3][2].
 __global__ void __launch_bounds__(kThreads)
 measure_aos_kernel(Geom g, const double2* __restrict__ U, double2* __restrict__ D, double* __restrict__ out,
