@@ -26,8 +26,8 @@
 // FxCut.  For that every rounding is centred: inputs are rounded, halves go to
 // even, and products carry the mean of what they drop.
 //
-// 32^4, us: pass A 74 (FP64 pipe: 231), pass B 165 (463), pass C with g 113 (397);
-// 24x18x12x27: 24, 41, 33 (54, 94, 78).  Bound by latency: about 400 instructions
+// 32^4, us: pass A 72 (FP64 pipe: 231), pass B 160 (463), pass C with g 110 (397);
+// 24x18x12x27: 23, 40, 33 (54, 94, 78).  Bound by latency: about 400 instructions
 // per element of pass A, 800 of pass B, at 1.9 to 2.1 a clock and SM of the 4 it
 // can issue; the 13 to 20 warps that are active wait on fixed latencies and on
 // memory.  80 registers a thread (pass B at 96: 151 us at 32^4, but 53 at 24x18x12x27; at
@@ -60,7 +60,12 @@ struct FxPlanes {  // a pass holds up to two transforms
 };
 static_assert(sizeof(FxPlanes) == FX_PLANE_BYTES, "header of the FP64 plane passes");
 
-__device__ __forceinline__ uint32_t fx_headroom(int N) { return 33u - (uint32_t)__clz(N - 1); }
+// ceil(log2 N) + 1
+static uint32_t fx_headroom(int N) {
+  uint32_t h = 1;
+  while ((1 << (h - 1)) < N) ++h;
+  return h;
+}
 
 // The word of a plane after fx_classify: the biased exponent that its input
 // is scaled by and, above bit 16, what was done to a plane out of the ordinary:
@@ -96,11 +101,43 @@ struct FxCut {
   int first;        // stages before the cut (all of them where there is none)
   uint32_t h0, h1;  // headroom of the two parts
 };
-template <bool DIT> __device__ __forceinline__ FxCut fx_cut(const FFTDir& d) {
+static FxCut fx_cut(const FFTDir& d, bool dit) {
   if (d.N <= FX_CUT_ABOVE) return FxCut{d.nst, fx_headroom(d.N), 0u};
   const int q = (int)d.ns[d.nst - 2].d;  // the product of all radices but the last two
   const uint32_t ha = fx_headroom(q), hb = fx_headroom(d.N / q);
-  return DIT ? FxCut{d.nst - 2, ha, hb} : FxCut{2, hb, ha};
+  return dit ? FxCut{d.nst - 2, ha, hb} : FxCut{2, hb, ha};
+}
+
+// The stages of a plane transform in order, made on the host, so that a kernel
+// reads from constant memory what each stage does and keeps no state of its own
+// (registers bound these kernels).  A step: axis, stage of the axis from bit 4,
+// headroom of its part of the direction from bit 8; bit 16: raw FP64 input,
+// scaled by FxTransform::in; from bit 20, m > 0: integers to be shifted by what
+// mid[m - 1] measured; from bit 24, m > 0: record the bits of the outputs in
+// mid[m - 1]; bit 28: the last stage.
+struct FxProgram {
+  int n;
+  uint32_t step[16];
+  uint32_t h[3], h0;  // headroom behind each measurement (0: none), and of the first stages
+};
+static FxProgram fx_program(const FFTDir d[2], int first, bool dit) {
+  FxProgram P{};
+  for (int k = 0; k < 2; ++k) {
+    const int ax = first ^ k;
+    const FxCut c = fx_cut(d[ax], dit);
+    for (int i = 0; i < d[ax].nst; ++i) {
+      const bool start = i == 0, cut = i == c.first, end = i == d[ax].nst - 1;
+      const uint32_t h = i < c.first ? c.h0 : c.h1;
+      const uint32_t shift = cut ? 2 * k + 1 : start && k == 1 ? 2 : 0;
+      const uint32_t mid = end ? (k == 0 ? 2 : 0) : i == c.first - 1 ? 2 * k + 1 : 0;
+      const uint32_t st = (uint32_t)(dit ? i : d[ax].nst - 1 - i);
+      P.step[P.n++] = (uint32_t)ax | st << 4 | h << 8 | (uint32_t)(start && k == 0) << 16 | shift << 20 | mid << 24 |
+                      (uint32_t)(end && k == 1) << 28;
+      if (shift) P.h[shift - 1] = h;
+    }
+    if (k == 0) P.h0 = c.h0;
+  }
+  return P;
 }
 
 __device__ __forceinline__ I2 fx_in(double2 v, uint32_t base) {
@@ -108,14 +145,13 @@ __device__ __forceinline__ I2 fx_in(double2 v, uint32_t base) {
 }
 
 // The word of a plane after its transform: the exponent of its integers (of the
-// scaled plane) and the class of fx_classify.  c0 and c1 are the cuts of its two
-// directions; a part that is not there has no shift.
-__device__ __forceinline__ uint32_t fx_finish(const FxTransform* t, int pl, const FxCut& c0, const FxCut& c1) {
+// scaled plane) and the class of fx_classify.
+__device__ __forceinline__ uint32_t fx_finish(const FxTransform* t, int pl, const FxProgram& P) {
   const uint32_t code = t->in[pl];
-  uint32_t sh = fx_mid_shift(t->mid[1][pl], c1.h0);
-  if (c0.h1 != 0u) sh += fx_mid_shift(t->mid[0][pl], c0.h1);
-  if (c1.h1 != 0u) sh += fx_mid_shift(t->mid[2][pl], c1.h1);
-  return (code & 0xffff0000u) | (sh + c0.h0 + fx_exp_of(code) - 1083u + 4096u);
+  uint32_t sh = fx_mid_shift(t->mid[1][pl], P.h[1]);
+  if (P.h[0] != 0u) sh += fx_mid_shift(t->mid[0][pl], P.h[0]);
+  if (P.h[2] != 0u) sh += fx_mid_shift(t->mid[2][pl], P.h[2]);
+  return (code & 0xffff0000u) | (sh + P.h0 + fx_exp_of(code) - 1083u + 4096u);
 }
 __device__ __forceinline__ int fx_out_exp(uint32_t word) { return (int)(word & 0xffffu) - 4096; }
 // The exponent of the plane as it was, large where it holds infinities or NaN.
@@ -238,20 +274,11 @@ template <int SIGN> struct IDFT<8, SIGN> {
   }
 };
 
-// How a direction's first stage takes its input and its last leaves it.
-struct FxStageIO {
-  FxTransform* t;
-  uint32_t h;     // headroom of this part of the direction
-  bool raw;       // raw FP64 input, scaled by t->in
-  int shift;      // >= 0: integers to be shifted by what t->mid[shift] measured
-  int mid;        // >= 0: record the bits of the outputs in t->mid[mid]
-};
-
-// One stage, as ct_stage of lgf_fft.cu.  The plane of line l is l / inner
+// One stage, as ct_stage of lgf_fft.cu; io: the step of FxProgram.  The plane of line l is l / inner
 // (PLO) or l % inner.
 template <int RAD, int SIGN, bool DIT, bool PLO>
 __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln, const int N, const FastDiv fns,
-                                         const int4* __restrict__ tw, const FxStageIO io) {
+                                         const int4* __restrict__ tw, const uint32_t io, FxTransform* t) {
   const int Ns = (int)fns.d;
   const int nbl = N / RAD;
   const int NB = ln.nlines * nbl;
@@ -264,16 +291,16 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
     const int base = lo * ln.outer_stride + li * ln.inner_stride + (grp * Ns * RAD + j) * ln.es;
     const int step = Ns * ln.es;
     I2 v[RAD];
-    if (io.raw) {
+    if (io & (1u << 16)) {
       const double2* raw = reinterpret_cast<const double2*>(tile);
-      const uint32_t sc = 3u + io.h + fx_exp_of(io.t->in[pl]);
+      const uint32_t sc = 3u + ((io >> 8) & 15u) + fx_exp_of(t->in[pl]);
 #pragma unroll
       for (int r = 0; r < RAD; ++r) v[r] = fx_in(raw[base + r * step], sc);
     } else {
 #pragma unroll
       for (int r = 0; r < RAD; ++r) v[r] = tile[base + r * step];
-      if (io.shift >= 0) {
-        const uint32_t sh = fx_mid_shift(io.t->mid[io.shift][pl], io.h);
+      if (io & (3u << 20)) {
+        const uint32_t sh = fx_mid_shift(t->mid[((io >> 20) & 3u) - 1u][pl], (io >> 8) & 15u);
         if (sh != 0u) {
 #pragma unroll
           for (int r = 0; r < RAD; ++r) v[r] = make_longlong2(ishift(v[r].x, sh), ishift(v[r].y, sh));
@@ -291,8 +318,8 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
     }
 #pragma unroll
     for (int r = 0; r < RAD; ++r) tile[base + r * step] = v[r];
-    if (io.mid >= 0) {
-      uint32_t* mid = io.t->mid[io.mid];
+    if (io & (3u << 24)) {
+      uint32_t* mid = t->mid[((io >> 24) & 3u) - 1u];
       uint32_t m = 0;
 #pragma unroll
       for (int r = 0; r < RAD; ++r) {
@@ -322,48 +349,30 @@ __device__ __forceinline__ void fx_stage(I2* __restrict__ tile, const Lines& ln,
 struct FxPass {
   FFTDir d[2];
   Lines l[2];
+  FxProgram p[2];  // its transforms, in order
 };
 
-// Both directions of a plane transform from raw FP64 input, axis `first` and
-// then the other; DIT takes digit-reversed input and gives natural order, DIF
-// the reverse.  One loop over the directions: the stages of a radix are the
-// same code for both (the instruction cache held neither copy otherwise).
-// Leaves the word of each plane (fx_finish) in t->in; ends with a __syncthreads.
+// Both directions of a plane transform from raw FP64 input; DIT takes
+// digit-reversed input and gives natural order, DIF the reverse.  One loop over
+// the stages of both: those of a radix are the same code (the instruction cache
+// held neither copy otherwise).  Leaves the word of each plane (fx_finish) in
+// t->in; ends with a __syncthreads.
 template <int SIGN, bool DIT, bool PLO>
-__device__ __forceinline__ void fx_plane(I2* tile, const FxPass& P, const int4* tw, int first, int nplanes,
+__device__ __forceinline__ void fx_plane(I2* tile, const FxPass& P, const FxProgram& prog, const int4* tw, int nplanes,
                                          FxTransform* t) {
 #pragma unroll 1
-  for (int k = 0; k < 2; ++k) {
-    const int ax = first ^ k;
+  for (int i = 0; i < prog.n; ++i) {
+    const uint32_t io = prog.step[i];
+    const int ax = (int)(io & 1u), st = (int)(io >> 4) & 15;
     const FFTDir& d = P.d[ax];
     const Lines& ln = P.l[ax];
     const int4* w = ax == 0 ? tw : tw + P.d[0].N;
-    const FxCut cut = fx_cut<DIT>(d);
-    FxStageIO s;
-    s.t = t;
-    s.h = cut.h0;
-    s.raw = k == 0;
-    s.shift = k == 0 ? -1 : 1;
-#pragma unroll 1
-    for (int i = 0; i < d.nst; ++i) {
-      const int st = DIT ? i : d.nst - 1 - i;
-      s.mid = -1;
-      if (i == d.nst - 1) s.mid = k == 0 ? 1 : -1;
-      else if (i == cut.first - 1) s.mid = 2 * k;
-      // every measurement is complete before the last stage
-      if (k == 1 && i == d.nst - 1 && (int)threadIdx.x < nplanes)
-        t->in[threadIdx.x] = fx_finish(t, threadIdx.x, fx_cut<DIT>(P.d[first]), cut);
-      if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
-      else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
-      else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
-      else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, s);
-      s.raw = false;
-      s.shift = -1;
-      if (i == cut.first - 1) {
-        s.shift = 2 * k;
-        s.h = cut.h1;
-      }
-    }
+    // every measurement is complete before the last stage
+    if (io >> 28 && (int)threadIdx.x < nplanes) t->in[threadIdx.x] = fx_finish(t, threadIdx.x, prog);
+    if (d.radix[st] == 8) fx_stage<8, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, io, t);
+    else if (d.radix[st] == 4) fx_stage<4, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, io, t);
+    else if (d.radix[st] == 3) fx_stage<3, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, io, t);
+    else fx_stage<2, SIGN, DIT, PLO>(tile, ln, d.N, d.ns[st], w, io, t);
   }
 }
 
@@ -468,7 +477,7 @@ __global__ void __launch_bounds__(FX_MAX_THREADS, 2) fft_xy_fx_kernel(Geom g, co
       dst);
   __syncthreads();
   const bool odd = fx_prepare(tile, n, fpb, ps->t[0].in, dst);
-  fx_plane<SIGN, true, true>(tile, P, tw, 0, fpb, &ps->t[0]);
+  fx_plane<SIGN, true, true>(tile, P, P.p[0], tw, fpb, &ps->t[0]);
   auto out = [&](auto convert) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const int f = (int)cd.a.div((uint32_t)i), r = i - f * plane, y = (int)cd.b.div((uint32_t)r), x = r - y * Lx;
@@ -518,7 +527,7 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
       dst);
   __syncthreads();
   bool odd = fx_prepare(tile, n, xc, ps->t[0].in, dst);
-  fx_plane<(MODE > 0 ? +1 : -1), true, false>(tile, P, tw, 0, xc, &ps->t[0]);
+  fx_plane<(MODE > 0 ? +1 : -1), true, false>(tile, P, P.p[0], tw, xc, &ps->t[0]);
   if (MODE != 0) {
     auto out = [&](auto convert) {
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -566,7 +575,7 @@ fft_zt_filter_fx_kernel(Geom g, const __grid_constant__ FxPass P, double2* __res
     pl = xi;
     return t * TS + z * xc + xi;
   });
-  fx_plane<+1, false, false>(tile, P, tw, 1, xc, &ps->t[1]);
+  fx_plane<+1, false, false>(tile, P, P.p[1], tw, xc, &ps->t[1]);
   auto out = [&](auto convert) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       LGF_ZT_IDX(i)
@@ -613,7 +622,7 @@ fft_xy_inv_gauge_fx_kernel(Geom g, const __grid_constant__ FxPass P, const doubl
       dst);
   __syncthreads();
   fx_prepare(tile, 4 * plane, 4, ps->t[0].in, dst);
-  fx_plane<+1, false, true>(tile, P, tw, 0, 4, &ps->t[0]);
+  fx_plane<+1, false, true>(tile, P, P.p[0], tw, 4, &ps->t[0]);
   for (int i = threadIdx.x; i < plane; i += blockDim.x) {
     const int y = (int)cd.b.div((uint32_t)i), x = i - y * Lx;
     const int o = pos[Lx + y] * RS + pos[x];
@@ -663,9 +672,11 @@ static const int4* fx_table(const Geom& g, const double2* tw) {
 }
 
 // The (x, y) planes of nf fields side by side in a tile.
-static FxPass xy_pass(const FFTPlan& p, int Lx, int Ly, int nf) {
+static FxPass xy_pass(const FFTPlan& p, int Lx, int Ly, int nf, bool dit) {
   const int RS = Lx + 1, PS = Ly * RS;
-  return FxPass{{p.d[0], p.d[1]}, {make_lines(nf * Ly, Ly, RS, PS, 1), make_lines(nf * Lx, Lx, 1, PS, RS)}};
+  return FxPass{{p.d[0], p.d[1]},
+                {make_lines(nf * Ly, Ly, RS, PS, 1), make_lines(nf * Lx, Lx, 1, PS, RS)},
+                {fx_program(p.d, 0, dit), FxProgram{}}};
 }
 
 template <typename K, typename... Args>
@@ -683,7 +694,7 @@ cudaError_t launch_fft_xy_fx(const Geom& g, const FFTPlan& p, double2* data, con
   const int Lx = g.L[0], Ly = g.L[1];
   const size_t smem = plane_header_bytes(Lx, Ly, 8) + (size_t)fpb * Ly * (Lx + 1) * sizeof(double2);
   const dim3 grid((unsigned)(g.L[2] * g.L[3]), (unsigned)(nfields / fpb), (unsigned)B.n);
-  const FxPass P = xy_pass(p, Lx, Ly, fpb);
+  const FxPass P = xy_pass(p, Lx, Ly, fpb, true);
   const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
   return fx_launch(sign < 0 ? fft_xy_fx_kernel<-1> : fft_xy_fx_kernel<+1>, grid, p.threads_xy, smem, s, g, P, data,
                    fx_table(g, tw), pos, fpb, cd, B);
@@ -696,7 +707,9 @@ cudaError_t launch_fft_zt_fx(const Geom& g, const FFTPlan& p, double2* data, con
   const bool lrn = mode == 0 && (lio.mtab != nullptr || lio.snap != nullptr);
   const int4 H = make_int4(g.L[0] / 2 + 1, g.L[1] / 2 + 1, g.L[2] / 2 + 1, g.L[3] / 2 + 1);
   const int xc = p.xc, Lz = g.L[2], Lt = g.L[3], TS = Lz * xc + 1;
-  const FxPass P{{p.d[2], p.d[3]}, {make_lines(Lt * xc, xc, 1, TS, xc), make_lines(Lz * xc, xc, 1, xc, TS)}};
+  const FxPass P{{p.d[2], p.d[3]},
+                 {make_lines(Lt * xc, xc, 1, TS, xc), make_lines(Lz * xc, xc, 1, xc, TS)},
+                 {fx_program(p.d + 2, 0, true), fx_program(p.d + 2, 1, false)}};
   const CopyDiv cd{FastDiv::make((uint32_t)xc), FastDiv::make((uint32_t)Lz)};
   auto kernel = mode < 0   ? fft_zt_filter_fx_kernel<-1, false>
                 : mode > 0 ? fft_zt_filter_fx_kernel<+1, false>
@@ -709,7 +722,7 @@ cudaError_t launch_xy_inv_gauge_fx(const Geom& g, const FFTPlan& p, const double
                                    const short* pos, double2* gfield, double2* Gfield, const DevState* st,
                                    cudaStream_t s, const Batch& B, bool exact_exp) {
   const int Lx = g.L[0], Ly = g.L[1];
-  const FxPass P = xy_pass(p, Lx, Ly, 4);
+  const FxPass P = xy_pass(p, Lx, Ly, 4, false);
   const CopyDiv cd{FastDiv::make((uint32_t)(Lx * Ly)), FastDiv::make((uint32_t)Lx)};
   const dim3 grid((unsigned)(g.L[2] * g.L[3]), 1, (unsigned)B.n);
   return fx_launch(exact_exp ? fft_xy_inv_gauge_fx_kernel<true> : fft_xy_inv_gauge_fx_kernel<false>, grid, p.threads_c,
