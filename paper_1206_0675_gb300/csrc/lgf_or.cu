@@ -325,8 +325,8 @@ or_half_sweep_kernel(Geom g, C2<R>* __restrict__ U0, C2<R>* __restrict__ U1, con
 // With FP64 arithmetic, one thread a site for all of it, the FP64 pipe was 93 %
 // busy (1199 operations a site and sweep).  One fixed-point kernel with the
 // hits between two barriers left three of four warps waiting for them.
-// A sweep, us (FP64 arithmetic before): 18-real 24^4 335 (724), 32^4 964 (2142),
-// 16^4 79 (168), 8^4 38 (93); 12-real 32^4 811 (2311).  theta of 8^4 levels off
+// A sweep, us (FP64 arithmetic before): 18-real 24^4 329 (724), 32^4 939 (2142),
+// 16^4 79 (168), 8^4 38 (93); 12-real 32^4 804 (2311).  theta of 8^4 levels off
 // (omega = 1.7) at 1.1e-32 (FP64: 1.2e-31) for eps = 0.5, 3.4e-33 (2.8e-32) for 0.25,
 // 3e-33 (6e-33) for 0.12; with operands of w / 64 and of r in [1/4, 1/2) it was
 // 2e-31 for all of them, and a sweep 2 % shorter.  The CTAs per SM are the
@@ -344,17 +344,19 @@ __device__ __forceinline__ int fx_lz4(const int64_t v[4]) {
   return __clzll((long long)mag);
 }
 
-// v / |v| of four integers of any common scale, lz = fx_lz4(v).  The components
-// are shifted until the largest lies in [1/2, 1), where an operand is finest:
-// |v|^2 is then in [1/4, 4) and 1 / (2 |v|) in (1/4, 1].  Every rounding here
-// turns g(x), and theta of a converged field is the square of that.
-__device__ __forceinline__ void fx_unit4(const int64_t v[4], int lz, Fx u[4]) {
+// v / |v| of four integers, lz = fx_lz4(v).  The components are shifted to where
+// an operand is finest, the largest to [1/2, 1) (UP: from below 9/8, which stays
+// as it is; otherwise from [2^59, 2^63) down): |v|^2 is then in [1/4, 5.1) and
+// 1 / (2 |v|) in (1/5, 1].  Every rounding here turns g(x), and theta of a
+// converged field is the square of that.
+template <bool UP> __device__ __forceinline__ void fx_unit4(const int64_t v[4], int lz, Fx u[4]) {
   uint32_t t = 0;
   Fx r[4];
   FxAcc n = fx_zero();
+  const int sh = UP ? max(lz - 4, 0) : 4 - lz;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    r[k] = fx_operand(lz >= 4 ? v[k] << (lz - 4) : (v[k] + ((int64_t)1 << (3 - lz))) >> (4 - lz));
+    r[k] = fx_operand(UP ? v[k] << sh : (v[k] + ((1 << sh) >> 1)) >> sh);
     fx_mac(n, r[k], r[k]);
   }
   const Fx y = fx_operand(fx_half_rsqrt(max(fx_sum60(n, t) >> 2, (int64_t)1 << 56)) >> 1);
@@ -378,8 +380,8 @@ __device__ __forceinline__ void or_subgroup_fx(const FxC& mii, const FxC& mij, c
   const int lz = fx_lz4(v);
   ok = ok && lz <= 24;
   Fx r[4];
-  fx_unit4(v, lz, r);
-  int64_t q[4];  // units of 2^-62
+  fx_unit4<true>(v, lz, r);
+  int64_t q[4];  // units of 2^-62: the largest component is at least 7/32, above 2^59
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     FxAcc p = fx_zero_x4();
@@ -387,7 +389,7 @@ __device__ __forceinline__ void or_subgroup_fx(const FxC& mii, const FxC& mij, c
     fx_mac(p, w7, r[k]);
     q[k] = fx_sum60_x4(p);
   }
-  fx_unit4(q, fx_lz4(q), r);
+  fx_unit4<false>(q, fx_lz4(q), r);
   a = FxC{r[0], r[3]};
   b = FxC{r[2], r[1]};
 }
@@ -456,7 +458,16 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
 #pragma unroll
   for (int e = 0; e < 9; ++e) W[e][0] = W[e][1] = 0;
   uint32_t m = 0, t = 0;
-  bool near_id = false;
+  // before the loop: a way out of it costs the loads' order (32^4 957 -> 939 us a sweep)
+  const bool near_id = __any_sync(
+      0xffffffffu, fx_max(fx_max(fx_max(0u, __ldg(&U.p[U.off(0, 0, 1, s)])), __ldg(&U.p[U.off(0, 0, 2, s)])),
+                          __ldg(&U.p[U.off(0, 1, 2, s)])) < FX_NEAR_HI);
+  if (near_id) {
+    if (!in) return;
+    or_gauge_fp64<ROWS>(g, U, s, gf, omega);
+    if (G != nullptr) accumulate_gauge_fp64(g.V, s, reinterpret_cast<const int4*>(gf) + s, g.V, G);
+    return;
+  }
 #pragma unroll 1
   for (int k = 0; k < 8; ++k) {
     const int mu = k >> 1;
@@ -467,10 +478,6 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
     for (int r = 0; r < ROWS; ++r)
 #pragma unroll
       for (int q = 0; q < 3; ++q) u[r][q] = __ldg(&U.p[U.off(mu, r, q, sl)]);
-    if (k == 0 && __any_sync(0xffffffffu, fx_max(fx_max(fx_max(0u, u[0][1]), u[0][2]), u[1][2]) < FX_NEAR_HI)) {
-      near_id = true;
-      break;
-    }
     int64_t x[3][3][2];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
@@ -507,12 +514,6 @@ or_gauge_fx_kernel(Geom g, MatField<double, ROWS> U, double2* __restrict__ gf, d
         W[e][1] -= x[e % 3][e / 3][1];
       }
     }
-  }
-  if (near_id) {
-    if (!in) return;
-    or_gauge_fp64<ROWS>(g, U, s, gf, omega);
-    if (G != nullptr) accumulate_gauge_fp64(g.V, s, reinterpret_cast<const int4*>(gf) + s, g.V, G);
-    return;
   }
   FxC M[3][3], gx[3][3];
 #pragma unroll
